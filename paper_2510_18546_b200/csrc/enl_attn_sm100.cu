@@ -214,36 +214,42 @@ __device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap *tm, int x, in
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after()  { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-// D[tmem] (+)= A[smem] * B[smem] and D[tmem] (+)= A[tmem] * B[smem].  The whole warp executes the surrounding code
-// and these wrappers; only the lane with `issue` != 0 issues the instruction.  Issuing from inside a one-lane branch
-// was measured at ~60 cycles per MMA (a diverged warp pays the full latency of every instruction and cannot use the
-// uniform datapath for the descriptors), against ~10 cycles this way; the pipe retires an MMA every ~65 cycles.
-// The shared-memory descriptors are given as (low word, high word): the high word is constant and the low word (the
-// start address field) moves by a small constant from one MMA to the next.
+// One lane of the converged warp, chosen by elect.sync.  The choice has to come from that instruction and right where a
+// tcgen05 instruction is issued: the compiler then knows that exactly one thread issues and keeps the operands in uniform
+// registers.  With a predicate of our own (lane == 0) an MMA took 87 cycles to issue and a commit 100, with elect.sync
+// the issue keeps up with the pipe (64): the loop without any softmax work went from 3389 to 2662 cycles per key tile.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(r));
+    return r != 0;
+}
+// D[tmem] (+)= A[smem] * B[smem] and D[tmem] (+)= A[tmem] * B[smem], called by the whole warp.  The shared-memory
+// descriptors are given as (low word, high word): the high word is constant and the low word (the start address field)
+// moves by a small constant from one MMA to the next.
 __device__ __forceinline__ void mma_ss2(uint32_t d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
-                                        uint32_t idesc, uint32_t acc, uint32_t issue)
+                                        uint32_t idesc, uint32_t acc)
 {
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\t"
-        "mov.b64 da, {%1, %2};\n\tmov.b64 db, {%3, %4};\n\tsetp.ne.b32 p, %6, 0;\n\tsetp.ne.b32 q, %7, 0;\n\t"
-        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}"
-        ::"r"(d), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(acc), "r"(issue) : "memory");
+    if (elect_one())
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+            "mov.b64 da, {%1, %2};\n\tmov.b64 db, {%3, %4};\n\tsetp.ne.b32 p, %6, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}"
+            ::"r"(d), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(acc) : "memory");
 }
-__device__ __forceinline__ void mma_ts2(uint32_t d, uint32_t a, uint32_t b_lo, uint32_t b_hi, uint32_t idesc, uint32_t acc,
-                                        uint32_t issue)
+__device__ __forceinline__ void mma_ts2(uint32_t d, uint32_t a, uint32_t b_lo, uint32_t b_hi, uint32_t idesc, uint32_t acc)
 {
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t.reg .b64 db;\n\t"
-        "mov.b64 db, {%2, %3};\n\tsetp.ne.b32 p, %5, 0;\n\tsetp.ne.b32 q, %6, 0;\n\t"
-        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, p;\n\t}"
-        ::"r"(d), "r"(a), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(acc), "r"(issue) : "memory");
+    if (elect_one())
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t.reg .b64 db;\n\t"
+            "mov.b64 db, {%2, %3};\n\tsetp.ne.b32 p, %5, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, p;\n\t}"
+            ::"r"(d), "r"(a), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(acc) : "memory");
 }
-__device__ __forceinline__ void tc_commit_if(uint32_t bar, uint32_t issue)
+__device__ __forceinline__ void tc_commit(uint32_t bar)
 {
-    asm volatile(
-        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
-        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
-        ::"r"(bar), "r"(issue) : "memory");
+    if (elect_one())
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ float ex2(float x)
 {
@@ -493,7 +499,6 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
             const uint32_t dk_lo = static_cast<uint32_t>(dk0), dk_hi = static_cast<uint32_t>(dk0 >> 32);
             const uint32_t dv_lo = static_cast<uint32_t>(dv0), dv_hi = static_cast<uint32_t>(dv0 >> 32);
             constexpr uint32_t kTileUnits = C::kTileBytes >> 4;
-            const uint32_t issue = lane == 0 ? 1u : 0u;
             auto issue_qk = [&](int i, int st) {
                 const uint32_t a = dq_lo + static_cast<uint32_t>(i) * kTileUnits, b = dk_lo + static_cast<uint32_t>(st) * kTileUnits;
                 const uint32_t d = tmem_s(i);
@@ -501,9 +506,9 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                 for (int kk = 0; kk < D / 16; ++kk) {
                     constexpr uint32_t kHalfUnits = C::kHalfBytes >> 4;
                     const uint32_t off = static_cast<uint32_t>((kk >> 2) * kHalfUnits + (kk & 3) * 2);   // 32 bytes per 16 channels
-                    mma_ss2(d, a + off, dq_hi, b + off, dk_hi, idesc_qk, kk > 0 ? 1u : 0u, issue);
+                    mma_ss2(d, a + off, dq_hi, b + off, dk_hi, idesc_qk, kk > 0 ? 1u : 0u);
                 }
-                tc_commit_if(bar_s_full(i), issue);
+                tc_commit(bar_s_full(i));
             };
             // O_i (+)= P_i[:, 64 hf .. 64 hf + 63] V[64 hf .. 64 hf + 63, :]; P of keys 2c, 2c+1 sits in column c of S_i
             auto issue_pv = [&](int i, int st, int hf, bool first_tile) {
@@ -512,9 +517,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
 #pragma unroll
                 for (int k4 = 0; k4 < 4; ++k4)                          // 16 keys = 16 rows of 128 B = 128 address units, 8 columns of P
                     mma_ts2(d, a + static_cast<uint32_t>(k4 * 8), b + static_cast<uint32_t>(k4 * 128), dv_hi, idesc_pv,
-                            (first_tile && hf == 0 && k4 == 0) ? 0u : 1u, issue);
+                            (first_tile && hf == 0 && k4 == 0) ? 0u : 1u);
             };
-            auto commit_to = [&](uint32_t bar) { tc_commit_if(bar, issue); };
             auto wait_full = [&](int f) {
                 return mbar_wait(bar_kv_full(f % C::kStages), static_cast<uint32_t>((f / C::kStages) & 1),
                                  abort_flag, p.status);
@@ -536,7 +540,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
             if (ok) {
                 tc_fence_after();
                 for (int i = 0; i < n_qt; ++i) issue_qk(i, 0);
-                commit_to(bar_kv_empty(0));
+                tc_commit(bar_kv_empty(0));
             }
             Pending w_v = arm(full_bar(1), full_par(1));                // V of the first tile
             Pending w_p = arm(bar_p_half(0, 0), 0u);                    // first half of P_0
@@ -559,8 +563,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                     if (more && i == 0) w_k = arm(full_bar(fk), full_par(fk));
                     if (!more && !last_i) w_p = arm(bar_p_half(i + 1, 0), par);
                     issue_pv(i, fv % C::kStages, 1, false);
-                    if (last_i) commit_to(bar_kv_empty(fv % C::kStages));
-                    if (!more) commit_to(bar_o_done(i));
+                    if (last_i) tc_commit(bar_kv_empty(fv % C::kStages));
+                    if (!more) tc_commit(bar_o_done(i));
                     if (more) {
                         ok = await(w_k);
                         if (!ok) break;
@@ -573,7 +577,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                             w_p = arm(bar_p_half(0, 0), par ^ 1u);
                         }
                         issue_qk(i, fk % C::kStages);
-                        if (last_i) commit_to(bar_kv_empty(fk % C::kStages));
+                        if (last_i) tc_commit(bar_kv_empty(fk % C::kStages));
                     }
                 }
             }
