@@ -4,6 +4,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <cstring>
 
 #include "enl_internal.h"
 
@@ -200,7 +201,47 @@ __global__ void page_copy_kernel(const uint8_t *src_k, const uint8_t *src_v, uin
         *reinterpret_cast<uint4 *>(d + i) = *reinterpret_cast<const uint4 *>(s + i);
 }
 
+// The gather plan as kernel parameters -> device memory.  It waits for the kernel before (which may read the previous plan
+// in the same place) and does not let its successor start early: the successor reads the plan in its set-up.
+template <int kBytes>
+struct PlanBlob {
+    uint4 *dst;
+    int32_t n;                                              // 16-byte words
+    int32_t pad;
+    uint4 data[kBytes / 16];
+};
+template <int kBytes>
+__global__ void __launch_bounds__(128) plan_write_kernel(const __grid_constant__ PlanBlob<kBytes> p)
+{
+    const int i = blockIdx.x * 128 + threadIdx.x;
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (i < p.n) v = p.data[i];
+    pdl_wait();
+    if (i < p.n) p.dst[i] = v;
+}
+
+template <int kBytes>
+cudaError_t plan_write(void *dst, const void *src, size_t bytes, cudaStream_t st)
+{
+    static thread_local PlanBlob<kBytes> blob;              // too large for the stack of every caller
+    blob.dst = static_cast<uint4 *>(dst);
+    blob.n = static_cast<int32_t>((bytes + 15) / 16);
+    std::memcpy(blob.data, src, bytes);
+    return launch_pdl(plan_write_kernel<kBytes>, dim3((blob.n + 127) / 128), dim3(128), 0, st, blob);
+}
+
 }  // namespace
+
+// Three sizes: what a launch costs grows with the parameters it carries.
+cudaError_t launch_plan_write(void *dst, const void *src, size_t bytes, cudaStream_t st)
+{
+    if (bytes == 0) return cudaSuccess;
+    if (bytes > kPlanParamBytes) return cudaErrorInvalidValue;
+    const cudaError_t e = bytes <= 2048   ? plan_write<2048>(dst, src, bytes, st)
+                          : bytes <= 8192 ? plan_write<8192>(dst, src, bytes, st)
+                                          : plan_write<kPlanParamBytes>(dst, src, bytes, st);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
 
 cudaError_t launch_page_copy(const uint8_t *src_k, const uint8_t *src_v, uint8_t *dst_k, uint8_t *dst_v,
                              size_t src_layer_bytes, size_t dst_layer_bytes, const int2 *pairs, int n_pairs,

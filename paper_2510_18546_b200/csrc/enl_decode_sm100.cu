@@ -219,6 +219,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(const __grid_consta
     auto bar_full = [&](int s) { return bar0 + 8u * (warp * kStages + s); };
     auto stage_addr = [&](int s) { return sbase + static_cast<uint32_t>((warp * kStages + s) * C::kStageBytes); };
 
+    if (p.fresh_plan) pdl_wait();
     // grid = (splits, kv heads, episodes); a single episode travels in the parameters
     struct { int ep, kvh, split; } it = {static_cast<int>(blockIdx.z), static_cast<int>(blockIdx.y), static_cast<int>(blockIdx.x)};
     EpInfo ep;

@@ -89,17 +89,20 @@ struct MapCache {
     MapKey key[kSlots] = {};
     CUtensorMap map[kSlots];
     bool used[kSlots] = {};
+    uint32_t turn = 0;
     // 3-D bf16 map [d2][d1][d0] with box {b0, b1, b2}
     bool get(CUtensorMap *out, const void *base, const cuuint64_t *dims, const cuuint64_t *strides, const cuuint32_t *box)
     {
         const MapKey k{base, dims[0], dims[1], dims[2], box[0], box[1], box[2]};
         const size_t h = (reinterpret_cast<uintptr_t>(base) >> 8) * 0x9E3779B97F4A7C15ull >> 56;
+        int victim = -1;                                    // the same tensor with another length (decoding), else a free slot
         for (int probe = 0; probe < 4; ++probe) {
             const int i = static_cast<int>((h + probe) % kSlots);
             if (used[i] && key[i] == k) { *out = map[i]; return true; }
+            if (victim < 0 && (!used[i] || key[i].base == base)) victim = i;
         }
         if (!encode_map(out, base, 3, dims, strides, box)) return false;
-        const int i = static_cast<int>(h % kSlots);
+        const int i = victim >= 0 ? victim : static_cast<int>((h + (turn++ & 3u)) % kSlots);
         key[i] = k;
         map[i] = *out;
         used[i] = true;
@@ -125,9 +128,14 @@ struct enl_cache {
     // gather plan: host image (pinned when there is a GPU), device copy, capacities
     int32_t cap_entries = 0, cap_items = 0;
     uint8_t *plan_host = nullptr, *plan_dev = nullptr;
-    size_t off_eps = 0, off_items = 0, off_stream = 0, off_meta = 0, off_rowslots = 0, off_rowobj = 0, plan_bytes = 0;
+    // sections of the current plan, back to back in the order of their offsets
+    size_t off_eps = 0, off_items = 0, off_stream = 0, off_meta = 0, off_rowslots = 0, off_rowobj = 0, plan_used = 0;
+    size_t plan_bytes = 0;                  // capacity
     cudaEvent_t plan_copied = nullptr;
+    bool plan_copying = false;              // a copy out of plan_host may be under way (until plan_copied)
     bool plan_valid = false, plan_on_device = false;
+    std::vector<uint8_t> plan_layer_ok;     // layers whose group lengths have been compared with the plan's
+    std::vector<int32_t> sel_len;           // working space of a call
     uint64_t plan_epoch = 0;
     int32_t plan_split_hint = 0;
     bool plan_has_mass = false;
@@ -251,13 +259,9 @@ extern "C" int enl_cache_create(const enl_cache_desc_t *desc, enl_cache_t **out)
     c->cap_entries = static_cast<int32_t>(std::min<int64_t>(2 * c->n_pages + kPagesPerTile * (d.max_batch + 1), 0x7ffffff0));
     c->cap_items = std::max(4096, (d.max_q_tokens / tpc + d.max_batch + 1) * d.n_kv_heads);
     auto align256 = [](size_t x) { return (x + 255) & ~static_cast<size_t>(255); };
-    c->off_eps = 0;
-    c->off_items = align256(c->off_eps + sizeof(EpInfo) * d.max_batch);
-    c->off_stream = align256(c->off_items + sizeof(Item) * c->cap_items);
-    c->off_meta = align256(c->off_stream + sizeof(int32_t) * c->cap_entries);
-    c->off_rowslots = align256(c->off_meta + sizeof(int32_t) * c->cap_entries);
-    c->off_rowobj = align256(c->off_rowslots + sizeof(int32_t) * d.max_q_tokens);
-    c->plan_bytes = align256(c->off_rowobj + sizeof(int32_t) * d.max_q_tokens);
+    c->plan_bytes = align256(sizeof(EpInfo) * d.max_batch) + align256(sizeof(Item) * c->cap_items) +
+                    2 * align256(sizeof(int32_t) * c->cap_entries) + 2 * align256(sizeof(int32_t) * d.max_q_tokens);
+    c->plan_layer_ok.assign(d.n_layers, 0);
 
     if (!c->gpu) {
         c->plan_host = new (std::nothrow) uint8_t[c->plan_bytes];
@@ -543,46 +547,51 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
     }
     const bool direct = has_sum || mass_only;       // these results leave the attention kernel itself: no KV splits
 
+    // ---- gather plan: reuse when nothing it was built from has changed ----
+    const bool has_mass = a->group_mass != nullptr;
+    const size_t cu_bytes = sizeof(int32_t) * (B + 1);
+    const bool same_obj = has_sum ? c->key_obj.size() == static_cast<size_t>(a->n_obj) + 1 &&
+                                        std::memcmp(c->key_obj.data(), a->obj_off, sizeof(int32_t) * (a->n_obj + 1)) == 0
+                                  : true;
+    bool reuse = c->plan_valid && c->plan_epoch == c->epoch && c->plan_split_hint == a->split_hint &&
+                 c->plan_has_mass == has_mass && c->plan_direct == direct && same_obj && c->plan_batch == B &&
+                 c->key_sel.size() == static_cast<size_t>(a->n_sel) &&
+                 (a->n_sel == 0 || std::memcmp(c->key_sel.data(), a->sel_ids, sizeof(int32_t) * a->n_sel) == 0) &&
+                 std::memcmp(c->key_cu.data(), cu_sel, cu_bytes) == 0 &&
+                 std::memcmp(c->key_cu.data() + B + 1, cu_q, cu_bytes) == 0 &&
+                 std::memcmp(c->key_cu.data() + 2 * (B + 1), cu_new, cu_bytes) == 0;
+
     // ---- select list: ids, duplicates, lengths (Sec. 3.4: a group is selected at most once) ----
-    std::vector<int32_t> sel_len(a->n_sel);
-    for (int b = 0; b < B; ++b) {
-        if (++c->stamp == 0x7fffffff) { std::fill(c->seen.begin(), c->seen.end(), 0); c->stamp = 1; }
-        for (int s = cu_sel[b]; s < cu_sel[b + 1]; ++s) {
-            const int32_t gid = a->sel_ids[s];
-            if (gid < 0 || gid >= d.max_groups) return ENL_E_NOGROUP;
-            const Group &g = c->groups[gid];
-            if (g.len.empty() || g.len[a->layer] < 0) return ENL_E_NOGROUP;
-            if (!g.resident) return ENL_E_EVICTED;
-            if (c->seen[gid] == c->stamp) return ENL_E_INVAL;
-            c->seen[gid] = c->stamp;
-            sel_len[s] = g.len[a->layer];
+    // The plan's own list at the plan's own epoch has been looked over; a layer it has not been used for yet may hold
+    // the groups at other lengths.
+    std::vector<int32_t> &sel_len = c->sel_len;
+    if (!reuse || !c->plan_layer_ok[a->layer]) {
+        sel_len.resize(a->n_sel);
+        for (int b = 0; b < B; ++b) {
+            if (++c->stamp == 0x7fffffff) { std::fill(c->seen.begin(), c->seen.end(), 0); c->stamp = 1; }
+            for (int s = cu_sel[b]; s < cu_sel[b + 1]; ++s) {
+                const int32_t gid = a->sel_ids[s];
+                if (gid < 0 || gid >= d.max_groups) return ENL_E_NOGROUP;
+                const Group &g = c->groups[gid];
+                if (g.len.empty() || g.len[a->layer] < 0) return ENL_E_NOGROUP;
+                if (!g.resident) return ENL_E_EVICTED;
+                if (c->seen[gid] == c->stamp) return ENL_E_INVAL;
+                c->seen[gid] = c->stamp;
+                sel_len[s] = g.len[a->layer];
+            }
         }
+        reuse = reuse && c->key_len == sel_len;
+        if (reuse) c->plan_layer_ok[a->layer] = 1;
     }
     if (a->sel_off_out) {
+        const std::vector<int32_t> &lens = reuse ? c->key_len : sel_len;
         int32_t *o = a->sel_off_out;
         for (int b = 0; b < B; ++b) {
             int32_t acc = 0;
             *o++ = 0;
-            for (int s = cu_sel[b]; s < cu_sel[b + 1]; ++s) { acc += sel_len[s]; *o++ = acc; }
+            for (int s = cu_sel[b]; s < cu_sel[b + 1]; ++s) { acc += lens[s]; *o++ = acc; }
         }
     }
-
-    // ---- gather plan: reuse when nothing it was built from has changed ----
-    std::vector<int32_t> cu_key;
-    cu_key.reserve(3 * (B + 1));
-    cu_key.insert(cu_key.end(), cu_sel, cu_sel + B + 1);
-    cu_key.insert(cu_key.end(), cu_q, cu_q + B + 1);
-    cu_key.insert(cu_key.end(), cu_new, cu_new + B + 1);
-    const bool has_mass = a->group_mass != nullptr;
-    bool same_obj = !has_sum;
-    if (has_sum)
-        same_obj = c->key_obj.size() == static_cast<size_t>(a->n_obj) + 1 &&
-                   std::memcmp(c->key_obj.data(), a->obj_off, sizeof(int32_t) * (a->n_obj + 1)) == 0;
-    const bool reuse = c->plan_valid && c->plan_epoch == c->epoch && c->plan_split_hint == a->split_hint &&
-                       c->plan_has_mass == has_mass && c->plan_direct == direct && same_obj &&
-                       c->key_cu == cu_key && c->key_len == sel_len &&
-                       c->key_sel.size() == static_cast<size_t>(a->n_sel) &&
-                       (a->n_sel == 0 || std::memcmp(c->key_sel.data(), a->sel_ids, sizeof(int32_t) * a->n_sel) == 0);
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     DeviceGuard dg(c->gpu ? d.device : -1);
 
@@ -642,8 +651,28 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
             while (n_splits > 1 && !fits(n_splits)) --n_splits;
         }
 
-        if (c->gpu && cudaEventSynchronize(c->plan_copied) != cudaSuccess) { cudaGetLastError(); return ENL_E_CUDA; }
+        if (c->plan_copying) {
+            if (cudaEventSynchronize(c->plan_copied) != cudaSuccess) { cudaGetLastError(); return ENL_E_CUDA; }
+            c->plan_copying = false;
+        }
         c->plan_valid = false;
+        // Two splits of a head_dim-128 call are launched as clusters of two CTAs, which exchange their partial
+        // results through distributed shared memory: no scratch round trip and no merge kernel.  Every CTA must
+        // have at least one tile, and the items of a pair must be neighbours (they are: same tile count, stable sort).
+        const bool pair = !decode && n_splits == 2 && d.head_dim == 128 && min_tiles >= 2 && (c->pairs_ok || !c->gpu);
+        const int64_t n_items = decode ? static_cast<int64_t>(B) * d.n_kv_heads * n_splits : base_items * n_splits;
+        {   // sections: what the kernels of this plan read (the decode kernel takes its CTA's place from the grid)
+            auto align16 = [](size_t x) { return (x + 15) & ~static_cast<size_t>(15); };
+            size_t at = 0;
+            auto section = [&](size_t bytes) { const size_t o = at; at += align16(bytes); return o; };
+            c->off_eps = section(sizeof(EpInfo) * B);
+            c->off_items = section(decode ? 0 : sizeof(Item) * n_items);
+            c->off_stream = section(sizeof(int32_t) * n_entries);
+            c->off_meta = section(sizeof(int32_t) * n_entries);
+            c->off_rowslots = section(!decode && n_splits > 1 && !pair ? sizeof(int32_t) * a->n_q : 0);
+            c->off_rowobj = section(has_sum ? sizeof(int32_t) * a->n_q : 0);
+            c->plan_used = at;
+        }
         EpInfo *eps = c->h_eps();
         int32_t *stream = c->h_stream();
         int32_t *smeta = c->h_meta();
@@ -671,7 +700,8 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
             }
             while ((ne - e.stream_off) % kPagesPerTile) { stream[ne] = kZeroPage; smeta[ne++] = (e.n_slots - 1) << 8; }
             e.n_ctiles = (ne - e.stream_off) / kPagesPerTile;
-            for (int r = e.q_off; r < e.q_off + e.n_q; ++r) rowslots[r] = e.n_slots;
+            if (!decode && n_splits > 1 && !pair)
+                for (int r = e.q_off; r < e.q_off + e.n_q; ++r) rowslots[r] = e.n_slots;
         }
         if (has_sum) {
             int32_t *rowobj = c->h_rowobj();
@@ -682,28 +712,27 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         } else {
             c->key_obj.clear();
         }
-        // CTAs, heaviest first (late token blocks see more new-token tiles)
-        struct Work { Item it; int tiles; };
-        std::vector<Work> work;
-        work.reserve(static_cast<size_t>(base_items) * n_splits);
-        for (int b = 0; b < B && decode; ++b)
-            for (int h = 0; h < d.n_kv_heads; ++h)
-                for (int sp = 0; sp < n_splits; ++sp) work.push_back({Item{b, h, 0, sp}, eps[b].n_ctiles});
-        for (int b = 0; b < B && !decode; ++b) {
-            const EpInfo &e = eps[b];
-            for (int t0 = 0; t0 < e.n_q; t0 += tpc) {
-                const int t_hi = std::min(t0 + tpc, e.n_q);
-                const int tiles = e.n_ctiles + (e.n_new - e.n_q + t_hi - 1) / kTileKeys + 1;
-                for (int h = 0; h < d.n_kv_heads; ++h)
-                    for (int sp = 0; sp < n_splits; ++sp) work.push_back({Item{b, h, t0, sp}, tiles});
+        if (!decode) {
+            // CTAs, heaviest first (late token blocks see more new-token tiles)
+            struct Work { Item it; int tiles; };
+            std::vector<Work> work;
+            work.reserve(static_cast<size_t>(n_items));
+            for (int b = 0; b < B; ++b) {
+                const EpInfo &e = eps[b];
+                for (int t0 = 0; t0 < e.n_q; t0 += tpc) {
+                    const int t_hi = std::min(t0 + tpc, e.n_q);
+                    const int tiles = e.n_ctiles + (e.n_new - e.n_q + t_hi - 1) / kTileKeys + 1;
+                    for (int h = 0; h < d.n_kv_heads; ++h)
+                        for (int sp = 0; sp < n_splits; ++sp) work.push_back({Item{b, h, t0, sp}, tiles});
+                }
             }
+            std::stable_sort(work.begin(), work.end(), [](const Work &x, const Work &y) { return x.tiles > y.tiles; });
+            Item *items = c->h_items();
+            for (size_t i = 0; i < work.size(); ++i) items[i] = work[i].it;
         }
-        std::stable_sort(work.begin(), work.end(), [](const Work &x, const Work &y) { return x.tiles > y.tiles; });
-        Item *items = c->h_items();
-        for (size_t i = 0; i < work.size(); ++i) items[i] = work[i].it;
 
         c->plan_entries = ne;
-        c->plan_items = static_cast<int32_t>(work.size());
+        c->plan_items = static_cast<int32_t>(n_items);
         c->plan_splits = n_splits;
         c->plan_batch = B;
         c->plan_max_slots = max_slots;
@@ -712,32 +741,31 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         c->plan_has_mass = has_mass;
         c->plan_direct = direct;
         c->plan_decode = decode;
-        // Two splits of a head_dim-128 call are launched as clusters of two CTAs, which exchange their partial
-        // results through distributed shared memory: no scratch round trip and no merge kernel.  Every CTA must
-        // have at least one tile, and the items of a pair must be neighbours (they are: same tile count, stable sort).
-        c->plan_pair = !decode && n_splits == 2 && d.head_dim == 128 && min_tiles >= 2 && (c->pairs_ok || !c->gpu);
+        c->plan_pair = pair;
         c->key_sel.assign(a->sel_ids, a->sel_ids + a->n_sel);
-        c->key_cu = cu_key;
+        c->key_cu.assign(cu_sel, cu_sel + B + 1);
+        c->key_cu.insert(c->key_cu.end(), cu_q, cu_q + B + 1);
+        c->key_cu.insert(c->key_cu.end(), cu_new, cu_new + B + 1);
         c->key_len = sel_len;
+        std::fill(c->plan_layer_ok.begin(), c->plan_layer_ok.end(), 0);
+        c->plan_layer_ok[a->layer] = 1;
         c->plan_valid = true;
         c->plan_on_device = false;
     }
     if (plan_only) return ENL_OK;
 
-    if (!c->plan_on_device) {
-        // one copy covers episodes, items, stream and row->slots (unused gaps travel too; they are small)
-        const size_t ent_bytes = sizeof(int32_t) * c->plan_entries;
-        bool okc = cudaMemcpyAsync(c->plan_dev, c->plan_host, c->off_stream, cudaMemcpyHostToDevice, st) == cudaSuccess &&
-                   (ent_bytes == 0 ||
-                    (cudaMemcpyAsync(c->plan_dev + c->off_stream, c->plan_host + c->off_stream, ent_bytes,
-                                     cudaMemcpyHostToDevice, st) == cudaSuccess &&
-                     cudaMemcpyAsync(c->plan_dev + c->off_meta, c->plan_host + c->off_meta, ent_bytes,
-                                     cudaMemcpyHostToDevice, st) == cudaSuccess)) &&
-                   cudaMemcpyAsync(c->plan_dev + c->off_rowslots, c->plan_host + c->off_rowslots,
-                                   sizeof(int32_t) * a->n_q, cudaMemcpyHostToDevice, st) == cudaSuccess &&
-                   (!has_sum || cudaMemcpyAsync(c->plan_dev + c->off_rowobj, c->plan_host + c->off_rowobj,
-                                                sizeof(int32_t) * a->n_q, cudaMemcpyHostToDevice, st) == cudaSuccess) &&
-                   cudaEventRecord(c->plan_copied, st) == cudaSuccess;
+    // The plan goes to the device with the first launch that uses it: as parameters of a small kernel, or, when it is too
+    // large for that (beyond some 3500 pages of 16 tokens), as one copy, before which this buffer must not be rebuilt.
+    const bool fresh = !c->plan_on_device;
+    if (fresh) {
+        bool okc;
+        if (c->plan_used <= static_cast<size_t>(kPlanParamBytes)) {
+            okc = launch_plan_write(c->plan_dev, c->plan_host, c->plan_used, st) == cudaSuccess;
+        } else {
+            okc = cudaMemcpyAsync(c->plan_dev, c->plan_host, c->plan_used, cudaMemcpyHostToDevice, st) == cudaSuccess &&
+                  cudaEventRecord(c->plan_copied, st) == cudaSuccess;
+            c->plan_copying = true;
+        }
         if (!okc) { cudaGetLastError(); c->plan_valid = false; return ENL_E_CUDA; }
         c->plan_on_device = true;
     }
@@ -779,6 +807,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         dp.slot_stride = slot_stride;
         dp.mass_stride = a->mass_stride;
         dp.n_splits = c->plan_splits;
+        dp.fresh_plan = fresh ? 1 : 0;
         dp.scale_log2 = 1.4426950408889634f / sqrtf(static_cast<float>(d.head_dim));
         if (launch_decode(dp, d.head_dim, c->plan_batch, st) != cudaSuccess) { cudaGetLastError(); return ENL_E_CUDA; }
         return ENL_OK;
@@ -823,6 +852,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
     p.sum_stride = a->sum_stride;
     p.mass_only = mass_only ? 1 : 0;
     p.first_wave = c->n_sm;
+    p.fresh_plan = fresh ? 1 : 0;
     const bool scratch_merge = p.n_splits > 1 && !c->plan_pair;
     if (scratch_merge) {
         const size_t rows = static_cast<size_t>(p.n_splits) * a->n_q * d.n_q_heads;

@@ -59,6 +59,7 @@ struct AttnParams {
     const int32_t *row_obj; // [n_q_total]: object of every query row, -1 = none (only with mass_sum)
     int32_t sum_stride;
     int32_t mass_only;      // 1: the output rows are not written
+    int32_t fresh_plan;     // 1: the kernel before wrote the gather plan, wait for it before the plan is read
     int32_t first_wave;     // CTAs that start while the previous kernel of the stream may still run (the number of SMs)
 };
 
@@ -88,6 +89,7 @@ struct DecodeParams {
     int32_t slot_stride;    // row stride of part_slot
     int32_t mass_stride;    // row stride of mass
     int32_t n_splits;
+    int32_t fresh_plan;     // as in AttnParams
     float   scale_log2;
 };
 
@@ -129,7 +131,8 @@ inline cudaError_t launch_pdl(Kernel kernel, dim3 grid, dim3 block, size_t smem,
         attr[1].val.clusterDim.z = 1;
         cfg.numAttrs = 2;
     }
-    return cudaLaunchKernelEx(&cfg, kernel, prm);
+    void *args[1] = {const_cast<Params *>(&prm)};           // not the typed form: that copies the parameters once more
+    return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void *>(kernel), args);
 }
 // the same for kernels that take several plain arguments
 template <typename... KArgs, typename... Args>
@@ -179,6 +182,10 @@ cudaError_t launch_page_scatter_layers(void *kpool, void *vpool, size_t layer_by
 cudaError_t launch_page_copy(const uint8_t *src_k, const uint8_t *src_v, uint8_t *dst_k, uint8_t *dst_v,
                              size_t src_layer_bytes, size_t dst_layer_bytes, const int2 *pairs, int n_pairs,
                              int n_layers, int page_bytes, cudaStream_t st);
+// Writes a gather plan of up to kPlanParamBytes to device memory out of the kernel's own parameters: no staging buffer
+// that the host would have to wait for, and (unlike a copy) it chains to its neighbours by programmatic dependent launch.
+constexpr int kPlanParamBytes = 28672;        // of the 32764 that a launch may carry
+cudaError_t launch_plan_write(void *dst, const void *src, size_t bytes, cudaStream_t st);
 size_t attention_smem_bytes(int head_dim);
 // Opts the attention kernel into its dynamic shared memory size on the current device.
 cudaError_t prepare_attention(int head_dim);

@@ -1,4 +1,5 @@
-"""Thin ctypes binding over ``libenl.so``: same names as the C ABI, argument marshalling only.
+"""Thin binding over ``libenl.so``: same names as the C ABI, argument marshalling only.  The calls made per layer or per
+group go through ``_enl.so`` (their marshalling in C), the others through ctypes.
 
 Every step of the path (page scatter, gather plan upload, attention, split merge) runs inside the
 library; nothing here computes.  There is no fallback: if the library is missing, loading raises.
@@ -72,6 +73,7 @@ class EnlError(RuntimeError):
 
 
 _lib = None
+_native = None          # the _enl extension module
 _n_layers = {}          # cache handle -> layer count (the all-layers store takes one pointer per layer)
 
 
@@ -131,6 +133,17 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+def _binding():
+    """The extension module (raises ImportError if it has not been built: there is no other path)."""
+    global _native
+    if _native is None:
+        lib()
+        from . import _enl
+        _enl.set_int32_converter(_i32)
+        _native = _enl
+    return _native
+
+
 def strerror(code: int) -> str:
     return lib().enl_strerror(int(code)).decode()
 
@@ -164,8 +177,7 @@ def enl_cache_create(n_layers: int, n_q_heads: int, n_kv_heads: int, head_dim: i
 def enl_group_store(cache: int, group_id: int, layer: int, k, v, mode: int = ENL_REPLACE,
                     stream: int = 0, n_tokens: Optional[int] = None) -> None:
     """``k``/``v``: ``[n, Hkv, D]`` bf16 CUDA tensors (or None with ``n_tokens`` on a bookkeeping cache)."""
-    n = int(k.shape[0]) if k is not None else int(n_tokens)
-    rc = lib().enl_group_store(cache, group_id, layer, n, _ptr(k), _ptr(v), mode, stream or None)
+    rc = (_native or _binding()).store(cache, group_id, layer, n_tokens, k, v, mode, stream or None)
     if rc != ENL_OK:
         raise EnlError(rc, "enl_group_store")
 
@@ -175,17 +187,12 @@ def enl_group_store_all_layers(cache: int, group_id: int, ks, vs, mode: int = EN
     """``ks``/``vs``: one ``[n, Hkv, D]`` bf16 CUDA tensor per layer (or None with ``n_tokens`` on a bookkeeping
     cache).  Every layer of the group is written by one launch."""
     if ks is None:
-        n, kp, vp = int(n_tokens), None, None
+        rc = lib().enl_group_store_all_layers(cache, group_id, int(n_tokens), None, None, mode, stream or None)
     else:
-        n = int(ks[0].shape[0])
-        if any(int(t.shape[0]) != n for t in list(ks) + list(vs)):
-            raise ValueError("every layer must bring the same number of rows")
-        n_layers = _n_layers.get(int(cache), n_layers)
+        n_layers = _n_layers.get(cache, n_layers)
         if n_layers is not None and (len(ks) != n_layers or len(vs) != n_layers):
             raise ValueError("one K and one V tensor per layer of the cache")
-        kp = (ctypes.c_void_p * len(ks))(*[_ptr(t) for t in ks])
-        vp = (ctypes.c_void_p * len(vs))(*[_ptr(t) for t in vs])
-    rc = lib().enl_group_store_all_layers(cache, group_id, n, kp, vp, mode, stream or None)
+        rc = (_native or _binding()).store_all_layers(cache, group_id, ks, vs, mode, stream or None)
     if rc != ENL_OK:
         raise EnlError(rc, "enl_group_store_all_layers")
 
@@ -197,31 +204,18 @@ def enl_attend(cache: int, layer: int, sel_ids: Sequence[int], q, k_new, v_new, 
     """One attend call.  Returns ``sel_off`` (numpy int32 ``[n_sel + batch]``) when asked, else None.
     ``group_mass_sum``: fp32 CUDA tensor ``[n_obj, stride]`` the call adds per-object mass sums to, with
     ``obj_off`` the ``n_obj + 1`` row offsets of the objects."""
-    sel = _i32(sel_ids)
-    cs, cq, cn = _i32(cu_sel), _i32(cu_q), _i32(cu_new)
-    batch = 1 if cq is None else len(cq) - 1
-    nq = int(n_q) if n_q is not None else int(q.shape[0])
-    nn = int(n_new) if n_new is not None else int(k_new.shape[0])
-    so = np.zeros(len(sel) + batch, np.int32) if want_sel_off else None
-    a = AttendArgs()
-    a.layer, a.batch = layer, batch
-    a.sel_ids, a.cu_sel, a.cu_q, a.cu_new = _np_ptr(sel), _np_ptr(cs), _np_ptr(cq), _np_ptr(cn)
-    a.n_sel, a.n_q, a.n_new = len(sel), nq, nn
-    a.q, a.k_new, a.v_new, a.out = _ptr(q), _ptr(k_new), _ptr(v_new), _ptr(out)
-    a.group_mass = _ptr(group_mass)
-    a.mass_stride = int(mass_stride) if mass_stride is not None else (
-        int(group_mass.shape[-1]) if group_mass is not None else 0)
-    a.sel_off_out = _np_ptr(so)
-    a.split_hint, a.flags = split_hint, flags
-    oo = _i32(obj_off)
-    a.group_mass_sum = _ptr(group_mass_sum)
-    a.sum_stride = int(group_mass_sum.shape[-1]) if group_mass_sum is not None else 0
-    a.n_obj = (len(oo) - 1) if oo is not None else 0
-    a.obj_off = _np_ptr(oo)
-    rc = lib().enl_attend(cache, ctypes.byref(a), stream or None)
+    if want_sel_off:
+        kept = []
+
+        def sel_off(n):
+            kept.append(np.zeros(n, np.int32))
+            return kept[0]
+    rc = (_native or _binding()).attend(cache, layer, sel_ids, q, k_new, v_new, out, group_mass, cu_sel, cu_q, cu_new, n_q, n_new,
+                                        mass_stride, sel_off if want_sel_off else None, split_hint, flags, stream or None,
+                                        group_mass_sum, obj_off)
     if rc != ENL_OK:
         raise EnlError(rc, "enl_attend")
-    return so
+    return kept[0] if want_sel_off else None
 
 
 def enl_attend_static(seg_len: Sequence[int], n_new: int, q, k, v, out, group_mass=None, stream: int = 0) -> None:
@@ -230,12 +224,7 @@ def enl_attend_static(seg_len: Sequence[int], n_new: int, q, k, v, out, group_ma
     ``q``/``out``: ``[Hq, D]`` bf16; ``k``/``v``: ``[sum(seg_len) + n_new, Hkv, D]`` bf16;
     ``group_mass``: ``[Hq, len(seg_len) + 1]`` fp32 or None.  Calls share the built-in array, so issue
     them on one stream (or order them); sizes beyond the fixed maxima raise ``ENL_E_LIMIT``."""
-    sl = _i32(seg_len)
-    a = StaticArgs()
-    a.n_q_heads, a.n_kv_heads, a.head_dim = int(q.shape[-2]), int(k.shape[-2]), int(q.shape[-1])
-    a.n_seg, a.seg_len, a.n_new = len(sl), _np_ptr(sl) if len(sl) else None, int(n_new)
-    a.q, a.k, a.v, a.out, a.group_mass = _ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(group_mass)
-    rc = lib().enl_attend_static(ctypes.byref(a), stream or None)
+    rc = (_native or _binding()).attend_static(seg_len, n_new, q, k, v, out, group_mass, stream or None)
     if rc != ENL_OK:
         raise EnlError(rc, "enl_attend_static")
 
