@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + C::kBarOff + 8 * (13 + 2 * C::kStages));
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
 
-    if (p.fresh_plan) pdl_wait();
+    if (p.wait_first) pdl_wait();
     // work item
     const Item it = p.items[blockIdx.x];
     const EpInfo ep = p.eps[it.ep];

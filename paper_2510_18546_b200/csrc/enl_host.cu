@@ -112,6 +112,14 @@ struct MapCache {
 
 }  // namespace
 
+bool enl::encode_key_map(CUtensorMap *tm, const void *base, int D, int Hkv, int n)
+{
+    const cuuint64_t dims[3] = {static_cast<cuuint64_t>(D), static_cast<cuuint64_t>(Hkv), static_cast<cuuint64_t>(n)};
+    const cuuint64_t strides[2] = {static_cast<cuuint64_t>(D) * 2, static_cast<cuuint64_t>(D) * 2 * Hkv};
+    const cuuint32_t box[3] = {64, 1, kPageTokens};
+    return encode_map(tm, base, 3, dims, strides, box);
+}
+
 struct enl_cache {
     enl_cache_desc_t d{};
     bool gpu = false;
@@ -142,6 +150,10 @@ struct enl_cache {
     bool plan_direct = false;               // built for a call that wants mass sums or no output: one split, general kernel
     std::vector<int32_t> key_obj;           // object spans the row -> object map was built from
     bool plan_decode = false;               // the plan is for the one-token decode kernel
+    int32_t plan_cluster = 0;               // decode: CTAs per cluster, 0 = the streaming kernel
+    int32_t plan_list_pages = 0;            // decode by clusters: most pages one of the CTAs covers
+    ClusterCaps cluster_caps = {};          // decode by clusters: how many run at once (none on a bookkeeping-only cache)
+    bool pool_written = true;               // a launch that writes the pool has been enqueued since the last attention launch
     bool plan_pair = false;                 // two splits whose CTAs merge inside the attention kernel (cluster of two)
     bool pairs_ok = false;                  // the device can co-schedule two of the attention kernel's CTAs as a cluster
     std::vector<int32_t> key_sel, key_cu, key_len;   // what the current plan was built from
@@ -307,7 +319,8 @@ extern "C" int enl_cache_create(const enl_cache_desc_t *desc, enl_cache_t **out)
             return ENL_E_CUDA;
         }
     }
-    if (prepare_attention(d.head_dim) != cudaSuccess || prepare_decode(d.head_dim) != cudaSuccess) { cudaGetLastError(); destroy(c); return ENL_E_CUDA; }
+    if (prepare_attention(d.head_dim) != cudaSuccess || prepare_decode(d.head_dim) != cudaSuccess ||
+        prepare_decode_cluster(d.head_dim, &c->cluster_caps) != cudaSuccess) { cudaGetLastError(); destroy(c); return ENL_E_CUDA; }
     c->pairs_ok = d.head_dim == 128 && attention_pairs_supported();   // else two splits go through the scratch buffer
     if (cudaDeviceSynchronize() != cudaSuccess) { cudaGetLastError(); destroy(c); return ENL_E_CUDA; }
     *out = c;
@@ -405,6 +418,7 @@ extern "C" int enl_group_store(enl_cache_t *c, int32_t group_id, int32_t layer, 
     ++c->epoch;
 
     if (!c->gpu || n_tokens == 0) return ENL_OK;
+    c->pool_written = true;
     DeviceGuard dg(c->d.device);
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const size_t row_bytes = static_cast<size_t>(c->d.n_kv_heads) * c->d.head_dim * 2;
@@ -471,6 +485,7 @@ extern "C" int enl_group_store_all_layers(enl_cache_t *c, int32_t group_id, int3
     ++c->epoch;
 
     if (!c->gpu || n_tokens == 0) return ENL_OK;
+    c->pool_written = true;
     DeviceGuard dg(c->d.device);
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const size_t row_bytes = static_cast<size_t>(c->d.n_kv_heads) * c->d.head_dim * 2;
@@ -622,7 +637,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         // One query token per episode: the streaming decode kernel, whose CTAs cover at most kDecodeMaxPages
         // pages each and always hand their partial results to the merge kernel.
         bool decode = c->rep <= 8 && !direct;
-        int need = 1, fewest = 0x7fffffff;
+        int need = 1, fewest = 0x7fffffff, most = 1;
         for (int b = 0; b < B && decode; ++b) {
             if (cu_q[b + 1] - cu_q[b] != 1) decode = false;
             int64_t e = 0;
@@ -630,9 +645,31 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
             e = (e + kPagesPerTile - 1) / kPagesPerTile * kPagesPerTile + ceil_div(cu_new[b + 1] - cu_new[b], kPageTokens);
             need = std::max<int64_t>(need, (e + kDecodeMaxPages - 1) / kDecodeMaxPages);
             fewest = std::min<int64_t>(fewest, e);
+            most = std::max<int64_t>(most, std::min<int64_t>(e, 0x7fffffff));
         }
-        int n_splits = 1;
-        if (decode) {
+        int n_splits = 1, cluster = 0;
+        int list_pages = 0;
+        if (decode && a->split_hint == 0) {
+            // Splits merged by a thread-block cluster: as many CTAs per (episode, kv head) as run at once.  When they do not fill
+            // two CTAs per SM the streaming kernel, whose CTAs keep more in flight, is faster from some 40 pages per CTA
+            // on (one episode, 8 kv heads, 10k keys: 15.4 against 15.6 us; 33k keys: 32.2 against 31.4); below, and wherever they do,
+            // the merge through memory costs more (2200 keys: 8.5 against 10.4; four episodes of 9900 keys: 31.7 against 34.9).
+            const int n = B * d.n_kv_heads;
+            for (int i = 4; i >= 0 && !cluster; --i) {
+                if ((1 << i) > fewest) continue;
+                list_pages = (ceil_div(most, 1 << i) + 1) & ~1;
+                if (list_pages > kClusterMaxPages) break;
+                const int cap = c->cluster_caps.get(i, decode_cluster_smem(d.head_dim, list_pages, std::min(list_pages, max_slots + 1), c->rep));
+                // (where the streaming kernel would need a second wave too, one here is the better one: 8 episodes of 9900 keys
+                // 56 against 82 us)
+                if (cap < n && !(cap > 0 && n * need > c->n_sm && (n << i) <= 2 * c->n_sm)) continue;
+                if (2 * (n << i) < 3 * c->n_sm && list_pages > 40) break;
+                cluster = 1 << i;
+            }
+        }
+        if (cluster) {
+            n_splits = cluster;
+        } else if (decode) {
             const int slots = c->n_sm;                                            // one CTA per SM, one wave
             n_splits = a->split_hint >= 1 ? a->split_hint : std::max(1, slots / (B * d.n_kv_heads));
             n_splits = std::min(std::min(std::max(n_splits, need), fewest), kMaxSplits);
@@ -741,6 +778,8 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         c->plan_has_mass = has_mass;
         c->plan_direct = direct;
         c->plan_decode = decode;
+        c->plan_cluster = cluster;
+        c->plan_list_pages = list_pages;
         c->plan_pair = pair;
         c->key_sel.assign(a->sel_ids, a->sel_ids + a->n_sel);
         c->key_cu.assign(cu_sel, cu_sel + B + 1);
@@ -769,8 +808,43 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         if (!okc) { cudaGetLastError(); c->plan_valid = false; return ENL_E_CUDA; }
         c->plan_on_device = true;
     }
+    // Launches that find plan and pool as the attention launch before left them may read both before the kernel before them
+    // has ended.  Ones that do not wait for it first and hold their own successor back until then, so that this carries over.
+    const bool wait_first = fresh || c->pool_written;
+    c->pool_written = false;
 
     const int slot_stride = c->plan_max_slots + 1;
+    if (c->plan_decode && c->plan_cluster) {
+        ClusterDecodeParams dp;
+        std::memset(&dp, 0, sizeof dp);
+        const cuuint64_t nd[3] = {static_cast<cuuint64_t>(d.head_dim), static_cast<cuuint64_t>(d.n_kv_heads),
+                                  static_cast<cuuint64_t>(a->n_new)};
+        const cuuint64_t ns[2] = {static_cast<cuuint64_t>(d.head_dim) * 2,
+                                  static_cast<cuuint64_t>(d.head_dim) * 2 * d.n_kv_heads};
+        const cuuint32_t nb[3] = {64, 1, kPageTokens};
+        if (!c->maps.get(&dp.tm_knew, a->k_new, nd, ns, nb) || !c->maps.get(&dp.tm_vnew, a->v_new, nd, ns, nb))
+            return ENL_E_CUDA;
+        dp.tm_kpool = c->tm_k[a->layer];
+        dp.tm_vpool = c->tm_v[a->layer];
+        dp.ep0 = c->h_eps()[0];
+        dp.eps = reinterpret_cast<const EpInfo *>(c->plan_dev + c->off_eps);
+        dp.stream_page = reinterpret_cast<const int32_t *>(c->plan_dev + c->off_stream);
+        dp.stream_meta = reinterpret_cast<const int32_t *>(c->plan_dev + c->off_meta);
+        dp.q = a->q;
+        dp.out = a->out;
+        dp.mass = a->group_mass;
+        dp.status = c->status_dev;
+        dp.Hq = d.n_q_heads;
+        dp.Hkv = d.n_kv_heads;
+        dp.rep = c->rep;
+        dp.mass_stride = a->mass_stride;
+        dp.list_pages = c->plan_list_pages;
+        dp.list_slots = std::min(c->plan_list_pages, c->plan_max_slots + 1);
+        dp.wait_first = wait_first ? 1 : 0;
+        dp.scale_log2 = 1.4426950408889634f / sqrtf(static_cast<float>(d.head_dim));
+        if (launch_decode_cluster(dp, d.head_dim, c->plan_batch, c->plan_cluster, st) != cudaSuccess) { cudaGetLastError(); return ENL_E_CUDA; }
+        return ENL_OK;
+    }
     if (c->plan_decode) {
         DecodeParams dp;
         std::memset(&dp, 0, sizeof dp);
@@ -807,7 +881,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         dp.slot_stride = slot_stride;
         dp.mass_stride = a->mass_stride;
         dp.n_splits = c->plan_splits;
-        dp.fresh_plan = fresh ? 1 : 0;
+        dp.wait_first = wait_first ? 1 : 0;
         dp.scale_log2 = 1.4426950408889634f / sqrtf(static_cast<float>(d.head_dim));
         if (launch_decode(dp, d.head_dim, c->plan_batch, st) != cudaSuccess) { cudaGetLastError(); return ENL_E_CUDA; }
         return ENL_OK;
@@ -852,7 +926,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
     p.sum_stride = a->sum_stride;
     p.mass_only = mass_only ? 1 : 0;
     p.first_wave = c->n_sm;
-    p.fresh_plan = fresh ? 1 : 0;
+    p.wait_first = wait_first ? 1 : 0;
     const bool scratch_merge = p.n_splits > 1 && !c->plan_pair;
     if (scratch_merge) {
         const size_t rows = static_cast<size_t>(p.n_splits) * a->n_q * d.n_q_heads;
@@ -1091,6 +1165,7 @@ extern "C" int enl_step_prepare(enl_cache_t *c, const int32_t *sel_ids, int32_t 
             g.resident = true;                                         // host copy stays current until the next store
             stt.bytes_h2d += static_cast<int64_t>(np) * page_bytes_of(c) * 2 * c->d.n_layers;
         }
+        c->pool_written = true;
         const int rc = enqueue_moves(c, n, false, st);
         if (rc != ENL_OK) return rc;
     }

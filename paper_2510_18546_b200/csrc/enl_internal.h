@@ -59,7 +59,8 @@ struct AttnParams {
     const int32_t *row_obj; // [n_q_total]: object of every query row, -1 = none (only with mass_sum)
     int32_t sum_stride;
     int32_t mass_only;      // 1: the output rows are not written
-    int32_t fresh_plan;     // 1: the kernel before wrote the gather plan, wait for it before the plan is read
+    int32_t wait_first;     // 1: the plan or the pool has been written since the last attention launch: wait for the kernel before
+                            // at the very start; 0: both may be read while it still runs
     int32_t first_wave;     // CTAs that start while the previous kernel of the stream may still run (the number of SMs)
 };
 
@@ -89,8 +90,38 @@ struct DecodeParams {
     int32_t slot_stride;    // row stride of part_slot
     int32_t mass_stride;    // row stride of mass
     int32_t n_splits;
-    int32_t fresh_plan;     // as in AttnParams
+    int32_t wait_first;     // as in AttnParams
     float   scale_log2;
+};
+
+// The same for calls whose splits fit a thread-block cluster (see enl_decode_cluster_sm100.cu): no partial results in memory.
+struct ClusterDecodeParams {
+    CUtensorMap tm_knew;    // [n_new][Hkv][D]   box {64, 1, 16}
+    CUtensorMap tm_vnew;
+    CUtensorMap tm_kpool;   // [pages*Hkv*16][D] box {64, 16}   (one layer)
+    CUtensorMap tm_vpool;
+    EpInfo ep0;             // episode 0 (used when the call has one episode; grid = cluster x kv heads x episodes)
+    const EpInfo *eps;
+    const int32_t *stream_page;
+    const int32_t *stream_meta;
+    const void *q;          // bf16 [n_q][Hq][D], one row per episode
+    void   *out;            // bf16 [n_q][Hq][D]
+    float  *mass;           // fp32 or null
+    int32_t *status;
+    int32_t Hq, Hkv, rep;
+    int32_t mass_stride;
+    int32_t list_pages;     // most pages a CTA of this launch covers, and most slots they can touch (sizes of its lists)
+    int32_t list_slots;
+    int32_t wait_first;     // as in AttnParams
+    float   scale_log2;
+};
+constexpr int kMaxCluster = 16;
+// Contiguous keys in segments instead of pool pages (the entry point that allocates nothing).
+constexpr int kStaticMaxSeg = 255;
+struct StaticDecodeParams {
+    ClusterDecodeParams d;                  // tm_knew / tm_vnew cover the whole stream, ep0.n_slots = segments
+    int32_t seg_off[kStaticMaxSeg + 2];     // first key of every slot (slot n_seg = the new keys), then the total
+    int32_t page_off[kStaticMaxSeg + 2];    // the same in pages (16 keys of one slot, the last one of a slot partly filled)
 };
 
 struct CombineParams {
@@ -151,11 +182,27 @@ inline cudaError_t launch_pdl_n(void (*kernel)(KArgs...), dim3 grid, dim3 block,
 }
 #endif
 
+// Tensor map of a caller's [n][Hkv][D] bf16 keys or values with boxes of one head's 16 rows x 64 channels (in enl_host.cu)
+bool encode_key_map(CUtensorMap *tm, const void *base, int D, int Hkv, int n);
+
 // launchers (defined in the .cu files of the kernels)
 cudaError_t launch_attention(const AttnParams &p, int head_dim, int n_items, cudaStream_t st);
 cudaError_t launch_combine(const CombineParams &p, cudaStream_t st);
 cudaError_t launch_decode(const DecodeParams &p, int head_dim, int batch, cudaStream_t st);
 cudaError_t prepare_decode(int head_dim);
+// cluster: CTAs per (episode, kv head), 1, 2, 4, 8 or 16
+cudaError_t launch_decode_cluster(const ClusterDecodeParams &p, int head_dim, int batch, int cluster, cudaStream_t st);
+cudaError_t launch_decode_static(const StaticDecodeParams &p, int head_dim, int cluster, cudaStream_t st);
+constexpr int kClusterMaxPages = 288;         // pages of a CTA of these kernels
+int decode_cluster_smem(int head_dim, int list_pages, int list_slots, int rep);
+constexpr int kClusterPairSmem = 113800;      // two CTAs of up to this much fit an SM
+// How many clusters of 2^i CTAs the current device runs at once: with two CTAs per SM, and with one (larger lists).
+struct ClusterCaps {
+    int two[5], one[5];
+    int get(int i, int smem) const { return smem <= kClusterPairSmem ? two[i] : one[i]; }
+};
+// Opts the kernels in and asks the device for its capacities.
+cudaError_t prepare_decode_cluster(int head_dim, ClusterCaps *caps);
 size_t decode_smem_bytes(int head_dim);
 // Page ids of (part of) one group, passed by value to the scatter kernel.
 constexpr int kScatterPages = 64;

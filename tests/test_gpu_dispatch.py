@@ -45,3 +45,94 @@ def test_gather_plan_reaches_the_device(pages, n_q):
             ks, vs = ([x[i] for i in sel] for x in s.host_kv[(0, 0)])
             ro, rm = orc.attend_slots(4, 1, 64, ks, vs, q.cpu(), kn.cpu(), vn.cpu(), rows=rows)
             check_close(out[rows], ro, mass[rows], rm, what=f"{wl.name}, {len(sel)} groups")
+
+
+# One-token steps merged by clusters: slots that reach over several CTAs' ranges, ranges that begin and end on slot
+# boundaries, empty groups, more slots than pages in a range, every number of q heads per kv head, streams from one page up to
+# where the streaming kernel takes over.
+STEP = {
+    "one_page": dict(Hq=4, Hkv=1, D=128, pool=[[10]], sel=[[]], n_new=[3]),
+    "two_pages": dict(Hq=2, Hkv=2, D=64, pool=[[5]], n_new=[1]),
+    "sixteen_pages": dict(Hq=8, Hkv=2, D=128, pool=[[16] * 8], n_new=[128]),
+    "one_slot_over_all_ranges": dict(Hq=8, Hkv=1, D=128, pool=[[3000]], n_new=[1]),
+    "slots_of_one_key": dict(Hq=16, Hkv=8, D=64, pool=[[1] * 200], n_new=[17]),
+    "empty_groups": dict(Hq=4, Hkv=4, D=128, pool=[[0, 0, 300, 0, 17, 0, 0]], n_new=[40]),
+    "long_new": dict(Hq=32, Hkv=8, D=128, pool=[[90, 33]], n_new=[700]),
+    "below_the_line": dict(Hq=32, Hkv=8, D=128, pool=[[639 * 16 // 4] * 4], n_new=[16]),
+    "above_the_line": dict(Hq=32, Hkv=8, D=128, pool=[[656 * 16 // 4] * 4], n_new=[16]),
+    "batch": dict(Hq=8, Hkv=2, D=128, pool=[[30, 60, 90], [5, 5, 5, 5], [200], [], [700, 1]], n_new=[1, 10, 129, 16, 33]),
+    "many_clusters": dict(Hq=16, Hkv=8, D=64, pool=[[40, 25]] * 20, n_new=[9] * 20),
+}
+
+
+@pytest.mark.parametrize("want_mass", [True, False])
+@pytest.mark.parametrize("name", sorted(STEP))
+def test_one_token_steps(name, want_mass):
+    c = STEP[name]
+    n = len(c["pool"])
+    wl = synth.make_small(41, 1, c["Hq"], c["Hkv"], c["D"], c["pool"],
+                          c.get("sel") or [list(range(len(x)))[::-1] for x in c["pool"]], [1] * n, c["n_new"], name=name)
+    with Session(wl, [0]) as s:
+        q, kn, vn = wl.new_qkv(0, s.device)
+        cn = wl.cu()[2]
+        for _ in range(2):                                  # the second call finds plan and pool as the first left them
+            out, mass, _ = s.attend(0, q, kn, vn, want_mass=want_mass)
+        torch.cuda.synchronize()
+        assert enl.enl_cache_status(s.cache) == enl.ENL_OK
+        for b in range(n):
+            ro, rm, _ = s.oracle(0, b, q[b:b + 1], kn[cn[b]:cn[b + 1]], vn[cn[b]:cn[b + 1]])
+            G = len(wl.sel_local[b])
+            check_close(out[b:b + 1], ro, mass[b:b + 1, :, :G + 1] if want_mass else None, rm if want_mass else None, what=name)
+
+
+def test_stores_between_one_token_steps_are_seen():
+    """A store directly before a step, and steps directly after one another: what may be read before the previous launch has
+    ended is exactly what no launch in between has written."""
+    wl = synth.make_small(43, 1, 8, 2, 128, [[60, 90, 33]], [[0, 1, 2]], [1], [1], name="store between steps")
+    with Session(wl, [0]) as s:
+        q, kn, vn = wl.new_qkv(0, s.device)
+        k, v = wl.pool_kv(0, 0, s.device)
+        outs, want = [], []
+        gen = torch.Generator(device=s.device).manual_seed(5)
+        for i in range(6):
+            if i % 2 == 0:
+                k[60:150] = torch.randn(90, 2, 128, generator=gen, device=s.device).to(k.dtype)
+                rows = k[60:150].clone()
+                enl.enl_group_store(s.cache, 1, 0, rows, v[60:150])
+            out = torch.empty_like(q)
+            enl.enl_attend(s.cache, 0, [0, 1, 2], q, kn, vn, out)
+            outs.append(out)
+            ks = [k[a:b].cpu().clone() for a, b in ((0, 60), (60, 150), (150, 183))]
+            vs = [v[a:b].cpu() for a, b in ((0, 60), (60, 150), (150, 183))]
+            want.append((ks, vs))
+        torch.cuda.synchronize()
+        for out, (ks, vs) in zip(outs, want):
+            ro, _ = orc.attend_slots(8, 2, 128, ks, vs, q.cpu(), kn.cpu(), vn.cpu())
+            check_close(out, ro, None, None, what="store between steps")
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("rep", [1, 2, 8])
+@pytest.mark.parametrize("lens, n_new", [([], 1), ([0, 5, 0, 0, 16, 1], 1), ([1] * 255, 2), ([700, 15, 17], 33), ([40000], 9)])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_static_step(D, rep, lens, n_new, shift):
+    """Segments that start anywhere; with shift the tensors start off a 16-byte boundary (the other kernel)."""
+    if shift and sum(lens) > 10000:
+        pytest.skip("one long stream is enough")
+    hkv = 2
+    n = sum(lens) + n_new
+    gen = torch.Generator(device="cuda").manual_seed(n)
+
+    def rand(*shape):
+        x = torch.randn(int(np.prod(shape)) + shift, generator=gen, device="cuda").to(torch.bfloat16)
+        return x[shift:].view(*shape)
+
+    q, k, v = rand(hkv * rep, D), rand(n, hkv, D), rand(n, hkv, D)
+    out = torch.full_like(q, float("nan"))
+    mass = torch.full((hkv * rep, len(lens) + 1), float("nan"), device="cuda")
+    enl.enl_attend_static(lens, n_new, q, k, v, out, mass)
+    torch.cuda.synchronize()
+    offs = np.concatenate([[0], np.cumsum(lens)]).astype(int)
+    ks, vs = ([x[a:b].cpu() for a, b in zip(offs[:-1], offs[1:])] for x in (k, v))
+    ro, rm = orc.attend_slots(hkv * rep, hkv, D, ks, vs, q[None].cpu(), k[offs[-1]:].cpu(), v[offs[-1]:].cpu())
+    check_close(out[None], ro, mass[None], rm, what="static")
