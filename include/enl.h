@@ -149,7 +149,7 @@ typedef struct {
     /* Sec. 3.3 consumes only an average of the mass over an object's tokens, the q heads and  */
     /* the scored layers.  With group_mass_sum the call ADDS, for every object o and slot s,   */
     /* the sum over the object's query rows and all q heads of the row's mass on s to          */
-    /* group_mass_sum[o * sum_stride + s] (one reduction inside the attention kernel, one      */
+    /* group_mass_sum[o * sum_stride + s] (while the masses are finished, one               */
     /* atomic add per warp, object and slot), so that the caller zeroes the array once, lets   */
     /* the scored layers accumulate and never reads the per-row masses back:                   */
     /* enl_cluster_assign_sums turns the sums into averages and decisions.                     */

@@ -137,7 +137,7 @@ struct enl_cache {
     int32_t cap_entries = 0, cap_items = 0;
     uint8_t *plan_host = nullptr, *plan_dev = nullptr;
     // sections of the current plan, back to back in the order of their offsets
-    size_t off_eps = 0, off_items = 0, off_stream = 0, off_meta = 0, off_rowslots = 0, off_rowobj = 0, plan_used = 0;
+    size_t off_eps = 0, off_items = 0, off_stream = 0, off_meta = 0, off_rowslots = 0, off_rowobj = 0, off_words = 0, plan_used = 0;
     size_t plan_bytes = 0;                  // capacity
     cudaEvent_t plan_copied = nullptr;
     bool plan_copying = false;              // a copy out of plan_host may be under way (until plan_copied)
@@ -147,7 +147,9 @@ struct enl_cache {
     uint64_t plan_epoch = 0;
     int32_t plan_split_hint = 0;
     bool plan_has_mass = false;
-    bool plan_direct = false;               // built for a call that wants mass sums or no output: one split, general kernel
+    bool plan_mass_only = false, plan_sums = false;      // what the call wants besides or instead of outputs
+    bool plan_park = false;                 // every CTA walks few slots: it parks their sums in shared memory and writes the masses itself
+    bool plan_finish = false;               // else a kernel behind the attention kernel turns log-sums into masses
     std::vector<int32_t> key_obj;           // object spans the row -> object map was built from
     bool plan_decode = false;               // the plan is for the one-token decode kernel
     int32_t plan_cluster = 0;               // decode: CTAs per cluster, 0 = the streaming kernel
@@ -174,6 +176,9 @@ struct enl_cache {
     uint64_t tick = 0;
 
     float *scratch = nullptr;
+    float *finish_lse = nullptr;            // rows' log-sum-exps for that kernel, and the splits' parts of shared slots
+    float2 *finish_bnd = nullptr;
+    int64_t finish_cap = 0;                 // entries of either
     int32_t *status_dev = nullptr;
     int32_t *counters_dev = nullptr;        // decode: finished splits per (episode, kv head)
 
@@ -182,6 +187,7 @@ struct enl_cache {
     int32_t *h_stream() { return reinterpret_cast<int32_t *>(plan_host + off_stream); }
     int32_t *h_meta() { return reinterpret_cast<int32_t *>(plan_host + off_meta); }
     int32_t *h_rowslots() { return reinterpret_cast<int32_t *>(plan_host + off_rowslots); }
+    int2 *h_words() { return reinterpret_cast<int2 *>(plan_host + off_words); }
     int32_t *h_rowobj() { return reinterpret_cast<int32_t *>(plan_host + off_rowobj); }
 };
 
@@ -198,6 +204,8 @@ void destroy(enl_cache *c)
         if (c->plan_dev) cudaFree(c->plan_dev);
         if (c->plan_host) cudaFreeHost(c->plan_host);
         if (c->scratch) cudaFree(c->scratch);
+        if (c->finish_lse) cudaFree(c->finish_lse);
+        if (c->finish_bnd) cudaFree(c->finish_bnd);
         if (c->status_dev) cudaFree(c->status_dev);
         if (c->counters_dev) cudaFree(c->counters_dev);
         if (c->plan_copied) cudaEventDestroy(c->plan_copied);
@@ -272,7 +280,7 @@ extern "C" int enl_cache_create(const enl_cache_desc_t *desc, enl_cache_t **out)
     c->cap_items = std::max(4096, (d.max_q_tokens / tpc + d.max_batch + 1) * d.n_kv_heads);
     auto align256 = [](size_t x) { return (x + 255) & ~static_cast<size_t>(255); };
     c->plan_bytes = align256(sizeof(EpInfo) * d.max_batch) + align256(sizeof(Item) * c->cap_items) +
-                    2 * align256(sizeof(int32_t) * c->cap_entries) + 2 * align256(sizeof(int32_t) * d.max_q_tokens);
+                    2 * align256(sizeof(int32_t) * c->cap_entries) + align256(c->cap_entries + sizeof(int2)) + 2 * align256(sizeof(int32_t) * d.max_q_tokens);
     c->plan_layer_ok.assign(d.n_layers, 0);
 
     if (!c->gpu) {
@@ -291,11 +299,14 @@ extern "C" int enl_cache_create(const enl_cache_desc_t *desc, enl_cache_t **out)
         delete c;
         return ENL_E_CUDA;
     }
+    c->finish_cap = std::max<int64_t>(static_cast<int64_t>(d.max_q_tokens) * d.n_q_heads, 256ll * c->n_sm);
     const size_t pool_bytes = c->layer_bytes * d.n_layers;
     bool okm = cudaMalloc(&c->kpool, pool_bytes) == cudaSuccess && cudaMalloc(&c->vpool, pool_bytes) == cudaSuccess &&
                cudaMalloc(&c->plan_dev, c->plan_bytes) == cudaSuccess &&
                cudaMallocHost(&c->plan_host, c->plan_bytes) == cudaSuccess &&
                cudaMalloc(&c->scratch, static_cast<size_t>(d.scratch_bytes)) == cudaSuccess &&
+               cudaMalloc(&c->finish_lse, sizeof(float) * c->finish_cap) == cudaSuccess &&
+               cudaMalloc(&c->finish_bnd, sizeof(float2) * c->finish_cap) == cudaSuccess &&
                cudaMalloc(&c->status_dev, sizeof(int32_t)) == cudaSuccess &&
                cudaMalloc(&c->counters_dev, sizeof(int32_t) * d.max_batch * d.n_kv_heads) == cudaSuccess;
     if (!okm) { cudaGetLastError(); destroy(c); return ENL_E_NOMEM; }
@@ -319,7 +330,7 @@ extern "C" int enl_cache_create(const enl_cache_desc_t *desc, enl_cache_t **out)
             return ENL_E_CUDA;
         }
     }
-    if (prepare_attention(d.head_dim) != cudaSuccess || prepare_decode(d.head_dim) != cudaSuccess ||
+    if (prepare_attention(d.head_dim) != cudaSuccess || prepare_decode(d.head_dim) != cudaSuccess || prepare_mass(d.head_dim) != cudaSuccess ||
         prepare_decode_cluster(d.head_dim, &c->cluster_caps) != cudaSuccess) { cudaGetLastError(); destroy(c); return ENL_E_CUDA; }
     c->pairs_ok = d.head_dim == 128 && attention_pairs_supported();   // else two splits go through the scratch buffer
     if (cudaDeviceSynchronize() != cudaSuccess) { cudaGetLastError(); destroy(c); return ENL_E_CUDA; }
@@ -560,7 +571,6 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         for (int o = 0; o < a->n_obj; ++o)
             if (a->obj_off[o + 1] < a->obj_off[o]) return ENL_E_INVAL;
     }
-    const bool direct = has_sum || mass_only;       // these results leave the attention kernel itself: no KV splits
 
     // ---- gather plan: reuse when nothing it was built from has changed ----
     const bool has_mass = a->group_mass != nullptr;
@@ -569,7 +579,8 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
                                         std::memcmp(c->key_obj.data(), a->obj_off, sizeof(int32_t) * (a->n_obj + 1)) == 0
                                   : true;
     bool reuse = c->plan_valid && c->plan_epoch == c->epoch && c->plan_split_hint == a->split_hint &&
-                 c->plan_has_mass == has_mass && c->plan_direct == direct && same_obj && c->plan_batch == B &&
+                 c->plan_has_mass == has_mass && c->plan_mass_only == mass_only &&
+                 c->plan_sums == has_sum && same_obj && c->plan_batch == B &&
                  c->key_sel.size() == static_cast<size_t>(a->n_sel) &&
                  (a->n_sel == 0 || std::memcmp(c->key_sel.data(), a->sel_ids, sizeof(int32_t) * a->n_sel) == 0) &&
                  std::memcmp(c->key_cu.data(), cu_sel, cu_bytes) == 0 &&
@@ -636,7 +647,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         };
         // One query token per episode: the streaming decode kernel, whose CTAs cover at most kDecodeMaxPages
         // pages each and always hand their partial results to the merge kernel.
-        bool decode = c->rep <= 8 && !direct;
+        bool decode = c->rep <= 8 && !mass_only && !has_sum;
         int need = 1, fewest = 0x7fffffff, most = 1;
         for (int b = 0; b < B && decode; ++b) {
             if (cu_q[b + 1] - cu_q[b] != 1) decode = false;
@@ -680,12 +691,19 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         }
         if (!decode) {
             n_splits = 1;
-            if (direct) n_splits = 1;
+            const bool few = base_items * 5 < c->n_sm * 4;         // a launch that leaves SMs idle splits the key stream
+            // (two key tiles per split are worth it where the merge is cheap; the kernel that finishes masses takes a few us itself)
+            const int filling = std::max(1, std::min(static_cast<int>(c->n_sm / base_items), min_tiles / (mass_only || has_sum ? 8 : 2)));
+            if (has_sum && !mass_only) n_splits = few && a->split_hint != 1 && c->pairs_ok && filling >= 2 ? 2 : 1;   // a pair or none
             else if (a->split_hint >= 1) n_splits = std::min(a->split_hint, std::max(1, min_tiles));   // no CTA without a tile
-            else if (base_items * 5 < c->n_sm * 4) n_splits = std::max(1, std::min(static_cast<int>(c->n_sm / base_items), min_tiles / 2));
+            else if (few) n_splits = filling;
+            if (mass_only) {                                       // no outputs to merge: the kernel that finishes the masses adds the splits up
+                n_splits = std::min(n_splits, kFinishSplits);
+                while (n_splits > 1 && static_cast<int64_t>(n_splits) * a->n_q * d.n_q_heads > c->finish_cap) --n_splits;
+            }
             n_splits = std::min<int64_t>(n_splits, std::max<int64_t>(1, c->cap_items / base_items));
             n_splits = std::min(n_splits, kMaxSplits);
-            while (n_splits > 1 && !fits(n_splits)) --n_splits;
+            while (n_splits > 1 && !mass_only && !fits(n_splits)) --n_splits;
         }
 
         if (c->plan_copying) {
@@ -696,7 +714,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         // Two splits of a head_dim-128 call are launched as clusters of two CTAs, which exchange their partial
         // results through distributed shared memory: no scratch round trip and no merge kernel.  Every CTA must
         // have at least one tile, and the items of a pair must be neighbours (they are: same tile count, stable sort).
-        const bool pair = !decode && n_splits == 2 && d.head_dim == 128 && min_tiles >= 2 && (c->pairs_ok || !c->gpu);
+        const bool pair = !decode && !mass_only && n_splits == 2 && d.head_dim == 128 && min_tiles >= 2 && (c->pairs_ok || !c->gpu);
         const int64_t n_items = decode ? static_cast<int64_t>(B) * d.n_kv_heads * n_splits : base_items * n_splits;
         {   // sections: what the kernels of this plan read (the decode kernel takes its CTA's place from the grid)
             auto align16 = [](size_t x) { return (x + 15) & ~static_cast<size_t>(15); };
@@ -706,7 +724,9 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
             c->off_items = section(decode ? 0 : sizeof(Item) * n_items);
             c->off_stream = section(sizeof(int32_t) * n_entries);
             c->off_meta = section(sizeof(int32_t) * n_entries);
-            c->off_rowslots = section(!decode && n_splits > 1 && !pair ? sizeof(int32_t) * a->n_q : 0);
+            const bool merged = n_splits > 1 && !pair && !mass_only;
+            c->off_words = section(mass_only ? sizeof(int2) * (n_entries / kPagesPerTile) : 0);
+            c->off_rowslots = section(!decode && (merged || (has_mass && B > 1)) ? sizeof(int32_t) * a->n_q : 0);
             c->off_rowobj = section(has_sum ? sizeof(int32_t) * a->n_q : 0);
             c->plan_used = at;
         }
@@ -737,7 +757,17 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
             }
             while ((ne - e.stream_off) % kPagesPerTile) { stream[ne] = kZeroPage; smeta[ne++] = (e.n_slots - 1) << 8; }
             e.n_ctiles = (ne - e.stream_off) / kPagesPerTile;
-            if (!decode && n_splits > 1 && !pair)
+            for (int j = 0; j < e.n_ctiles && mass_only; ++j) {
+                uint32_t keys = 0, hide = 0, chg = 0;
+                for (int x = 0; x < kPagesPerTile; ++x) {
+                    const int at = e.stream_off + j * kPagesPerTile + x, n = smeta[at] & 0xff;
+                    keys |= static_cast<uint32_t>(n & 15) << (4 * x);
+                    if (n < kPageTokens) hide |= 1u << x;
+                    if (at > e.stream_off && (smeta[at] >> 8) != (smeta[at - 1] >> 8)) chg |= 1u << x;
+                }
+                c->h_words()[e.stream_off / kPagesPerTile + j] = make_int2(static_cast<int>(keys), static_cast<int>(hide | chg << 8));
+            }
+            if (!decode && ((n_splits > 1 && !pair && !mass_only) || (has_mass && B > 1)))
                 for (int r = e.q_off; r < e.q_off + e.n_q; ++r) rowslots[r] = e.n_slots;
         }
         if (has_sum) {
@@ -776,7 +806,11 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         c->plan_epoch = c->epoch;
         c->plan_split_hint = a->split_hint;
         c->plan_has_mass = has_mass;
-        c->plan_direct = direct;
+        c->plan_mass_only = mass_only;
+        c->plan_sums = has_sum;
+        const bool merged = !decode && n_splits > 1 && !pair && !mass_only;
+        c->plan_park = has_mass && !mass_only && (!has_sum || merged) && max_slots + 1 <= attention_park_slots();
+        c->plan_finish = has_mass && !decode && !c->plan_park && !merged;
         c->plan_decode = decode;
         c->plan_cluster = cluster;
         c->plan_list_pages = list_pages;
@@ -921,13 +955,11 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
     p.n_splits = c->plan_splits;
     p.pair_merge = c->plan_pair ? 1 : 0;
     p.scale_log2 = 1.4426950408889634f / sqrtf(static_cast<float>(d.head_dim));
-    p.mass_sum = a->group_mass_sum;
-    p.row_obj = has_sum ? reinterpret_cast<const int32_t *>(c->plan_dev + c->off_rowobj) : nullptr;
-    p.sum_stride = a->sum_stride;
-    p.mass_only = mass_only ? 1 : 0;
+    p.park_smem = c->plan_park ? 1 : 0;
+    p.lse_out = c->finish_lse;
     p.first_wave = c->n_sm;
     p.wait_first = wait_first ? 1 : 0;
-    const bool scratch_merge = p.n_splits > 1 && !c->plan_pair;
+    const bool scratch_merge = p.n_splits > 1 && !c->plan_pair && !mass_only;
     if (scratch_merge) {
         const size_t rows = static_cast<size_t>(p.n_splits) * a->n_q * d.n_q_heads;
         p.part_o = c->scratch;
@@ -935,7 +967,47 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         p.part_slot = has_mass ? c->scratch + rows * (d.head_dim + 1) : nullptr;
         p.mass_stride = slot_stride;                 // the partial slot buffer is packed
     }
-    if (launch_attention(p, d.head_dim, c->plan_items, st) != cudaSuccess) { cudaGetLastError(); return ENL_E_CUDA; }
+    if (mass_only) {
+        MassParams mp;
+        std::memset(&mp, 0, sizeof mp);
+        mp.tm_q = p.tm_q;
+        mp.tm_knew = p.tm_knew;
+        mp.tm_kpool = p.tm_kpool;
+        mp.items = p.items;
+        mp.eps = p.eps;
+        mp.stream_page = p.stream_page;
+        mp.stream_meta = p.stream_meta;
+        mp.tile_words = reinterpret_cast<const int2 *>(c->plan_dev + c->off_words);
+        mp.mass = a->group_mass;
+        mp.lse_out = c->finish_lse;
+        mp.bnd_out = c->finish_bnd;
+        mp.status = c->status_dev;
+        mp.n_q_total = a->n_q;
+        mp.Hq = d.n_q_heads;
+        mp.Hkv = d.n_kv_heads;
+        mp.rep = c->rep;
+        mp.mass_stride = a->mass_stride;
+        mp.n_splits = p.n_splits;
+        mp.wait_first = p.wait_first;
+        mp.scale_log2 = p.scale_log2;
+        if (launch_mass(mp, d.head_dim, c->plan_items, st) != cudaSuccess) { cudaGetLastError(); return ENL_E_CUDA; }
+    } else if (launch_attention(p, d.head_dim, c->plan_items, st) != cudaSuccess) { cudaGetLastError(); return ENL_E_CUDA; }
+    if (c->plan_finish) {
+        FinishParams fp;
+        fp.mass = a->group_mass;
+        fp.lse = c->finish_lse;
+        fp.bnd = c->finish_bnd;
+        fp.row_slots = c->plan_batch > 1 ? reinterpret_cast<const int32_t *>(c->plan_dev + c->off_rowslots) : nullptr;
+        fp.row_obj = has_sum ? reinterpret_cast<const int32_t *>(c->plan_dev + c->off_rowobj) : nullptr;
+        fp.mass_sum = a->group_mass_sum;
+        fp.n_q_total = a->n_q;
+        fp.Hq = d.n_q_heads;
+        fp.mass_stride = a->mass_stride;
+        fp.sum_stride = a->sum_stride;
+        fp.n_splits = mass_only ? p.n_splits : 1;
+        fp.max_slots = c->plan_max_slots;
+        if (launch_mass_finish(fp, st) != cudaSuccess) { cudaGetLastError(); return ENL_E_CUDA; }
+    }
     if (scratch_merge) {
         CombineParams cp;
         cp.part_o = p.part_o;
@@ -1183,7 +1255,7 @@ extern "C" int enl_plan_inspect(const enl_cache_t *cc, int32_t cap_entries, int3
     if (n_entries) *n_entries = c->plan_entries;
     if (n_splits) *n_splits = c->plan_splits;
     if (n_items) *n_items = c->plan_items;
-    if (merge_kind) *merge_kind = c->plan_decode ? 3 : c->plan_pair ? 2 : c->plan_splits > 1 ? 1 : 0;
+    if (merge_kind) *merge_kind = c->plan_decode ? 3 : c->plan_pair ? 2 : c->plan_splits > 1 && !c->plan_mass_only ? 1 : 0;
     const int32_t *s = c->h_stream(), *m = c->h_meta();
     for (int i = 0; i < c->plan_entries && i < cap_entries; ++i) {
         if (stream_pages) stream_pages[i] = s[i];

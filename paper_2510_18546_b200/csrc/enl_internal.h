@@ -55,13 +55,36 @@ struct AttnParams {
     int32_t n_splits;
     int32_t pair_merge;     // 1: two splits, launched as clusters of two CTAs that merge through distributed shared memory
     float   scale_log2;     // log2(e) / sqrt(D)
-    float  *mass_sum;       // fp32 [n_obj][sum_stride] or null: per object the masses summed over its rows and the q heads (added to)
-    const int32_t *row_obj; // [n_q_total]: object of every query row, -1 = none (only with mass_sum)
-    int32_t sum_stride;
-    int32_t mass_only;      // 1: the output rows are not written
+    int32_t park_smem;      // 1: the call has at most attention_park_slots() slots: the kernel turns their log-sums into masses itself;
+                            // 0: log-sums go to mass, log-sum-exps to lse_out, and mass_finish_kernel does
+    float  *lse_out;        // [n_q_total][Hq] log2-sum-exp of every row
     int32_t wait_first;     // 1: the plan or the pool has been written since the last attention launch: wait for the kernel before
                             // at the very start; 0: both may be read while it still runs
     int32_t first_wave;     // CTAs that start while the previous kernel of the stream may still run (the number of SMs)
+};
+
+// Masses without outputs (see enl_attn_mass_sm100.cu)
+struct MassParams {
+    CUtensorMap tm_q;       // [n_q][Hq][D]      box {64, rep, 128/rep}
+    CUtensorMap tm_knew;    // [n_new][Hkv][D]   box {64, 1, 128}
+    CUtensorMap tm_kpool;   // [pages*Hkv*16][D] box {64, 16}   (one layer)
+    const Item   *items;
+    const EpInfo *eps;
+    const int32_t *stream_page;
+    const int32_t *stream_meta;
+    const int2 *tile_words; // per cached tile: visible keys of its pages (4 bits each, of 16), then pages that hide keys (8 bits)
+                            // and pages whose slot differs from the page before (8 bits)
+    float  *mass;           // log2-sums of the slots, for mass_finish_kernel
+    float  *lse_out;        // [split][n_q_total][Hq] log2-sum-exp of every row
+    float2 *bnd_out;        // with splits: [split][n_q_total][Hq] the split's part of the slot it shares with the split before it
+                            // (log2), and that slot (or -1)
+    int32_t *status;
+    int32_t n_q_total;
+    int32_t Hq, Hkv, rep;
+    int32_t mass_stride;
+    int32_t n_splits;
+    int32_t wait_first;     // as in AttnParams
+    float   scale_log2;
 };
 
 // Decode (one query token per episode): pages of the key stream one CTA may cover, and the most splits
@@ -182,6 +205,19 @@ inline cudaError_t launch_pdl_n(void (*kernel)(KArgs...), dim3 grid, dim3 block,
 }
 #endif
 
+// Parked log-sums -> masses, and their sums per object (see mass_finish_kernel)
+struct FinishParams {
+    float *mass;                // [n_q_total][Hq][mass_stride]: log2-sums of the slots, replaced by shares of the row's total
+    const float *lse;           // [split][n_q_total][Hq]
+    const float2 *bnd;          // [split][n_q_total][Hq] (only with splits)
+    const int32_t *row_slots;   // [n_q_total]: G_b of the row's episode, or null: max_slots
+    const int32_t *row_obj;     // [n_q_total]: object of every query row, -1 = none (only with mass_sum)
+    float *mass_sum;            // fp32 [n_obj][sum_stride] or null: added to
+    int32_t n_q_total, Hq, mass_stride, sum_stride, n_splits, max_slots;
+};
+constexpr int kFinishSplits = 8;
+cudaError_t launch_mass_finish(const FinishParams &p, cudaStream_t st);
+
 // Tensor map of a caller's [n][Hkv][D] bf16 keys or values with boxes of one head's 16 rows x 64 channels (in enl_host.cu)
 bool encode_key_map(CUtensorMap *tm, const void *base, int D, int Hkv, int n);
 
@@ -233,7 +269,9 @@ cudaError_t launch_page_copy(const uint8_t *src_k, const uint8_t *src_v, uint8_t
 // that the host would have to wait for, and (unlike a copy) it chains to its neighbours by programmatic dependent launch.
 constexpr int kPlanParamBytes = 28672;        // of the 32764 that a launch may carry
 cudaError_t launch_plan_write(void *dst, const void *src, size_t bytes, cudaStream_t st);
-size_t attention_smem_bytes(int head_dim);
+int attention_park_slots();
+cudaError_t launch_mass(const MassParams &p, int head_dim, int n_items, cudaStream_t st);
+cudaError_t prepare_mass(int head_dim);
 // Opts the attention kernel into its dynamic shared memory size on the current device.
 cudaError_t prepare_attention(int head_dim);
 // can the device run the head_dim-128 kernel as clusters of two CTAs (the in-kernel merge of two KV splits)?

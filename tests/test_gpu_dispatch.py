@@ -136,3 +136,40 @@ def test_static_step(D, rep, lens, n_new, shift):
     ks, vs = ([x[a:b].cpu() for a, b in zip(offs[:-1], offs[1:])] for x in (k, v))
     ro, rm = orc.attend_slots(hkv * rep, hkv, D, ks, vs, q[None].cpu(), k[offs[-1]:].cpu(), v[offs[-1]:].cpu())
     check_close(out[None], ro, mass[None], rm, what="static")
+
+
+# Masses without outputs: slots that end anywhere in a key tile, that reach over several splits, one Q tile and two, rows at
+# the causal limit, scores that jump by hundreds between tiles.
+MASS = {
+    "one_tile": dict(Hq=4, Hkv=1, D=128, pool=[[5, 16, 1]], n_q=[7], n_new=[7]),
+    "ragged": dict(Hq=8, Hkv=2, D=128, pool=[[1, 50, 16, 33, 7, 120, 15, 17, 300]], n_q=[77], n_new=[200]),
+    "slot_over_all_splits": dict(Hq=4, Hkv=2, D=64, pool=[[20, 2500, 3]], n_q=[130], n_new=[130]),
+    "many_slots": dict(Hq=8, Hkv=8, D=128, pool=[[1 + i % 9 for i in range(300)]], n_q=[129], n_new=[129]),
+    "batch": dict(Hq=16, Hkv=2, D=128, pool=[[30, 0, 90], [700, 5, 250], [200]], n_q=[70, 3, 129], n_new=[70, 10, 129]),
+}
+
+
+@pytest.mark.parametrize("split", [0, 1, 3, 8])
+@pytest.mark.parametrize("name", sorted(MASS))
+def test_masses_without_outputs(name, split):
+    c = MASS[name]
+    n = len(c["pool"])
+    wl = synth.make_small(47, 1, c["Hq"], c["Hkv"], c["D"], c["pool"], [list(range(len(x)))[::-1] for x in c["pool"]], c["n_q"],
+                          c["n_new"], name=name)
+    with Session(wl, [0]) as s:
+        q, kn, vn = wl.new_qkv(0, s.device)
+        if name == "ragged":
+            q = (q.float() * torch.linspace(1, 40, q.shape[0], device=s.device)[:, None, None]).to(q.dtype)
+        cs, cq, cn = wl.cu()
+        G = max(len(x) for x in wl.sel_local)
+        mass = torch.full((q.shape[0], wl.n_q_heads, G + 1), float("nan"), device=s.device)
+        enl.enl_attend(s.cache, 0, wl.sel_ids(), q, kn, vn, None, mass, cu_sel=cs if n > 1 else None, cu_q=cq if n > 1 else None,
+                       cu_new=cn if n > 1 else None, split_hint=split, flags=enl.ENL_MASS_ONLY)
+        torch.cuda.synchronize()
+        assert enl.enl_cache_status(s.cache) == enl.ENL_OK
+        for b in range(n):
+            rows = sorted({0, c["n_q"][b] // 2, c["n_q"][b] - 1, min(63, c["n_q"][b] - 1)})
+            _, rm, _ = s.oracle(0, b, q[cq[b]:cq[b + 1]], kn[cn[b]:cn[b + 1]], vn[cn[b]:cn[b + 1]], rows=rows)
+            g = len(wl.sel_local[b])
+            got = mass[cq[b]:cq[b + 1]][rows, :, :g + 1].cpu().numpy()
+            assert np.abs(got - rm).max() < 1e-4, f"{name} episode {b}"
