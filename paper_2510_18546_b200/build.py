@@ -11,7 +11,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libenl.so")
 BINDING = os.path.join(HERE, "_enl.so")
 BINDING_SOURCE = os.path.join(CSRC, "enl_py.c")
-SOURCES = ["enl_host.cu", "enl_attn_sm100.cu", "enl_attn_mass_sm100.cu", "enl_decode_sm100.cu", "enl_decode_cluster_sm100.cu", "enl_aux_kernels.cu", "enl_static_scratch.cu", "enl_cluster.cu", "enl_rope.cu", "enl_select.cpp"]
+SOURCES = ["enl_host.cu", "enl_attn_sm100.cu", "enl_attn_mass_sm100.cu", "enl_attn_small_sm100.cu", "enl_decode_sm100.cu", "enl_decode_cluster_sm100.cu", "enl_aux_kernels.cu", "enl_static_scratch.cu", "enl_cluster.cu", "enl_rope.cu", "enl_select.cpp"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-shared"]
 

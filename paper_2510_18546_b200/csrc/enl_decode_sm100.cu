@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(const __grid_consta
         const int4 *src = reinterpret_cast<const int4 *>(p.eps + it.ep);
         const int4 e0 = __ldg(src), e1 = __ldg(src + 1);
         ep.stream_off = e0.x; ep.n_ctiles = e0.y; ep.n_slots = e0.z; ep.q_off = e0.w;
-        ep.n_q = e1.x; ep.new_off = e1.y; ep.n_new = e1.z; ep.pad = e1.w;
+        ep.n_q = e1.x; ep.new_off = e1.y; ep.n_new = e1.z; ep.n_entries = e1.w;
     }
     if (threadIdx.x == 0) {
         asm volatile("prefetch.tensormap [%0];" ::"l"(&p.tm_kpool) : "memory");

@@ -152,6 +152,7 @@ struct enl_cache {
     bool plan_finish = false;               // else a kernel behind the attention kernel turns log-sums into masses
     std::vector<int32_t> key_obj;           // object spans the row -> object map was built from
     bool plan_decode = false;               // the plan is for the one-token decode kernel
+    int32_t plan_small_blocks = 0;          // > 0: the plan is for the kernel of short calls, with this many row blocks per kv head
     int32_t plan_cluster = 0;               // decode: CTAs per cluster, 0 = the streaming kernel
     int32_t plan_list_pages = 0;            // decode by clusters: most pages one of the CTAs covers
     ClusterCaps cluster_caps = {};          // decode by clusters: how many run at once (none on a bookkeeping-only cache)
@@ -331,6 +332,7 @@ extern "C" int enl_cache_create(const enl_cache_desc_t *desc, enl_cache_t **out)
         }
     }
     if (prepare_attention(d.head_dim) != cudaSuccess || prepare_decode(d.head_dim) != cudaSuccess || prepare_mass(d.head_dim) != cudaSuccess ||
+        prepare_small(d.head_dim) != cudaSuccess ||
         prepare_decode_cluster(d.head_dim, &c->cluster_caps) != cudaSuccess) { cudaGetLastError(); destroy(c); return ENL_E_CUDA; }
     c->pairs_ok = d.head_dim == 128 && attention_pairs_supported();   // else two splits go through the scratch buffer
     if (cudaDeviceSynchronize() != cudaSuccess) { cudaGetLastError(); destroy(c); return ENL_E_CUDA; }
@@ -689,12 +691,31 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
                 static_cast<int64_t>(B) * d.n_kv_heads * n_splits > c->cap_items)
                 decode = false;                                                    // too long for one merge: general kernel
         }
+        // Short calls: all the keys of an episode fit a CTA's shared memory and the row blocks fill the device at most once.
+        int small_blocks = 0;
+        if (!decode && c->gpu && a->split_hint == 0 && !mass_only && !has_sum) {
+            int64_t ctas = 0;
+            int pages = 0, blocks = 0;
+            for (int b = 0; b < B; ++b) {
+                int64_t e = 0;
+                for (int s = cu_sel[b]; s < cu_sel[b + 1]; ++s) e += std::max(1, ceil_div(sel_len[s], kPageTokens));
+                pages = static_cast<int>(std::min<int64_t>(0x7fffffff, std::max<int64_t>(pages, e + ceil_div(cu_new[b + 1] - cu_new[b], kPageTokens))));
+                const int n = ceil_div((cu_q[b + 1] - cu_q[b]) * c->rep, small_rows());
+                blocks = std::max(blocks, n);
+                ctas += static_cast<int64_t>(n) * d.n_kv_heads;
+            }
+            if (pages <= kSmallMaxPages && ctas <= c->n_sm) {
+                small_blocks = blocks;
+                list_pages = pages;
+            }
+        }
         if (!decode) {
             n_splits = 1;
             const bool few = base_items * 5 < c->n_sm * 4;         // a launch that leaves SMs idle splits the key stream
             // (two key tiles per split are worth it where the merge is cheap; the kernel that finishes masses takes a few us itself)
             const int filling = std::max(1, std::min(static_cast<int>(c->n_sm / base_items), min_tiles / (mass_only || has_sum ? 8 : 2)));
-            if (has_sum && !mass_only) n_splits = few && a->split_hint != 1 && c->pairs_ok && filling >= 2 ? 2 : 1;   // a pair or none
+            if (small_blocks) n_splits = 1;
+            else if (has_sum && !mass_only) n_splits = few && a->split_hint != 1 && c->pairs_ok && filling >= 2 ? 2 : 1;   // a pair or none
             else if (a->split_hint >= 1) n_splits = std::min(a->split_hint, std::max(1, min_tiles));   // no CTA without a tile
             else if (few) n_splits = filling;
             if (mass_only) {                                       // no outputs to merge: the kernel that finishes the masses adds the splits up
@@ -715,18 +736,19 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         // results through distributed shared memory: no scratch round trip and no merge kernel.  Every CTA must
         // have at least one tile, and the items of a pair must be neighbours (they are: same tile count, stable sort).
         const bool pair = !decode && !mass_only && n_splits == 2 && d.head_dim == 128 && min_tiles >= 2 && (c->pairs_ok || !c->gpu);
+        const bool by_grid = decode || small_blocks > 0;               // kernels that take their CTA's place from the grid
         const int64_t n_items = decode ? static_cast<int64_t>(B) * d.n_kv_heads * n_splits : base_items * n_splits;
         {   // sections: what the kernels of this plan read (the decode kernel takes its CTA's place from the grid)
             auto align16 = [](size_t x) { return (x + 15) & ~static_cast<size_t>(15); };
             size_t at = 0;
             auto section = [&](size_t bytes) { const size_t o = at; at += align16(bytes); return o; };
             c->off_eps = section(sizeof(EpInfo) * B);
-            c->off_items = section(decode ? 0 : sizeof(Item) * n_items);
+            c->off_items = section(by_grid ? 0 : sizeof(Item) * n_items);
             c->off_stream = section(sizeof(int32_t) * n_entries);
             c->off_meta = section(sizeof(int32_t) * n_entries);
             const bool merged = n_splits > 1 && !pair && !mass_only;
             c->off_words = section(mass_only ? sizeof(int2) * (n_entries / kPagesPerTile) : 0);
-            c->off_rowslots = section(!decode && (merged || (has_mass && B > 1)) ? sizeof(int32_t) * a->n_q : 0);
+            c->off_rowslots = section(!by_grid && (merged || (has_mass && B > 1)) ? sizeof(int32_t) * a->n_q : 0);
             c->off_rowobj = section(has_sum ? sizeof(int32_t) * a->n_q : 0);
             c->plan_used = at;
         }
@@ -743,7 +765,6 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
             e.n_q = cu_q[b + 1] - cu_q[b];
             e.new_off = cu_new[b];
             e.n_new = cu_new[b + 1] - cu_new[b];
-            e.pad = 0;
             for (int s = cu_sel[b]; s < cu_sel[b + 1]; ++s) {
                 const int slot = s - cu_sel[b];
                 const Group &g = c->groups[a->sel_ids[s]];
@@ -755,6 +776,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
                     smeta[ne++] = (slot << 8) | nv;
                 }
             }
+            e.n_entries = ne - e.stream_off;
             while ((ne - e.stream_off) % kPagesPerTile) { stream[ne] = kZeroPage; smeta[ne++] = (e.n_slots - 1) << 8; }
             e.n_ctiles = (ne - e.stream_off) / kPagesPerTile;
             for (int j = 0; j < e.n_ctiles && mass_only; ++j) {
@@ -767,7 +789,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
                 }
                 c->h_words()[e.stream_off / kPagesPerTile + j] = make_int2(static_cast<int>(keys), static_cast<int>(hide | chg << 8));
             }
-            if (!decode && ((n_splits > 1 && !pair && !mass_only) || (has_mass && B > 1)))
+            if (!by_grid && ((n_splits > 1 && !pair && !mass_only) || (has_mass && B > 1)))
                 for (int r = e.q_off; r < e.q_off + e.n_q; ++r) rowslots[r] = e.n_slots;
         }
         if (has_sum) {
@@ -779,7 +801,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         } else {
             c->key_obj.clear();
         }
-        if (!decode) {
+        if (!by_grid) {
             // CTAs, heaviest first (late token blocks see more new-token tiles)
             struct Work { Item it; int tiles; };
             std::vector<Work> work;
@@ -809,8 +831,9 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         c->plan_mass_only = mass_only;
         c->plan_sums = has_sum;
         const bool merged = !decode && n_splits > 1 && !pair && !mass_only;
+        c->plan_small_blocks = small_blocks;
         c->plan_park = has_mass && !mass_only && (!has_sum || merged) && max_slots + 1 <= attention_park_slots();
-        c->plan_finish = has_mass && !decode && !c->plan_park && !merged;
+        c->plan_finish = has_mass && !by_grid && !c->plan_park && !merged;
         c->plan_decode = decode;
         c->plan_cluster = cluster;
         c->plan_list_pages = list_pages;
@@ -848,7 +871,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
     c->pool_written = false;
 
     const int slot_stride = c->plan_max_slots + 1;
-    if (c->plan_decode && c->plan_cluster) {
+    if (c->plan_small_blocks || (c->plan_decode && c->plan_cluster)) {
         ClusterDecodeParams dp;
         std::memset(&dp, 0, sizeof dp);
         const cuuint64_t nd[3] = {static_cast<cuuint64_t>(d.head_dim), static_cast<cuuint64_t>(d.n_kv_heads),
@@ -876,7 +899,8 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         dp.list_slots = std::min(c->plan_list_pages, c->plan_max_slots + 1);
         dp.wait_first = wait_first ? 1 : 0;
         dp.scale_log2 = 1.4426950408889634f / sqrtf(static_cast<float>(d.head_dim));
-        if (launch_decode_cluster(dp, d.head_dim, c->plan_batch, c->plan_cluster, st) != cudaSuccess) { cudaGetLastError(); return ENL_E_CUDA; }
+        if ((c->plan_small_blocks ? launch_small(dp, d.head_dim, c->plan_small_blocks, c->plan_batch, st)
+                                  : launch_decode_cluster(dp, d.head_dim, c->plan_batch, c->plan_cluster, st)) != cudaSuccess) { cudaGetLastError(); return ENL_E_CUDA; }
         return ENL_OK;
     }
     if (c->plan_decode) {

@@ -21,7 +21,7 @@ struct EpInfo {
     int32_t n_slots;        // selected groups G_b; mass slot G_b = new tokens
     int32_t q_off, n_q;     // first query row (global) and count
     int32_t new_off, n_new; // first new-token key (global) and count
-    int32_t pad;
+    int32_t n_entries;      // stream entries without the null ones that fill the last tile
 };
 
 // One CTA of the attention launch.
@@ -133,6 +133,7 @@ struct ClusterDecodeParams {
     int32_t *status;
     int32_t Hq, Hkv, rep;
     int32_t mass_stride;
+    // (the small kernel takes these parameters too; its list is every page that a CTA's rows see)
     int32_t list_pages;     // most pages a CTA of this launch covers, and most slots they can touch (sizes of its lists)
     int32_t list_slots;
     int32_t wait_first;     // as in AttnParams
@@ -230,6 +231,11 @@ cudaError_t prepare_decode(int head_dim);
 cudaError_t launch_decode_cluster(const ClusterDecodeParams &p, int head_dim, int batch, int cluster, cudaStream_t st);
 cudaError_t launch_decode_static(const StaticDecodeParams &p, int head_dim, int cluster, cudaStream_t st);
 constexpr int kClusterMaxPages = 288;         // pages of a CTA of these kernels
+// Short calls (see enl_attn_small_sm100.cu): every page a CTA sees in shared memory at once.
+constexpr int kSmallMaxPages = 24;
+int small_rows();                             // query rows (tokens x q heads of a kv head) per CTA
+cudaError_t prepare_small(int head_dim);
+cudaError_t launch_small(const ClusterDecodeParams &p, int head_dim, int row_blocks, int batch, cudaStream_t st);
 int decode_cluster_smem(int head_dim, int list_pages, int list_slots, int rep);
 constexpr int kClusterPairSmem = 113800;      // two CTAs of up to this much fit an SM
 // How many clusters of 2^i CTAs the current device runs at once: with two CTAs per SM, and with one (larger lists).

@@ -173,3 +173,42 @@ def test_masses_without_outputs(name, split):
             g = len(wl.sel_local[b])
             got = mass[cq[b]:cq[b + 1]][rows, :, :g + 1].cpu().numpy()
             assert np.abs(got - rm).max() < 1e-4, f"{name} episode {b}"
+
+
+# Short calls: rows at the edges of a CTA's 64, key streams up to the 24 pages that stay resident and one beyond, empty lists and groups, every number
+# of q heads per kv head, episodes of different sizes, queries that are only the last of the new tokens.
+SHORT = {
+    "one_row_pair": dict(Hq=2, Hkv=2, D=64, pool=[[3]], sel=[[0]], n_q=[2], n_new=[2]),
+    "rows_63": dict(Hq=2, Hkv=2, D=128, pool=[[40, 17]], sel=[[1, 0]], n_q=[63], n_new=[63]),
+    "rows_64": dict(Hq=8, Hkv=2, D=128, pool=[[40, 17]], sel=[[0, 1]], n_q=[16], n_new=[16]),
+    "rows_65": dict(Hq=1, Hkv=1, D=64, pool=[[40, 17]], sel=[[0, 1]], n_q=[65], n_new=[65]),
+    "rep16": dict(Hq=32, Hkv=2, D=128, pool=[[33, 50]], sel=[[0, 1]], n_q=[9], n_new=[9]),
+    "rep8": dict(Hq=32, Hkv=4, D=64, pool=[[33, 50]], sel=[[0, 1]], n_q=[41], n_new=[41]),
+    "pages_24": dict(Hq=32, Hkv=8, D=128, pool=[[160, 128]], sel=[[0, 1]], n_q=[61], n_new=[96]),
+    "pages_25": dict(Hq=32, Hkv=8, D=128, pool=[[160, 128]], sel=[[0, 1]], n_q=[61], n_new=[97]),
+    "slots_as_pages": dict(Hq=8, Hkv=2, D=128, pool=[[1] * 20], sel=[list(range(20))], n_q=[30], n_new=[30]),
+    "empty_select": dict(Hq=8, Hkv=2, D=128, pool=[[10]], sel=[[]], n_q=[100], n_new=[100]),
+    "empty_groups": dict(Hq=8, Hkv=2, D=64, pool=[[0, 0, 40, 0, 5, 0]], sel=[[0, 1, 2, 3, 4, 5]], n_q=[20], n_new=[20]),
+    "prior": dict(Hq=8, Hkv=2, D=128, pool=[[30]], sel=[[0]], n_q=[5], n_new=[200]),
+    "batch": dict(Hq=8, Hkv=2, D=128, pool=[[30, 60, 90], [5, 5, 5, 5], [200]], sel=[[2, 0], [0, 1, 2, 3], []],
+                  n_q=[70, 3, 129], n_new=[70, 10, 129]),
+}
+
+
+@pytest.mark.parametrize("want_mass", [True, False])
+@pytest.mark.parametrize("name", sorted(SHORT))
+def test_short_calls(name, want_mass):
+    c = SHORT[name]
+    wl = synth.make_small(53, 1, c["Hq"], c["Hkv"], c["D"], c["pool"], c["sel"], c["n_q"], c["n_new"], name=name)
+    with Session(wl, [0]) as s:
+        q, kn, vn = wl.new_qkv(0, s.device)
+        q = q * 3
+        _, cq, cn = wl.cu()
+        for _ in range(2):                                  # the second call finds plan and pool as the first left them
+            out, mass, _ = s.attend(0, q, kn, vn, want_mass=want_mass)
+        torch.cuda.synchronize()
+        assert enl.enl_cache_status(s.cache) == enl.ENL_OK
+        for b in range(wl.batch):
+            ro, rm, _ = s.oracle(0, b, q[cq[b]:cq[b + 1]], kn[cn[b]:cn[b + 1]], vn[cn[b]:cn[b + 1]])
+            G = len(wl.sel_local[b])
+            check_close(out[cq[b]:cq[b + 1]], ro, mass[cq[b]:cq[b + 1], :, :G + 1] if want_mass else None, rm if want_mass else None, what=name)
