@@ -4,12 +4,13 @@
 // Same computation and row layout as enl_attn_sm100.cu.  There such a call took 11 us for two key tiles: 3 us a tile through
 // a chain of roles (loader, MMA issuer, softmax warps, accumulator in TMEM) whose unrolled code is fetched anew by every
 // launch, and 2 us of epilogue.  The tensor work is nothing here (0.1 us of the pipe), so this kernel has no roles and little
-// code: a CTA takes 64 query rows of one kv head, loads every page of K and V the rows can see at once (they fit shared
-// memory: up to kSmallMaxPages pages), and its 12 warps are 4 row groups x 3 key ranges, each walking its pages with everything in registers:
+// code: a CTA takes 16, 32 or 64 query rows of one kv head, loads every page of K and V the rows can see at once (they fit
+// shared memory: up to kSmallMaxPages pages), and its 12 warps are 1, 2 or 4 row groups x 12, 6 or 3 key ranges, each walking
+// its pages with everything in registers (the fewest rows with which all the CTAs run at once: a page costs a warp 0.5 us):
 //   S = Q K^T      mma.sync m16n8k16, A = 16 query rows, B = the K page (ldmatrix)
 //   p = exp2(S-m)  running maximum per row kept by the warp, O and the sums rescaled when it grows
 //   O += P V       A = P straight from the S accumulators, B = the V page (ldmatrix.trans)
-// then the three ranges are merged through shared memory (their outputs lie where the pages lay).  A range's pages are in
+// then the ranges are merged through shared memory (their outputs lie where the pages lay).  A range's pages are in
 // stream order, so a row has one open slot; its log2-sum is parked when it ends.
 // When neither plan nor pool have been written since the last attention launch the cached pages are fetched before the wait
 // for the previous kernel.
@@ -22,11 +23,8 @@
 namespace enl {
 namespace {
 
-constexpr int kRowGroups = 4;                             // of 16 rows
-constexpr int kKeyRanges = 3;
-constexpr int kWarps     = kRowGroups * kKeyRanges;
+constexpr int kWarps     = 12;
 constexpr int kThreads   = kWarps * 32;
-constexpr int kRows      = kRowGroups * 16;               // query rows per CTA
 constexpr float kRescaleThreshold = 8.0f;                 // log2 units
 
 __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
@@ -51,10 +49,13 @@ __device__ __forceinline__ void plain_load_3d(uint32_t dst, const CUtensorMap *t
 
 // Shared memory: pages [K, V] (later the ranges' outputs) | barriers | page list | per range and row (m, l) | row log-sum-exp |
 // parked log-sums [range][slot][row]
-template <int D>
+// kRowGroups: groups of 16 query rows per CTA
+template <int D, int kRowGroups>
 struct Cfg {
+    static constexpr int kKeyRanges  = kWarps / kRowGroups;
+    static constexpr int kRows       = kRowGroups * 16;
     static constexpr int kStageBytes = D * kPageTokens * 2;            // one page of one head
-    static constexpr int kORow       = D + 4;                          // row of a range's output: no two rows of a store share banks
+    static constexpr int kORow       = D + 8;                          // row of a range's output: no two rows of a store share banks
     static constexpr int kOutBytes   = kKeyRanges * kRows * kORow * 4;
     static __host__ __device__ constexpr int pages_bytes(int pages)
     {
@@ -69,10 +70,11 @@ struct Cfg {
     }
 };
 
-template <int D>
+template <int D, int kRowGroups>
 __global__ void __launch_bounds__(kThreads, 1) small_kernel(const __grid_constant__ ClusterDecodeParams p)
 {
-    using C = Cfg<D>;
+    using C = Cfg<D, kRowGroups>;
+    constexpr int kKeyRanges = C::kKeyRanges, kRows = C::kRows;
     constexpr int kHalves = D / 64;                       // TMA boxes (64 channels) per page
     constexpr int kSteps  = D / 16;                       // k16 steps of Q K^T
     constexpr int kNB     = D / 8;                        // 8-channel blocks of O
@@ -343,25 +345,40 @@ __global__ void __launch_bounds__(kThreads, 1) small_kernel(const __grid_constan
 
 }  // namespace
 
+namespace {
+template <int D>
+cudaError_t opt_in()
+{
+    cudaError_t e = cudaFuncSetAttribute(small_kernel<D, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<D, 1>::smem_bytes(kSmallMaxPages));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(small_kernel<D, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<D, 2>::smem_bytes(kSmallMaxPages));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(small_kernel<D, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<D, 4>::smem_bytes(kSmallMaxPages));
+    return e;
+}
+template <int D>
+cudaError_t launch(const ClusterDecodeParams &p, int row_groups, dim3 grid, cudaStream_t st)
+{
+    if (row_groups == 1) return launch_pdl(small_kernel<D, 1>, grid, dim3(kThreads), Cfg<D, 1>::smem_bytes(p.list_pages), st, p);
+    if (row_groups == 2) return launch_pdl(small_kernel<D, 2>, grid, dim3(kThreads), Cfg<D, 2>::smem_bytes(p.list_pages), st, p);
+    return launch_pdl(small_kernel<D, 4>, grid, dim3(kThreads), Cfg<D, 4>::smem_bytes(p.list_pages), st, p);
+}
+}  // namespace
+
 cudaError_t prepare_small(int head_dim)
 {
-    if (head_dim == 128)
-        return cudaFuncSetAttribute(small_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<128>::smem_bytes(kSmallMaxPages));
-    if (head_dim == 64)
-        return cudaFuncSetAttribute(small_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<64>::smem_bytes(kSmallMaxPages));
+    if (head_dim == 128) return opt_in<128>();
+    if (head_dim == 64) return opt_in<64>();
     return cudaErrorInvalidValue;
 }
 
-int small_rows() { return kRows; }
-
-cudaError_t launch_small(const ClusterDecodeParams &p, int head_dim, int row_blocks, int batch, cudaStream_t st)
+cudaError_t launch_small(const ClusterDecodeParams &p, int head_dim, int row_groups, int row_blocks, int batch, cudaStream_t st)
 {
     if (batch <= 0 || row_blocks <= 0) return cudaSuccess;
-    if (p.list_pages > kSmallMaxPages || kRows % p.rep) return cudaErrorInvalidValue;
+    if (p.list_pages > kSmallMaxPages || (16 * row_groups) % p.rep || (row_groups != 1 && row_groups != 2 && row_groups != 4))
+        return cudaErrorInvalidValue;
     const dim3 grid(row_blocks, p.Hkv, batch);
     cudaError_t e;
-    if (head_dim == 128) e = launch_pdl(small_kernel<128>, grid, dim3(kThreads), Cfg<128>::smem_bytes(p.list_pages), st, p);
-    else if (head_dim == 64) e = launch_pdl(small_kernel<64>, grid, dim3(kThreads), Cfg<64>::smem_bytes(p.list_pages), st, p);
+    if (head_dim == 128) e = launch<128>(p, row_groups, grid, st);
+    else if (head_dim == 64) e = launch<64>(p, row_groups, grid, st);
     else return cudaErrorInvalidValue;
     return e != cudaSuccess ? e : cudaGetLastError();
 }

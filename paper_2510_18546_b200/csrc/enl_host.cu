@@ -153,6 +153,7 @@ struct enl_cache {
     std::vector<int32_t> key_obj;           // object spans the row -> object map was built from
     bool plan_decode = false;               // the plan is for the one-token decode kernel
     int32_t plan_small_blocks = 0;          // > 0: the plan is for the kernel of short calls, with this many row blocks per kv head
+    int32_t plan_small_groups = 0;          // ... of this many times 16 rows
     int32_t plan_cluster = 0;               // decode: CTAs per cluster, 0 = the streaming kernel
     int32_t plan_list_pages = 0;            // decode by clusters: most pages one of the CTAs covers
     ClusterCaps cluster_caps = {};          // decode by clusters: how many run at once (none on a bookkeeping-only cache)
@@ -692,20 +693,25 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
                 decode = false;                                                    // too long for one merge: general kernel
         }
         // Short calls: all the keys of an episode fit a CTA's shared memory and the row blocks fill the device at most once.
-        int small_blocks = 0;
+        int small_blocks = 0, small_groups = 0;
         if (!decode && c->gpu && a->split_hint == 0 && !mass_only && !has_sum) {
-            int64_t ctas = 0;
-            int pages = 0, blocks = 0;
+            int pages = 0;
             for (int b = 0; b < B; ++b) {
                 int64_t e = 0;
                 for (int s = cu_sel[b]; s < cu_sel[b + 1]; ++s) e += std::max(1, ceil_div(sel_len[s], kPageTokens));
                 pages = static_cast<int>(std::min<int64_t>(0x7fffffff, std::max<int64_t>(pages, e + ceil_div(cu_new[b + 1] - cu_new[b], kPageTokens))));
-                const int n = ceil_div((cu_q[b + 1] - cu_q[b]) * c->rep, small_rows());
-                blocks = std::max(blocks, n);
-                ctas += static_cast<int64_t>(n) * d.n_kv_heads;
             }
-            if (pages <= kSmallMaxPages && ctas <= c->n_sm) {
+            for (int rg = 1; rg <= 4 && pages <= kSmallMaxPages && !small_blocks; rg *= 2) {
+                int64_t ctas = 0;
+                int blocks = 0;
+                for (int b = 0; b < B; ++b) {
+                    const int n = ceil_div((cu_q[b + 1] - cu_q[b]) * c->rep, 16 * rg);
+                    blocks = std::max(blocks, n);
+                    ctas += static_cast<int64_t>(n) * d.n_kv_heads;
+                }
+                if (ctas > c->n_sm) continue;
                 small_blocks = blocks;
+                small_groups = rg;
                 list_pages = pages;
             }
         }
@@ -832,6 +838,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         c->plan_sums = has_sum;
         const bool merged = !decode && n_splits > 1 && !pair && !mass_only;
         c->plan_small_blocks = small_blocks;
+        c->plan_small_groups = small_groups;
         c->plan_park = has_mass && !mass_only && (!has_sum || merged) && max_slots + 1 <= attention_park_slots();
         c->plan_finish = has_mass && !by_grid && !c->plan_park && !merged;
         c->plan_decode = decode;
@@ -899,7 +906,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         dp.list_slots = std::min(c->plan_list_pages, c->plan_max_slots + 1);
         dp.wait_first = wait_first ? 1 : 0;
         dp.scale_log2 = 1.4426950408889634f / sqrtf(static_cast<float>(d.head_dim));
-        if ((c->plan_small_blocks ? launch_small(dp, d.head_dim, c->plan_small_blocks, c->plan_batch, st)
+        if ((c->plan_small_blocks ? launch_small(dp, d.head_dim, c->plan_small_groups, c->plan_small_blocks, c->plan_batch, st)
                                   : launch_decode_cluster(dp, d.head_dim, c->plan_batch, c->plan_cluster, st)) != cudaSuccess) { cudaGetLastError(); return ENL_E_CUDA; }
         return ENL_OK;
     }

@@ -233,9 +233,9 @@ cudaError_t launch_decode_static(const StaticDecodeParams &p, int head_dim, int 
 constexpr int kClusterMaxPages = 288;         // pages of a CTA of these kernels
 // Short calls (see enl_attn_small_sm100.cu): every page a CTA sees in shared memory at once.
 constexpr int kSmallMaxPages = 24;
-int small_rows();                             // query rows (tokens x q heads of a kv head) per CTA
 cudaError_t prepare_small(int head_dim);
-cudaError_t launch_small(const ClusterDecodeParams &p, int head_dim, int row_blocks, int batch, cudaStream_t st);
+// row_groups: 1, 2 or 4 groups of 16 query rows (tokens x q heads of a kv head) per CTA
+cudaError_t launch_small(const ClusterDecodeParams &p, int head_dim, int row_groups, int row_blocks, int batch, cudaStream_t st);
 int decode_cluster_smem(int head_dim, int list_pages, int list_slots, int rep);
 constexpr int kClusterPairSmem = 113800;      // two CTAs of up to this much fit an SM
 // How many clusters of 2^i CTAs the current device runs at once: with two CTAs per SM, and with one (larger lists).
