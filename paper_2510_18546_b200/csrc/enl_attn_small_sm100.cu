@@ -14,7 +14,8 @@
 // stream order, so a row has one open slot; its log2-sum is parked when it ends.
 // When neither plan nor pool have been written since the last attention launch the cached pages are fetched before the wait
 // for the previous kernel.
-// Measured per launch in a chain of layers (D 128, 32 q / 8 kv heads): MEASURED_SMALL
+// Measured per launch in a chain of layers (D 128, 32 q / 8 kv heads, large kernel -> this one): 41 rows over 121 keys 10.4 -> 6.9 us,
+// 61 over 301 12.9 -> 8.6, 128 over 308 14.4 -> 9.4, 256 over 276 13.6 -> 11.5.
 #include <cuda_bf16.h>
 
 #include "decode_ops.cuh"

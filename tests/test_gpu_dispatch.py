@@ -212,3 +212,18 @@ def test_short_calls(name, want_mass):
             ro, rm, _ = s.oracle(0, b, q[cq[b]:cq[b + 1]], kn[cn[b]:cn[b + 1]], vn[cn[b]:cn[b + 1]])
             G = len(wl.sel_local[b])
             check_close(out[cq[b]:cq[b + 1]], ro, mass[cq[b]:cq[b + 1], :, :G + 1] if want_mass else None, rm if want_mass else None, what=name)
+
+
+@pytest.mark.parametrize("interleaved", [False, True])
+@pytest.mark.parametrize("heads, D, n", [(32, 128, 5), (8, 128, 5), (1, 16, 9), (3, 48, 7), (2, 256, 3), (2, 24, 6), (40, 256, 2)])
+def test_rope_pieces(heads, D, n, interleaved):
+    """Sizes around the rows and heads that a CTA takes, and head sizes that do not split into 16-byte pieces."""
+    gen = torch.Generator(device="cuda").manual_seed(D)
+    x = torch.randn(n, heads, D, generator=gen, device="cuda").to(torch.bfloat16)
+    pos = torch.tensor([(i * 7919) % 120_000 for i in range(n)], dtype=torch.int32, device="cuda")
+    want = orc.rope_rotate(x.float().cpu().numpy(), pos.cpu().numpy(), 10000.0, interleaved)
+    got = x.clone()
+    enl.enl_rope_rotate(got, positions=pos, interleaved=interleaved)
+    torch.cuda.synchronize()
+    err = np.abs(got.float().cpu().numpy() - want)
+    assert (err <= np.maximum(np.abs(want) * 2.0 ** -8, 1e-4)).all(), err.max()
