@@ -183,7 +183,8 @@ __global__ void __launch_bounds__(kThreads, 1) small_kernel(const __grid_constan
     for (int nb = 0; nb < kNB; ++nb) { o[nb][0] = o[nb][1] = o[nb][2] = o[nb][3] = 0.f; }
     float m[2] = {kNegInf, kNegInf};                                          // references of the two rows (the same in a quad)
     float l[2] = {0.f, 0.f}, acc[2] = {0.f, 0.f};                             // lane-local parts of the row sums and of the open slot's
-    const int pg_beg = total * kr / kKeyRanges, pg_end = total * (kr + 1) / kKeyRanges;
+    const int n_ranges = min(total, kKeyRanges);                              // no range without a page
+    const int pg_beg = kr < n_ranges ? total * kr / n_ranges : total, pg_end = kr < n_ranges ? total * (kr + 1) / n_ranges : total;
     const int slot_first = pg_end > pg_beg ? pg_list[pg_beg].y >> 8 : 0;
     int cur_slot = slot_first;
     bool ok = true;
@@ -290,26 +291,28 @@ __global__ void __launch_bounds__(kThreads, 1) small_kernel(const __grid_constan
     __syncthreads();                                                          // every page has been read: the outputs may go there
     if (*abort_flag) return;
     float *obuf = reinterpret_cast<float *>(smem);                            // [range][row][kORow]
+    if (kr < n_ranges) {
 #pragma unroll
-    for (int nb = 0; nb < kNB; ++nb) {
-        *reinterpret_cast<float2 *>(obuf + (kr * kRows + r0) * C::kORow + nb * 8 + 2 * tq) = make_float2(o[nb][0], o[nb][1]);
-        *reinterpret_cast<float2 *>(obuf + (kr * kRows + r1) * C::kORow + nb * 8 + 2 * tq) = make_float2(o[nb][2], o[nb][3]);
+        for (int nb = 0; nb < kNB; ++nb) {
+            *reinterpret_cast<float2 *>(obuf + (kr * kRows + r0) * C::kORow + nb * 8 + 2 * tq) = make_float2(o[nb][0], o[nb][1]);
+            *reinterpret_cast<float2 *>(obuf + (kr * kRows + r1) * C::kORow + nb * 8 + 2 * tq) = make_float2(o[nb][2], o[nb][3]);
+        }
     }
     // weights of the ranges (exp2(m - lse): they take the unnormalised outputs straight to the result)
-    if (threadIdx.x < kRows) {
-        const int r = threadIdx.x;
-        float mm[kKeyRanges], M = kNegInf, L = 0.f;
+    constexpr int kLanes = kKeyRanges > 8 ? 16 : kKeyRanges > 4 ? 8 : 4;      // lanes per row, one range each
+    {
+        const int r = threadIdx.x / kLanes, k = lane % kLanes;                // kRows * kLanes = 256
+        const bool on = r < kRows && k < n_ranges;
+        const float mk = on ? wm[k * kRows + r] : kNegInf;
+        float M = mk;
 #pragma unroll
-        for (int k = 0; k < kKeyRanges; ++k) { mm[k] = wm[k * kRows + r]; M = fmaxf(M, mm[k]); }
+        for (int of = kLanes / 2; of > 0; of >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, of));
+        const float f = (mk == kNegInf) ? 0.f : ex2(mk - M);
+        float L = on ? f * wl[k * kRows + r] : 0.f;
 #pragma unroll
-        for (int k = 0; k < kKeyRanges; ++k) {
-            mm[k] = (mm[k] == kNegInf) ? 0.f : ex2(mm[k] - M);
-            L += mm[k] * wl[k * kRows + r];
-        }
-        const float inv = (L > 0.f) ? 1.f / L : 0.f;
-#pragma unroll
-        for (int k = 0; k < kKeyRanges; ++k) wm[k * kRows + r] = mm[k] * inv;
-        lse[r] = (L > 0.f) ? M + lg2(L) : kNegInf;
+        for (int of = kLanes / 2; of > 0; of >>= 1) L += __shfl_xor_sync(0xffffffffu, L, of);
+        if (on) wm[k * kRows + r] = (L > 0.f) ? f / L : 0.f;
+        if (on && k == 0) lse[r] = (L > 0.f) ? M + lg2(L) : kNegInf;
     }
     __syncthreads();
     const long long row_h0 = static_cast<long long>(ep.q_off + t0) * p.Hq + kvh * rep;        // + (r / rep) * Hq + r % rep
@@ -319,6 +322,7 @@ __global__ void __launch_bounds__(kThreads, 1) small_kernel(const __grid_constan
         float a[8] = {};
 #pragma unroll
         for (int k = 0; k < kKeyRanges; ++k) {
+            if (k >= n_ranges) break;
             const float w = wm[k * kRows + r];
             const float4 *src = reinterpret_cast<const float4 *>(obuf + (k * kRows + r) * C::kORow + c8 * 8);
             const float4 x = src[0], y = src[1];
@@ -333,10 +337,8 @@ __global__ void __launch_bounds__(kThreads, 1) small_kernel(const __grid_constan
     for (int idx = threadIdx.x; idx < n_rows * (G + 1); idx += kThreads) {
         const int r = idx / (G + 1), s = idx % (G + 1);
         float w = 0.f;
-#pragma unroll
-        for (int k = 0; k < kKeyRanges; ++k) {
-            const int b = total * k / kKeyRanges, e = total * (k + 1) / kKeyRanges;
-            if (e <= b) continue;
+        for (int k = 0; k < n_ranges; ++k) {
+            const int b = total * k / n_ranges, e = total * (k + 1) / n_ranges;
             const int first = pg_list[b].y >> 8, last = pg_list[e - 1].y >> 8;
             if (s >= first && s <= last) w += ex2(parked[(k * range_slots + s - first) * kRows + r] - lse[r]);
         }
