@@ -67,10 +67,11 @@ __device__ __forceinline__ float ex2f(float x)
     return y;
 }
 
-// One warp per (query row, q head): lane l merges channels 4l..4l+3 (D = 128) or 2l, 2l+1 (D = 64),
-// then the lanes stride over the slots.
-template <int D>
-__global__ void combine_kernel(const CombineParams p)
+// One warp per (query row, q head): lane l merges channels 4l..4l+3 (D = 128) or 2l, 2l+1 (D = 64), and slot l, l + 32, ...
+// Splits are taken kBatch at a time, their partial outputs and the log-sums of 32 slots on the way together, the first ones with
+// the log-sum-exps: up to eight splits cost one memory round trip (four or fewer are not charged for eight).
+template <int D, int kBatch>
+__global__ void __launch_bounds__(256) combine_kernel(const CombineParams p)
 {
     constexpr int V = D / 32;                               // channels per lane
     const int lane = threadIdx.x & 31;
@@ -79,71 +80,29 @@ __global__ void combine_kernel(const CombineParams p)
     pdl_trigger();
     pdl_wait();                                             // the partial results come from the previous kernel
     if (rh >= split_stride) return;
-    const int row = static_cast<int>(rh / p.Hq);
     const float ninf = -__builtin_huge_valf();
-
-    // Few splits (the usual case): every load of the warp -- log-sum-exps, partial outputs, the first 32 slot
-    // log-sums -- is issued before anything is computed, so the warp pays one memory round trip, not five.
-    if (p.n_splits <= 4) {
-        const float *slot0 = p.part_slot ? p.part_slot + rh * p.slot_stride + lane : nullptr;
-        const int G = p.mass ? p.row_slots[row] : -1;
-        float lv[4], sv[4], ov[4][V];
+    const int G = p.mass ? p.row_slots[static_cast<int>(rh / p.Hq)] : -1;
+    const float *o0 = p.part_o + rh * D + lane * V;
+    const float *s0 = p.part_slot ? p.part_slot + rh * p.slot_stride + lane : nullptr;
+    float ov[kBatch][V], sv[kBatch];
+    auto fetch = [&](int k0) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const bool on = k < p.n_splits;
-            lv[k] = on ? __ldcg(p.part_lse + k * split_stride + rh) : ninf;
-            sv[k] = (on && p.mass && lane <= G) ? __ldcg(slot0 + k * split_stride * p.slot_stride) : ninf;
-            const float *src = p.part_o + ((on ? k : 0) * split_stride + rh) * D + lane * V;
+        for (int j = 0; j < kBatch; ++j) {
+            const int k = k0 + j < p.n_splits ? k0 + j : 0; // (a split beyond the last has weight 0)
             if constexpr (V == 4) {
-                const float4 t = __ldcg(reinterpret_cast<const float4 *>(src));
-                ov[k][0] = t.x; ov[k][1] = t.y; ov[k][2] = t.z; ov[k][3] = t.w;
+                const float4 t = __ldcg(reinterpret_cast<const float4 *>(o0 + k * split_stride * D));
+                ov[j][0] = t.x; ov[j][1] = t.y; ov[j][2] = t.z; ov[j][3] = t.w;
             } else {
-                const float2 t = __ldcg(reinterpret_cast<const float2 *>(src));
-                ov[k][0] = t.x; ov[k][1] = t.y;
+                const float2 t = __ldcg(reinterpret_cast<const float2 *>(o0 + k * split_stride * D));
+                ov[j][0] = t.x; ov[j][1] = t.y;
             }
+            sv[j] = (lane <= G && k0 + j < p.n_splits) ? __ldcg(s0 + k * split_stride * p.slot_stride) : ninf;
         }
-        const float mxv = fmaxf(fmaxf(lv[0], lv[1]), fmaxf(lv[2], lv[3]));
-        float sum = 0.f;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) sum += (lv[k] != ninf) ? ex2f(lv[k] - mxv) : 0.f;
-        const float lse = mxv + log2f(sum);
-        const float lse_s = (lse > ninf) ? lse : 0.f;
-        float acc[V];
-#pragma unroll
-        for (int x = 0; x < V; ++x) acc[x] = 0.f;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            // a split that saw no key has weight 0 and never wrote its partial output: what sits there is stale
-            const float w = (lv[k] != ninf) ? ex2f(lv[k] - lse) : 0.f;
-#pragma unroll
-            for (int x = 0; x < V; ++x) acc[x] = (w != 0.f) ? fmaf(w, ov[k][x], acc[x]) : acc[x];
-        }
-        __nv_bfloat16 *dst = static_cast<__nv_bfloat16 *>(p.out) + rh * D + lane * V;
-#pragma unroll
-        for (int x = 0; x < V; x += 2)
-            *reinterpret_cast<__nv_bfloat162 *>(dst + x) = __floats2bfloat162_rn(acc[x], acc[x + 1]);
-        if (p.mass) {
-            if (lane <= G) {
-                float w = 0.f;
-#pragma unroll
-                for (int k = 0; k < 4; ++k) w += ex2f(sv[k] - lse_s);       // exp2(-inf) = 0: absent slots drop out
-                p.mass[rh * p.mass_stride + lane] = w;
-            }
-            for (int s = lane + 32; s <= G; s += 32) {                      // more than 32 slots: the rest, as below
-                float w = 0.f;
-                for (int k = 0; k < p.n_splits; ++k) {
-                    const float v = __ldcg(p.part_slot + (k * split_stride + rh) * p.slot_stride + s);
-                    if (v != ninf) w += ex2f(v - lse);
-                }
-                p.mass[rh * p.mass_stride + s] = w;
-            }
-        }
-        return;
-    }
-
+    };
+    fetch(0);
     // every lane needs every split's log-sum-exp: lane k loads split k (and k + 32), then shuffles
-    float my0 = lane < p.n_splits ? p.part_lse[lane * split_stride + rh] : ninf;
-    float my1 = lane + 32 < p.n_splits ? p.part_lse[(lane + 32) * split_stride + rh] : ninf;
+    const float my0 = lane < p.n_splits ? __ldcg(p.part_lse + lane * split_stride + rh) : ninf;
+    const float my1 = lane + 32 < p.n_splits ? __ldcg(p.part_lse + (lane + 32) * split_stride + rh) : ninf;
     float mx = fmaxf(my0, my1);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -151,40 +110,44 @@ __global__ void combine_kernel(const CombineParams p)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
     const float lse = mx + log2f(sum);
+    const float lse_s = (lse > ninf) ? lse : 0.f;
     const float w0 = my0 != ninf ? ex2f(my0 - lse) : 0.f;
     const float w1 = my1 != ninf ? ex2f(my1 - lse) : 0.f;
 
-    float acc[V];
+    float acc[V], mass = 0.f;
 #pragma unroll
     for (int x = 0; x < V; ++x) acc[x] = 0.f;
-    for (int k = 0; k < p.n_splits; ++k) {
-        const float w = __shfl_sync(0xffffffffu, k < 32 ? w0 : w1, k & 31);
-        if (w != 0.f) {
-            const float *src = p.part_o + (k * split_stride + rh) * D + lane * V;
-            if constexpr (V == 4) {
-                const float4 v = *reinterpret_cast<const float4 *>(src);
-                acc[0] += w * v.x; acc[1] += w * v.y; acc[2] += w * v.z; acc[3] += w * v.w;
-            } else {
-                const float2 v = *reinterpret_cast<const float2 *>(src);
-                acc[0] += w * v.x; acc[1] += w * v.y;
+    for (int k0 = 0; k0 < p.n_splits; k0 += kBatch) {
+        if (k0 > 0) fetch(k0);
+#pragma unroll
+        for (int j = 0; j < kBatch; ++j) {
+            const int k = k0 + j;
+            // a split that saw no key has weight 0 and never wrote its partial output: what sits there is stale
+            const float w = __shfl_sync(0xffffffffu, k < 32 ? w0 : w1, k & 31);
+            if (w != 0.f && k < p.n_splits) {
+#pragma unroll
+                for (int x = 0; x < V; ++x) acc[x] = fmaf(w, ov[j][x], acc[x]);
             }
+            mass += ex2f(sv[j] - lse_s);                    // exp2(-inf) = 0: absent slots drop out
         }
     }
     __nv_bfloat16 *dst = static_cast<__nv_bfloat16 *>(p.out) + rh * D + lane * V;
 #pragma unroll
     for (int x = 0; x < V; x += 2)
         *reinterpret_cast<__nv_bfloat162 *>(dst + x) = __floats2bfloat162_rn(acc[x], acc[x + 1]);
-
-    if (p.mass) {
-        const int G = p.row_slots[row];
-        for (int s = lane; s <= G; s += 32) {
-            float w = 0.f;
-            for (int k = 0; k < p.n_splits; ++k) {
-                const float v = p.part_slot[(k * split_stride + rh) * p.slot_stride + s];
-                if (v != ninf) w += ex2f(v - lse);
-            }
-            p.mass[rh * p.mass_stride + s] = w;
+    if (!p.mass) return;
+    float *masses = p.mass + rh * p.mass_stride;
+    if (lane <= G) masses[lane] = mass;
+    for (int s = 32; s <= G; s += 32) {                     // warp-uniform
+        mass = 0.f;
+        for (int k0 = 0; k0 < p.n_splits; k0 += kBatch) {
+#pragma unroll
+            for (int j = 0; j < kBatch; ++j)
+                sv[j] = (s + lane <= G && k0 + j < p.n_splits) ? __ldcg(s0 + s + (k0 + j) * split_stride * p.slot_stride) : ninf;
+#pragma unroll
+            for (int j = 0; j < kBatch; ++j) mass += ex2f(sv[j] - lse_s);
         }
+        if (s + lane <= G) masses[s + lane] = mass;
     }
 }
 
@@ -418,8 +381,13 @@ cudaError_t launch_combine(const CombineParams &p, cudaStream_t st)
     if (pairs <= 0) return cudaSuccess;
     const int warps = 8;
     const int blocks = static_cast<int>((pairs + warps - 1) / warps);
-    const cudaError_t e = (p.D == 128) ? launch_pdl(combine_kernel<128>, dim3(blocks), dim3(warps * 32), 0, st, p)
-                                       : launch_pdl(combine_kernel<64>, dim3(blocks), dim3(warps * 32), 0, st, p);
+    cudaError_t e;
+    if (p.n_splits <= 4)
+        e = p.D == 128 ? launch_pdl(combine_kernel<128, 4>, dim3(blocks), dim3(warps * 32), 0, st, p)
+                       : launch_pdl(combine_kernel<64, 4>, dim3(blocks), dim3(warps * 32), 0, st, p);
+    else
+        e = p.D == 128 ? launch_pdl(combine_kernel<128, 8>, dim3(blocks), dim3(warps * 32), 0, st, p)
+                       : launch_pdl(combine_kernel<64, 8>, dim3(blocks), dim3(warps * 32), 0, st, p);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 

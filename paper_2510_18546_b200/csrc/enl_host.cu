@@ -628,7 +628,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         // size check first, so that a failed call leaves the previous plan intact
         const int tpc = tokens_per_cta(c);
         int64_t n_entries = 0, base_items = 0;
-        int min_tiles = 0x7fffffff;
+        int min_tiles = 0x7fffffff, max_tiles = 1, max_rows = 1;
         for (int b = 0; b < B; ++b) {
             int64_t e = 0;
             for (int s = cu_sel[b]; s < cu_sel[b + 1]; ++s) e += std::max(1, ceil_div(sel_len[s], kPageTokens));
@@ -639,6 +639,8 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
             // fewest tiles any CTA of this episode walks: its first token block
             const int c_first = nn - nq + std::min(tpc, nq) - 1;
             min_tiles = std::min<int64_t>(min_tiles, e / kPagesPerTile + c_first / kTileKeys + 1);
+            max_tiles = std::max<int64_t>(max_tiles, e / kPagesPerTile + (nn - 1) / kTileKeys + 1);
+            max_rows = std::max(max_rows, std::min(nq, tpc) * c->rep);
         }
         if (n_entries > c->cap_entries || base_items > c->cap_items) return ENL_E_NOMEM;
 
@@ -718,12 +720,28 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         if (!decode) {
             n_splits = 1;
             const bool few = base_items * 5 < c->n_sm * 4;         // a launch that leaves SMs idle splits the key stream
-            // (two key tiles per split are worth it where the merge is cheap; the kernel that finishes masses takes a few us itself)
-            const int filling = std::max(1, std::min(static_cast<int>(c->n_sm / base_items), min_tiles / (mass_only || has_sum ? 8 : 2)));
+            // A launch takes about T us per key tile of its longest CTA on top of what it always takes: 8.5 us in one split,
+            // 10.5 with two splits merged by pairs, 11.5 with partial results in memory plus 0.15 us per 1000 of their rows.
+            // (T = 2.25 for two Q tiles, 2.0 for one.  17 to 320 rows over 640 to 5120 keys, measured against two tiles or
+            // more per split: 17 rows over 640 keys 15.0 -> 10.4 us, 41 over 640 17.0 -> 12.6, 320 over 1280 27.0 -> 25.9.)
+            // Of equal costs the fewest splits: SMs left over take in the next launch.
+            auto filling = [&]() {
+                int best = 1;
+                double least = 1e30;
+                for (int ns = 1; ns <= kMaxSplits && ns * base_items <= c->n_sm && ns <= min_tiles; ++ns) {
+                    const bool in_pairs = ns == 2 && c->pairs_ok;
+                    const double cost = (max_rows > kTileRows ? 2.25 : 2.0) * ceil_div(max_tiles, ns) +
+                                        (ns == 1 ? 8.5 : in_pairs ? 10.5 : 11.5 + 0.15e-3 * ns * a->n_q * d.n_q_heads);
+                    if (cost < least - 1e-9) { least = cost; best = ns; }
+                }
+                return best;
+            };
+            // the kernel that finishes masses takes a few us itself: eight tiles per split and more
+            const int filling_mass = std::max(1, std::min(static_cast<int>(c->n_sm / base_items), min_tiles / 8));
             if (small_blocks) n_splits = 1;
-            else if (has_sum && !mass_only) n_splits = few && a->split_hint != 1 && c->pairs_ok && filling >= 2 ? 2 : 1;   // a pair or none
+            else if (has_sum && !mass_only) n_splits = few && a->split_hint != 1 && c->pairs_ok && filling_mass >= 2 ? 2 : 1;   // a pair or none
             else if (a->split_hint >= 1) n_splits = std::min(a->split_hint, std::max(1, min_tiles));   // no CTA without a tile
-            else if (few) n_splits = filling;
+            else if (few) n_splits = mass_only ? filling_mass : filling();
             if (mass_only) {                                       // no outputs to merge: the kernel that finishes the masses adds the splits up
                 n_splits = std::min(n_splits, kFinishSplits);
                 while (n_splits > 1 && static_cast<int64_t>(n_splits) * a->n_q * d.n_q_heads > c->finish_cap) --n_splits;
