@@ -7,7 +7,8 @@
 // list order (eight 16-token pages per 128-key tile, fetched as separate TMA boxes from wherever the
 // pages lie in the pool), then the new-token keys up to the causal limit.  Per tile:
 //   S_i = Q_i K^T            tcgen05.mma, operands in shared memory, accumulator in TMEM
-//   p   = exp2(S * c - m)    one thread per row, fp32; padding and causally hidden columns -> 0
+//                            (after an MMA of one K step that puts -inf under page padding)
+//   p   = exp2(S * c - m)    one thread per row, fp32; causally hidden columns -> 0
 //   O_i += P_i V             tcgen05.mma, P (bf16) read from TMEM, V from shared memory
 // The row sum of p is split by the slot (selected group, or the new tokens) each 16-key page belongs
 // to; when a slot ends its log2-sum-exp is parked: in shared memory for calls with few slots, whose values are turned into
@@ -41,7 +42,7 @@ constexpr int kRegsOther    = 80;
 constexpr int kProducerWarp = 8;
 constexpr int kMmaWarp      = 9;
 constexpr uint32_t kTmemCols = 512;
-constexpr int kParkSlots = 28;                // calls with up to this many mass slots park their slot sums in shared memory
+constexpr int kParkSlots = 25;                // calls with up to this many mass slots park their slot sums in shared memory
 constexpr float kRescaleThreshold = 8.0f;     // log2 units: p stays below 2^8 between updates of the reference
 
 template <int D>
@@ -53,9 +54,15 @@ struct Cfg {
     static constexpr int kBarOff    = (kQTiles + kStages) * kTileBytes;
     // pair merge: what the other CTA of the cluster knows about this CTA's rows, [tile][128] x (m, l, shared-slot log-sum, -)
     static constexpr int kXpeerOff  = kBarOff + 512;
+    // the operands of the MMA that hides page padding, 16 bytes per row: 1 for 8 queries (behind the barriers; every group of
+    // 8 rows reads them), 0 or -inf for every key of a K stage
+    static constexpr int kOnesOff   = kBarOff + 256;
+    static constexpr int kHideOff   = kXpeerOff + kQTiles * 128 * 16;
+    static constexpr int kHideBytes = kTileKeys * 16;
     // slot log-sums of calls with at most kParkSlots slots, [tile][slot][128 rows] fp32 (what is left of the 227 KB)
-    static constexpr int kParkOff   = kXpeerOff + kQTiles * 128 * 16;
+    static constexpr int kParkOff   = kHideOff + kStages / 2 * kHideBytes;
     static constexpr int kSmemBytes = kParkOff + kQTiles * kParkSlots * 128 * 4 + 1024;   // + alignment slack
+    static_assert(8 * (13 + 2 * kStages) + 8 <= 256 && kOnesOff + 128 <= kXpeerOff && kSmemBytes <= 232448, "shared memory");
 };
 
 // ---- the kernel ----------------------------------------------------------------------------
@@ -124,6 +131,9 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
             mbar_expect_tx(bar_peer_o, 4u * 16384u);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (threadIdx.x < 8) {
+        *reinterpret_cast<uint4 *>(smem + C::kOnesOff + threadIdx.x * 16) = make_uint4(0x3f80u, 0u, 0u, 0u);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     if (warp == kMmaWarp) {
@@ -180,9 +190,11 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
             int fill = 0;
             for (int j = j_beg; j < j_end && ok; ++j) {
                 const bool cached = j < ep.n_ctiles;
-                int page = 0;
-                if (cached && lane < kPagesPerTile)
+                int page = 0, valid = 0;                             // page of this lane (0..7) and its keys
+                if (cached && lane < kPagesPerTile) {
                     page = p.stream_page[ep.stream_off + j * kPagesPerTile + lane];
+                    valid = __ldg(p.stream_meta + ep.stream_off + j * kPagesPerTile + lane) & 0xff;
+                }
                 for (int kv = 0; kv < 2; ++kv, ++fill) {
                     const int st = fill % C::kStages;
                     if (fill >= C::kStages) {
@@ -191,6 +203,16 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                         if (!ok) break;
                     }
                     const uint32_t full = bar_kv_full(st);
+                    if (cached && kv == 0) {                         // what hides the padding of these keys: see issue_qk
+                        uint4 *hide = reinterpret_cast<uint4 *>(smem + C::kHideOff + st / 2 * C::kHideBytes);
+#pragma unroll
+                        for (int x = 0; x < kTileKeys / 32; ++x) {
+                            const int n = __shfl_sync(kFull, valid, 2 * x + (lane >> 4));
+                            hide[x * 32 + lane] = make_uint4((lane & 15) < n ? 0u : 0xff80u, 0u, 0u, 0u);
+                        }
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                        __syncwarp();
+                    }
                     if (lane == 0) mbar_expect_tx(full, static_cast<uint32_t>(C::kTileBytes));
                     __syncwarp();
                     const uint32_t dst = stage_addr(st);
@@ -234,14 +256,27 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
             const uint32_t dk_lo = static_cast<uint32_t>(dk0), dk_hi = static_cast<uint32_t>(dk0 >> 32);
             const uint32_t dv_lo = static_cast<uint32_t>(dv0), dv_hi = static_cast<uint32_t>(dv0 >> 32);
             constexpr uint32_t kTileUnits = C::kTileBytes >> 4;
-            auto issue_qk = [&](int i, int st) {
+            // operands of 16 channels without a swizzle: the 16 bytes of a row are channels 0..7 and (offset 0) again 8..15
+            auto plain_desc = [&](uint32_t addr, uint32_t group_bytes) {
+                return (1ull << 46) | (static_cast<uint64_t>(group_bytes >> 4) << 32) | ((addr & 0x3FFFFu) >> 4);
+            };
+            const uint64_t d_ones = plain_desc(sbase + C::kOnesOff, 0u), d_hide = plain_desc(sbase + C::kHideOff, 128u);
+            // S_i = Q_i K^T; with cached pages (`hide`) an MMA of one K step before it puts -inf under the padding keys and 0 under
+            // the others.  It costs the pipe 1/16 of a tile's work and takes the compares and selects of ragged
+            // pages out of the softmax warps, which are what a tile waits for: 4374 -> 3999 cycles per key tile and pair of Q tiles
+            // (pages of objects of 20..200 tokens), with masses 4436 -> 4146.
+            auto issue_qk = [&](int i, int st, bool hide) {
                 const uint32_t a = dq_lo + static_cast<uint32_t>(i) * kTileUnits, b = dk_lo + static_cast<uint32_t>(st) * kTileUnits;
                 const uint32_t d = tmem_s(i);
+                if (hide)
+                    mma_ss2(d, static_cast<uint32_t>(d_ones), static_cast<uint32_t>(d_ones >> 32),
+                            static_cast<uint32_t>(d_hide) + static_cast<uint32_t>(st / 2) * (C::kHideBytes >> 4),
+                            static_cast<uint32_t>(d_hide >> 32), idesc_qk, 0u);
 #pragma unroll
                 for (int kk = 0; kk < D / 16; ++kk) {
                     constexpr uint32_t kHalfUnits = C::kHalfBytes >> 4;
                     const uint32_t off = static_cast<uint32_t>((kk >> 2) * kHalfUnits + (kk & 3) * 2);   // 32 bytes per 16 channels
-                    mma_ss2(d, a + off, dq_hi, b + off, dk_hi, idesc_qk, kk > 0 ? 1u : 0u);
+                    mma_ss2(d, a + off, dq_hi, b + off, dk_hi, idesc_qk, kk > 0 || hide ? 1u : 0u);
                 }
                 tc_commit(bar_s_full(i));
             };
@@ -274,7 +309,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
             if (ok) ok = wait_full(0);
             if (ok) {
                 tc_fence_after();
-                for (int i = 0; i < n_qt; ++i) issue_qk(i, 0);
+                for (int i = 0; i < n_qt; ++i) issue_qk(i, 0, j_beg < ep.n_ctiles);
                 tc_commit(bar_kv_empty(0));
             }
             Pending w_v = arm(full_bar(1), full_par(1));                // V of the first tile
@@ -311,7 +346,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                             w_v = arm(full_bar(fv + 2), full_par(fv + 2));
                             w_p = arm(bar_p_half(0, 0), par ^ 1u);
                         }
-                        issue_qk(i, fk % C::kStages);
+                        issue_qk(i, fk % C::kStages, j_beg + jj + 1 < ep.n_ctiles);
                         if (last_i) tc_commit(bar_kv_empty(fk % C::kStages));
                     }
                 }
@@ -388,23 +423,13 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
         for (int jj = 0; jj < n_tiles; ++jj) {
             const int j = j_beg + jj;
             const bool cached = j < ep.n_ctiles;
-            // From the page words two warp-uniform masks: pages with padding, pages whose slot differs from the
-            // page before.  The pages of a new-token tile are masked from the causal limit of the tile's first row on.
+            // From the page words a warp-uniform mask: pages whose slot differs from the page before.  The pages of a new-token tile
+            // are masked from the causal limit of the tile's first row on.
             const int meta = meta_next;
             if (jj + 1 < n_tiles) meta_next = load_meta(j + 1);
             int prev = __shfl_up_sync(kFull, meta >> 8, 1);
             if (lane == 0) prev = cur_slot;
             const uint32_t chg_mask = __ballot_sync(kFull, (meta >> 8) != prev) & 0xffu;
-            uint32_t mask_pages;
-            int vis = kTileKeys;                                    // visible keys of this row in a new-token tile
-            if (cached) {
-                mask_pages = __ballot_sync(kFull, (meta & 0xff) < kPageTokens) & 0xffu;
-            } else {
-                const int kbase = (j - ep.n_ctiles) * kTileKeys;
-                vis = c - kbase + 1;
-                const int vis_lo = c_lo - kbase + 1;               // <= vis of every row of the tile
-                mask_pages = vis_lo >= kTileKeys ? 0u : (0xffu << (max(vis_lo, 0) / kPageTokens)) & 0xffu;
-            }
 
             ok = mbar_wait(bar_s_full(i), static_cast<uint32_t>(jj & 1), abort_flag, p.status);
             if (!ok) break;
@@ -422,20 +447,15 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
 #pragma unroll
             for (int x = 0; x < kTileKeys; ++x) s[x] = __uint_as_float(su[x]);
 
-            // hide page padding / keys after the causal limit
-            for (uint32_t todo = mask_pages; todo; todo &= todo - 1u) {
-                const int e = __ffs(static_cast<int>(todo)) - 1;    // warp-uniform
-                const int nv_e = __shfl_sync(kFull, meta & 0xff, e);
-                const int bound = cached ? nv_e : vis - e * kPageTokens;
-                switch (e) {
-#define ENL_MASK_PAGE(E)                                                          \
-                    case E:                                                       \
-                        _Pragma("unroll") for (int x = 0; x < kPageTokens; ++x)   \
-                            if (x >= bound) s[E * kPageTokens + x] = kNegInf;     \
-                        break;
-                    ENL_MASK_PAGE(0) ENL_MASK_PAGE(1) ENL_MASK_PAGE(2) ENL_MASK_PAGE(3)
-                    ENL_MASK_PAGE(4) ENL_MASK_PAGE(5) ENL_MASK_PAGE(6) ENL_MASK_PAGE(7)
-#undef ENL_MASK_PAGE
+            // hide keys after the causal limit (page padding is hidden in S already)
+            if (!cached) {
+                const int kbase = (j - ep.n_ctiles) * kTileKeys;
+                const int vis = c - kbase + 1;                      // visible keys of this row
+                const int vis_lo = c_lo - kbase + 1;                // <= vis of every row of the tile
+                if (vis_lo < kTileKeys) {
+#pragma unroll
+                    for (int x = 0; x < kTileKeys; ++x)
+                        if (x >= vis) s[x] = kNegInf;
                 }
             }
 
