@@ -233,7 +233,8 @@ typedef struct {
  * a resident group is a hit, any other is loaded from the slow tier once, for all layers; when the
  * device pool is short, the least recently selected groups outside the list are evicted first.  The
  * cache hit rate of the step (Sec. 3.4, last paragraph) is n_hit / n_sel.
- * All copies are enqueued on the stream (kernels that read or write the pinned pool directly).
+ * All copies are asynchronous (kernels that read or write the pinned pool directly).  They start behind what the stream
+ * holds; large loads then run beside it, layer by layer, and every call on the cache is ordered behind those it needs.
  * enl_attend / enl_group_store on a group that is only in the slow tier return ENL_E_EVICTED.
  * Errors: ENL_E_INVAL, ENL_E_NOGROUP, ENL_E_NOMEM (host pool or device pool too small for the
  * request; residency is unchanged then), ENL_E_CUDA.

@@ -240,17 +240,28 @@ __global__ void __launch_bounds__(256) mass_finish_kernel(const FinishParams p)
         if (run_obj >= 0 && run != 0.f) atomicAdd(p.mass_sum + static_cast<long long>(run_obj) * p.sum_stride + s, run);
 }
 
-// grid (pairs, layers, 2): one CTA moves one page of K or V of one layer, 16 bytes per thread and trip
-__global__ void page_copy_kernel(const uint8_t *src_k, const uint8_t *src_v, uint8_t *dst_k, uint8_t *dst_v,
-                                 size_t src_layer_bytes, size_t dst_layer_bytes, const int2 *pairs, int page_bytes)
+// Pages between the pool and the pinned host pool: pairs (from, to) of layers layer0 .. layer0 + n_layers - 1, K and V, 2 KB per
+// warp and trip.  Bound by the host link, whose latency 64 warps with 2 KB in flight each cover (32: 34 GB/s, 64: 50.5, more: 51).
+constexpr int kCopyThreads = 256;
+constexpr int kPieceChunks = 128;                           // a page is a multiple of 2 KB
+__global__ void __launch_bounds__(kCopyThreads) page_copy_kernel(const uint4 *src_k, const uint4 *src_v, uint4 *dst_k, uint4 *dst_v, size_t src_layer,
+                                                                 size_t dst_layer, const int2 *pairs, int n_pairs, int layer0, long long total, int pieces)
 {
-    pdl_trigger();
-    pdl_wait();
-    const int2 pr = pairs[blockIdx.x];
-    const uint8_t *s = (blockIdx.z ? src_v : src_k) + src_layer_bytes * blockIdx.y + static_cast<size_t>(pr.x) * page_bytes;
-    uint8_t *d = (blockIdx.z ? dst_v : dst_k) + dst_layer_bytes * blockIdx.y + static_cast<size_t>(pr.y) * page_bytes;
-    for (int i = threadIdx.x * 16; i < page_bytes; i += blockDim.x * 16)
-        *reinterpret_cast<uint4 *>(d + i) = *reinterpret_cast<const uint4 *>(s + i);
+    const int lane = threadIdx.x & 31;
+#pragma unroll 1
+    for (long long i = blockIdx.x * (kCopyThreads / 32) + (threadIdx.x >> 5); i < total; i += gridDim.x * (kCopyThreads / 32)) {
+        const int page = static_cast<int>(i / pieces), piece = static_cast<int>(i - static_cast<long long>(page) * pieces);
+        const int layer = layer0 + (page >> 1) / n_pairs;                // K and V of a page follow one another
+        const int2 pr = pairs[(page >> 1) % n_pairs];
+        const size_t off = static_cast<size_t>(piece) * kPieceChunks + lane;
+        const uint4 *s = ((page & 1) ? src_v : src_k) + src_layer * layer + static_cast<size_t>(pr.x) * pieces * kPieceChunks + off;
+        uint4 *d = ((page & 1) ? dst_v : dst_k) + dst_layer * layer + static_cast<size_t>(pr.y) * pieces * kPieceChunks + off;
+        uint4 v[kPieceChunks / 32];
+#pragma unroll
+        for (int u = 0; u < kPieceChunks / 32; ++u) v[u] = s[u * 32];
+#pragma unroll
+        for (int u = 0; u < kPieceChunks / 32; ++u) d[u * 32] = v[u];
+    }
 }
 
 // The gather plan as kernel parameters -> device memory.  It waits for the kernel before (which may read the previous plan
@@ -296,13 +307,18 @@ cudaError_t launch_plan_write(void *dst, const void *src, size_t bytes, cudaStre
 }
 
 cudaError_t launch_page_copy(const uint8_t *src_k, const uint8_t *src_v, uint8_t *dst_k, uint8_t *dst_v,
-                             size_t src_layer_bytes, size_t dst_layer_bytes, const int2 *pairs, int n_pairs,
-                             int n_layers, int page_bytes, cudaStream_t st)
+                             size_t src_layer_bytes, size_t dst_layer_bytes, const int2 *pairs, int n_pairs, int layer0,
+                             int n_layers, int page_bytes, int ctas, cudaStream_t st)
 {
-    if (n_pairs <= 0) return cudaSuccess;
-    const cudaError_t e = launch_pdl_n(page_copy_kernel, dim3(n_pairs, n_layers, 2), dim3(256), st, src_k, src_v, dst_k, dst_v,
-                                       src_layer_bytes, dst_layer_bytes, pairs, page_bytes);
-    return e != cudaSuccess ? e : cudaGetLastError();
+    if (n_pairs <= 0 || n_layers <= 0) return cudaSuccess;
+    const int pieces = page_bytes / (16 * kPieceChunks);
+    const long long total = 2ll * n_pairs * n_layers * pieces;
+    const long long need = (total + kCopyThreads / 32 - 1) / (kCopyThreads / 32);
+    // an ordinary launch: the CTAs of dependent ones would take their places early and keep attention CTAs out
+    page_copy_kernel<<<static_cast<unsigned>(std::min<long long>(ctas, need)), kCopyThreads, 0, st>>>(
+        reinterpret_cast<const uint4 *>(src_k), reinterpret_cast<const uint4 *>(src_v), reinterpret_cast<uint4 *>(dst_k),
+        reinterpret_cast<uint4 *>(dst_v), src_layer_bytes / 16, dst_layer_bytes / 16, pairs, n_pairs, layer0, total, pieces);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_page_scatter(void *kpool_layer, void *vpool_layer, const void *k, const void *v,

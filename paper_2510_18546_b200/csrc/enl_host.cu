@@ -175,6 +175,10 @@ struct enl_cache {
     int2 *pairs_host = nullptr, *pairs_dev = nullptr;        // page moves of one enqueue (pinned staging + device copy)
     int32_t cap_pairs = 0;
     cudaEvent_t pairs_copied = nullptr;
+    // loads of several megabytes run beside the caller's stream, a few layers at a time (see enqueue_loads)
+    cudaStream_t load_stream[2] = {nullptr, nullptr};
+    std::vector<cudaEvent_t> load_done;                     // per chunk of layers
+    int load_chunks = 0, load_layers = 1;                   // chunks not known to be complete (0: none pending), layers of a chunk
     uint64_t tick = 0;
 
     float *scratch = nullptr;
@@ -215,6 +219,9 @@ void destroy(enl_cache *c)
         if (c->host_v) cudaFreeHost(c->host_v);
         if (c->pairs_host) cudaFreeHost(c->pairs_host);
         if (c->pairs_dev) cudaFree(c->pairs_dev);
+        for (cudaStream_t q : c->load_stream)
+            if (q) { cudaStreamSynchronize(q); cudaStreamDestroy(q); }
+        for (cudaEvent_t e : c->load_done) cudaEventDestroy(e);
         if (c->pairs_copied) cudaEventDestroy(c->pairs_copied);
     } else {
         delete[] c->plan_host;
@@ -356,6 +363,39 @@ extern "C" int32_t enl_group_len(const enl_cache_t *c, int32_t group_id, int32_t
     return g.len.empty() ? -1 : g.len[layer];
 }
 
+namespace {
+
+// Puts work of `st` that is about to be enqueued behind the loads that are still under way: those of one layer, or (-1) all.
+int join_loads(enl_cache *c, cudaStream_t st, int layer)
+{
+    if (c->load_chunks == 0) return ENL_OK;
+    const int last = c->load_chunks - 1, other = std::max(0, last - 1);       // the last chunk of either load stream
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) { cudaGetLastError(); cap = cudaStreamCaptureStatusNone; }
+    if (cap == cudaStreamCaptureStatusActive) {
+        // a graph cannot wait for work outside it, so the host does
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        bool ok = cudaThreadExchangeStreamCaptureMode(&mode) == cudaSuccess;
+        ok = ok && cudaEventSynchronize(c->load_done[other]) == cudaSuccess && cudaEventSynchronize(c->load_done[last]) == cudaSuccess;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (!ok) { cudaGetLastError(); return ENL_E_CUDA; }
+        c->load_chunks = 0;
+        return ENL_OK;
+    }
+    if (cudaEventQuery(c->load_done[last]) == cudaSuccess && cudaEventQuery(c->load_done[other]) == cudaSuccess) {
+        c->load_chunks = 0;
+        return ENL_OK;
+    }
+    cudaGetLastError();                                                        // "not ready"
+    const bool ok = layer >= 0 ? cudaStreamWaitEvent(st, c->load_done[layer / c->load_layers], 0) == cudaSuccess
+                               : cudaStreamWaitEvent(st, c->load_done[other], 0) == cudaSuccess &&
+                                     cudaStreamWaitEvent(st, c->load_done[last], 0) == cudaSuccess;
+    if (!ok) { cudaGetLastError(); return ENL_E_CUDA; }
+    return ENL_OK;
+}
+
+}  // namespace
+
 extern "C" int enl_cache_status(enl_cache_t *c)
 {
     if (!c) return ENL_E_INVAL;
@@ -435,6 +475,7 @@ extern "C" int enl_group_store(enl_cache_t *c, int32_t group_id, int32_t layer, 
     c->pool_written = true;
     DeviceGuard dg(c->d.device);
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    if (join_loads(c, st, -1) != ENL_OK) return ENL_E_CUDA;
     const size_t row_bytes = static_cast<size_t>(c->d.n_kv_heads) * c->d.head_dim * 2;
     int pos = first_pos;
     while (pos < new_len) {
@@ -502,6 +543,7 @@ extern "C" int enl_group_store_all_layers(enl_cache_t *c, int32_t group_id, int3
     c->pool_written = true;
     DeviceGuard dg(c->d.device);
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    if (join_loads(c, st, -1) != ENL_OK) return ENL_E_CUDA;
     const size_t row_bytes = static_cast<size_t>(c->d.n_kv_heads) * c->d.head_dim * 2;
     for (int layer0 = 0; layer0 < L; layer0 += kScatterLayers) {
         const int nl = std::min(kScatterLayers, L - layer0);
@@ -874,6 +916,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         c->plan_on_device = false;
     }
     if (plan_only) return ENL_OK;
+    if (join_loads(c, st, a->layer) != ENL_OK) return ENL_E_CUDA;
 
     // The plan goes to the device with the first launch that uses it: as parameters of a small kernel, or, when it is too
     // large for that (beyond some 3500 pages of 16 tokens), as one copy, before which this buffer must not be rebuilt.
@@ -1083,23 +1126,63 @@ namespace {
 
 int page_bytes_of(const enl_cache *c) { return c->d.n_kv_heads * kPageTokens * c->d.head_dim * 2; }
 
-// Enqueues the page moves collected in c->pairs_host[0 .. n): direction to_host or to_device.
-int enqueue_moves(enl_cache *c, int n, bool to_host, cudaStream_t st)
+// Uploads the page moves collected in c->pairs_host[0 .. n): the pinned staging list is free again as soon as this upload has
+// run (the event), the device list when the copy kernels behind it have.
+bool upload_moves(enl_cache *c, int n, cudaStream_t st)
+{
+    return cudaMemcpyAsync(c->pairs_dev, c->pairs_host, sizeof(int2) * n, cudaMemcpyHostToDevice, st) == cudaSuccess &&
+           cudaEventRecord(c->pairs_copied, st) == cudaSuccess;
+}
+
+constexpr int kCopyCtas = 32;                               // of a copy that has the stream to itself
+
+// Write-backs: on the caller's stream, whose next launches may reuse the pages.
+int enqueue_evictions(enl_cache *c, int n, cudaStream_t st)
 {
     if (!c->gpu || n == 0) return ENL_OK;
-    // the pinned staging list is free again as soon as this upload has run (the event), the device list when the
-    // copy kernel behind it has (stream order)
-    if (cudaMemcpyAsync(c->pairs_dev, c->pairs_host, sizeof(int2) * n, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaEventRecord(c->pairs_copied, st) != cudaSuccess) {
+    if (!upload_moves(c, n, st) ||
+        launch_page_copy(c->kpool, c->vpool, c->host_k, c->host_v, c->layer_bytes, c->host_layer_bytes, c->pairs_dev, n, 0,
+                         c->d.n_layers, page_bytes_of(c), kCopyCtas, st) != cudaSuccess) {
         cudaGetLastError();
         return ENL_E_CUDA;
     }
-    const cudaError_t e = to_host
-        ? launch_page_copy(c->kpool, c->vpool, c->host_k, c->host_v, c->layer_bytes, c->host_layer_bytes, c->pairs_dev, n,
-                           c->d.n_layers, page_bytes_of(c), st)
-        : launch_page_copy(c->host_k, c->host_v, c->kpool, c->vpool, c->host_layer_bytes, c->layer_bytes, c->pairs_dev, n,
-                           c->d.n_layers, page_bytes_of(c), st);
-    if (e != cudaSuccess) { cudaGetLastError(); return ENL_E_CUDA; }
+    return ENL_OK;
+}
+
+// Loads are bound by the host link (about 51 GB/s of scattered pages), while the attention that follows needs its layer only.
+// So they run on streams of their own behind what the caller's stream holds, in chunks of layers, and a layer's attention waits
+// for its chunk.  Two steps of 20 layers (46 MB each) with attends of 128 rows: 2356 -> 1867 us.
+// - A chunk has at least kLoadChunkBytes: two streams that take turns hide the gaps between chunks down to that size.  What fits
+//   into one chunk stays on the caller's stream.
+// - As few bytes in flight as the link needs (two streams of 32 warps with 2 KB each): what waits for the link stands in the way
+//   of the attention's own loads (four times as many: attends of 24 us take 70 and more, and the two steps 2266 us).
+// - High priority: the few CTAs have to get their places between those of the attention and merge kernels, or chunks come late
+//   (2114 us).
+constexpr int64_t kLoadChunkBytes = 2 << 20;
+constexpr int kLoadCtas = 4;                                // of each load stream
+
+int enqueue_loads(enl_cache *c, int n, cudaStream_t st)
+{
+    if (!c->gpu || n == 0) return ENL_OK;
+    const int L = c->d.n_layers;
+    const int64_t layer_moved = 2ll * n * page_bytes_of(c);
+    const int per = static_cast<int>(std::min<int64_t>(L, (kLoadChunkBytes + layer_moved - 1) / layer_moved));
+    bool ok = upload_moves(c, n, st);
+    if (ok && per == L)
+        ok = launch_page_copy(c->host_k, c->host_v, c->kpool, c->vpool, c->host_layer_bytes, c->layer_bytes, c->pairs_dev, n, 0, L,
+                              page_bytes_of(c), kCopyCtas, st) == cudaSuccess;
+    else if (ok) {
+        for (cudaStream_t q : c->load_stream) ok = ok && cudaStreamWaitEvent(q, c->pairs_copied, 0) == cudaSuccess;
+        c->load_layers = per;
+        for (int l = 0, k = 0; ok && l < L; l += per, ++k) {
+            cudaStream_t q = c->load_stream[k & 1];
+            ok = launch_page_copy(c->host_k, c->host_v, c->kpool, c->vpool, c->host_layer_bytes, c->layer_bytes, c->pairs_dev, n, l,
+                                  std::min(per, L - l), page_bytes_of(c), kLoadCtas, q) == cudaSuccess &&
+                 cudaEventRecord(c->load_done[k], q) == cudaSuccess;
+            if (ok) c->load_chunks = k + 1;
+        }
+    }
+    if (!ok) { cudaGetLastError(); return ENL_E_CUDA; }
     return ENL_OK;
 }
 
@@ -1122,11 +1205,19 @@ extern "C" int enl_tier_enable(enl_cache_t *c, int64_t host_tokens)
     if (c->gpu) {
         DeviceGuard g(c->d.device);
         const size_t bytes = c->host_layer_bytes * c->d.n_layers;
-        const bool okm = cudaMallocHost(&c->host_k, bytes) == cudaSuccess && cudaMallocHost(&c->host_v, bytes) == cudaSuccess &&
+        bool okm = cudaMallocHost(&c->host_k, bytes) == cudaSuccess && cudaMallocHost(&c->host_v, bytes) == cudaSuccess &&
                          cudaMallocHost(&c->pairs_host, sizeof(int2) * c->cap_pairs) == cudaSuccess &&
                          cudaMalloc(&c->pairs_dev, sizeof(int2) * c->cap_pairs) == cudaSuccess &&
                          cudaEventCreateWithFlags(&c->pairs_copied, cudaEventDisableTiming) == cudaSuccess &&
                          cudaEventRecord(c->pairs_copied, 0) == cudaSuccess;
+        int prio_low = 0, prio_high = 0;
+        okm = okm && cudaDeviceGetStreamPriorityRange(&prio_low, &prio_high) == cudaSuccess;
+        for (cudaStream_t &q : c->load_stream) okm = okm && cudaStreamCreateWithPriority(&q, cudaStreamNonBlocking, prio_high) == cudaSuccess;
+        for (int l = 0; l < c->d.n_layers && okm; ++l) {
+            cudaEvent_t e;
+            okm = cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
+            if (okm) c->load_done.push_back(e);
+        }
         if (!okm) {
             cudaGetLastError();
             if (c->host_k) cudaFreeHost(c->host_k);
@@ -1134,6 +1225,9 @@ extern "C" int enl_tier_enable(enl_cache_t *c, int64_t host_tokens)
             if (c->pairs_host) cudaFreeHost(c->pairs_host);
             if (c->pairs_dev) cudaFree(c->pairs_dev);
             if (c->pairs_copied) cudaEventDestroy(c->pairs_copied);
+            for (cudaStream_t &q : c->load_stream) { if (q) cudaStreamDestroy(q); q = nullptr; }
+            for (cudaEvent_t e : c->load_done) cudaEventDestroy(e);
+            c->load_done.clear();
             c->host_k = c->host_v = nullptr;
             c->pairs_host = c->pairs_dev = nullptr;
             c->pairs_copied = nullptr;
@@ -1194,7 +1288,8 @@ extern "C" int enl_group_evict(enl_cache_t *c, int32_t group_id, void *cuda_stre
     const int n = evict_one(c, g, 0, &d2h);
     if (n < 0) return n;
     ++c->epoch;
-    return enqueue_moves(c, n, true, static_cast<cudaStream_t>(cuda_stream));
+    if (c->gpu && join_loads(c, static_cast<cudaStream_t>(cuda_stream), -1) != ENL_OK) return ENL_E_CUDA;
+    return enqueue_evictions(c, n, static_cast<cudaStream_t>(cuda_stream));
 }
 
 extern "C" int enl_step_prepare(enl_cache_t *c, const int32_t *sel_ids, int32_t n_sel, void *cuda_stream,
@@ -1260,7 +1355,10 @@ extern "C" int enl_step_prepare(enl_cache_t *c, const int32_t *sel_ids, int32_t 
     }
     DeviceGuard dg(c->gpu ? c->d.device : -1);
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    if (!victims.empty() || !misses.empty()) ++c->epoch;
+    if (!victims.empty() || !misses.empty()) {
+        ++c->epoch;
+        if (c->gpu && join_loads(c, st, -1) != ENL_OK) return ENL_E_CUDA;
+    }
     if (!victims.empty()) {
         if (!staging_free(c)) { cudaGetLastError(); return ENL_E_CUDA; }
         int n = 0;
@@ -1269,7 +1367,7 @@ extern "C" int enl_step_prepare(enl_cache_t *c, const int32_t *sel_ids, int32_t 
             if (n < 0) return n;                                       // cannot happen: sizes were checked above
             ++stt.n_evicted;
         }
-        const int rc = enqueue_moves(c, n, true, st);
+        const int rc = enqueue_evictions(c, n, st);
         if (rc != ENL_OK) return rc;
     }
     if (!misses.empty()) {
@@ -1287,7 +1385,7 @@ extern "C" int enl_step_prepare(enl_cache_t *c, const int32_t *sel_ids, int32_t 
             stt.bytes_h2d += static_cast<int64_t>(np) * page_bytes_of(c) * 2 * c->d.n_layers;
         }
         c->pool_written = true;
-        const int rc = enqueue_moves(c, n, false, st);
+        const int rc = enqueue_loads(c, n, st);
         if (rc != ENL_OK) return rc;
     }
     for (int s = 0; s < n_sel; ++s) c->groups[sel_ids[s]].last_use = c->tick;

@@ -269,8 +269,8 @@ cudaError_t launch_page_scatter_layers(void *kpool, void *vpool, size_t layer_by
 // Copies whole pages (all kv heads) between two pools of the page format, every layer, K and V: pairs[i] =
 // {source page, destination page}; the pools may be device memory or pinned host memory.
 cudaError_t launch_page_copy(const uint8_t *src_k, const uint8_t *src_v, uint8_t *dst_k, uint8_t *dst_v,
-                             size_t src_layer_bytes, size_t dst_layer_bytes, const int2 *pairs, int n_pairs,
-                             int n_layers, int page_bytes, cudaStream_t st);
+                             size_t src_layer_bytes, size_t dst_layer_bytes, const int2 *pairs, int n_pairs, int layer0,
+                             int n_layers, int page_bytes, int ctas, cudaStream_t st);
 // Writes a gather plan of up to kPlanParamBytes to device memory out of the kernel's own parameters: no staging buffer
 // that the host would have to wait for, and (unlike a copy) it chains to its neighbours by programmatic dependent launch.
 constexpr int kPlanParamBytes = 28672;        // of the 32764 that a launch may carry

@@ -227,3 +227,74 @@ def test_rope_pieces(heads, D, n, interleaved):
     torch.cuda.synchronize()
     err = np.abs(got.float().cpu().numpy() - want)
     assert (err <= np.maximum(np.abs(want) * 2.0 ** -8, 1e-4)).all(), err.max()
+
+
+@pytest.mark.parametrize("splits", [0, 3, 4, 5, 8, 9, 17])
+@pytest.mark.parametrize("n_q", [40, 150])
+def test_splits_and_ragged_pages(n_q, splits):
+    """Merging up to four, eight and more splits (0: as many as the library likes), more than 32 slots, and groups of 1 to 45
+    tokens, so that pages of every fill stand in the key tiles."""
+    lens = list(range(1, 46))
+    wl = synth.make_small(61, 1, 8, 2, 128, [lens + [700, 800]], [list(range(47))[::-1]], [n_q], [n_q], name=f"{splits} splits")
+    check(wl, split_hint=splits)
+
+
+@pytest.mark.parametrize("slots", [24, 25, 26, 27])
+def test_slots_parked_in_shared_memory(slots):
+    wl = synth.make_small(62, 1, 8, 2, 128, [[30] * (slots - 1)], [list(range(slots - 1))], [300], [300], name=f"{slots} slots")
+    check(wl, rows=[0, 127, 128, 299])
+
+
+@pytest.mark.parametrize("pages", [3, 17, 33, 70])
+def test_loads_beside_the_stream(pages):
+    """Loads of one chunk and of chunks of several layers and of one (64 KB per page and layer, 2 MB per chunk): layers in any
+    order right behind the load, another stream, a captured graph, a store and an eviction that overtake nothing."""
+    L, half = 5, pages * 8 + 5                              # the two groups of a list fill `pages` pages, and one more
+    wl = synth.make_small(63, L, 8, 8, 128, [[half] * 4], [[0, 1]], [20], [20], name=f"load {pages} pages")
+    with Session(wl, list(range(L)), extra_tokens=64) as s:
+        enl.enl_tier_enable(s.cache, 8 * half)
+        q, kn, vn = wl.new_qkv(0, s.device)
+
+        def attend(sel, layer, stream=None):
+            out = torch.empty_like(q)
+            enl.enl_attend(s.cache, layer, sel, q, kn, vn, out, stream=torch.cuda.current_stream().cuda_stream if stream is None else stream)
+            return out
+
+        def swap(i):                                        # the other list out, this one in
+            for g in sels[1 - i]:
+                enl.enl_group_evict(s.cache, g)
+            enl.enl_step_prepare(s.cache, sels[i])
+
+        sels = ([0, 1], [2, 3])
+        want = [[attend(sel, l) for l in range(L)] for sel in sels]
+        torch.cuda.synchronize()
+        for i in (0, 1, 0):
+            swap(i)
+            got = {l: attend(sels[i], l) for l in (4, 0, 2, 1, 3)}
+            torch.cuda.synchronize()
+            assert all(torch.equal(got[l], want[i][l]) for l in range(L))
+        swap(1)
+        swap(0)                                             # nothing has waited for the load before
+        side = torch.cuda.Stream()
+        side.wait_stream(torch.cuda.current_stream())
+        out = attend(sels[0], 4, stream=side.cuda_stream)
+        torch.cuda.synchronize()
+        assert torch.equal(out, want[0][4])
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            out = attend(sels[0], 3)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(out, want[0][3])
+        rows = torch.zeros(half, 8, 128, device=s.device, dtype=torch.bfloat16)
+        swap(1)
+        swap(0)
+        for l in range(L):                                  # over what has just been loaded
+            enl.enl_group_store(s.cache, 0, l, rows, rows)
+        got = [attend([0], l) for l in range(L)]
+        torch.cuda.synchronize()
+        assert enl.enl_cache_status(s.cache) == enl.ENL_OK
+        zero = rows.cpu()
+        ro, _ = orc.attend_slots(8, 8, 128, [zero], [zero], q.cpu(), kn.cpu(), vn.cpu())
+        for out in got:
+            check_close(out, ro, None, None, what=wl.name)
