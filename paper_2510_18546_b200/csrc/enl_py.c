@@ -12,7 +12,7 @@
 
 #include "../../include/enl.h"
 
-static PyObject *s_data_ptr, *s_size, *minus_one, *to_int32;
+static PyObject *s_data_ptr, *s_shape, *to_int32;
 
 /* 0 and NULL for None */
 static int tensor_ptr(PyObject *t, void **out)
@@ -26,22 +26,31 @@ static int tensor_ptr(PyObject *t, void **out)
     return (!*out && PyErr_Occurred()) ? -1 : 0;
 }
 
-static int last_dim(PyObject *t, int32_t *out)
+/* one dimension of a tensor, counted from the end if negative (by `shape`: len() and size() of a tensor take three times as long) */
+static int dim_of(PyObject *t, Py_ssize_t at, int32_t *out)
 {
-    PyObject *v = PyObject_CallMethodOneArg(t, s_size, minus_one);
+    PyObject *shape = PyObject_GetAttr(t, s_shape);
+    if (!shape) return -1;
+    PyObject *v = NULL;
+    if (PyTuple_Check(shape)) {
+        const Py_ssize_t n = PyTuple_GET_SIZE(shape), i = at < 0 ? n + at : at;
+        if (i >= 0 && i < n) {
+            v = PyTuple_GET_ITEM(shape, i);
+            Py_INCREF(v);
+        } else {
+            PyErr_SetString(PyExc_IndexError, "tensor has too few dimensions");
+        }
+    } else {
+        v = PySequence_GetItem(shape, at);
+    }
+    Py_DECREF(shape);
     if (!v) return -1;
     *out = (int32_t)PyLong_AsLong(v);
     Py_DECREF(v);
     return (*out == -1 && PyErr_Occurred()) ? -1 : 0;
 }
-
-static int first_dim(PyObject *t, int32_t *out)
-{
-    const Py_ssize_t n = PyObject_Length(t);
-    if (n < 0) return -1;
-    *out = (int32_t)n;
-    return 0;
-}
+static int last_dim(PyObject *t, int32_t *out) { return dim_of(t, -1, out); }
+static int first_dim(PyObject *t, int32_t *out) { return dim_of(t, 0, out); }
 
 static int int_arg(PyObject *o, int32_t *out)
 {
@@ -199,15 +208,7 @@ static PyObject *py_attend_static(PyObject *self, PyObject *const *v, Py_ssize_t
     void *stream, *p;
     if (ints_get(v[0], &seg) || int_arg(v[1], &a.n_new)) goto done;
     if (last_dim(v[2], &a.head_dim)) goto done;
-    {   /* q[-2] and k[-2] */
-        PyObject *minus_two = PyLong_FromLong(-2), *x;
-        x = minus_two ? PyObject_CallMethodOneArg(v[2], s_size, minus_two) : NULL;
-        if (x) { a.n_q_heads = (int32_t)PyLong_AsLong(x); Py_DECREF(x); }
-        x = x ? PyObject_CallMethodOneArg(v[3], s_size, minus_two) : NULL;
-        if (x) { a.n_kv_heads = (int32_t)PyLong_AsLong(x); Py_DECREF(x); }
-        Py_XDECREF(minus_two);
-        if (!x) goto done;
-    }
+    if (dim_of(v[2], -2, &a.n_q_heads) || dim_of(v[3], -2, &a.n_kv_heads)) goto done;
     a.n_seg = (int32_t)seg.n;
     a.seg_len = seg.n ? seg.p : NULL;
     if (tensor_ptr(v[2], &p)) goto done;
@@ -318,8 +319,7 @@ static struct PyModuleDef module = {PyModuleDef_HEAD_INIT, "_enl", NULL, -1, met
 PyMODINIT_FUNC PyInit__enl(void)
 {
     s_data_ptr = PyUnicode_InternFromString("data_ptr");
-    s_size = PyUnicode_InternFromString("size");
-    minus_one = PyLong_FromLong(-1);
-    if (!s_data_ptr || !s_size || !minus_one) return NULL;
+    s_shape = PyUnicode_InternFromString("shape");
+    if (!s_data_ptr || !s_shape) return NULL;
     return PyModule_Create(&module);
 }
