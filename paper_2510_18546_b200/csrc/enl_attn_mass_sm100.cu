@@ -14,7 +14,7 @@
 //     every split's log2-sum-exp go to mass_finish_kernel, which turns log-sums into masses.
 // Bound by the exponentials and the issue slots around them, not by the tensor pipe.  Measured against the general kernel
 // that skipped its output: 512 rows x 32 heads over 200 groups (16 000 keys) 375 -> 165 us a layer, of which the two-way split of the
-// keys is half; per key tile and pair of Q tiles 4400 -> 3650 cycles.
+// keys is half; per key tile and pair of Q tiles 4400 -> 3080 cycles.
 #include <cuda_bf16.h>
 
 #include "attn_ops.cuh"
@@ -28,9 +28,7 @@ constexpr int kSoftmaxWarps = 16;             // two warpgroups per Q tile: keys
 constexpr int kProducerWarp = 16;
 constexpr int kMmaWarp      = 17;
 constexpr int kSlotWarp     = 18;             // + Q tile
-constexpr int kThreads      = 20 * 32;        // launched with 96 registers a thread
-constexpr int kRegsSoftmax  = 104;            // 512 x 104 + 128 x 64 = 640 x 96, what the launch allocates
-constexpr int kRegsOther    = 64;
+constexpr int kThreads      = 20 * 32;        // 96 registers a thread, for all roles: the slot warps use them, too (with 64 they took 1.2 of a softmax warp's time)
 constexpr uint32_t kTmemCols = 512;
 constexpr float kRescaleThreshold = 8.0f;     // log2 units: a reference that lags the maximum by more moves before the next tile
 constexpr float kJumpThreshold = 64.0f;       // log2 units: scores further above the reference make the tile start over
@@ -125,7 +123,6 @@ __global__ void __launch_bounds__(kThreads, 1) mass_kernel(const __grid_constant
     bool ok = true;
 
     if (warp >= kSoftmaxWarps) {
-      asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsOther));
       if (warp == kProducerWarp) {
         // ================= TMA producer =================
         if (lane == 0) {
@@ -196,12 +193,14 @@ __global__ void __launch_bounds__(kThreads, 1) mass_kernel(const __grid_constant
       } else if (warp - kSlotWarp < n_qt) {
         // ================= slot book-keeping: four rows per lane =================
         const int i = warp - kSlotWarp;
+        float m_half[4][2], f_half[4][2];                              // the halves' references, what their sums are scaled by
         float acc[4], m_acc[4], bnd[4];                                // open slot's sum, its reference; log-sum of the slot shared with the split before
         int idx[4];                                                    // (row, head) index, -1 beyond the episode's queries
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             acc[q] = 0.f;
-            m_acc[q] = kNegInf;
+            m_acc[q] = m_half[q][0] = m_half[q][1] = kNegInf;
+            f_half[q][0] = f_half[q][1] = 1.f;
             bnd[q] = kNegInf;
             const int r = q * 32 + lane, t = it.t0 + i * tile_tokens + r / rep;
             idx[q] = t < ep.n_q ? (ep.q_off + t) * p.Hq + it.kvh * rep + r % rep : -1;
@@ -234,39 +233,40 @@ __global__ void __launch_bounds__(kThreads, 1) mass_kernel(const __grid_constant
             chg_next = load_chg(j_beg + jj + 1);
             ok = mbar_wait(bar_sums(i, buf), static_cast<uint32_t>((jj >> 1) & 1), abort_flag, p.status);
             if (!ok) break;
-            float ps[4][kPagesPerTile];
+            float ps[4][kPagesPerTile], ma[4], mb[4];
+            bool moved = false;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const float4 *sums = reinterpret_cast<const float4 *>(smem + C::kSumOff + buf * C::kSumBytes) + i * 256 + q * 32 + lane;
                 const float *refs = reinterpret_cast<const float *>(smem + C::kRefOff + buf * (C::kSumBytes / 4)) + i * 256 + q * 32 + lane;
+                ma[q] = refs[0];
+                mb[q] = refs[128];
                 const float4 a = sums[0], b = sums[128];
-                const float ma = refs[0], mb = refs[128];
-                const float m = fmaxf(ma, mb);
-                // everything relative to the larger of the two references; a half that has seen nothing yet has sums of 0
-                const float fa = (ma == m) ? 1.f : ex2(ma - m), fb = (mb == m) ? 1.f : ex2(mb - m);
-                if (m != m_acc[q]) acc[q] = acc[q] > 0.f ? acc[q] * ex2(m_acc[q] - m) : 0.f;
-                m_acc[q] = m;
-                ps[q][0] = a.x * fa; ps[q][1] = a.y * fa; ps[q][2] = a.z * fa; ps[q][3] = a.w * fa;
-                ps[q][4] = b.x * fb; ps[q][5] = b.y * fb; ps[q][6] = b.z * fb; ps[q][7] = b.w * fb;
+                moved = moved || ma[q] != m_half[q][0] || mb[q] != m_half[q][1];
+                ps[q][0] = a.x; ps[q][1] = a.y; ps[q][2] = a.z; ps[q][3] = a.w;
+                ps[q][4] = b.x; ps[q][5] = b.y; ps[q][6] = b.z; ps[q][7] = b.w;
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_taken(i, buf));
-            // runs of pages of one slot
-            uint32_t todo = 0xffu;                                     // pages not added yet
-#pragma unroll 1
-            for (uint32_t left = chg;; left &= left - 1u) {
-                const uint32_t upto = left ? (1u << (__ffs(static_cast<int>(left)) - 1)) - 1u : 0xffu;
-                const uint32_t run = todo & upto;
+            // Everything is relative to the larger of the two halves' references (a half that has seen nothing yet has sums of
+            // 0).  They seldom move.
+            if (__any_sync(kFull, moved)) {
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    float t = 0.f;
-#pragma unroll
-                    for (int e = 0; e < kPagesPerTile; ++e) t += ((run >> e) & 1u) ? ps[q][e] : 0.f;
-                    acc[q] += t;
+                    const float m = fmaxf(ma[q], mb[q]);
+                    m_half[q][0] = ma[q];
+                    m_half[q][1] = mb[q];
+                    f_half[q][0] = (ma[q] == m) ? 1.f : ex2(ma[q] - m);
+                    f_half[q][1] = (mb[q] == m) ? 1.f : ex2(mb[q] - m);
+                    if (m != m_acc[q]) acc[q] = acc[q] > 0.f ? acc[q] * ex2(m_acc[q] - m) : 0.f;
+                    m_acc[q] = m;
                 }
-                todo &= ~upto;
-                if (!left) break;
-                park();
+            }
+#pragma unroll
+            for (int e = 0; e < kPagesPerTile; ++e) {
+                if ((chg >> e) & 1u) park();                           // the same in every lane
+#pragma unroll
+                for (int q = 0; q < 4; ++q) acc[q] = fmaf(ps[q][e], f_half[q][e / kHalfPages], acc[q]);
             }
         }
         if (ok) {
@@ -280,7 +280,6 @@ __global__ void __launch_bounds__(kThreads, 1) mass_kernel(const __grid_constant
         }
       }
     } else {
-      asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsSoftmax));
       if ((warp >> 3) < n_qt) {
         // ================= softmax: two threads per query row, 64 keys of every tile each =================
         const int i = warp >> 3;                                   // Q tile
