@@ -262,6 +262,12 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo_bytes)
     d |= static_cast<uint64_t>(2) << 61;                               // 128-byte swizzle
     return d;
 }
+// K-major operand of one K step without a swizzle, of which only channel 0 counts: a row is 16 bytes (channels 0..7, and at
+// offset 0 again as 8..15), groups of 8 rows are group_bytes apart (0: every group reads the same rows).
+__device__ __forceinline__ uint64_t smem_desc_plain(uint32_t addr, uint32_t group_bytes)
+{
+    return (static_cast<uint64_t>(1) << 46) | (static_cast<uint64_t>(group_bytes >> 4) << 32) | ((addr & 0x3FFFFu) >> 4);
+}
 // Instruction descriptor, kind::f16: bf16 x bf16 -> fp32, M = 128.
 __host__ __device__ constexpr uint32_t make_idesc(int n, bool b_mn_major)
 {

@@ -4,6 +4,8 @@
 // output.  Half the tensor work of enl_attn_sm100.cu and none of what P V brings with it (P, its way to the MMA issuer, the
 // accumulator and its rescaling) is left, so the split of the work is another one:
 //   - S of both Q tiles is double-buffered in TMEM (4 x 128 columns): the next Q K^T runs under a tile's softmax;
+//   - page padding is hidden by an MMA of one K step that S starts from (see enl_attn_sm100.cu; added in the softmax warps, the
+//     same took 130 of 3080 cycles per tile);
 //   - two threads per query row take 64 keys each, sixteen softmax warps in all, and share nothing: with no accumulator there is no need
 //     for a common reference.  A thread takes its exponentials against the reference of the tiles before and finds the tile's
 //     maximum beside them; any reference is exact as long as nothing overflows, so only scores more than 64 (log2) above it
@@ -14,7 +16,7 @@
 //     every split's log2-sum-exp go to mass_finish_kernel, which turns log-sums into masses.
 // Bound by the exponentials and the issue slots around them, not by the tensor pipe.  Measured against the general kernel
 // that skipped its output: 512 rows x 32 heads over 200 groups (16 000 keys) 375 -> 165 us a layer, of which the two-way split of the
-// keys is half; per key tile and pair of Q tiles 4400 -> 3080 cycles.
+// keys is half; per key tile and pair of Q tiles 4400 -> 2940 cycles.
 #include <cuda_bf16.h>
 
 #include "attn_ops.cuh"
@@ -42,10 +44,12 @@ struct Cfg {
     static constexpr int kTileBytes = kHalves * kHalfBytes;
     static constexpr int kStages    = 4;
     static constexpr int kBarOff    = (kQTiles + kStages) * kTileBytes;
-    // what is added to the scores of a page with v visible keys, [v = 0 .. 16][16] fp32: 0 or -inf
+    // operands of the MMA that hides page padding, 16 bytes per row: 1 for 8 queries, 0 or -inf for every key of a stage
+    static constexpr int kOnesOff   = kBarOff + 256;
     static constexpr int kHideOff   = kBarOff + 512;
+    static constexpr int kHideBytes = kTileKeys * 16;
     // what the softmax threads leave for the slot warps: [buffer][tile][half][128] page sums x 4, and their references
-    static constexpr int kSumOff    = kHideOff + (kPageTokens + 1) * kPageTokens * 4;
+    static constexpr int kSumOff    = kHideOff + kStages * kHideBytes;
     static constexpr int kSumBytes  = kQTiles * 2 * 128 * 16;
     static constexpr int kRefOff    = kSumOff + 2 * kSumBytes;
     static constexpr int kLseOff    = kRefOff + 2 * kSumBytes / 4;     // [tile][128] log2-sum-exps of the second half
@@ -90,11 +94,11 @@ __global__ void __launch_bounds__(kThreads, 1) mass_kernel(const __grid_constant
                 mbar_init(bar_taken(i, b), 1);
             }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (threadIdx.x < 8) {
+        *reinterpret_cast<uint4 *>(smem + C::kOnesOff + threadIdx.x * 16) = make_uint4(0x3f80u, 0u, 0u, 0u);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    if (threadIdx.x < (kPageTokens + 1) * kPageTokens)
-        reinterpret_cast<float *>(smem + C::kHideOff)[threadIdx.x] =
-            static_cast<int>(threadIdx.x % kPageTokens) < static_cast<int>(threadIdx.x / kPageTokens) ? 0.f : kNegInf;
     if (warp == kMmaWarp) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      ::"r"(smem_u32(tmem_slot)), "r"(kTmemCols) : "memory");
@@ -138,12 +142,24 @@ __global__ void __launch_bounds__(kThreads, 1) mass_kernel(const __grid_constant
             const bool cached = j < ep.n_ctiles;
             // lane = (64-channel half, page): every box of a tile leaves in one instruction
             const int hf = lane / kPagesPerTile;
-            int row = 0;
-            if (cached && hf < C::kHalves)
+            int row = 0, valid = 0;
+            if (cached && hf < C::kHalves) {
                 row = (p.stream_page[ep.stream_off + j * kPagesPerTile + lane % kPagesPerTile] * p.Hkv + it.kvh) * kPageTokens;
+                valid = __ldg(p.stream_meta + ep.stream_off + j * kPagesPerTile + lane % kPagesPerTile) & 0xff;
+            }
             if (jj >= C::kStages) {
                 ok = mbar_wait(bar_k_empty(st), static_cast<uint32_t>((jj / C::kStages - 1) & 1), abort_flag, p.status);
                 if (!ok) break;
+            }
+            if (cached) {                                            // what hides the padding of these keys
+                uint4 *hide = reinterpret_cast<uint4 *>(smem + C::kHideOff + st * C::kHideBytes);
+#pragma unroll
+                for (int x = 0; x < kTileKeys / 32; ++x) {
+                    const int n = __shfl_sync(kFull, valid, 2 * x + (lane >> 4));
+                    hide[x * 32 + lane] = make_uint4((lane & 15) < n ? 0u : 0xff80u, 0u, 0u, 0u);
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
             }
             if (lane == 0) mbar_expect_tx(bar_k_full(st), static_cast<uint32_t>(C::kTileBytes));
             __syncwarp();
@@ -169,6 +185,7 @@ __global__ void __launch_bounds__(kThreads, 1) mass_kernel(const __grid_constant
         const uint64_t dq0 = smem_desc(q_addr(0), 16), dk0 = smem_desc(stage_addr(0), 16);
         const uint32_t dq_lo = static_cast<uint32_t>(dq0), dq_hi = static_cast<uint32_t>(dq0 >> 32);
         const uint32_t dk_lo = static_cast<uint32_t>(dk0), dk_hi = static_cast<uint32_t>(dk0 >> 32);
+        const uint64_t d_ones = smem_desc_plain(sbase + C::kOnesOff, 0u), d_hide = smem_desc_plain(sbase + C::kHideOff, 128u);
         ok = mbar_wait(bar_q_full, 0, abort_flag, p.status);
         for (int jj = 0; jj < n_tiles && ok; ++jj) {
             const int st = jj % C::kStages, buf = jj & 1;
@@ -177,11 +194,16 @@ __global__ void __launch_bounds__(kThreads, 1) mass_kernel(const __grid_constant
                 if (jj >= 2) ok = mbar_wait(bar_s_free(i, buf), static_cast<uint32_t>((jj / 2 - 1) & 1), abort_flag, p.status);
                 if (!ok) break;
                 tc_fence_after();
+                const bool hide = j_beg + jj < ep.n_ctiles;
+                if (hide)
+                    mma_ss2(tmem_base + static_cast<uint32_t>((2 * buf + i) * 128), static_cast<uint32_t>(d_ones),
+                            static_cast<uint32_t>(d_ones >> 32), static_cast<uint32_t>(d_hide) + static_cast<uint32_t>(st) * (C::kHideBytes >> 4),
+                            static_cast<uint32_t>(d_hide >> 32), idesc_qk, 0u);
 #pragma unroll
                 for (int kk = 0; kk < D / 16; ++kk) {
                     const uint32_t off = static_cast<uint32_t>((kk >> 2) * (C::kHalfBytes >> 4) + (kk & 3) * 2);   // 32 bytes per 16 channels
                     mma_ss2(tmem_base + static_cast<uint32_t>((2 * buf + i) * 128), dq_lo + static_cast<uint32_t>(i) * kTileUnits + off, dq_hi,
-                            dk_lo + static_cast<uint32_t>(st) * kTileUnits + off, dk_hi, idesc_qk, kk > 0 ? 1u : 0u);
+                            dk_lo + static_cast<uint32_t>(st) * kTileUnits + off, dk_hi, idesc_qk, kk > 0 || hide ? 1u : 0u);
                 }
                 tc_commit(bar_s_full(i, buf));
             }
@@ -223,8 +245,7 @@ __global__ void __launch_bounds__(kThreads, 1) mass_kernel(const __grid_constant
             ++slot;
         };
         auto load_chg = [&](int j) -> uint32_t {
-            return j < ep.n_ctiles ? static_cast<uint32_t>(__ldg(p.tile_words + ep.stream_off / kPagesPerTile + j).y) >> 8
-                                   : (j == ep.n_ctiles ? 1u : 0u);
+            return j < ep.n_ctiles ? __ldg(p.tile_chg + ep.stream_off / kPagesPerTile + j) : (j == ep.n_ctiles ? 1u : 0u);
         };
         uint32_t chg_next = load_chg(j_beg) & ~1u;                     // the first page opens its slot
         for (int jj = 0; jj < n_tiles; ++jj) {
@@ -293,22 +314,10 @@ __global__ void __launch_bounds__(kThreads, 1) mass_kernel(const __grid_constant
         const uint64_t sc2 = pack2(scale, scale);
         float m = kNegInf, m_run = kNegInf;                        // reference and maximum so far (log2 units)
         float l = 0.f;                                             // sum, relative to m
-        // Words of a cached tile (from the gather plan): visible keys of its pages (4 bits each, of 16), pages that hide keys.
-        // Fetched one tile ahead.  A new-token tile hides keys from the causal limit of the Q tile's first row on.
-        auto load_words = [&](int j) -> int2 {
-            if (j < ep.n_ctiles) return __ldg(p.tile_words + ep.stream_off / kPagesPerTile + j);
-            const int vis_lo = ep.n_new - ep.n_q + it.t0 + i * tile_tokens - (j - ep.n_ctiles) * kTileKeys + 1;   // <= visible keys of every row
-            return make_int2(0, vis_lo >= kTileKeys ? 0 : (0xff << (max(vis_lo, 0) / kPageTokens)) & 0xff);
-        };
-        int2 words = load_words(j_beg);
-        const float *hide_tab = reinterpret_cast<const float *>(smem + C::kHideOff);
-
         for (int jj = 0; jj < n_tiles; ++jj) {
             const int j = j_beg + jj, buf = jj & 1;
             const uint32_t t_s = t_s0 + static_cast<uint32_t>(buf * 256);
             const uint32_t par = static_cast<uint32_t>((jj >> 1) & 1);
-            const int2 w = words;
-            words = load_words(j + 1);
             auto move_reference = [&](float to) {
                 const float m_new = fmaxf(m, to);
                 l *= (m_new == kNegInf) ? 1.f : ex2(m - m_new);
@@ -328,24 +337,12 @@ __global__ void __launch_bounds__(kThreads, 1) mass_kernel(const __grid_constant
                 tmem_ld_wait();
                 tmem_ld32_arrived(*reinterpret_cast<uint32_t(*)[32]>(&s[0]));
                 tmem_ld32_arrived(*reinterpret_cast<uint32_t(*)[32]>(&s[32]));
-                // hide page padding / keys after the causal limit: a row of the table (0 or -inf) is added
-                if ((w.y >> (half * kHalfPages)) & 15) {
+                // hide keys after the causal limit (page padding is hidden in S already)
+                if (j >= ep.n_ctiles) {
+                    const int vis = c - (j - ep.n_ctiles) * kTileKeys + 1 - half * kHalfKeys;
 #pragma unroll
-                    for (int e = 0; e < kHalfPages; ++e) {
-                        const int pe = half * kHalfPages + e;
-                        if ((w.y >> pe) & 1) {
-                            const int n = j < ep.n_ctiles ? (w.x >> (4 * pe)) & 15
-                                                          : min(max(c - (j - ep.n_ctiles) * kTileKeys + 1 - pe * kPageTokens, 0), kPageTokens);
-                            const float4 *row = reinterpret_cast<const float4 *>(hide_tab + n * kPageTokens);
-#pragma unroll
-                            for (int x = 0; x < 4; ++x) {
-                                const float4 v = row[x];
-                                float *d = s + e * kPageTokens + 4 * x;
-                                unpack2(add2(pack2(d[0], d[1]), pack2(v.x, v.y)), d[0], d[1]);
-                                unpack2(add2(pack2(d[2], d[3]), pack2(v.z, v.w)), d[2], d[3]);
-                            }
-                        }
-                    }
+                    for (int x = 0; x < kHalfKeys; ++x)
+                        if (x >= vis) s[x] = kNegInf;
                 }
                 const float m_use = (m == kNegInf) ? 0.f : m;
                 const uint64_t nm2 = pack2(-m_use, -m_use);

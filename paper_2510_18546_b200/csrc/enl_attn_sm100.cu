@@ -256,11 +256,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
             const uint32_t dk_lo = static_cast<uint32_t>(dk0), dk_hi = static_cast<uint32_t>(dk0 >> 32);
             const uint32_t dv_lo = static_cast<uint32_t>(dv0), dv_hi = static_cast<uint32_t>(dv0 >> 32);
             constexpr uint32_t kTileUnits = C::kTileBytes >> 4;
-            // operands of 16 channels without a swizzle: the 16 bytes of a row are channels 0..7 and (offset 0) again 8..15
-            auto plain_desc = [&](uint32_t addr, uint32_t group_bytes) {
-                return (1ull << 46) | (static_cast<uint64_t>(group_bytes >> 4) << 32) | ((addr & 0x3FFFFu) >> 4);
-            };
-            const uint64_t d_ones = plain_desc(sbase + C::kOnesOff, 0u), d_hide = plain_desc(sbase + C::kHideOff, 128u);
+            const uint64_t d_ones = smem_desc_plain(sbase + C::kOnesOff, 0u), d_hide = smem_desc_plain(sbase + C::kHideOff, 128u);
             // S_i = Q_i K^T; with cached pages (`hide`) an MMA of one K step before it puts -inf under the padding keys and 0 under
             // the others.  It costs the pipe 1/16 of a tile's work and takes the compares and selects of ragged
             // pages out of the softmax warps, which are what a tile waits for: 4374 -> 3999 cycles per key tile and pair of Q tiles

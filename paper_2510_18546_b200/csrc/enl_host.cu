@@ -137,7 +137,7 @@ struct enl_cache {
     int32_t cap_entries = 0, cap_items = 0;
     uint8_t *plan_host = nullptr, *plan_dev = nullptr;
     // sections of the current plan, back to back in the order of their offsets
-    size_t off_eps = 0, off_items = 0, off_stream = 0, off_meta = 0, off_rowslots = 0, off_rowobj = 0, off_words = 0, plan_used = 0;
+    size_t off_eps = 0, off_items = 0, off_stream = 0, off_meta = 0, off_rowslots = 0, off_rowobj = 0, off_chg = 0, plan_used = 0;
     size_t plan_bytes = 0;                  // capacity
     cudaEvent_t plan_copied = nullptr;
     bool plan_copying = false;              // a copy out of plan_host may be under way (until plan_copied)
@@ -193,7 +193,7 @@ struct enl_cache {
     int32_t *h_stream() { return reinterpret_cast<int32_t *>(plan_host + off_stream); }
     int32_t *h_meta() { return reinterpret_cast<int32_t *>(plan_host + off_meta); }
     int32_t *h_rowslots() { return reinterpret_cast<int32_t *>(plan_host + off_rowslots); }
-    int2 *h_words() { return reinterpret_cast<int2 *>(plan_host + off_words); }
+    uint8_t *h_chg() { return plan_host + off_chg; }
     int32_t *h_rowobj() { return reinterpret_cast<int32_t *>(plan_host + off_rowobj); }
 };
 
@@ -289,7 +289,7 @@ extern "C" int enl_cache_create(const enl_cache_desc_t *desc, enl_cache_t **out)
     c->cap_items = std::max(4096, (d.max_q_tokens / tpc + d.max_batch + 1) * d.n_kv_heads);
     auto align256 = [](size_t x) { return (x + 255) & ~static_cast<size_t>(255); };
     c->plan_bytes = align256(sizeof(EpInfo) * d.max_batch) + align256(sizeof(Item) * c->cap_items) +
-                    2 * align256(sizeof(int32_t) * c->cap_entries) + align256(c->cap_entries + sizeof(int2)) + 2 * align256(sizeof(int32_t) * d.max_q_tokens);
+                    2 * align256(sizeof(int32_t) * c->cap_entries) + align256(c->cap_entries / kPagesPerTile + 1) + 2 * align256(sizeof(int32_t) * d.max_q_tokens);
     c->plan_layer_ok.assign(d.n_layers, 0);
 
     if (!c->gpu) {
@@ -813,7 +813,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
             c->off_stream = section(sizeof(int32_t) * n_entries);
             c->off_meta = section(sizeof(int32_t) * n_entries);
             const bool merged = n_splits > 1 && !pair && !mass_only;
-            c->off_words = section(mass_only ? sizeof(int2) * (n_entries / kPagesPerTile) : 0);
+            c->off_chg = section(mass_only ? n_entries / kPagesPerTile : 0);
             c->off_rowslots = section(!by_grid && (merged || (has_mass && B > 1)) ? sizeof(int32_t) * a->n_q : 0);
             c->off_rowobj = section(has_sum ? sizeof(int32_t) * a->n_q : 0);
             c->plan_used = at;
@@ -846,14 +846,12 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
             while ((ne - e.stream_off) % kPagesPerTile) { stream[ne] = kZeroPage; smeta[ne++] = (e.n_slots - 1) << 8; }
             e.n_ctiles = (ne - e.stream_off) / kPagesPerTile;
             for (int j = 0; j < e.n_ctiles && mass_only; ++j) {
-                uint32_t keys = 0, hide = 0, chg = 0;
+                uint32_t chg = 0;
                 for (int x = 0; x < kPagesPerTile; ++x) {
-                    const int at = e.stream_off + j * kPagesPerTile + x, n = smeta[at] & 0xff;
-                    keys |= static_cast<uint32_t>(n & 15) << (4 * x);
-                    if (n < kPageTokens) hide |= 1u << x;
+                    const int at = e.stream_off + j * kPagesPerTile + x;
                     if (at > e.stream_off && (smeta[at] >> 8) != (smeta[at - 1] >> 8)) chg |= 1u << x;
                 }
-                c->h_words()[e.stream_off / kPagesPerTile + j] = make_int2(static_cast<int>(keys), static_cast<int>(hide | chg << 8));
+                c->h_chg()[e.stream_off / kPagesPerTile + j] = static_cast<uint8_t>(chg);
             }
             if (!by_grid && ((n_splits > 1 && !pair && !mass_only) || (has_mass && B > 1)))
                 for (int r = e.q_off; r < e.q_off + e.n_q; ++r) rowslots[r] = e.n_slots;
@@ -1069,7 +1067,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         mp.eps = p.eps;
         mp.stream_page = p.stream_page;
         mp.stream_meta = p.stream_meta;
-        mp.tile_words = reinterpret_cast<const int2 *>(c->plan_dev + c->off_words);
+        mp.tile_chg = c->plan_dev + c->off_chg;
         mp.mass = a->group_mass;
         mp.lse_out = c->finish_lse;
         mp.bnd_out = c->finish_bnd;

@@ -72,8 +72,7 @@ struct MassParams {
     const EpInfo *eps;
     const int32_t *stream_page;
     const int32_t *stream_meta;
-    const int2 *tile_words; // per cached tile: visible keys of its pages (4 bits each, of 16), then pages that hide keys (8 bits)
-                            // and pages whose slot differs from the page before (8 bits)
+    const uint8_t *tile_chg; // per cached tile: pages whose slot is not that of the page before (a bit each)
     float  *mass;           // log2-sums of the slots, for mass_finish_kernel
     float  *lse_out;        // [split][n_q_total][Hq] log2-sum-exp of every row
     float2 *bnd_out;        // with splits: [split][n_q_total][Hq] the split's part of the slot it shares with the split before it
