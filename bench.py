@@ -530,26 +530,26 @@ def run_cuda(args, workload, steps, warmup, want_e2e, want_cpu, rank, world, loc
             for gid in ids:
                 enl.enl_group_evict(cache, gid, stream=stream)
             torch.cuda.synchronize(dev)
-            ta, tb = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-            ta.record()
+            t0 = time.perf_counter()                        # loads run beside the stream: its events would not see them
             st_ = enl.enl_step_prepare(cache, ids, stream=stream)
-            tb.record()
             torch.cuda.synchronize(dev)
-            t_ms.append(ta.elapsed_time(tb))
+            t_ms.append((time.perf_counter() - t0) * 1e3)
             moved = st_["bytes_h2d"]
         again = enl.enl_step_prepare(cache, ids, stream=stream)
         tier = {"load_ms": float(np.median(t_ms)), "bytes_h2d": int(moved), "gbs": moved / (np.median(t_ms) * 1e-3) / 1e9,
                 "groups": len(ids), "layers": L, "hit_rate_when_repeated": again["n_hit"] / max(len(ids), 1),
-                "note": "enl_step_prepare after evicting the step's selected groups: one kernel copies their pages "
-                        "of all layers from the pinned host pool"}
+                "note": "enl_step_prepare after evicting the step's selected groups, until all their pages of all layers "
+                        "have come from the pinned host pool (host clock)"}
 
     cpu = None
     if rank == 0 and world == 1 and want_cpu:
         wl0 = synth.make(workload)
         _, _, _, cpu = oracle_sample(wl0)
 
-    # attention (+ merge kernel when the splits go through the scratch buffer) + page scatter
-    launches_per_step = L * (1 + (1 if plan["merge_kind"] == 1 else 0)) + store_launches
+    # attention (+ merge kernel when the splits go through the scratch buffer, or the kernel that finishes the masses of more
+    # than 25 slots) + page scatter; the launch that carries a step's gather plan is not counted
+    second = plan["merge_kind"] == 1 or (plan["merge_kind"] in (0, 2) and not wl.decode_steps and G + 1 > 25)
+    launches_per_step = L * (2 if second else 1) + store_launches
     enl.enl_cache_free(cache)
     del qs, kns, vns, outs, masses, store_src
     torch.cuda.empty_cache()
