@@ -4,6 +4,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <cstring>
 
 #include "enl_internal.h"
@@ -200,42 +201,62 @@ __global__ void __launch_bounds__(256) mass_finish_kernel(const FinishParams p)
             lse = __ldcg(p.lse + mine);
         }
     }
+    const int n_here = static_cast<int>(max(0ll, min(32ll, n_pairs - first)));
+    // splits (bit k) that share a slot of this warp's with the one before: seldom any
+    uint32_t shared = 0;
+    if constexpr (kSplits) {
+#pragma unroll
+        for (int k = 1; k < kFinishSplits; ++k)
+            if (__any_sync(0xffffffffu, (__float_as_int(bnd[k].y) >> 5) == static_cast<int>(blockIdx.y))) shared |= 1u << k;
+    }
     float run = 0.f;                                        // this slot's sum over the rows of the current object
     int run_obj = -1;
-    const int n_here = static_cast<int>(min(32ll, n_pairs - first));
-    for (int x0 = 0; x0 < n_here; x0 += 8) {
-        float v[8];
+    float *const col = p.mass + first * p.mass_stride + s;
+    auto turn = [&](auto one_row) {
+        constexpr bool kOneRow = decltype(one_row)::value;  // the pairs have one slot count and one object
+        if (kOneRow) run_obj = obj;
+        for (int x0 = 0; x0 < n_here; x0 += 8) {
+            float v[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int g = __shfl_sync(0xffffffffu, G, x0 + u);
-            v[u] = s <= g ? __ldcg(p.mass + (first + x0 + u) * p.mass_stride + s) : ninf;
-        }
+            for (int u = 0; u < 8; ++u) {
+                const int g = kOneRow ? G : __shfl_sync(0xffffffffu, G, x0 + u);
+                v[u] = s <= g ? __ldcg(col + static_cast<long long>(x0 + u) * p.mass_stride) : ninf;
+            }
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int x = x0 + u, g = __shfl_sync(0xffffffffu, G, x);
-            const float ref = __shfl_sync(0xffffffffu, lse, x);
-            float w = (ref != ninf) ? ex2f(v[u] - ref) : 0.f;
-            if constexpr (kSplits) {
+            for (int u = 0; u < 8; ++u) {
+                const int x = x0 + u, g = kOneRow ? G : __shfl_sync(0xffffffffu, G, x);
+                const float ref = __shfl_sync(0xffffffffu, lse, x);
+                float w = (ref != ninf) ? ex2f(v[u] - ref) : 0.f;
+                if constexpr (kSplits) {
+                    if (shared) {
 #pragma unroll
-                for (int k = 1; k < kFinishSplits; ++k) {
-                    if (k >= p.n_splits) break;
-                    const float b = __shfl_sync(0xffffffffu, bnd[k].x, x);
-                    const int bs = __shfl_sync(0xffffffffu, __float_as_int(bnd[k].y), x);
-                    if (s == bs) w += b;
+                        for (int k = 1; k < kFinishSplits; ++k) {
+                            if (!((shared >> k) & 1u)) continue;
+                            const float b = __shfl_sync(0xffffffffu, bnd[k].x, x);
+                            const int bs = __shfl_sync(0xffffffffu, __float_as_int(bnd[k].y), x);
+                            if (s == bs) w += b;
+                        }
+                    }
+                }
+                if (s <= g) col[static_cast<long long>(x) * p.mass_stride] = w;
+                if constexpr (kSums) {
+                    if (!kOneRow) {
+                        const int o = __shfl_sync(0xffffffffu, obj, x);
+                        if (o != run_obj) {                 // the same in every lane
+                            if (run_obj >= 0 && run != 0.f) atomicAdd(p.mass_sum + static_cast<long long>(run_obj) * p.sum_stride + s, run);
+                            run = 0.f;
+                            run_obj = o;
+                        }
+                    }
+                    if (s <= g) run += w;
                 }
             }
-            if (s <= g) p.mass[(first + x) * p.mass_stride + s] = w;
-            if constexpr (kSums) {
-                const int o = __shfl_sync(0xffffffffu, obj, x);
-                if (o != run_obj) {                         // the same in every lane
-                    if (run_obj >= 0 && run != 0.f) atomicAdd(p.mass_sum + static_cast<long long>(run_obj) * p.sum_stride + s, run);
-                    run = 0.f;
-                    run_obj = o;
-                }
-                if (s <= g) run += w;
-            }
         }
-    }
+    };
+    // A row's 32 q heads are one warp's pairs in many models; then nothing has to be looked up pair by pair (four layers of 512 rows over 200 groups 526 -> 513 us in all).
+    const int G0 = __shfl_sync(0xffffffffu, G, 0), obj0 = __shfl_sync(0xffffffffu, obj, 0);
+    if (n_here == 32 && __all_sync(0xffffffffu, G == G0 && obj == obj0)) turn(std::true_type{});
+    else turn(std::false_type{});
     if constexpr (kSums)
         if (run_obj >= 0 && run != 0.f) atomicAdd(p.mass_sum + static_cast<long long>(run_obj) * p.sum_stride + s, run);
 }
