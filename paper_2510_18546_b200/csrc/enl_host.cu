@@ -918,7 +918,9 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
 
     // The plan goes to the device with the first launch that uses it: as parameters of a small kernel, or, when it is too
     // large for that (beyond some 3500 pages of 16 tokens), as one copy, before which this buffer must not be rebuilt.
-    const bool fresh = !c->plan_on_device;
+    // (A short call of one episode takes it along in its own parameters.)
+    const bool plan_inside = c->plan_small_blocks && c->plan_batch == 1;
+    const bool fresh = !c->plan_on_device && !plan_inside;
     if (fresh) {
         bool okc;
         if (c->plan_used <= static_cast<size_t>(kPlanParamBytes)) {
@@ -938,7 +940,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
 
     const int slot_stride = c->plan_max_slots + 1;
     if (c->plan_small_blocks || (c->plan_decode && c->plan_cluster)) {
-        ClusterDecodeParams dp;
+        SmallParams dp;
         std::memset(&dp, 0, sizeof dp);
         const cuuint64_t nd[3] = {static_cast<cuuint64_t>(d.head_dim), static_cast<cuuint64_t>(d.n_kv_heads),
                                   static_cast<cuuint64_t>(a->n_new)};
@@ -953,6 +955,10 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         dp.eps = reinterpret_cast<const EpInfo *>(c->plan_dev + c->off_eps);
         dp.stream_page = reinterpret_cast<const int32_t *>(c->plan_dev + c->off_stream);
         dp.stream_meta = reinterpret_cast<const int32_t *>(c->plan_dev + c->off_meta);
+        if (plan_inside) {
+            dp.n_list = std::min(dp.ep0.n_entries, kSmallMaxPages);
+            for (int i = 0; i < dp.n_list; ++i) dp.list[i] = make_int2(c->h_stream()[i], c->h_meta()[i]);
+        }
         dp.q = a->q;
         dp.out = a->out;
         dp.mass = a->group_mass;

@@ -138,6 +138,11 @@ struct ClusterDecodeParams {
     int32_t wait_first;     // as in AttnParams
     float   scale_log2;
 };
+constexpr int kSmallMaxPages = 24;
+struct SmallParams : ClusterDecodeParams {
+    int32_t n_list;             // the cached pages of a single episode travel here (else 0: they are in the gather plan)
+    int2    list[kSmallMaxPages];   // page id, slot << 8 | valid keys
+};
 constexpr int kMaxCluster = 16;
 // Contiguous keys in segments instead of pool pages (the entry point that allocates nothing).
 constexpr int kStaticMaxSeg = 255;
@@ -231,10 +236,9 @@ cudaError_t launch_decode_cluster(const ClusterDecodeParams &p, int head_dim, in
 cudaError_t launch_decode_static(const StaticDecodeParams &p, int head_dim, int cluster, cudaStream_t st);
 constexpr int kClusterMaxPages = 288;         // pages of a CTA of these kernels
 // Short calls (see enl_attn_small_sm100.cu): every page a CTA sees in shared memory at once.
-constexpr int kSmallMaxPages = 24;
 cudaError_t prepare_small(int head_dim);
 // row_groups: 1, 2 or 4 groups of 16 query rows (tokens x q heads of a kv head) per CTA
-cudaError_t launch_small(const ClusterDecodeParams &p, int head_dim, int row_groups, int row_blocks, int batch, cudaStream_t st);
+cudaError_t launch_small(const SmallParams &p, int head_dim, int row_groups, int row_blocks, int batch, cudaStream_t st);
 int decode_cluster_smem(int head_dim, int list_pages, int list_slots, int rep);
 constexpr int kClusterPairSmem = 113800;      // two CTAs of up to this much fit an SM
 // How many clusters of 2^i CTAs the current device runs at once: with two CTAs per SM, and with one (larger lists).

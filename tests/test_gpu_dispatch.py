@@ -298,3 +298,27 @@ def test_loads_beside_the_stream(pages):
         ro, _ = orc.attend_slots(8, 8, 128, [zero], [zero], q.cpu(), kn.cpu(), vn.cpu())
         for out in got:
             check_close(out, ro, None, None, what=wl.name)
+
+
+def test_short_calls_between_long_ones_and_stores():
+    """A short call takes its pages along, a long one reads them from device memory: either after the other and after a store."""
+    wl = synth.make_small(64, 1, 8, 2, 128, [[40, 30, 600]], [[0, 1, 2]], [20], [20], name="short and long in turn")
+    with Session(wl, [0]) as s:
+        q, kn, vn = wl.new_qkv(0, s.device)
+        k, v = wl.pool_kv(0, 0, s.device)
+        gen = torch.Generator(device=s.device).manual_seed(6)
+        spans, outs, want = ((0, 40), (40, 70), (70, 670)), [], []
+        for i in range(8):
+            if i % 3 == 0:
+                k[:40] = torch.randn(40, 2, 128, generator=gen, device=s.device).to(k.dtype)
+                enl.enl_group_store(s.cache, 0, 0, k[:40].clone(), v[:40])
+            sel = ([0, 1], [0, 2], [1, 0], [2, 0])[i % 4]
+            out = torch.empty_like(q)
+            enl.enl_attend(s.cache, 0, sel, q, kn, vn, out)
+            outs.append(out)
+            want.append([[x[a:b].cpu().clone() for a, b in (spans[g] for g in sel)] for x in (k, v)])
+        torch.cuda.synchronize()
+        assert enl.enl_cache_status(s.cache) == enl.ENL_OK
+        for out, (ks, vs) in zip(outs, want):
+            ro, _ = orc.attend_slots(8, 2, 128, ks, vs, q.cpu(), kn.cpu(), vn.cpu())
+            check_close(out, ro, None, None, what=wl.name)
