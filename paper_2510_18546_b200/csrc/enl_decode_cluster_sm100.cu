@@ -26,6 +26,8 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <map>
+#include <mutex>
 #include <type_traits>
 
 #include "decode_ops.cuh"
@@ -575,6 +577,18 @@ cudaError_t prepare(ClusterCaps *caps)
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     if (e != cudaSuccess) return e;
     const bool wide = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    // a device's answers are asked for once: ten occupancy queries per kernel are most of what making a small cache takes
+    static std::mutex lock;
+    static std::map<int, ClusterCaps> known;
+    int dev = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    const std::lock_guard<std::mutex> guard(lock);
+    const auto found = known.find(dev);
+    if (found != known.end()) {
+        *caps = found->second;
+        cudaGetLastError();
+        return cudaSuccess;
+    }
     for (int i = 0; i < 5; ++i)
         for (int two = 0; two < 2; ++two) {
             cudaLaunchConfig_t cfg = {};
@@ -592,6 +606,7 @@ cudaError_t prepare(ClusterCaps *caps)
             if ((i == 4 && !wide) || cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) n = 0;
             (two ? caps->two : caps->one)[i] = n;
         }
+    known[dev] = *caps;
     cudaGetLastError();
     return cudaSuccess;
 }

@@ -127,6 +127,7 @@ struct enl_cache {
     int n_sm = 148;                         // multiprocessors of the device (grid sizes, split counts)
     int64_t n_pages = 0;
     size_t layer_bytes = 0;                 // one layer of one pool
+    uint8_t *work = nullptr;                // the device allocation that holds all but the pools
     uint8_t *kpool = nullptr, *vpool = nullptr;
     std::vector<int32_t> free_pages;        // stack of free page ids (page 0 is never in it)
     std::vector<Group> groups;
@@ -207,13 +208,8 @@ void destroy(enl_cache *c)
         cudaDeviceSynchronize();
         if (c->kpool) cudaFree(c->kpool);
         if (c->vpool) cudaFree(c->vpool);
-        if (c->plan_dev) cudaFree(c->plan_dev);
+        if (c->work) cudaFree(c->work);
         if (c->plan_host) cudaFreeHost(c->plan_host);
-        if (c->scratch) cudaFree(c->scratch);
-        if (c->finish_lse) cudaFree(c->finish_lse);
-        if (c->finish_bnd) cudaFree(c->finish_bnd);
-        if (c->status_dev) cudaFree(c->status_dev);
-        if (c->counters_dev) cudaFree(c->counters_dev);
         if (c->plan_copied) cudaEventDestroy(c->plan_copied);
         if (c->host_k) cudaFreeHost(c->host_k);
         if (c->host_v) cudaFreeHost(c->host_v);
@@ -311,17 +307,23 @@ extern "C" int enl_cache_create(const enl_cache_desc_t *desc, enl_cache_t **out)
     c->finish_cap = std::max<int64_t>(static_cast<int64_t>(d.max_q_tokens) * d.n_q_heads, 256ll * c->n_sm);
     const size_t pool_bytes = c->layer_bytes * d.n_layers;
     bool okm = cudaMalloc(&c->kpool, pool_bytes) == cudaSuccess && cudaMalloc(&c->vpool, pool_bytes) == cudaSuccess &&
-               cudaMalloc(&c->plan_dev, c->plan_bytes) == cudaSuccess &&
-               cudaMallocHost(&c->plan_host, c->plan_bytes) == cudaSuccess &&
-               cudaMalloc(&c->scratch, static_cast<size_t>(d.scratch_bytes)) == cudaSuccess &&
-               cudaMalloc(&c->finish_lse, sizeof(float) * c->finish_cap) == cudaSuccess &&
-               cudaMalloc(&c->finish_bnd, sizeof(float2) * c->finish_cap) == cudaSuccess &&
-               cudaMalloc(&c->status_dev, sizeof(int32_t)) == cudaSuccess &&
-               cudaMalloc(&c->counters_dev, sizeof(int32_t) * d.max_batch * d.n_kv_heads) == cudaSuccess;
+               cudaMallocHost(&c->plan_host, c->plan_bytes) == cudaSuccess;
+    // everything else in one allocation: each costs the driver up to a millisecond of mapping
+    size_t at = 0;
+    auto place = [&](size_t bytes) { const size_t o = at; at += align256(bytes); return o; };
+    const size_t at_status = place(sizeof(int32_t)), at_counters = place(sizeof(int32_t) * d.max_batch * d.n_kv_heads), zeroed = at,
+                 at_plan = place(c->plan_bytes), at_lse = place(sizeof(float) * c->finish_cap), at_bnd = place(sizeof(float2) * c->finish_cap),
+                 at_scratch = place(static_cast<size_t>(d.scratch_bytes));
+    okm = okm && cudaMalloc(&c->work, at) == cudaSuccess;
     if (!okm) { cudaGetLastError(); destroy(c); return ENL_E_NOMEM; }
+    c->status_dev = reinterpret_cast<int32_t *>(c->work + at_status);
+    c->counters_dev = reinterpret_cast<int32_t *>(c->work + at_counters);
+    c->plan_dev = c->work + at_plan;
+    c->finish_lse = reinterpret_cast<float *>(c->work + at_lse);
+    c->finish_bnd = reinterpret_cast<float2 *>(c->work + at_bnd);
+    c->scratch = reinterpret_cast<float *>(c->work + at_scratch);
     bool okc = cudaMemset(c->kpool, 0, pool_bytes) == cudaSuccess && cudaMemset(c->vpool, 0, pool_bytes) == cudaSuccess &&
-               cudaMemset(c->status_dev, 0, sizeof(int32_t)) == cudaSuccess &&
-               cudaMemset(c->counters_dev, 0, sizeof(int32_t) * d.max_batch * d.n_kv_heads) == cudaSuccess &&
+               cudaMemset(c->work, 0, zeroed) == cudaSuccess &&
                cudaEventCreateWithFlags(&c->plan_copied, cudaEventDisableTiming) == cudaSuccess &&
                cudaEventRecord(c->plan_copied, 0) == cudaSuccess;
     if (!okc) { cudaGetLastError(); destroy(c); return ENL_E_CUDA; }
