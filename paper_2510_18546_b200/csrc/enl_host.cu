@@ -715,7 +715,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
             // on (one episode, 8 kv heads, 10k keys: 15.4 against 15.6 us; 33k keys: 32.2 against 31.4); below, and wherever they do,
             // the merge through memory costs more (2200 keys: 8.5 against 10.4; four episodes of 9900 keys: 31.7 against 34.9).
             const int n = B * d.n_kv_heads;
-            for (int i = 4; i >= 0 && !cluster; --i) {
+            for (int i = widest_cluster_log(n, most, has_mass); i >= 0 && !cluster; --i) {
                 if ((1 << i) > fewest) continue;
                 list_pages = (ceil_div(most, 1 << i) + 1) & ~1;
                 if (list_pages > kClusterMaxPages) break;

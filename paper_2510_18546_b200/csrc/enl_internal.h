@@ -246,6 +246,12 @@ struct ClusterCaps {
     int two[5], one[5];
     int get(int i, int smem) const { return smem <= kClusterPairSmem ? two[i] : one[i]; }
 };
+// log2 of the widest cluster worth having for `heads` (kv heads x episodes) streams of up to `pages` pages.  Sixteen CTAs read a
+// stream fastest, but clusters of eight start and merge faster: where eight leave every warp one page (two with masses, whose
+// merge grows with the CTAs) they are the better ones.  One token, 8 kv heads, 640 keys in 24 groups: 7.2 against 6.1 us, with masses
+// 8.4 against 7.4; 2560 keys 8.7 against 9.2, with masses 10.4 against 10.1.  Up to four streams, whose sixteens take less than
+// half of the SMs, gain nothing (2 kv heads, 960 keys: 5.56 against 5.67).
+inline int widest_cluster_log(int heads, int pages, bool masses) { return heads > 4 && pages <= 8 * 12 * (masses ? 2 : 1) ? 3 : 4; }
 // Opts the kernels in and asks the device for its capacities.
 cudaError_t prepare_decode_cluster(int head_dim, ClusterCaps *caps);
 size_t decode_smem_bytes(int head_dim);

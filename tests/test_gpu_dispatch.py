@@ -61,6 +61,9 @@ STEP = {
     "below_the_line": dict(Hq=32, Hkv=8, D=128, pool=[[639 * 16 // 4] * 4], n_new=[16]),
     "above_the_line": dict(Hq=32, Hkv=8, D=128, pool=[[656 * 16 // 4] * 4], n_new=[16]),
     "batch": dict(Hq=8, Hkv=2, D=128, pool=[[30, 60, 90], [5, 5, 5, 5], [200], [], [700, 1]], n_new=[1, 10, 129, 16, 33]),
+    "eights_at_most": dict(Hq=32, Hkv=8, D=128, pool=[[90 * 16 // 4] * 4], n_new=[96]),
+    "eights_with_masses": dict(Hq=32, Hkv=8, D=128, pool=[[47 * 16] * 4], n_new=[64]),
+    "sixteens_again": dict(Hq=32, Hkv=8, D=128, pool=[[48 * 16] * 4], n_new=[16]),
     "many_clusters": dict(Hq=16, Hkv=8, D=64, pool=[[40, 25]] * 20, n_new=[9] * 20),
 }
 
