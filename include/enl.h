@@ -368,8 +368,9 @@ typedef struct {
  * kv head, and partials that fit the array (n_q_heads * (head_dim + n_seg + 2) * 4 bytes per
  * 1024 keys); anything larger returns ENL_E_LIMIT and enqueues nothing.
  *
- * The first call on a device looks up the array's device address (cudaGetSymbolAddress, with that
- * device current) and keeps it; make that first call outside any stream capture.  All calls share the
+ * The first call on a device with a head_dim asks the runtime what it has to know there (the device
+ * addresses of the library's own arrays, how many clusters of the kernel run at once) and keeps the
+ * answers in fixed arrays; make that first call outside any stream capture.  All calls share the
  * one array and it keeps the previous call's partials: a call overwrites everything it later reads,
  * so back-to-back calls on one stream are fine, but two calls whose kernels overlap on the GPU
  * (different streams, no dependency) race on it and give wrong results.  Use one stream, or order the

@@ -26,8 +26,6 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
-#include <map>
-#include <mutex>
 #include <type_traits>
 
 #include "decode_ops.cuh"
@@ -577,15 +575,16 @@ cudaError_t prepare(ClusterCaps *caps)
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     if (e != cudaSuccess) return e;
     const bool wide = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
-    // a device's answers are asked for once: ten occupancy queries per kernel are most of what making a small cache takes
-    static std::mutex lock;
-    static std::map<int, ClusterCaps> known;
+    // A device's answers are asked for once: ten occupancy queries per kernel are most of what making a small cache takes.  They
+    // are kept without the heap or a lock, since the entry point that promises to do without comes here, too (callers that race
+    // store the same values).
+    static ClusterCaps known[kMaxDevices];
+    static int ready[kMaxDevices];
     int dev = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    const std::lock_guard<std::mutex> guard(lock);
-    const auto found = known.find(dev);
-    if (found != known.end()) {
-        *caps = found->second;
+    const bool keep = dev >= 0 && dev < kMaxDevices;
+    if (keep && __atomic_load_n(&ready[dev], __ATOMIC_ACQUIRE)) {
+        *caps = known[dev];
         cudaGetLastError();
         return cudaSuccess;
     }
@@ -606,7 +605,10 @@ cudaError_t prepare(ClusterCaps *caps)
             if ((i == 4 && !wide) || cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) n = 0;
             (two ? caps->two : caps->one)[i] = n;
         }
-    known[dev] = *caps;
+    if (keep) {
+        known[dev] = *caps;
+        __atomic_store_n(&ready[dev], 1, __ATOMIC_RELEASE);
+    }
     cudaGetLastError();
     return cudaSuccess;
 }
@@ -620,12 +622,16 @@ int decode_cluster_smem(int head_dim, int list_pages, int list_slots, int rep)
 
 cudaError_t prepare_decode_cluster(int head_dim, ClusterCaps *caps)
 {
-    cudaError_t e;
-    if (head_dim == 128) e = prepare<128, true>(caps);
-    else if (head_dim == 64) e = prepare<64, true>(caps);
-    else return cudaErrorInvalidValue;
-    if (e != cudaSuccess) return e;
-    return head_dim == 128 ? prepare<128, false>(caps) : prepare<64, false>(caps);
+    if (head_dim == 128) return prepare<128, false>(caps);
+    if (head_dim == 64) return prepare<64, false>(caps);
+    return cudaErrorInvalidValue;
+}
+
+cudaError_t prepare_decode_static(int head_dim, ClusterCaps *caps)
+{
+    if (head_dim == 128) return prepare<128, true>(caps);
+    if (head_dim == 64) return prepare<64, true>(caps);
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_decode_cluster(const ClusterDecodeParams &p, int head_dim, int batch, int cluster, cudaStream_t st)

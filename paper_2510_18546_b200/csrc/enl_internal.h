@@ -144,6 +144,7 @@ struct SmallParams : ClusterDecodeParams {
     int2    list[kSmallMaxPages];   // page id, slot << 8 | valid keys
 };
 constexpr int kMaxCluster = 16;
+constexpr int kMaxDevices = 64;     // devices whose properties are kept in fixed arrays
 // Contiguous keys in segments instead of pool pages (the entry point that allocates nothing).
 constexpr int kStaticMaxSeg = 255;
 struct StaticDecodeParams {
@@ -252,8 +253,9 @@ struct ClusterCaps {
 // 8.4 against 7.4; 2560 keys 8.7 against 9.2, with masses 10.4 against 10.1.  Up to four streams, whose sixteens take less than
 // half of the SMs, gain nothing (2 kv heads, 960 keys: 5.56 against 5.67).
 inline int widest_cluster_log(int heads, int pages, bool masses) { return heads > 4 && pages <= 8 * 12 * (masses ? 2 : 1) ? 3 : 4; }
-// Opts the kernels in and asks the device for its capacities.
+// Opt the kernel for pool pages, and the one for contiguous keys, in on the current device and ask for its capacities there.
 cudaError_t prepare_decode_cluster(int head_dim, ClusterCaps *caps);
+cudaError_t prepare_decode_static(int head_dim, ClusterCaps *caps);
 size_t decode_smem_bytes(int head_dim);
 // Page ids of (part of) one group, passed by value to the scatter kernel.
 constexpr int kScatterPages = 64;

@@ -20,7 +20,7 @@
 
 namespace {
 
-constexpr int kMaxDevices   = 64;
+using enl::kMaxDevices;
 constexpr int kMaxSeg       = ENL_STATIC_MAX_SEGMENTS;
 constexpr int kMaxSplits    = 64;
 constexpr int kKeysPerSplit = 1024;                              // scores of one split live in shared memory
@@ -149,7 +149,8 @@ __global__ void __launch_bounds__(kThreads) static_partial_kernel(const StaticPa
 // Set by a bounded wait that expired (there is no cache object whose status call would read it).
 static __device__ int32_t g_static_status;
 
-// What the cluster kernels need to know of a device and head_dim, asked once (racing first calls store the same values).
+// What the cluster kernel needs to know of a device and head_dim, asked once, by the first call there (racing first calls store
+// the same values).
 struct ClusterInfo {
     int ready;
     enl::ClusterCaps caps;
@@ -162,7 +163,7 @@ const ClusterInfo *cluster_info(int dev, int head_dim)
     if (!__atomic_load_n(&c.ready, __ATOMIC_ACQUIRE)) {
         enl::ClusterCaps n = {};
         void *sym = nullptr;
-        if (enl::prepare_decode_cluster(head_dim, &n) != cudaSuccess || cudaGetSymbolAddress(&sym, g_static_status) != cudaSuccess) {
+        if (enl::prepare_decode_static(head_dim, &n) != cudaSuccess || cudaGetSymbolAddress(&sym, g_static_status) != cudaSuccess) {
             cudaGetLastError();
             return nullptr;
         }
