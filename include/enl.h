@@ -21,8 +21,8 @@
  *
  * Every device operation is enqueued on the stream the caller passes (a cudaStream_t cast to
  * void*; NULL = the legacy default stream).  No call synchronises the device except
- * enl_cache_create, enl_cache_free, enl_cache_status and enl_cache_selfcheck.  Validation
- * happens on the host before anything is enqueued: a call that returns a validation error
+ * enl_cache_create, enl_cache_free, enl_cache_status, enl_cache_selfcheck and
+ * enl_static_status.  Validation happens on the host before anything is enqueued: a call that returns a validation error
  * (ENL_E_INVAL, ENL_E_NOGROUP, ENL_E_NOMEM, ENL_E_LIMIT, ENL_E_EVICTED) has enqueued nothing
  * and has left the cache unchanged.  ENL_E_CUDA (a launch or copy that the runtime refused)
  * can come after the tables were updated and after earlier launches of the same call were
@@ -61,7 +61,8 @@ enum {                                            /* return codes               
     ENL_E_NOGROUP  = -2,   /* group id out of range, or never stored for that layer            */
     ENL_E_NOMEM    = -3,   /* page pool, plan buffers or a create-time allocation exhausted    */
     ENL_E_CUDA     = -4,   /* a CUDA call failed, or a GPU operation on a bookkeeping cache    */
-    ENL_E_TIMEOUT  = -5,   /* a bounded wait inside a kernel expired (see enl_cache_status)    */
+    ENL_E_TIMEOUT  = -5,   /* a bounded wait inside a kernel expired (see enl_cache_status and  */
+                           /* enl_static_status)                                               */
     ENL_E_LIMIT    = -6,   /* a size beyond the fixed maxima of enl_attend_static              */
                            /* -7 is not used                                                    */
     ENL_E_EVICTED  = -8,   /* the group's K/V is in the slow tier only (see enl_step_prepare)   */
@@ -376,8 +377,14 @@ typedef struct {
  * (different streams, no dependency) race on it and give wrong results.  Use one stream, or order the
  * calls with events.
  * Errors: ENL_E_INVAL (null pointer, bad shape, negative length), ENL_E_LIMIT, ENL_E_CUDA.
+ * A kernel-side bounded wait that ran out leaves wrong results; enl_static_status reports it.
  */
 int enl_attend_static(const enl_static_args_t *args, void *cuda_stream);
+
+/* What enl_cache_status is for a cache: synchronises the current device and returns ENL_OK, or ENL_E_TIMEOUT if
+ * a kernel of enl_attend_static gave up on a bounded wait there since the last call of this function (the flag is then
+ * cleared).  Allocates nothing; not during a stream capture.  ENL_E_CUDA. */
+int enl_static_status(void);
 
 #ifdef __cplusplus
 }

@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(kThreads) static_partial_kernel(const StaticPa
     }
 }
 
-// Set by a bounded wait that expired (there is no cache object whose status call would read it).
+// Set by a bounded wait that expired, read and cleared by enl_static_status.
 static __device__ int32_t g_static_status;
 
 // What the cluster kernel needs to know of a device and head_dim, asked once, by the first call there (racing first calls store
@@ -156,10 +156,10 @@ struct ClusterInfo {
     enl::ClusterCaps caps;
     int32_t *status;
 };
+ClusterInfo g_cluster_infos[kMaxDevices][2] = {};
 const ClusterInfo *cluster_info(int dev, int head_dim)
 {
-    static ClusterInfo infos[kMaxDevices][2] = {};
-    ClusterInfo &c = infos[dev][head_dim == 128 ? 1 : 0];
+    ClusterInfo &c = g_cluster_infos[dev][head_dim == 128 ? 1 : 0];
     if (!__atomic_load_n(&c.ready, __ATOMIC_ACQUIRE)) {
         enl::ClusterCaps n = {};
         void *sym = nullptr;
@@ -319,4 +319,22 @@ extern "C" int enl_attend_static(const enl_static_args_t *a, void *cuda_stream)
     cp.n_splits = n_splits;
     if (enl::launch_combine(cp, st) != cudaSuccess) { cudaGetLastError(); return ENL_E_CUDA; }
     return ENL_OK;
+}
+
+extern "C" int enl_static_status(void)
+{
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices || cudaDeviceSynchronize() != cudaSuccess) {
+        cudaGetLastError();
+        return ENL_E_CUDA;
+    }
+    for (const ClusterInfo &c : g_cluster_infos[dev]) {
+        if (!__atomic_load_n(&c.ready, __ATOMIC_ACQUIRE)) continue;
+        int32_t word = 0;                                        // one word per device, whichever head_dim
+        if (cudaMemcpy(&word, c.status, sizeof word, cudaMemcpyDeviceToHost) != cudaSuccess) { cudaGetLastError(); return ENL_E_CUDA; }
+        if (word == 0) return ENL_OK;
+        if (cudaMemset(c.status, 0, sizeof word) != cudaSuccess) { cudaGetLastError(); return ENL_E_CUDA; }
+        return ENL_E_TIMEOUT;
+    }
+    return ENL_OK;                                               // no kernel that waits has been launched here
 }

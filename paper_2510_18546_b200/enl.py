@@ -24,7 +24,7 @@ ENL_OK, ENL_E_INVAL, ENL_E_NOGROUP, ENL_E_NOMEM, ENL_E_CUDA, ENL_E_TIMEOUT, ENL_
 ENL_STATIC_MAX_SEGMENTS, ENL_STATIC_MAX_KEYS, ENL_STATIC_SCRATCH_BYTES = 255, 65536, 4 << 20
 
 EXPORTS = ("enl_cache_create", "enl_group_store", "enl_attend", "enl_cache_free", "enl_strerror",
-           "enl_group_store_all_layers", "enl_group_len", "enl_cache_status", "enl_cache_selfcheck", "enl_plan_inspect", "enl_attend_static", "enl_cluster_assign",
+           "enl_group_store_all_layers", "enl_group_len", "enl_cache_status", "enl_cache_selfcheck", "enl_plan_inspect", "enl_attend_static", "enl_static_status", "enl_cluster_assign",
            "enl_cluster_assign_sums", "enl_select_knapsack", "enl_rope_rotate", "enl_tier_enable", "enl_group_evict", "enl_step_prepare", "enl_group_resident")
 
 
@@ -108,6 +108,8 @@ def lib() -> ctypes.CDLL:
         L.enl_plan_inspect.restype = ctypes.c_int
         L.enl_attend_static.argtypes = [ctypes.POINTER(StaticArgs), ctypes.c_void_p]
         L.enl_attend_static.restype = ctypes.c_int
+        L.enl_static_status.argtypes = []
+        L.enl_static_status.restype = ctypes.c_int
         L.enl_cluster_assign.argtypes = [ctypes.POINTER(ClusterArgs), ctypes.c_void_p]
         L.enl_cluster_assign.restype = ctypes.c_int
         L.enl_cluster_assign_sums.argtypes = [ctypes.c_void_p, ctypes.c_int32, ctypes.c_int32, ctypes.c_int32, ctypes.c_void_p,
@@ -227,6 +229,11 @@ def enl_attend_static(seg_len: Sequence[int], n_new: int, q, k, v, out, group_ma
     rc = (_native or _binding()).attend_static(seg_len, n_new, q, k, v, out, group_mass, stream or None)
     if rc != ENL_OK:
         raise EnlError(rc, "enl_attend_static")
+
+
+def enl_static_status() -> int:
+    """ENL_OK, or ENL_E_TIMEOUT when a wait inside a kernel of ``enl_attend_static`` has run out on the current device."""
+    return int(lib().enl_static_status())
 
 
 def enl_cluster_assign(masses: Sequence, obj_off: Sequence[int], n_groups: int, threshold: float, avg, assign,

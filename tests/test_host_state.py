@@ -55,3 +55,18 @@ def test_static_call_uses_no_heap(host, D):
         assert host.enl_attend_static(ctypes.byref(a), None) == enl.ENL_OK
         assert host.fake_heap() == 0, f"call {call}"
     assert host.fake_launches() == 3 and host.fake_kind(0) == ord("c")
+
+
+def test_static_call_that_gave_up_is_reported(host):
+    """An expired wait shows once in the status call, whichever head_dim launched the kernel, and not in later ones."""
+    assert host.enl_static_status() == enl.ENL_OK               # before any call
+    for D in (64, 128):
+        a = static_args(D)
+        assert host.enl_attend_static(ctypes.byref(a), None) == enl.ENL_OK
+        assert host.enl_static_status() == enl.ENL_OK
+        host.fake_expire(1)
+        assert host.enl_attend_static(ctypes.byref(a), None) == enl.ENL_OK
+        host.fake_expire(0)
+        assert host.enl_attend_static(ctypes.byref(a), None) == enl.ENL_OK      # a later call does not hide it
+        assert host.enl_static_status() == enl.ENL_E_TIMEOUT
+        assert host.enl_static_status() == enl.ENL_OK
