@@ -28,6 +28,10 @@
  * can come after the tables were updated and after earlier launches of the same call were
  * enqueued: treat the cache as unusable then.
  *
+ * Calls may be captured into a CUDA graph.  The tables change when a call is captured; its launches run
+ * when the graph does, on the pages that the groups had then.  A captured enl_attend takes its gather
+ * plan along, and calls outside the graph rely on nothing that was only captured.
+ *
  * No position encoding is applied here: cached K is stored as the caller produced it (already
  * rotated at whatever positions the caller assigned to the group), so results do not depend
  * on the order of the select list except for the order of the mass slots.

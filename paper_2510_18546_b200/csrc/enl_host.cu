@@ -158,7 +158,12 @@ struct enl_cache {
     int32_t plan_cluster = 0;               // decode: CTAs per cluster, 0 = the streaming kernel
     int32_t plan_list_pages = 0;            // decode by clusters: most pages one of the CTAs covers
     ClusterCaps cluster_caps = {};          // decode by clusters: how many run at once (none on a bookkeeping-only cache)
-    bool pool_written = true;               // a launch that writes the pool has been enqueued since the last attention launch
+    // Order of launches, outside captures: a launch that writes the plan or the pool has been enqueued since the last attention
+    // launch.  What a capture records runs when its graph does, so calls inside one go by what the same capture holds.
+    bool written = true;
+    unsigned long long settled_graph = 0;   // capture that holds an attention launch behind everything written so far
+    unsigned long long plan_graph = 0;      // capture that holds the write of the current plan
+    bool plan_in_graphs = false;            // some graph may write its plan over the one on the device at any time
     bool plan_pair = false;                 // two splits whose CTAs merge inside the attention kernel (cluster of two)
     bool pairs_ok = false;                  // the device can co-schedule two of the attention kernel's CTAs as a cluster
     std::vector<int32_t> key_sel, key_cu, key_len;   // what the current plan was built from
@@ -195,6 +200,7 @@ struct enl_cache {
     int32_t *h_meta() { return reinterpret_cast<int32_t *>(plan_host + off_meta); }
     int32_t *h_rowslots() { return reinterpret_cast<int32_t *>(plan_host + off_rowslots); }
     uint8_t *h_chg() { return plan_host + off_chg; }
+    void pool_written() { written = true; settled_graph = 0; }
     int32_t *h_rowobj() { return reinterpret_cast<int32_t *>(plan_host + off_rowobj); }
 };
 
@@ -367,20 +373,36 @@ extern "C" int32_t enl_group_len(const enl_cache_t *c, int32_t group_id, int32_t
 
 namespace {
 
+// The capture that `st` is in, 0 = none (a graph's launches run when the graph does, not now).
+unsigned long long capture_of(cudaStream_t st)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    if (cudaStreamGetCaptureInfo(st, &cap, &id) != cudaSuccess) { cudaGetLastError(); return 0; }
+    return cap == cudaStreamCaptureStatusActive ? id + 1 : 0;
+}
+
+// Waits on the host for an event that was recorded outside any capture; legal while a stream is being captured.
+bool host_waits(cudaEvent_t e)
+{
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    bool ok = cudaThreadExchangeStreamCaptureMode(&mode) == cudaSuccess;
+    if (ok) {
+        ok = cudaEventSynchronize(e) == cudaSuccess;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+    }
+    if (!ok) cudaGetLastError();
+    return ok;
+}
+
 // Puts work of `st` that is about to be enqueued behind the loads that are still under way: those of one layer, or (-1) all.
 int join_loads(enl_cache *c, cudaStream_t st, int layer)
 {
     if (c->load_chunks == 0) return ENL_OK;
     const int last = c->load_chunks - 1, other = std::max(0, last - 1);       // the last chunk of either load stream
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) { cudaGetLastError(); cap = cudaStreamCaptureStatusNone; }
-    if (cap == cudaStreamCaptureStatusActive) {
+    if (capture_of(st)) {
         // a graph cannot wait for work outside it, so the host does
-        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-        bool ok = cudaThreadExchangeStreamCaptureMode(&mode) == cudaSuccess;
-        ok = ok && cudaEventSynchronize(c->load_done[other]) == cudaSuccess && cudaEventSynchronize(c->load_done[last]) == cudaSuccess;
-        cudaThreadExchangeStreamCaptureMode(&mode);
-        if (!ok) { cudaGetLastError(); return ENL_E_CUDA; }
+        if (!host_waits(c->load_done[other]) || !host_waits(c->load_done[last])) return ENL_E_CUDA;
         c->load_chunks = 0;
         return ENL_OK;
     }
@@ -474,7 +496,7 @@ extern "C" int enl_group_store(enl_cache_t *c, int32_t group_id, int32_t layer, 
     ++c->epoch;
 
     if (!c->gpu || n_tokens == 0) return ENL_OK;
-    c->pool_written = true;
+    c->pool_written();
     DeviceGuard dg(c->d.device);
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     if (join_loads(c, st, -1) != ENL_OK) return ENL_E_CUDA;
@@ -542,7 +564,7 @@ extern "C" int enl_group_store_all_layers(enl_cache_t *c, int32_t group_id, int3
     ++c->epoch;
 
     if (!c->gpu || n_tokens == 0) return ENL_OK;
-    c->pool_written = true;
+    c->pool_written();
     DeviceGuard dg(c->d.device);
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     if (join_loads(c, st, -1) != ENL_OK) return ENL_E_CUDA;
@@ -796,7 +818,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         }
 
         if (c->plan_copying) {
-            if (cudaEventSynchronize(c->plan_copied) != cudaSuccess) { cudaGetLastError(); return ENL_E_CUDA; }
+            if (!host_waits(c->plan_copied)) return ENL_E_CUDA;
             c->plan_copying = false;
         }
         c->plan_valid = false;
@@ -914,31 +936,43 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         c->plan_layer_ok[a->layer] = 1;
         c->plan_valid = true;
         c->plan_on_device = false;
+        c->plan_graph = 0;
     }
     if (plan_only) return ENL_OK;
     if (join_loads(c, st, a->layer) != ENL_OK) return ENL_E_CUDA;
 
     // The plan goes to the device with the first launch that uses it: as parameters of a small kernel, or, when it is too
     // large for that (beyond some 3500 pages of 16 tokens), as one copy, before which this buffer must not be rebuilt.
-    // (A short call of one episode takes it along in its own parameters.)
+    // (A short call of one episode takes it along in its own parameters.)  A graph that is being captured gets its own writes,
+    // as parameters of as many kernels as it takes: it may run at any time, or never.
+    const unsigned long long graph = capture_of(st);
     const bool plan_inside = c->plan_small_blocks && c->plan_batch == 1;
-    const bool fresh = !c->plan_on_device && !plan_inside;
+    const bool fresh = !plan_inside && (graph ? c->plan_graph != graph : !c->plan_on_device || c->plan_in_graphs);
     if (fresh) {
-        bool okc;
-        if (c->plan_used <= static_cast<size_t>(kPlanParamBytes)) {
-            okc = launch_plan_write(c->plan_dev, c->plan_host, c->plan_used, st) == cudaSuccess;
+        bool okc = true;
+        if (graph || c->plan_used <= static_cast<size_t>(kPlanParamBytes)) {
+            for (size_t at = 0; okc && at < c->plan_used; at += kPlanParamBytes)
+                okc = launch_plan_write(c->plan_dev + at, c->plan_host + at, std::min<size_t>(kPlanParamBytes, c->plan_used - at), st) == cudaSuccess;
         } else {
             okc = cudaMemcpyAsync(c->plan_dev, c->plan_host, c->plan_used, cudaMemcpyHostToDevice, st) == cudaSuccess &&
                   cudaEventRecord(c->plan_copied, st) == cudaSuccess;
             c->plan_copying = true;
         }
         if (!okc) { cudaGetLastError(); c->plan_valid = false; return ENL_E_CUDA; }
-        c->plan_on_device = true;
+        if (graph) {
+            c->plan_graph = graph;
+            c->plan_in_graphs = true;
+            c->settled_graph = 0;
+        } else {
+            c->plan_on_device = true;
+            c->written = true;
+        }
     }
     // Launches that find plan and pool as the attention launch before left them may read both before the kernel before them
-    // has ended.  Ones that do not wait for it first and hold their own successor back until then, so that this carries over.
-    const bool wait_first = fresh || c->pool_written;
-    c->pool_written = false;
+    // has ended.  Ones that do not wait for it first and hold their own successor back until then, so that this carries over:
+    // from an attention launch that was made, not from one that was refused.
+    const bool wait_first = graph ? c->settled_graph != graph : c->written;
+    auto settled = [&]() { if (graph) c->settled_graph = graph; else c->written = false; };
 
     const int slot_stride = c->plan_max_slots + 1;
     if (c->plan_small_blocks || (c->plan_decode && c->plan_cluster)) {
@@ -975,6 +1009,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         dp.scale_log2 = 1.4426950408889634f / sqrtf(static_cast<float>(d.head_dim));
         if ((c->plan_small_blocks ? launch_small(dp, d.head_dim, c->plan_small_groups, c->plan_small_blocks, c->plan_batch, st)
                                   : launch_decode_cluster(dp, d.head_dim, c->plan_batch, c->plan_cluster, st)) != cudaSuccess) { cudaGetLastError(); return ENL_E_CUDA; }
+        settled();
         return ENL_OK;
     }
     if (c->plan_decode) {
@@ -1016,6 +1051,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         dp.wait_first = wait_first ? 1 : 0;
         dp.scale_log2 = 1.4426950408889634f / sqrtf(static_cast<float>(d.head_dim));
         if (launch_decode(dp, d.head_dim, c->plan_batch, st) != cudaSuccess) { cudaGetLastError(); return ENL_E_CUDA; }
+        settled();
         return ENL_OK;
     }
 
@@ -1090,6 +1126,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         mp.scale_log2 = p.scale_log2;
         if (launch_mass(mp, d.head_dim, c->plan_items, st) != cudaSuccess) { cudaGetLastError(); return ENL_E_CUDA; }
     } else if (launch_attention(p, d.head_dim, c->plan_items, st) != cudaSuccess) { cudaGetLastError(); return ENL_E_CUDA; }
+    settled();
     if (c->plan_finish) {
         FinishParams fp;
         fp.mass = a->group_mass;
@@ -1390,7 +1427,7 @@ extern "C" int enl_step_prepare(enl_cache_t *c, const int32_t *sel_ids, int32_t 
             g.resident = true;                                         // host copy stays current until the next store
             stt.bytes_h2d += static_cast<int64_t>(np) * page_bytes_of(c) * 2 * c->d.n_layers;
         }
-        c->pool_written = true;
+        c->pool_written();
         const int rc = enqueue_loads(c, n, st);
         if (rc != ENL_OK) return rc;
     }

@@ -13,7 +13,7 @@ struct Record { char kind; int wait_first; size_t bytes; };      // launch ('w' 
 Record g_log[4096];
 int g_n_log;
 int g_heap;                      // allocations of the library's code since the last look
-int g_fail_kind;                 // launches of this kind are refused
+int g_fail_kind;                 // launches of this kind are refused ('e': tensor maps)
 int g_wait_expires;              // the next one-token kernel gives up on a wait
 unsigned long long g_capture;    // the stream is being captured (as this graph)
 bool g_captured_event;           // the last record of any event was captured
@@ -27,7 +27,7 @@ cudaError_t note(char kind, int wait_first, size_t bytes = 0)
 CUresult encode(CUtensorMap *tm, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
                 const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill)
 {
-    if (g_fail_kind == 'm') return CUDA_ERROR_INVALID_VALUE;
+    if (g_fail_kind == 'e') return CUDA_ERROR_INVALID_VALUE;
     std::memset(tm, 0, sizeof *tm);
     return CUDA_SUCCESS;
 }
@@ -100,6 +100,12 @@ cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus *s)
 {
     *s = g_capture ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
     return cudaSuccess;
+}
+cudaError_t cudaStreamGetCaptureInfo(cudaStream_t st, cudaStreamCaptureStatus *s, unsigned long long *id, cudaGraph_t *, const cudaGraphNode_t **,
+                                     size_t *)
+{
+    *id = g_capture;
+    return cudaStreamIsCapturing(st, s);
 }
 cudaError_t cudaThreadExchangeStreamCaptureMode(cudaStreamCaptureMode *) { return cudaSuccess; }
 cudaError_t cudaFuncSetAttribute(const void *, cudaFuncAttribute, int) { return cudaSuccess; }

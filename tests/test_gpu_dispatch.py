@@ -325,3 +325,34 @@ def test_short_calls_between_long_ones_and_stores():
         for out, (ks, vs) in zip(outs, want):
             ro, _ = orc.attend_slots(8, 2, 128, ks, vs, q.cpu(), kn.cpu(), vn.cpu())
             check_close(out, ro, None, None, what=wl.name)
+
+
+@pytest.mark.parametrize("n_q, pages", [(20, 4), (300, 60), (1, 60), (40, 3700)])
+def test_graphs_and_calls_beside_them(n_q, pages):
+    """A call captured into a graph that has not run yet, calls outside the graph before and after it runs, over either list: each
+    goes by its own gather plan (in the parameters, written in one piece, in several)."""
+    wl = synth.make_small(65, 1, 4, 1, 64, [[5, 40, 16 * pages]], [[0, 1, 2]], [n_q], [n_q], name=f"graph {n_q} rows, {pages} pages")
+    with Session(wl, [0]) as s:
+        q, kn, vn = wl.new_qkv(0, s.device)
+        lists = [np.asarray(x, np.int32) for x in ([2, 0], [1, 2])]
+
+        def attend(i):
+            out = torch.empty_like(q)
+            enl.enl_attend(s.cache, 0, lists[i], q, kn, vn, out, stream=torch.cuda.current_stream().cuda_stream)
+            return out
+
+        got = [(0, attend(0))]
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            in_graph = attend(1)
+        got += [(1, attend(1)), (0, attend(0))]
+        graph.replay()
+        got += [(0, attend(0)), (1, in_graph.clone()), (1, attend(1))]
+        torch.cuda.synchronize()
+        assert enl.enl_cache_status(s.cache) == enl.ENL_OK
+        rows = sorted({0, n_q // 2, n_q - 1})
+        for i, out in got:
+            ks, vs = ([x[g] for g in lists[i]] for x in s.host_kv[(0, 0)])
+            ro, _ = orc.attend_slots(4, 1, 64, ks, vs, q.cpu(), kn.cpu(), vn.cpu(), rows=rows)
+            check_close(out[rows], ro, None, None, what=f"{wl.name}, list {i}")

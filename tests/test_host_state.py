@@ -70,3 +70,91 @@ def test_static_call_that_gave_up_is_reported(host):
         assert host.enl_attend_static(ctypes.byref(a), None) == enl.ENL_OK      # a later call does not hide it
         assert host.enl_static_status() == enl.ENL_E_TIMEOUT
         assert host.enl_static_status() == enl.ENL_OK
+
+
+class Cache:
+    """A cache on the fake device: two groups of 64 rows and one of `long` rows, and calls over them that take each of the routes."""
+    ROUTES = dict(short=("a", [0, 1], 20, 0), prefill=("a", [0, 2], 300, 0), cluster=("c", [0, 1], 1, 0), stream=("d", [0, 2], 1, 8),
+                  masses=("m", [0, 2], 40, 0))
+
+    def __init__(self, host, long=4000):
+        self.host, self.h = host, ctypes.c_void_p()
+        d = enl.CacheDesc(2, 8, 2, 128, 0, 4, long + 200, enl.ENL_BF16, 0, 4, 512, 0)
+        assert host.enl_cache_create(ctypes.byref(d), ctypes.byref(self.h)) == enl.ENL_OK
+        for g, n in enumerate((64, 64, long)):
+            self.store(g, n)
+
+    def store(self, group, n):
+        for layer in range(2):
+            assert self.host.enl_group_store(self.h, group, layer, n, ctypes.c_void_p(1 << 20), ctypes.c_void_p(1 << 21), 0, None) == enl.ENL_OK
+
+    def attend(self, route, layer=0):
+        """Return code, and what was launched: (kind, wait_first) of every launch."""
+        kind, sel, n_q, split = self.ROUTES[route]
+        ids = np.asarray(sel, np.int32)
+        a = enl.AttendArgs()
+        a.layer, a.batch, a.n_sel, a.n_q, a.n_new, a.split_hint = layer, 1, len(ids), n_q, n_q, split
+        a.sel_ids, a.mass_stride = ids.ctypes.data, len(ids) + 1
+        a.q, a.k_new, a.v_new, a.out, a.group_mass = ((1 << 20) * i for i in range(1, 6))
+        a.flags = enl.ENL_MASS_ONLY if route == "masses" else 0
+        self.host.fake_clear()
+        rc = self.host.enl_attend(self.h, ctypes.byref(a), None)
+        return rc, [(chr(self.host.fake_kind(i)), self.host.fake_wait_first(i)) for i in range(self.host.fake_launches())]
+
+    def waits(self, route, layer=0):
+        """wait_first of a call that goes through, and whether it wrote the gather plan."""
+        rc, log = self.attend(route, layer)
+        assert rc == enl.ENL_OK
+        (first,) = [w for k, w in log if k == self.ROUTES[route][0]]
+        return first, any(k in "wp" for k, _ in log)
+
+
+@pytest.mark.parametrize("refused", ["launch", "map"])
+@pytest.mark.parametrize("route", sorted(Cache.ROUTES))
+def test_refused_launch_settles_nothing(host, route, refused):
+    """The pages stored before a call whose launch was refused may still be on their way in the call after it."""
+    c = Cache(host)
+    host.fake_fail(ord(Cache.ROUTES[route][0] if refused == "launch" else "e"))
+    assert c.attend(route)[0] == enl.ENL_E_CUDA
+    host.fake_fail(0)
+    assert c.waits(route)[0] == 1
+    assert c.waits(route, layer=1) == (0, False)
+    c.store(1, 60)
+    assert c.waits(route)[0] == 1
+
+
+@pytest.mark.parametrize("route", sorted(Cache.ROUTES))
+def test_captured_call_settles_nothing_outside_its_graph(host, route):
+    """A captured call has run when its graph runs, if it does: calls outside the graph go by what was launched outside it, and a
+    graph brings its gather plan along, however often and after whatever it runs."""
+    inside = route == "short"                                   # such a call carries its plan in its own parameters
+    c = Cache(host)
+    host.fake_capture(7)
+    assert c.waits(route) == (1, not inside)
+    assert c.waits(route, layer=1) == (0, False)                # behind the first one in the same graph
+    host.fake_capture(0)
+    assert c.waits(route) == (1, not inside)                    # the stores are still to be waited for, the plan to be written
+    if inside:
+        assert c.waits(route, layer=1) == (0, False)
+    else:
+        assert c.waits(route, layer=1) == (1, True)             # the graph may have run in between and written its own plan there
+    host.fake_capture(8)
+    assert c.waits(route) == (1, not inside)
+    c.store(1, 60)
+    assert c.waits(route)[0] == 1
+    host.fake_capture(0)
+    assert c.waits(route) == (1, not inside)
+
+
+def test_captured_plan_of_any_size_is_part_of_the_graph(host):
+    """A plan too large for one launch's parameters is copied from a buffer that the next plan overwrites; a graph may run later
+    than that, so it takes the plan along in pieces.  The next plan does not wait for what was captured."""
+    c = Cache(host, long=90000)
+    assert [k for k, _ in c.attend("prefill")[1]][:2] == ["p", "a"]
+    host.fake_capture(7)
+    rc, log = c.attend("prefill")
+    assert rc == enl.ENL_OK and [k for k, _ in log][:3] == ["w", "w", "a"]
+    assert 28672 == host.fake_bytes(0) >= host.fake_bytes(1) > 0
+    host.fake_capture(0)
+    c.store(2, 89000)
+    assert c.waits("prefill") == (1, True)
