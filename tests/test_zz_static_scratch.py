@@ -85,3 +85,61 @@ def test_limits_are_reported_not_enqueued():
     with pytest.raises(enl.EnlError) as e:
         enl.enl_attend_static([10], 0, q, kv, kv, out)
     assert e.value.code == enl.ENL_E_INVAL
+
+
+def rounded(p, terms):
+    """p as the sum of its first `terms` bf16 terms."""
+    got = np.zeros_like(p)
+    for _ in range(terms):
+        got += torch.tensor(p - got).to(torch.bfloat16).double().numpy()
+    return got
+
+
+@pytest.mark.parametrize("path", ["cluster", "general"])
+@pytest.mark.parametrize("D", [64, 128])
+def test_probabilities_are_fp32(D, path):
+    """Three neighbouring keys whose values all but cancel: v_b = -bf16(v_a p_a / p_b), v_c = -bf16 of what that leaves.  The rest
+    is some 2^-18 of v_a, so an output shows how exactly the probabilities went into the product: with two bf16 terms of them (17
+    bits) it is wrong altogether, while fp32 arithmetic keeps it within a few per cent."""
+    Hq, Hkv, seg, n_new, dev = 8, 2, [16, 5, 33], 10, torch.device("cuda:0")
+    n = sum(seg) + n_new
+    gen = torch.Generator().manual_seed(D)
+    q = torch.randn(Hkv, 1, D, generator=gen).repeat(1, Hq // Hkv, 1).reshape(Hq, D).to(torch.bfloat16)      # all heads of a kv head agree
+    k = (0.7 * torch.randn(n, Hkv, D, generator=gen)).to(torch.bfloat16)
+    v = (1.0 + torch.rand(n, Hkv, D, generator=gen)).to(torch.bfloat16)
+    s = np.einsum("hd,nhd->hn", q.reshape(Hkv, -1, D)[:, 0].double().numpy(), k.double().numpy()) / np.sqrt(D)
+    p = np.exp(s - s.max(axis=1, keepdims=True))
+    p /= p.sum(axis=1, keepdims=True)
+    ends = np.cumsum([0] + seg + [n_new])
+    pages = [(i, min(i + 16, e)) for a, e in zip(ends, ends[1:]) for i in range(a, e, 16)]
+    for a, e in pages:                                           # the three are of one page, so that one warp adds them up
+        v[a + (e - a) // 3 * 3:e] = 0                            # keys without partners
+        for i in range(a, e - 2, 3):
+            rest = v[i].double()                                 # what key i (then i + 1) leaves, in units of the next key's probability
+            for j in (i + 1, i + 2):
+                rest = rest * torch.tensor(p[:, j - 1] / p[:, j])[:, None]
+                v[j] = (-rest).to(torch.bfloat16)
+                rest = rest + v[j].double()
+    vd = v.double().numpy()
+    ks, vs = ([x[a:e] for a, e in zip(ends[:-2], ends[1:-1])] for x in (k, v))
+    want, _ = orc.attend_slots(Hq, Hkv, D, ks, vs, q[None], k[ends[-2]:], v[ends[-2]:])
+    want = want.reshape(Hkv, -1, D)[:, 0]
+    size = np.linalg.norm(want)
+    # one bf16 rounding of the output; scores (products and sums in fp32), ex2 and the sums of the second product each err by
+    # about 2^-23 of a probability, independently from key to key
+    bound = 2.0 ** -9 + 2.0 ** -21 * np.linalg.norm(np.sqrt(np.einsum("hn,nhd->hd", p ** 2, vd ** 2))) / size
+    for terms, enough in ((1, False), (2, False), (3, True)):
+        err = np.linalg.norm(np.einsum("hn,nhd->hd", rounded(p, terms), vd) - want) / size
+        assert (err < bound / 8) if enough else (err > 1.5 * bound), (terms, err, bound)
+    out = torch.empty(Hq, D, dtype=torch.bfloat16, device=dev)
+    flat = torch.empty(2, n * Hkv * D + 8, dtype=torch.bfloat16, device=dev)
+    at = 0 if path == "cluster" else 1                           # tensors off the 16-byte boundary take the general kernels
+    kd, vv = (x[at:at + n * Hkv * D].view(n, Hkv, D) for x in flat)
+    kd.copy_(k), vv.copy_(v)
+    enl.enl_attend_static(seg, n_new, q.to(dev), kd, vv, out, None)
+    torch.cuda.synchronize()
+    assert enl.enl_static_status() == enl.ENL_OK
+    got = out.double().cpu().numpy().reshape(Hkv, -1, D)
+    for h in range(Hq // Hkv):
+        err = np.linalg.norm(got[:, h] - want) / size
+        assert err <= bound, (h, err, bound)
