@@ -15,8 +15,9 @@
 //   - key ranges may be split over CTAs: a slot that two splits share is written by the earlier one, the later one's part and
 //     every split's log2-sum-exp go to mass_finish_kernel, which turns log-sums into masses.
 // Bound by the exponentials and the issue slots around them, not by the tensor pipe.  Measured against the general kernel
-// that skipped its output: 512 rows x 32 heads over 200 groups (16 000 keys) 375 -> 165 us a layer, of which the two-way split of the
-// keys is half; per key tile and pair of Q tiles 4400 -> 2940 cycles.
+// that skipped its output: 512 rows x 32 heads over 200 groups (16 000 keys) 375 -> 122 us a layer, mass_finish_kernel included
+// (this kernel alone 117 in a serialised capture), of which the two-way split of the keys is half; per key tile and pair of Q tiles
+// 4400 -> 2940 cycles.
 #include <cuda_bf16.h>
 
 #include "attn_ops.cuh"

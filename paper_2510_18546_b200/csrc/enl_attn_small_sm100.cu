@@ -14,8 +14,10 @@
 // stream order, so a row has one open slot; its log2-sum is parked when it ends.
 // When neither plan nor pool have been written since the last attention launch the cached pages are fetched before the wait
 // for the previous kernel.
-// Measured per launch in a chain of layers (D 128, 32 q / 8 kv heads, large kernel -> this one): 41 rows over 121 keys 10.4 -> 6.9 us,
-// 61 over 301 12.9 -> 8.6, 128 over 308 14.4 -> 9.4, 256 over 276 13.6 -> 11.5.
+// Measured per launch in a chain of 20 layers (32 q / 8 kv heads, large kernel -> this one), one group, no masses: D 128, 41 rows
+// over 121 keys 9.5 -> 5.5 us, 61 over 301 11.1 -> 7.4, 128 over 308 12.4 -> 8.4, 256 over 276 12.5 -> 10.6; four groups with
+// masses 9.5 -> 7.1, 11.3 -> 8.3, 12.1 -> 9.4, 12.6 -> 11.7.  D 64, four groups with masses: 8.5 -> 5.4, 9.7 -> 6.2, 10.8 -> 6.9,
+// 10.7 -> 8.6.
 #include <cuda_bf16.h>
 
 #include "decode_ops.cuh"

@@ -6,13 +6,15 @@
 // The time of such a call is latency, not bandwidth: with 2600 keys all the CTAs' loads are in flight at once and the
 // streaming kernel spends 6 of its 8.6 us on merging -- partial results to memory, a fence, a counter, and the last CTA
 // reading them back (0.9 + 1.9 us), while the next launch cannot even start.  Here the splits of one (episode, kv head) are
-// the CTAs of one thread-block cluster: each merges its warps in its own shared memory, one cluster barrier later every CTA
-// reads its share of the others' results and writes it out.  And two CTAs fit an SM (12 warps of 80 registers, ~110 KB),
-// so the next launch is resident while this one runs: its set-up and its first pages (from the pool, which only this
-// library writes) are done before its wait for the previous kernel ends.
-// Measured per launch in a chain of layers (32 q / 8 kv heads, D 128, masses wanted, streaming kernel -> this one): 240 keys
-// 9.2 -> 8.0 us, 2200 keys 10.4 -> 8.4, 4900 keys 12.0 -> 10.8, 16 episodes of 3160 keys 39.1 -> 38.6, 8 of 3200 25.9 -> 23.1;
-// contiguous keys (the entry point that allocates nothing), 2500 keys 91 -> 11.0.
+// the CTAs of one thread-block cluster: each merges its warps in its own shared memory and pushes what the others need of
+// the result into theirs; behind the cluster barrier every CTA adds up its share of the output out of its own shared memory
+// and writes it out.  And two CTAs fit an SM (12 warps of 80 registers, ~110 KB), so the next launch is resident while this
+// one runs: its set-up and its first pages (from the pool, which only this library writes) are done before its wait for the
+// previous kernel ends.
+// Measured per launch in a chain of 20 layers (32 q / 8 kv heads, 24 groups, masses wanted, streaming kernel -> this one): D 128,
+// 640 keys 9.2 -> 6.0 us, 2200 keys 10.2 -> 8.1, 4900 keys 11.9 -> 10.1, 16 episodes of 3160 keys 38.1 -> 37.8, 8 of 3200
+// 24.5 -> 22.3; D 64, the same, 8.6 -> 5.5, 9.1 -> 6.9, 10.3 -> 8.5, 28.7 -> 22.8, 20.2 -> 14.7; contiguous keys (the entry point
+// that allocates nothing), D 128, 2500 keys 91 -> 9.3 (10.2 where every layer's keys come from memory).
 //
 // Per page, all in registers of one warp:
 //   S^T = K Q^T        mma.sync m16n8k16, A = the 16 keys (ldmatrix), B = the rep query rows padded to 8

@@ -716,8 +716,8 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
             return static_cast<int64_t>(ns) * a->n_q * d.n_q_heads * per_rh * 4 +
                    static_cast<int64_t>(ns) * B * d.n_kv_heads * 8 + 16 <= d.scratch_bytes;
         };
-        // One query token per episode: the streaming decode kernel, whose CTAs cover at most kDecodeMaxPages
-        // pages each and always hand their partial results to the merge kernel.
+        // One query token per episode: the streaming decode kernel, whose CTAs cover at most kDecodeMaxPages pages each (the
+        // last one of a kv head to finish merges their partial results), or the one merged by clusters.
         bool decode = c->rep <= 8 && !mass_only && !has_sum;
         int need = 1, fewest = 0x7fffffff, most = 1;
         for (int b = 0; b < B && decode; ++b) {
@@ -732,10 +732,13 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         int n_splits = 1, cluster = 0;
         int list_pages = 0;
         if (decode && a->split_hint == 0) {
-            // Splits merged by a thread-block cluster: as many CTAs per (episode, kv head) as run at once.  When they do not fill
-            // two CTAs per SM the streaming kernel, whose CTAs keep more in flight, is faster from some 40 pages per CTA
-            // on (one episode, 8 kv heads, 10k keys: 15.4 against 15.6 us; 33k keys: 32.2 against 31.4); below, and wherever they do,
-            // the merge through memory costs more (2200 keys: 8.5 against 10.4; four episodes of 9900 keys: 31.7 against 34.9).
+            // Splits merged by a thread-block cluster: the widest one worth having of which all (episode, kv head) pairs' run at
+            // once.  When they do not fill one and a half CTAs per SM the streaming kernel, whose CTAs keep more in flight, is faster
+            // from some 40 pages per CTA on; below, and wherever they do, its merge through memory costs more.  Measured with masses
+            // (clusters against streaming, us), one episode, 8 kv heads, D 128: 2200 keys 8.1 / 10.2, 7000 keys 12.3 / 13.3, 10k keys
+            // (40 pages) 14.6 / 14.4, 20k keys 21.1 / 19.4, 33k keys 30.0 / 26.3; four episodes of 9900 keys 29.3 / 30.3.  D 64: 6.9 / 9.1,
+            // 9.9 / 11.8, 11.3 / 12.4, 15.0 / 15.6, 20.0 / 19.3; 18.2 / 23.1, so there the line could lie at some 100 pages.  With few
+            // kv heads, too: D 128, 10k keys, 2 kv heads 10.5 / 15.7, 4 kv heads 12.3 / 14.9.
             const int n = B * d.n_kv_heads;
             for (int i = widest_cluster_log(n, most, has_mass); i >= 0 && !cluster; --i) {
                 if ((1 << i) > fewest) continue;
@@ -789,7 +792,10 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
             // A launch takes about T us per key tile of its longest CTA on top of what it always takes: 8.5 us in one split,
             // 10.5 with two splits merged by pairs, 11.5 with partial results in memory plus 0.15 us per 1000 of their rows.
             // (T = 2.25 for two Q tiles, 2.0 for one.  17 to 320 rows over 640 to 5120 keys, measured against two tiles or
-            // more per split: 17 rows over 640 keys 15.0 -> 10.4 us, 41 over 640 17.0 -> 12.6, 320 over 1280 27.0 -> 25.9.)
+            // more per split: 17 rows over 640 keys 15.0 -> 10.4 us, 41 over 640 17.0 -> 12.6, 320 over 1280 27.0 -> 25.9.  The same
+            // figures serve head_dim 64, whose tiles take 0.93 of the time: of 17, 41, 128 and 320 rows over 640, 1280, 2560 and
+            // 5120 keys the best of 1, 2, 3, 4, 6, 8, 12 and 16 splits takes 0.94 of the chosen number's time at worst, 1.00 in
+            // the middle; at head_dim 128 0.91 and 1.00.)
             // Of equal costs the fewest splits: SMs left over take in the next launch.
             auto filling = [&]() {
                 int best = 1;
@@ -1194,7 +1200,7 @@ int enqueue_evictions(enl_cache *c, int n, cudaStream_t st)
 
 // Loads are bound by the host link (about 51 GB/s of scattered pages), while the attention that follows needs its layer only.
 // So they run on streams of their own behind what the caller's stream holds, in chunks of layers, and a layer's attention waits
-// for its chunk.  Two steps of 20 layers (46 MB each) with attends of 128 rows: 2356 -> 1867 us.
+// for its chunk.  Two steps of 20 layers (46 MB each) with attends of 128 rows: 2356 -> 1857 us.
 // - A chunk has at least kLoadChunkBytes: two streams that take turns hide the gaps between chunks down to that size.  What fits
 //   into one chunk stays on the caller's stream.
 // - As few bytes in flight as the link needs (two streams of 32 warps with 2 KB each): what waits for the link stands in the way

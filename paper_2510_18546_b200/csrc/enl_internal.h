@@ -248,10 +248,14 @@ struct ClusterCaps {
     int get(int i, int smem) const { return smem <= kClusterPairSmem ? two[i] : one[i]; }
 };
 // log2 of the widest cluster worth having for `heads` (kv heads x episodes) streams of up to `pages` pages.  Sixteen CTAs read a
-// stream fastest, but clusters of eight start and merge faster: where eight leave every warp one page (two with masses, whose
-// merge grows with the CTAs) they are the better ones.  One token, 8 kv heads, 640 keys in 24 groups: 7.2 against 6.1 us, with masses
-// 8.4 against 7.4; 2560 keys 8.7 against 9.2, with masses 10.4 against 10.1.  Up to four streams, whose sixteens take less than
-// half of the SMs, gain nothing (2 kv heads, 960 keys: 5.56 against 5.67).
+// stream fastest, but clusters of eight start and merge faster.  Measured (one token, 24 groups, sixteens against eights, us):
+//   8 kv heads, D 128, 640 keys (a page a warp) 5.87 against 4.97, with masses 7.17 against 5.97; 1280 keys (two pages) 6.20
+//     against 6.31, with masses 7.46 against 7.39; 2560 keys 6.66 against 7.10, with masses 8.09 against 8.33
+//   8 kv heads, D 64, the same sizes: 5.16 / 4.44, 6.42 / 5.62; 5.32 / 5.34, 6.57 / 6.42; 5.76 / 5.99, 7.03 / 7.27
+//   6 kv heads, D 128, with masses: 640 keys 6.44 / 6.20, 1280 keys 6.67 / 7.40, 2560 keys 7.12 / 8.87
+//   2 kv heads, D 128: 640 keys 4.62 / 4.52, 960 keys 4.70 / 4.65
+// So a page a warp is where eights are the better ones, most of all at eight streams, whose sixteens leave an SM no room; the two pages
+// that the rule grants calls with masses are about even at eight streams and lose at five and six.
 inline int widest_cluster_log(int heads, int pages, bool masses) { return heads > 4 && pages <= 8 * 12 * (masses ? 2 : 1) ? 3 : 4; }
 // Opt the kernel for pool pages, and the one for contiguous keys, in on the current device and ask for its capacities there.
 cudaError_t prepare_decode_cluster(int head_dim, ClusterCaps *caps);

@@ -8,7 +8,8 @@
 //
 // The call is one launch of decode_cluster_kernel, which reads keys of any segment through tensor maps of the caller's
 // tensors and merges its splits through distributed shared memory: no partial results in memory at all.  (The kernels below
-// took 91 us for 2500 keys x 8 kv heads, one FMA per key, head and channel with uncoalesced reads of V; 11.0 us now.)
+// took 91 us for 2500 keys x 8 kv heads, one FMA per key, head and channel with uncoalesced reads of V; 9.3 us now, and 3.5 us of
+// host time per call, which the launches hide.)
 // They remain for what those maps cannot address: tensors that do not start on a 16-byte boundary, and devices that cannot
 // place a cluster.  Their partial results are held in a file-scope device array of fixed size, whose name is only a host-side
 // handle in host code; its device address is looked up once per device with cudaGetSymbolAddress.
