@@ -1,43 +1,15 @@
-// PTX wrappers shared by the tcgen05 kernels: barriers, TMA, MMA issue, packed arithmetic, descriptors.
+// PTX wrappers of the tcgen05 kernels: waits, pairs of CTAs, MMA issue, packed arithmetic, descriptors.
 #pragma once
-#include <cuda.h>
-#include <cuda_bf16.h>
-#include <stdint.h>
+#include "ptx_ops.cuh"
 
 namespace enl {
 namespace {
 
-constexpr unsigned long long kWaitLimitNs = 1000ull * 1000ull * 1000ull;
 constexpr uint32_t kFull = 0xffffffffu;
 
-__device__ __forceinline__ uint32_t smem_u32(const void *p)
-{
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
 __device__ __forceinline__ void mbar_arrive(uint32_t bar)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-// One poll: the thread may stay suspended inside the instruction for up to the hinted time, and is woken when
-// the phase completes; a longer hint means fewer polling instructions competing with the warps that work.
-constexpr uint32_t kSuspendHintNs = 20000;
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok) : "r"(bar), "r"(parity), "r"(kSuspendHintNs) : "memory");
-    return ok != 0;
 }
 // A test that never suspends (about 35 cycles until its result can be used, half of a poll with a suspend hint).
 __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity)
@@ -63,19 +35,12 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t par
         : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
 }
-// Distributed shared memory of a two-CTA cluster: address of the peer's copy of a local shared-memory location,
-// stores to it, and arrivals on its barriers.
+// Distributed shared memory of a two-CTA cluster: stores to the peer's, and arrivals on its barriers.
 __device__ __forceinline__ uint32_t cluster_rank()
 {
     uint32_t r;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
     return r;
-}
-__device__ __forceinline__ uint32_t peer_addr(uint32_t local, uint32_t rank)
-{
-    uint32_t a;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(local), "r"(rank));
-    return a;
 }
 // 16-byte store into the peer's shared memory whose completion is counted (in bytes) on a barrier of the peer: the
 // sender needs no release fence, which would also wait for its earlier global stores
@@ -103,12 +68,6 @@ __device__ __forceinline__ void cluster_sync_all()
 {
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ unsigned long long global_ns()
-{
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
 }
 // Bounded wait: gives up about kWaitLimitNs after its 16th failed poll, or when another role has raised the abort flag.
 // The result is made warp-uniform so that warp-collective tcgen05 instructions stay converged.
@@ -138,29 +97,6 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
         }
     }
     return __all_sync(kFull, ok);
-}
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *tm, int x, int y, uint32_t bar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-        ::"r"(dst), "l"(tm), "r"(x), "r"(y), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *tm, int x, int y, int z, uint32_t bar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
-        ::"r"(dst), "l"(tm), "r"(x), "r"(y), "r"(z), "r"(bar) : "memory");
-}
-// Bring a box into the L2 without a destination in the SM: nothing is observed, so these may run before the wait for
-// the previous kernel of the stream (the L2 is the point of coherence: a later write to those lines updates them).
-__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap *tm, int x, int y)
-{
-    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(tm), "r"(x), "r"(y) : "memory");
-}
-__device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap *tm, int x, int y, int z)
-{
-    asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];"
-                 ::"l"(tm), "r"(x), "r"(y), "r"(z) : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after()  { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -201,18 +137,6 @@ __device__ __forceinline__ void tc_commit(uint32_t bar)
     if (elect_one())
         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
-__device__ __forceinline__ float ex2(float x)
-{
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-__device__ __forceinline__ float lg2(float x)
-{
-    float y;
-    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
 
 // 3-input max and packed 2 x fp32 arithmetic (one issue slot for two lanes of work)
 __device__ __forceinline__ float fmax3(float a, float b, float c)
@@ -242,11 +166,6 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
     uint64_t d;
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
-}
-__device__ __forceinline__ uint32_t bf16x2(float lo, float hi)
-{
-    const __nv_bfloat162 b = __floats2bfloat162_rn(lo, hi);
-    return *reinterpret_cast<const uint32_t *>(&b);
 }
 
 // Shared-memory matrix descriptor, 128-byte swizzle, rows of 128 B, 8-row groups 1024 B apart.
@@ -278,7 +197,6 @@ __host__ __device__ constexpr uint32_t make_idesc(int n, bool b_mn_major)
          | (static_cast<uint32_t>(128 >> 4) << 24);  // M
 }
 
-constexpr float kNegInf = -__builtin_huge_valf();
 
 }  // namespace
 }  // namespace enl

@@ -505,7 +505,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                     a0 = ex2(a0);
                     a1 = ex2(a1);
                     const uint64_t p2 = pack2(a0, a1);
-                    pk[x] = bf16x2(a0, a1);
+                    pk[x] = pack_bf16(a0, a1);
                     ps2[e] = (x & 7) ? add2(ps2[e], p2) : p2;
                 }
                 tmem_st16(t_s + static_cast<uint32_t>(ch * 16), pk);
@@ -624,7 +624,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                                 tmem_ld32_wait(t_o + static_cast<uint32_t>(pc * 64 + k * 32), o);
 #pragma unroll
                                 for (int x = 0; x < 16; ++x)
-                                    w[k * 16 + x] = bf16x2(__uint_as_float(o[2 * x]) * inv, __uint_as_float(o[2 * x + 1]) * inv);
+                                    w[k * 16 + x] = pack_bf16(__uint_as_float(o[2 * x]) * inv, __uint_as_float(o[2 * x + 1]) * inv);
                             }
                             flush_piece(w, static_cast<uint8_t *>(p.out), D * 2, pc);
                         }
@@ -757,8 +757,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                                     const float4 a = *reinterpret_cast<const float4 *>(
                                         theirs + ((((pc * 2 + k) * 8 + cch) ^ (lane & 7)) << 4));
                                     auto mix = [&](uint32_t own, float th) { return fmaf(__uint_as_float(own), w_own, th * w_peer); };
-                                    w[k * 16 + 2 * cch] = bf16x2(mix(o[4 * cch], a.x), mix(o[4 * cch + 1], a.y));
-                                    w[k * 16 + 2 * cch + 1] = bf16x2(mix(o[4 * cch + 2], a.z), mix(o[4 * cch + 3], a.w));
+                                    w[k * 16 + 2 * cch] = pack_bf16(mix(o[4 * cch], a.x), mix(o[4 * cch + 1], a.y));
+                                    w[k * 16 + 2 * cch + 1] = pack_bf16(mix(o[4 * cch + 2], a.z), mix(o[4 * cch + 3], a.w));
                                 }
                             }
                             flush_piece(w, static_cast<uint8_t *>(p.out), D * 2, pc);

@@ -30,26 +30,6 @@ constexpr int kWarps     = 12;
 constexpr int kThreads   = kWarps * 32;
 constexpr float kRescaleThreshold = 8.0f;                 // log2 units
 
-__device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
-{
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
-// (no evict-first hint: the row blocks of a kv head share its pages)
-__device__ __forceinline__ void plain_load_2d(uint32_t dst, const CUtensorMap *tm, int x, int y, uint32_t bar)
-{
-    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                 ::"r"(dst), "l"(tm), "r"(x), "r"(y), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void plain_load_3d(uint32_t dst, const CUtensorMap *tm, int x, int y, int z, uint32_t bar)
-{
-    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
-                 ::"r"(dst), "l"(tm), "r"(x), "r"(y), "r"(z), "r"(bar) : "memory");
-}
-
 // Shared memory: pages [K, V] (later the ranges' outputs) | barriers | page list | per range and row (m, l) | row log-sum-exp |
 // parked log-sums [range][slot][row]
 // kRowGroups: groups of 16 query rows per CTA
@@ -150,8 +130,9 @@ __global__ void __launch_bounds__(kThreads, 1) small_kernel(const __grid_constan
             const bool v = x >= kHalves;
             const int ch = (x % kHalves) * 64;
             const uint32_t at = dst + static_cast<uint32_t>(x * kPageTokens * 128);
-            if (pg >= 0) plain_load_2d(at, v ? &p.tm_vpool : &p.tm_kpool, ch, (pg * p.Hkv + kvh) * kPageTokens, full);
-            else plain_load_3d(at, v ? &p.tm_vnew : &p.tm_knew, ch, kvh, ep.new_off + (-1 - pg), full);
+            // (no evict-first hint: the row blocks of a kv head share its pages)
+            if (pg >= 0) tma_load_2d(at, v ? &p.tm_vpool : &p.tm_kpool, ch, (pg * p.Hkv + kvh) * kPageTokens, full);
+            else tma_load_3d(at, v ? &p.tm_vnew : &p.tm_knew, ch, kvh, ep.new_off + (-1 - pg), full);
         }
     };
     // page i is fetched by lane 0 of warp i % kWarps: the cached ones while the previous kernel still runs

@@ -43,17 +43,6 @@ constexpr int kMaxRep  = 8;                               // q heads per kv head
 constexpr int kPrefetchPages = 24;                        // pages per CTA asked into the L2 before the previous kernel has ended
 constexpr float kRescaleThreshold = 8.0f;                 // log2 units
 
-__device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap *tm, int x, int y, int z)
-{
-    asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];"
-                 ::"l"(tm), "r"(x), "r"(y), "r"(z) : "memory");
-}
-__device__ __forceinline__ uint32_t peer_addr(uint32_t local, uint32_t rank)
-{
-    uint32_t a;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(local), "r"(rank));
-    return a;
-}
 __device__ __forceinline__ float peer_f32(uint32_t addr)
 {
     float v;
@@ -70,14 +59,6 @@ __device__ __forceinline__ void peer_push4(uint32_t addr, float4 v)
 }
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-// D (fp32, m16n8) += A (bf16, m16k16, row) * B (bf16, k16n8, col)
-__device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
-{
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
 // the 8 x 8 matrix of 16-bit values that the warp holds, transposed
 __device__ __forceinline__ uint32_t transpose8x8(uint32_t x)
 {

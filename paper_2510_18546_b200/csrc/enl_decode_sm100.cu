@@ -592,11 +592,6 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(const __grid_consta
 
 }  // namespace
 
-size_t decode_smem_bytes(int head_dim)
-{
-    return head_dim == 128 ? DecCfg<128>::kSmemBytes : DecCfg<64>::kSmemBytes;
-}
-
 cudaError_t prepare_decode(int head_dim)
 {
     if (head_dim == 128)

@@ -260,7 +260,6 @@ inline int widest_cluster_log(int heads, int pages, bool masses) { return heads 
 // Opt the kernel for pool pages, and the one for contiguous keys, in on the current device and ask for its capacities there.
 cudaError_t prepare_decode_cluster(int head_dim, ClusterCaps *caps);
 cudaError_t prepare_decode_static(int head_dim, ClusterCaps *caps);
-size_t decode_smem_bytes(int head_dim);
 // Page ids of (part of) one group, passed by value to the scatter kernel.
 constexpr int kScatterPages = 64;
 struct PageRun {
