@@ -363,23 +363,25 @@ typedef struct {
  * control loop with memory fixed at start-up, code hosted by another runtime that owns the whole
  * device heap, a process whose allocator is sealed after initialisation.  Such callers cannot create
  * a cache (the paged pool is an allocation), so they pass the key/value stream as ONE contiguous
- * buffer they own, and the split-KV partial results go to a fixed array of ENL_STATIC_SCRATCH_BYTES
- * that is part of the library image: every GPU that loads the library carries that array until the
- * process exits, whether or not this function is ever called.
+ * buffer they own.
  *
- * The work is split over up to 64 key ranges whose partial outputs, log-sum-exps and per-segment
- * sums are written to the built-in array and merged by a second kernel into out / group_mass.
+ * Where q, k, v and out start on 16-byte boundaries the call is one launch: the key ranges are the CTAs
+ * of a thread-block cluster, which merge their results among themselves.  Otherwise (and on a device
+ * that cannot place a cluster) the work is split over up to 64 key ranges whose partial outputs,
+ * log-sum-exps and per-segment sums go to a fixed array of ENL_STATIC_SCRATCH_BYTES and are merged by
+ * a second kernel into out / group_mass.  The array is part of the library image: every GPU that loads
+ * the library carries it until the process exits, whether or not this function is ever called.
  * Limits: at most ENL_STATIC_MAX_SEGMENTS segments, ENL_STATIC_MAX_KEYS keys in all, 8 q heads per
  * kv head, and partials that fit the array (n_q_heads * (head_dim + n_seg + 2) * 4 bytes per
  * 1024 keys); anything larger returns ENL_E_LIMIT and enqueues nothing.
  *
  * The first call on a device with a head_dim asks the runtime what it has to know there (the device
  * addresses of the library's own arrays, how many clusters of the kernel run at once) and keeps the
- * answers in fixed arrays; make that first call outside any stream capture.  All calls share the
- * one array and it keeps the previous call's partials: a call overwrites everything it later reads,
- * so back-to-back calls on one stream are fine, but two calls whose kernels overlap on the GPU
- * (different streams, no dependency) race on it and give wrong results.  Use one stream, or order the
- * calls with events.
+ * answers in fixed arrays; make that first call outside any stream capture.  All calls that split
+ * through the array share it and it keeps the previous call's partials: a call overwrites everything it
+ * later reads, so back-to-back calls on one stream are fine, but two such calls whose kernels overlap on
+ * the GPU (different streams, no dependency) race on it and give wrong results.  Use one stream, or order
+ * the calls with events.
  * Errors: ENL_E_INVAL (null pointer, bad shape, negative length), ENL_E_LIMIT, ENL_E_CUDA.
  * A kernel-side bounded wait that ran out leaves wrong results; enl_static_status reports it.
  */

@@ -221,11 +221,12 @@ def enl_attend(cache: int, layer: int, sel_ids: Sequence[int], q, k_new, v_new, 
 
 
 def enl_attend_static(seg_len: Sequence[int], n_new: int, q, k, v, out, group_mass=None, stream: int = 0) -> None:
-    """One query token over contiguous caller-owned K/V, for callers that must not allocate: the library
-    keeps its split-KV partials in a fixed built-in device array instead of allocated scratch.
+    """One query token over contiguous caller-owned K/V, for callers that must not allocate: split-KV partials are merged
+    inside a thread-block cluster or, for tensors off the 16-byte boundary, held in a fixed built-in device array.
     ``q``/``out``: ``[Hq, D]`` bf16; ``k``/``v``: ``[sum(seg_len) + n_new, Hkv, D]`` bf16;
     ``group_mass``: ``[Hq, len(seg_len) + 1]`` fp32 or None.  Calls share the built-in array, so issue
-    them on one stream (or order them); sizes beyond the fixed maxima raise ``ENL_E_LIMIT``."""
+    them on one stream (or order them); sizes beyond the fixed maxima raise ``ENL_E_LIMIT``; a wait that ran out
+    inside the kernel is reported by ``enl_static_status``."""
     rc = (_native or _binding()).attend_static(seg_len, n_new, q, k, v, out, group_mass, stream or None)
     if rc != ENL_OK:
         raise EnlError(rc, "enl_attend_static")
