@@ -168,15 +168,15 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
     return d;
 }
 
-// Shared-memory matrix descriptor, 128-byte swizzle, rows of 128 B, 8-row groups 1024 B apart.
+// Shared-memory matrix descriptor, 128-byte swizzle, rows of 128 B, 8-row groups 1024 B apart unless given.
 // K-major operand (the contraction dimension is contiguous): LBO unused.
 // MN-major operand: LBO = distance between 64-element column blocks.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo_bytes)
+__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo_bytes, uint32_t group_bytes = 1024u)
 {
     uint64_t d = 0;
     d |= static_cast<uint64_t>((addr & 0x3FFFFu) >> 4);               // start address
     d |= static_cast<uint64_t>((lbo_bytes >> 4) & 0x3FFFu) << 16;      // leading byte offset
-    d |= static_cast<uint64_t>(1024u >> 4) << 32;                      // stride byte offset
+    d |= static_cast<uint64_t>(group_bytes >> 4) << 32;                     // stride byte offset
     d |= static_cast<uint64_t>(1) << 46;                               // descriptor version (sm_100)
     d |= static_cast<uint64_t>(2) << 61;                               // 128-byte swizzle
     return d;

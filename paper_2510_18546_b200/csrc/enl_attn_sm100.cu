@@ -3,29 +3,41 @@
 // What it computes (paper, App. A: softmax(Q K^T / sqrt(D)) V; App. C: the prompt is the selected
 // groups followed by the new tokens; Sec. 3.3: attention between new tokens and a group):
 // one CTA takes two Q tiles of 128 rows each -- (128/rep) consecutive query tokens x the rep q heads
-// that read one kv head -- and walks the key stream of its episode: the selected groups' pages in
-// list order (eight 16-token pages per 128-key tile, fetched as separate TMA boxes from wherever the
-// pages lie in the pool), then the new-token keys up to the causal limit.  Per tile:
+// that read one kv head -- and walks the key stream of its episode in steps of 64 keys: the selected groups' pages in
+// list order (four 16-token pages a step, fetched as separate TMA boxes from wherever the pages lie in the pool), then the
+// new-token keys up to the causal limit.  Per step:
 //   S_i = Q_i K^T            tcgen05.mma, operands in shared memory, accumulator in TMEM
-//                            (after an MMA of one K step that puts -inf under page padding)
+//                            (after an MMA of one K step that puts -inf under page padding, where there is any)
 //   p   = exp2(S * c - m)    one thread per row, fp32; causally hidden columns -> 0
 //   O_i += P_i V             tcgen05.mma, P (bf16) read from TMEM, V from shared memory
 // The row sum of p is split by the slot (selected group, or the new tokens) each 16-key page belongs
 // to; when a slot ends its log2-sum-exp is parked: in shared memory for calls with few slots, whose values are turned into
-// probabilities after the last tile, else in the mass buffer, where mass_finish_kernel does.  With KV splits every split writes partial results that a
+// probabilities after the last step, else in the mass buffer, where mass_finish_kernel does.  With KV splits every split writes partial results that a
 // second kernel merges, or (two splits, head_dim 128) the two CTAs of a cluster merge in place.
 //
 // Roles (12 warps): warps 0-3 are the softmax warpgroup of Q tile 0, warps 4-7 that of Q tile 1: one
-// thread per query row holds the row's 128 scores of a tile in registers, so the row maximum, the
-// exponentials and the eight page sums need no exchange between threads.  Warp 8 is the TMA producer,
-// warp 9 the MMA issuer (and TMEM owner), warps 10-11 idle: they complete the third warpgroup so that
-// setmaxnreg can move its registers to the softmax warpgroups.
-// The two Q tiles alternate on the tensor pipe: while one tile's softmax runs, the pipe does the other
-// tile's P V and the next Q K^T.  P is handed over in two halves of 64 keys so that P V starts while
-// the second half's exponentials are still being taken; everything that is not needed for P (row and
-// page sums, slot book-keeping) is done after the hand-over, under the MMAs.
-// TMEM columns: S0 [0,128) S1 [128,256) O0 [256,384) O1 [384,512); P_i (bf16 pairs) overwrites columns
-// [0,64) of S_i once the row's scores are in registers.
+// thread per query row holds the row's 64 scores of a step in registers, so the row maximum, the
+// exponentials and the four page sums need no exchange between threads.  Warps 8 and 10 fetch K and V, warps 9 and 11 issue the
+// MMAs of tile 0 and tile 1 (9 owns the TMEM).
+//
+// What bounds it, and why it is split like this (all cycles per 128 keys and pair of Q tiles, 64 groups, 1024 rows; the tensor pipe
+// needs 2176, the special-function unit 2048):
+//  * S is double-buffered: Q K^T of step j + 2 is issued behind P V of step j, so a softmax warp finds its next scores waiting.  Tiles of
+//    128 keys leave no TMEM for that; their chain scores -> softmax -> P V -> Q K^T took 3640.
+//  * The issuers: issuing an MMA costs its scheduler about 13 issue slots, a wait its warp 100 cycles and more.  One warp that
+//    alternated between the tiles was what both waited for (4700 with these steps); one warp for Q K^T and one for P V slowed the
+//    two softmax warps of the former's scheduler to 4300.  An issuer per tile, on different schedulers, waits for nothing but its own tile.
+//  * The producers: a TMA box costs its warp 50 cycles and a fetch some 200 to 350 more.  One producer with two boxes of half a page
+//    per page needed 3800.
+//  * Turns: the warps of the two tiles that share a scheduler take their exponentials one after the other (a named barrier).  Left alone
+//    the tiles fall into step, both wanting the special-function unit and then both not: 4150 against 3500.
+// Long calls 251 -> 238 thousand cycles a launch (then at the power cap), the planner's 512 rows over 24 groups 33.5 -> 31.0 us.
+// Not kept: exponentials on the FMA pipe, a quarter of them 270 thousand cycles (the warps have issue slots, but a step is one chain);
+// the maximum beside the exponentials, with the reference a step behind: 6700 against 5860 us a pass; tiles of 128 keys with all of the
+// above: the same on long calls, 8 % slower on the planner's, whose ends waste half a tile.
+//
+// TMEM columns: S0 [0,128) S1 [128,256), two buffers of 64 columns each, O0 [256,384) O1 [384,512); P_i (bf16 pairs) overwrites the
+// first 32 columns of the buffer that held its scores once these are in registers.
 #include <cuda_bf16.h>
 
 #include "attn_ops.cuh"
@@ -37,32 +49,39 @@ namespace {
 
 constexpr int kThreads      = 384;
 constexpr int kSoftmaxWarps = 8;
-constexpr int kRegsSoftmax  = 208;            // 256 x 208 + 128 x 80 <= 384 x 168, what the launch allocates
-constexpr int kRegsOther    = 80;
-constexpr int kProducerWarp = 8;
-constexpr int kMmaWarp      = 9;
+constexpr int kRegsSoftmax  = 184;            // 256 x 184 + 128 x 128 <= 384 x 168, what the launch allocates
+constexpr int kRegsOther    = 128;
+constexpr int kKWarp        = 8;              // fetches K
+constexpr int kVWarp        = 10;             // fetches V
+constexpr int kMmaWarp      = 9;              // issues the MMAs of Q tile 0 (and owns the TMEM); those of tile 1 two warps on
 constexpr uint32_t kTmemCols = 512;
 constexpr int kParkSlots = 25;                // calls with up to this many mass slots park their slot sums in shared memory
+constexpr int kStepPages = kStepKeys / kPageTokens;
 constexpr float kRescaleThreshold = 8.0f;     // log2 units: p stays below 2^8 between updates of the reference
 
 template <int D>
 struct Cfg {
     static constexpr int kHalves    = D / 64;             // 64-channel (128-byte) column blocks
-    static constexpr int kHalfBytes = 128 * 128;          // 128 rows x 128 B
+    static constexpr int kHalfBytes = 128 * 128;          // Q tile: 128 rows x 128 B
     static constexpr int kTileBytes = kHalves * kHalfBytes;
-    static constexpr int kStages    = (D == 128) ? 4 : 8;
-    static constexpr int kBarOff    = (kQTiles + kStages) * kTileBytes;
+    // K or V of a step: eight groups of 8 rows, a group being one 8 x 128-byte block per 64 channels
+    static constexpr int kGroupBytes = kHalves * 1024;
+    static constexpr int kStepBytes = kStepKeys / 8 * kGroupBytes;
+    static constexpr int kRing      = 4;                  // steps whose K (and whose V) are in shared memory at once
+    static constexpr int kRingOff   = kQTiles * kTileBytes;
+    static constexpr int kBarOff    = kRingOff + 2 * kRing * kStepBytes;
+    // the operands of the MMA that hides page padding, 16 bytes per row: 1 for 8 queries (behind the barriers; every group of
+    // 8 rows reads them), 0 or -inf for every key of a step in the ring; and a word per step: has it padding at all?
+    static constexpr int kHideFlagOff = kBarOff + 352;
+    static constexpr int kOnesOff   = kBarOff + 384;
     // pair merge: what the other CTA of the cluster knows about this CTA's rows, [tile][128] x (m, l, shared-slot log-sum, -)
     static constexpr int kXpeerOff  = kBarOff + 512;
-    // the operands of the MMA that hides page padding, 16 bytes per row: 1 for 8 queries (behind the barriers; every group of
-    // 8 rows reads them), 0 or -inf for every key of a K stage
-    static constexpr int kOnesOff   = kBarOff + 256;
     static constexpr int kHideOff   = kXpeerOff + kQTiles * 128 * 16;
-    static constexpr int kHideBytes = kTileKeys * 16;
+    static constexpr int kHideBytes = kStepKeys * 16;
     // slot log-sums of calls with at most kParkSlots slots, [tile][slot][128 rows] fp32 (what is left of the 227 KB)
-    static constexpr int kParkOff   = kHideOff + kStages / 2 * kHideBytes;
+    static constexpr int kParkOff   = kHideOff + kRing * kHideBytes;
     static constexpr int kSmemBytes = kParkOff + kQTiles * kParkSlots * 128 * 4 + 1024;   // + alignment slack
-    static_assert(8 * (13 + 2 * kStages) + 8 <= 256 && kOnesOff + 128 <= kXpeerOff && kSmemBytes <= 232448, "shared memory");
+    static_assert(8 * 33 + 8 <= 352 && kSmemBytes <= 232448, "shared memory");
 };
 
 // ---- the kernel ----------------------------------------------------------------------------
@@ -79,22 +98,27 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
 
     // shared-memory map
     auto q_addr     = [&](int i) { return sbase + static_cast<uint32_t>(i * C::kTileBytes); };
-    auto stage_addr = [&](int s) { return sbase + static_cast<uint32_t>((kQTiles + s) * C::kTileBytes); };
+    auto k_addr = [&](int x) { return sbase + static_cast<uint32_t>(C::kRingOff + 2 * x * C::kStepBytes); };
+    auto v_addr = [&](int x) { return k_addr(x) + static_cast<uint32_t>(C::kStepBytes); };
     const uint32_t bar0 = sbase + C::kBarOff;
     const uint32_t bar_q_full = bar0;
-    auto bar_kv_full  = [&](int s) { return bar0 + 8u * (1 + s); };
-    auto bar_kv_empty = [&](int s) { return bar0 + 8u * (1 + C::kStages + s); };
-    auto bar_s_full   = [&](int i) { return bar0 + 8u * (1 + 2 * C::kStages + i); };
-    auto bar_p_half   = [&](int i, int hf) { return bar0 + 8u * (3 + 2 * C::kStages + 2 * i + hf); };   // keys 0..63 / 64..127 of P_i
-    auto bar_o_done   = [&](int i) { return bar0 + 8u * (7 + 2 * C::kStages + i); };
+    auto bar_k_full  = [&](int x) { return bar0 + 8u * (1 + x); };             // x: place in the ring
+    auto bar_k_empty = [&](int x) { return bar0 + 8u * (5 + x); };
+    auto bar_v_full  = [&](int x) { return bar0 + 8u * (9 + x); };
+    auto bar_v_empty = [&](int x) { return bar0 + 8u * (13 + x); };
+    auto bar_s_full  = [&](int i, int b) { return bar0 + 8u * (17 + 2 * i + b); };   // b: step & 1
+    auto bar_p_full  = [&](int i, int b) { return bar0 + 8u * (21 + 2 * i + b); };
+    auto bar_pv_done = [&](int i) { return bar0 + 8u * (25 + i); };            // P_i V of a step
+    auto bar_o_done  = [&](int i) { return bar0 + 8u * (27 + i); };            // of the last step
     // pair merge (cluster of two): the peer's row sums have arrived / the peer's partial output has arrived /
     // the peer's K/V ring is idle and may be written / the peer has received what this CTA staged for it
-    const uint32_t bar_peer_ml = bar0 + 8u * (9 + 2 * C::kStages);
-    const uint32_t bar_peer_o = bar0 + 8u * (10 + 2 * C::kStages);
-    const uint32_t bar_peer_free = bar0 + 8u * (11 + 2 * C::kStages);
-    const uint32_t bar_peer_ack = bar0 + 8u * (12 + 2 * C::kStages);
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + C::kBarOff + 8 * (13 + 2 * C::kStages));
+    const uint32_t bar_peer_ml = bar0 + 8u * 29;
+    const uint32_t bar_peer_o = bar0 + 8u * 30;
+    const uint32_t bar_peer_free = bar0 + 8u * 31;
+    const uint32_t bar_peer_ack = bar0 + 8u * 32;
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + C::kBarOff + 8 * 33);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
+    volatile uint32_t *hide_flag = reinterpret_cast<volatile uint32_t *>(smem + C::kHideFlagOff);
 
     if (p.wait_first) pdl_wait();
     // work item
@@ -105,21 +129,26 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
     const int t_hi = min(it.t0 + kQTiles * tile_tokens, ep.n_q);        // exclusive
     const int n_qt = (t_hi - it.t0 > tile_tokens) ? 2 : 1;
     const int c_max = ep.n_new - ep.n_q + t_hi - 1;                      // last new key any row sees
-    const int n_new_tiles = c_max / kTileKeys + 1;
-    const int total_tiles = ep.n_ctiles + n_new_tiles;
-    const int j_beg = static_cast<int>(static_cast<long long>(total_tiles) * it.split / p.n_splits);
-    const int j_end = static_cast<int>(static_cast<long long>(total_tiles) * (it.split + 1) / p.n_splits);
-    const int n_tiles = j_end - j_beg;
+    const int n_csteps = (ep.n_entries + kStepPages - 1) / kStepPages;  // steps over cached pages
+    const int total_steps = n_csteps + c_max / kStepKeys + 1;
+    const int j_beg = static_cast<int>(static_cast<long long>(total_steps) * it.split / p.n_splits);
+    const int j_end = static_cast<int>(static_cast<long long>(total_steps) * (it.split + 1) / p.n_splits);
+    const int n_steps = j_end - j_beg;
 
     // ---- set-up ----
     if (threadIdx.x == 0) {
         *abort_flag = 0;
         mbar_init(bar_q_full, 1);
-        for (int s = 0; s < C::kStages; ++s) { mbar_init(bar_kv_full(s), 1); mbar_init(bar_kv_empty(s), 1); }
+        for (int x = 0; x < C::kRing; ++x) {
+            mbar_init(bar_k_full(x), 1); mbar_init(bar_k_empty(x), n_qt);
+            mbar_init(bar_v_full(x), 1); mbar_init(bar_v_empty(x), n_qt);
+        }
         for (int i = 0; i < kQTiles; ++i) {
-            mbar_init(bar_s_full(i), 1);
-            mbar_init(bar_p_half(i, 0), 4);       // one arrival per softmax warp of the tile
-            mbar_init(bar_p_half(i, 1), 4);
+            for (int b = 0; b < 2; ++b) {
+                mbar_init(bar_s_full(i, b), 1);
+                mbar_init(bar_p_full(i, b), 4);       // one arrival per softmax warp of the tile
+            }
+            mbar_init(bar_pv_done(i), 1);
             mbar_init(bar_o_done(i), 1);
         }
         mbar_init(bar_peer_ml, 1);                                   // this thread's arrival below + 16 bytes per row from the peer
@@ -150,26 +179,19 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
     // everything above touched only shared memory, TMEM and the gather plan; from here on the caller's tensors,
     // the pool and the scratch are read and written, so the previous kernel of the stream must have finished
     pdl_trigger();
-    // While the previous kernel drains, ask what the first S tile needs into the L2: the Q tiles and the first two
-    // key tiles' K and V (cached pages; new-token tiles only when the stream starts with them).
+    // While the previous kernel drains, ask what the first steps need into the L2: the Q tiles and a ring full of
+    // K and V (new tokens only when the stream starts with them).
     // (Only CTAs of the first wave wait for the previous kernel; for the others this would be loads issued twice.)
-    if (warp == kProducerWarp && n_tiles > 0 && static_cast<int>(blockIdx.x) < p.first_wave) {
-        if (lane < n_qt * C::kHalves)
+    if ((warp == kKWarp || warp == kVWarp) && n_steps > 0 && static_cast<int>(blockIdx.x) < p.first_wave) {
+        if (warp == kKWarp && lane < n_qt * C::kHalves)
             tma_prefetch_3d(&p.tm_q, (lane % C::kHalves) * 64, it.kvh * rep, ep.q_off + it.t0 + (lane / C::kHalves) * tile_tokens);
-        for (int j = j_beg; j < min(j_beg + 2, j_end); ++j) {
-            if (j < ep.n_ctiles) {
-                if (lane < kPagesPerTile) {
-                    const int row = (p.stream_page[ep.stream_off + j * kPagesPerTile + lane] * p.Hkv + it.kvh) * kPageTokens;
-                    for (int hf = 0; hf < C::kHalves; ++hf) {
-                        tma_prefetch_2d(&p.tm_kpool, hf * 64, row);
-                        tma_prefetch_2d(&p.tm_vpool, hf * 64, row);
-                    }
-                }
-            } else if (lane < 2 * C::kHalves) {
-                tma_prefetch_3d(lane < C::kHalves ? &p.tm_knew : &p.tm_vnew, (lane % C::kHalves) * 64, it.kvh,
-                                ep.new_off + (j - ep.n_ctiles) * kTileKeys);
-            }
-        }
+        const int j = j_beg + lane / kStepPages;
+        if (lane < C::kRing * kStepPages && j < min(j_end, n_csteps))
+            tma_prefetch_4d(warp == kKWarp ? &p.tm_kpool : &p.tm_vpool, 0, 0, 0,
+                            (p.stream_page[ep.stream_off + j * kStepPages + lane % kStepPages] * p.Hkv + it.kvh) * 2);
+        const int jn = max(j_beg, n_csteps) + lane / 8;              // new tokens: eight rows a box
+        if (jn < min(j_beg + C::kRing, j_end))
+            tma_prefetch_4d(warp == kKWarp ? &p.tm_knew : &p.tm_vnew, 0, ep.new_off + (jn - n_csteps) * kStepKeys + lane % 8 * 8, 0, it.kvh);
     }
     pdl_wait();
 
@@ -177,180 +199,148 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
 
     if (warp >= kSoftmaxWarps) {
       asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsOther));
-      if (warp == kProducerWarp) {
-        // ================= TMA producer =================
-        if (n_tiles > 0) {
-            if (lane == 0) {
+      if (warp == kKWarp || warp == kVWarp) {
+        // ================= TMA producers =================
+        // K and V have a warp each, and a box is a whole page of a kv head: eight lanes with half a page each took 767 cycles per 16 KB,
+        // four with a page take 562 (the wait for the ring's place included).
+        const bool is_k = warp == kKWarp;
+        const CUtensorMap *tm_pool = is_k ? &p.tm_kpool : &p.tm_vpool, *tm_new = is_k ? &p.tm_knew : &p.tm_vnew;
+        const uint32_t ring = is_k ? k_addr(0) : v_addr(0), full0 = is_k ? bar_k_full(0) : bar_v_full(0),
+                       empty0 = is_k ? bar_k_empty(0) : bar_v_empty(0);
+        if (n_steps > 0) {
+            if (is_k && lane == 0) {
                 mbar_expect_tx(bar_q_full, static_cast<uint32_t>(n_qt * C::kTileBytes));
                 for (int i = 0; i < n_qt; ++i)
                     for (int hf = 0; hf < C::kHalves; ++hf)
                         tma_load_3d(q_addr(i) + hf * C::kHalfBytes, &p.tm_q, hf * 64, it.kvh * rep,
                                     ep.q_off + it.t0 + i * tile_tokens, bar_q_full);
             }
-            int fill = 0;
-            for (int j = j_beg; j < j_end && ok; ++j) {
-                const bool cached = j < ep.n_ctiles;
-                int page = 0, valid = 0;                             // page of this lane (0..7) and its keys
-                if (cached && lane < kPagesPerTile) {
-                    page = p.stream_page[ep.stream_off + j * kPagesPerTile + lane];
-                    valid = __ldg(p.stream_meta + ep.stream_off + j * kPagesPerTile + lane) & 0xff;
+            // Page words (id; slot << 8 | valid keys) of 32 pages at a time, one per lane, fetched eight steps ahead: a load in
+            // every step kept the ring waiting for the L2.
+            constexpr int kBatch = 32 / kStepPages;
+            auto words = [&](int jj, int &id, int &meta) {
+                const int e = (j_beg + jj) * kStepPages + lane;
+                id = kZeroPage;
+                meta = kPageTokens;
+                if (e < n_csteps * kStepPages) {
+                    id = __ldg(p.stream_page + ep.stream_off + e);
+                    meta = __ldg(p.stream_meta + ep.stream_off + e);
                 }
-                for (int kv = 0; kv < 2; ++kv, ++fill) {
-                    const int st = fill % C::kStages;
-                    if (fill >= C::kStages) {
-                        ok = mbar_wait(bar_kv_empty(st), static_cast<uint32_t>((fill / C::kStages - 1) & 1),
-                                       abort_flag, p.status);
-                        if (!ok) break;
-                    }
-                    const uint32_t full = bar_kv_full(st);
-                    if (cached && kv == 0) {                         // what hides the padding of these keys: see issue_qk
-                        uint4 *hide = reinterpret_cast<uint4 *>(smem + C::kHideOff + st / 2 * C::kHideBytes);
+            };
+            int id_cur = 0, meta_cur = 0, id_next, meta_next, fetched = 0;
+            words(0, id_next, meta_next);
+            for (int jj = 0; jj < n_steps; ++jj) {
+                const int j = j_beg + jj, x = jj % C::kRing;
+                if (jj % kBatch == 0) {
+                    id_cur = id_next;
+                    meta_cur = meta_next;
+                    words(jj + kBatch, id_next, meta_next);
+                }
+                const int pg = lane % kStepPages, at = jj % kBatch * kStepPages;
+                const int row8 = (__shfl_sync(kFull, id_cur, at + pg) * p.Hkv + it.kvh) * 2;
+                const int valid = __shfl_sync(kFull, meta_cur, at + pg) & 0xff;
+                if (jj >= C::kRing) ok = mbar_wait(empty0 + 8u * x, static_cast<uint32_t>((jj / C::kRing - 1) & 1), abort_flag, p.status);
+                if (!ok) break;
+                const uint32_t dst = ring + static_cast<uint32_t>(2 * x * C::kStepBytes), full = full0 + 8u * x;
+                if (is_k) {
+                    const bool padded = __any_sync(kFull, valid < kPageTokens);
+                    if (lane == 0) hide_flag[x] = padded ? 1u : 0u;
+                    if (padded) {                                    // what hides the padding of these keys: see issue_qk
+                        uint4 *hide = reinterpret_cast<uint4 *>(smem + C::kHideOff + x * C::kHideBytes);
 #pragma unroll
-                        for (int x = 0; x < kTileKeys / 32; ++x) {
-                            const int n = __shfl_sync(kFull, valid, 2 * x + (lane >> 4));
-                            hide[x * 32 + lane] = make_uint4((lane & 15) < n ? 0u : 0xff80u, 0u, 0u, 0u);
+                        for (int y = 0; y < kStepKeys / 32; ++y) {
+                            const int n = __shfl_sync(kFull, valid, 2 * y + (lane >> 4));
+                            hide[y * 32 + lane] = make_uint4((lane & 15) < n ? 0u : 0xff80u, 0u, 0u, 0u);
                         }
                         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                        __syncwarp();
                     }
-                    if (lane == 0) mbar_expect_tx(full, static_cast<uint32_t>(C::kTileBytes));
                     __syncwarp();
-                    const uint32_t dst = stage_addr(st);
-                    if (cached) {
-                        if (lane < kPagesPerTile) {
-                            const CUtensorMap *tm = kv ? &p.tm_vpool : &p.tm_kpool;
-                            const int row = (page * p.Hkv + it.kvh) * kPageTokens;
-                            for (int hf = 0; hf < C::kHalves; ++hf)
-                                tma_load_2d(dst + hf * C::kHalfBytes + lane * (kPageTokens * 128), tm,
-                                            hf * 64, row, full);
-                        }
-                    } else if (lane == 0) {
-                        const CUtensorMap *tm = kv ? &p.tm_vnew : &p.tm_knew;
-                        const int krow = ep.new_off + (j - ep.n_ctiles) * kTileKeys;
-                        for (int hf = 0; hf < C::kHalves; ++hf)
-                            tma_load_3d(dst + hf * C::kHalfBytes, tm, hf * 64, it.kvh, krow, full);
-                    }
                 }
+                if (lane == 0) mbar_expect_tx(full, static_cast<uint32_t>(C::kStepBytes));
+                if (j < n_csteps) {
+                    if (lane < kStepPages) tma_load_4d(dst + static_cast<uint32_t>(lane * 2 * C::kGroupBytes), tm_pool, 0, 0, 0, row8, full);
+                } else if (lane < 8) {
+                    tma_load_4d(dst + static_cast<uint32_t>(lane * C::kGroupBytes), tm_new, 0,
+                                ep.new_off + (j - n_csteps) * kStepKeys + lane * 8, 0, it.kvh, full);
+                }
+                ++fetched;
             }
             // error path only: let the copies already in flight land before the CTA retires
             if (!ok) {
-                const int first = fill > C::kStages ? fill - C::kStages : 0;
-                for (int f = first; f < fill; ++f) {
+                for (int f = max(0, fetched - C::kRing); f < fetched; ++f) {
                     const unsigned long long t0 = global_ns();
-                    while (!mbar_try_wait(bar_kv_full(f % C::kStages), static_cast<uint32_t>((f / C::kStages) & 1)) &&
+                    while (!mbar_try_wait(full0 + 8u * (f % C::kRing), static_cast<uint32_t>((f / C::kRing) & 1)) &&
                            global_ns() - t0 < 2000000ull) { }
                 }
             }
         }
-      } else if (warp == kMmaWarp) {
-        // ================= MMA issuer =================
-        if (n_tiles > 0) {
-            constexpr uint32_t idesc_qk = make_idesc(kTileKeys, false);
-            constexpr uint32_t idesc_pv = make_idesc(D, true);
-            auto tmem_s = [&](int i) { return tmem_base + static_cast<uint32_t>(i * 128); };
-            auto tmem_o = [&](int i) { return tmem_base + static_cast<uint32_t>(256 + i * 128); };
-            // descriptor words: Q tile i and ring stage st start (kTileBytes >> 4) address units apart
-            const uint64_t dq0 = smem_desc(q_addr(0), 16), dk0 = smem_desc(stage_addr(0), 16),
-                           dv0 = smem_desc(stage_addr(0), C::kHalfBytes);
+      } else {
+        // ================= MMA issuer of a Q tile =================
+        const int i = warp == kMmaWarp ? 0 : 1;
+        if (n_steps > 0 && i < n_qt) {
+            constexpr uint32_t idesc_qk = make_idesc(kStepKeys, false), idesc_pv = make_idesc(D, true);
+            // descriptor words: place x of the ring starts 2 * kStepUnits x address units behind place 0
+            constexpr uint32_t kStepUnits = C::kStepBytes >> 4, kGroupUnits = C::kGroupBytes >> 4;
+            const uint64_t dq0 = smem_desc(q_addr(i), 16), dk0 = smem_desc(k_addr(0), 16, C::kGroupBytes), dv0 = smem_desc(v_addr(0), 1024, C::kGroupBytes);
             const uint32_t dq_lo = static_cast<uint32_t>(dq0), dq_hi = static_cast<uint32_t>(dq0 >> 32);
             const uint32_t dk_lo = static_cast<uint32_t>(dk0), dk_hi = static_cast<uint32_t>(dk0 >> 32);
             const uint32_t dv_lo = static_cast<uint32_t>(dv0), dv_hi = static_cast<uint32_t>(dv0 >> 32);
-            constexpr uint32_t kTileUnits = C::kTileBytes >> 4;
             const uint64_t d_ones = smem_desc_plain(sbase + C::kOnesOff, 0u), d_hide = smem_desc_plain(sbase + C::kHideOff, 128u);
-            // S_i = Q_i K^T; with cached pages (`hide`) an MMA of one K step before it puts -inf under the padding keys and 0 under
-            // the others.  It costs the pipe 1/16 of a tile's work and takes the compares and selects of ragged
-            // pages out of the softmax warps, which are what a tile waits for: 4374 -> 3999 cycles per key tile and pair of Q tiles
-            // (pages of objects of 20..200 tokens), with masses 4436 -> 4146.
-            auto issue_qk = [&](int i, int st, bool hide) {
-                const uint32_t a = dq_lo + static_cast<uint32_t>(i) * kTileUnits, b = dk_lo + static_cast<uint32_t>(st) * kTileUnits;
-                const uint32_t d = tmem_s(i);
+            const uint32_t t_si = tmem_base + static_cast<uint32_t>(i * 128), t_oi = tmem_base + static_cast<uint32_t>(256 + i * 128);
+            // S_i = Q_i K^T into buffer b; where a page is padded (`hide`) an MMA of one K step before it puts -inf under the padding
+            // keys and 0 under the others.  It costs the pipe 1/8 of the step's Q K^T and takes the compares and selects of
+            // ragged pages out of the softmax warps (in the tiles of 128 keys: 4374 -> 3999 cycles).
+            auto issue_qk = [&](int x, int b, bool hide) {
+                const uint32_t ka = dk_lo + static_cast<uint32_t>(x) * (2u * kStepUnits), d = t_si + static_cast<uint32_t>(b * kStepKeys);
                 if (hide)
                     mma_ss2(d, static_cast<uint32_t>(d_ones), static_cast<uint32_t>(d_ones >> 32),
-                            static_cast<uint32_t>(d_hide) + static_cast<uint32_t>(st / 2) * (C::kHideBytes >> 4),
+                            static_cast<uint32_t>(d_hide) + static_cast<uint32_t>(x) * (C::kHideBytes >> 4),
                             static_cast<uint32_t>(d_hide >> 32), idesc_qk, 0u);
 #pragma unroll
                 for (int kk = 0; kk < D / 16; ++kk) {
-                    constexpr uint32_t kHalfUnits = C::kHalfBytes >> 4;
-                    const uint32_t off = static_cast<uint32_t>((kk >> 2) * kHalfUnits + (kk & 3) * 2);   // 32 bytes per 16 channels
-                    mma_ss2(d, a + off, dq_hi, b + off, dk_hi, idesc_qk, kk > 0 || hide ? 1u : 0u);
+                    const uint32_t in_row = static_cast<uint32_t>((kk & 3) * 2);                       // 32 bytes per 16 channels
+                    mma_ss2(d, dq_lo + static_cast<uint32_t>((kk >> 2) * (C::kHalfBytes >> 4)) + in_row, dq_hi,
+                            ka + static_cast<uint32_t>((kk >> 2) * (1024 >> 4)) + in_row, dk_hi, idesc_qk, kk > 0 || hide ? 1u : 0u);
                 }
-                tc_commit(bar_s_full(i));
+                tc_commit(bar_s_full(i, b));
+                tc_commit(bar_k_empty(x));
             };
-            // O_i (+)= P_i[:, 64 hf .. 64 hf + 63] V[64 hf .. 64 hf + 63, :]; P of keys 2c, 2c+1 sits in column c of S_i
-            auto issue_pv = [&](int i, int st, int hf, bool first_tile) {
-                const uint32_t b = dv_lo + static_cast<uint32_t>(st) * kTileUnits + static_cast<uint32_t>(hf) * (4u * 128u);
-                const uint32_t d = tmem_o(i), a = tmem_s(i) + static_cast<uint32_t>(hf * 32);
+            // O_i (+)= P_i V; P of keys 2c, 2c+1 sits in column c of the buffer that held their scores
+            auto issue_pv = [&](int x, int b, bool first) {
+                const uint32_t va = dv_lo + static_cast<uint32_t>(x) * (2u * kStepUnits), a = t_si + static_cast<uint32_t>(b * kStepKeys);
 #pragma unroll
-                for (int k4 = 0; k4 < 4; ++k4)                          // 16 keys = 16 rows of 128 B = 128 address units, 8 columns of P
-                    mma_ts2(d, a + static_cast<uint32_t>(k4 * 8), b + static_cast<uint32_t>(k4 * 128), dv_hi, idesc_pv,
-                            (first_tile && hf == 0 && k4 == 0) ? 0u : 1u);
+                for (int k4 = 0; k4 < kStepPages; ++k4)                  // 16 keys = two groups of 8 rows, 8 columns of P
+                    mma_ts2(t_oi, a + static_cast<uint32_t>(k4 * 8), va + static_cast<uint32_t>(k4 * 2) * kGroupUnits, dv_hi, idesc_pv,
+                            (first && k4 == 0) ? 0u : 1u);
+                tc_commit(bar_pv_done(i));
+                tc_commit(bar_v_empty(x));
             };
-            auto wait_full = [&](int f) {
-                return mbar_wait(bar_kv_full(f % C::kStages), static_cast<uint32_t>((f / C::kStages) & 1),
-                                 abort_flag, p.status);
-            };
-
-            // A barrier the issuer will need is tested one batch of MMAs ahead ("armed"), so that the test's latency
-            // passes while the batch is issued; only a barrier that was not complete then is waited for.  The queue in
-            // front of the pipe holds about four MMAs: a wait of a few hundred cycles between two batches empties it.
-            struct Pending { uint32_t bar, par; bool pre; };
-            auto arm = [&](uint32_t bar, uint32_t par) { return Pending{bar, par, mbar_test(bar, par)}; };
-            auto await = [&](const Pending &w) {
-                return __all_sync(kFull, w.pre) ? true : mbar_wait(w.bar, w.par, abort_flag, p.status);
-            };
-            auto full_bar = [&](int f) { return bar_kv_full(f % C::kStages); };
-            auto full_par = [&](int f) { return static_cast<uint32_t>((f / C::kStages) & 1); };
-
+            auto wait_k = [&](int jj) { return mbar_wait(bar_k_full(jj % C::kRing), static_cast<uint32_t>((jj / C::kRing) & 1), abort_flag, p.status); };
             ok = mbar_wait(bar_q_full, 0, abort_flag, p.status);
-            if (ok) ok = wait_full(0);
-            if (ok) {
+            for (int jj = 0; jj < min(2, n_steps) && ok; ++jj) {
+                ok = wait_k(jj);
+                if (!ok) break;
                 tc_fence_after();
-                for (int i = 0; i < n_qt; ++i) issue_qk(i, 0, j_beg < ep.n_ctiles);
-                tc_commit(bar_kv_empty(0));
+                issue_qk(jj, jj, hide_flag[jj] != 0u);
             }
-            Pending w_v = arm(full_bar(1), full_par(1));                // V of the first tile
-            Pending w_p = arm(bar_p_half(0, 0), 0u);                    // first half of P_0
-            for (int jj = 0; jj < n_tiles && ok; ++jj) {
-                const int fv = 2 * jj + 1, fk = 2 * jj + 2;             // ring slots of V_jj and K_{jj+1}
-                const bool more = jj + 1 < n_tiles;
-                const uint32_t par = static_cast<uint32_t>(jj & 1);
-                for (int i = 0; i < n_qt; ++i) {
-                    const bool last_i = i == n_qt - 1;
-                    if (i == 0) ok = await(w_v);
-                    if (ok) ok = await(w_p);
-                    if (!ok) break;
-                    tc_fence_after();
-                    const Pending w_h1 = arm(bar_p_half(i, 1), par);
-                    issue_pv(i, fv % C::kStages, 0, jj == 0);
-                    ok = await(w_h1);
-                    if (!ok) break;
-                    tc_fence_after();
-                    Pending w_k = {0u, 0u, true};
-                    if (more && i == 0) w_k = arm(full_bar(fk), full_par(fk));
-                    if (!more && !last_i) w_p = arm(bar_p_half(i + 1, 0), par);
-                    issue_pv(i, fv % C::kStages, 1, false);
-                    if (last_i) tc_commit(bar_kv_empty(fv % C::kStages));
-                    if (!more) tc_commit(bar_o_done(i));
-                    if (more) {
-                        ok = await(w_k);
-                        if (!ok) break;
-                        tc_fence_after();
-                        // what follows Q_i K^T: the next tile's P of this key tile, or (after the last Q tile) V and P_0 of the next
-                        if (!last_i) {
-                            w_p = arm(bar_p_half(i + 1, 0), par);
-                        } else {
-                            w_v = arm(full_bar(fv + 2), full_par(fv + 2));
-                            w_p = arm(bar_p_half(0, 0), par ^ 1u);
-                        }
-                        issue_qk(i, fk % C::kStages, j_beg + jj + 1 < ep.n_ctiles);
-                        if (last_i) tc_commit(bar_kv_empty(fk % C::kStages));
-                    }
-                }
+            for (int jj = 0; jj < n_steps && ok; ++jj) {
+                const int x = jj % C::kRing, x2 = (jj + 2) % C::kRing, b = jj & 1;
+                const bool more = jj + 2 < n_steps;
+                // P comes last: nothing but the MMAs themselves stands between its arrival and the next scores
+                ok = mbar_wait(bar_v_full(x), static_cast<uint32_t>((jj / C::kRing) & 1), abort_flag, p.status);
+                if (ok && more) ok = wait_k(jj + 2);
+                const bool hide = more && hide_flag[x2] != 0u;
+                if (ok) ok = mbar_wait(bar_p_full(i, b), static_cast<uint32_t>((jj >> 1) & 1), abort_flag, p.status);
+                if (!ok) break;
+                tc_fence_after();
+                issue_pv(x, b, jj == 0);
+                if (more) issue_qk(x2, b, hide);
+                else if (jj + 1 == n_steps) tc_commit(bar_o_done(i));
             }
             // pair merge: once every MMA of this CTA has completed, its K/V ring is idle and the peer may write
             // into it (only a CTA that finishes a Q tile receives anything)
-            if (ok && pair && it.split < n_qt) {
-                for (int i = 0; i < n_qt && ok; ++i) ok = mbar_wait(bar_o_done(i), 0, abort_flag, p.status);
+            if (ok && pair && i == 0 && it.split < n_qt) {
+                for (int t = 0; t < n_qt && ok; ++t) ok = mbar_wait(bar_o_done(t), 0, abort_flag, p.status);
                 if (ok && lane == 0) peer_arrive(peer_addr(bar_peer_free, cluster_rank() ^ 1u));
             }
         }
@@ -391,8 +381,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
         float bnd = kNegInf;
         if (pair) {
             const int jb = (it.split == 0) ? j_end : j_beg;         // first tile of split 1
-            const int last0 = (jb > ep.n_ctiles) ? G : (__ldg(p.stream_meta + ep.stream_off + jb * kPagesPerTile - 1) >> 8);
-            const int first1 = (jb < ep.n_ctiles) ? (__ldg(p.stream_meta + ep.stream_off + jb * kPagesPerTile) >> 8) : G;
+            const int last0 = (jb > n_csteps) ? G : (__ldg(p.stream_meta + ep.stream_off + jb * kStepPages - 1) >> 8);
+            const int first1 = (jb < n_csteps) ? (__ldg(p.stream_meta + ep.stream_off + jb * kStepPages) >> 8) : G;
             if (last0 == first1) { shared_slot = last0; if (it.split == 1) skip_slot = last0; }
         }
         float m = kNegInf, l = 0.f, acc = 0.f;                     // reference (log2 units), row sum, sum of the current slot
@@ -407,64 +397,76 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
             }
         };
 
-        // Page words of a tile, one per lane 0..7 (slot << 8 | valid keys); a new-token tile is one slot (G).  They
-        // are fetched one tile ahead: the load's latency would otherwise sit between two tiles of this warp.
-        auto load_meta = [&](int j) -> int {
-            int w = (G << 8) | kPageTokens;
-            if (j < ep.n_ctiles && lane < kPagesPerTile) w = __ldg(p.stream_meta + ep.stream_off + j * kPagesPerTile + lane);
-            return w;
+        // Slots of 32 pages at a time, one per lane, fetched eight steps ahead, and a warp-uniform mask of those pages whose slot differs
+        // from the page before.  The pages of a new-token step are one slot (G).
+        constexpr int kBatch = 32 / kStepPages;
+        auto load_slots = [&](int jj) -> int {
+            const int e = (j_beg + jj) * kStepPages + lane;
+            return e < n_csteps * kStepPages ? __ldg(p.stream_meta + ep.stream_off + e) >> 8 : G;
         };
-        int meta_next = n_tiles > 0 ? load_meta(j_beg) : 0;
+        int slots = -1, slots_next = load_slots(0);
+        uint32_t changes = 0;
+        // The two warps that share a scheduler (one of each tile) take their exponentials in turns: both at once leave its special-function
+        // unit idle while both do the rest.  (Named barriers 1..8: (tile, quadrant) may begin.)
+        auto await_turn = [&](int jj) {
+            if (n_qt == 2 && (i == 1 || jj > 0)) asm volatile("bar.sync %0, 64;" ::"r"(1 + q4 + 4 * i) : "memory");
+        };
+        auto pass_turn = [&](int jj) {
+            if (n_qt == 2 && (i == 0 || jj + 1 < n_steps)) asm volatile("bar.arrive %0, 64;" ::"r"(1 + q4 + 4 * (i ^ 1)) : "memory");
+        };
 
-        for (int jj = 0; jj < n_tiles; ++jj) {
+        int jj = 0;
+        for (; jj < n_steps; ++jj) {
             const int j = j_beg + jj;
-            const bool cached = j < ep.n_ctiles;
-            // From the page words a warp-uniform mask: pages whose slot differs from the page before.  The pages of a new-token tile
-            // are masked from the causal limit of the tile's first row on.
-            const int meta = meta_next;
-            if (jj + 1 < n_tiles) meta_next = load_meta(j + 1);
-            int prev = __shfl_up_sync(kFull, meta >> 8, 1);
-            if (lane == 0) prev = cur_slot;
-            const uint32_t chg_mask = __ballot_sync(kFull, (meta >> 8) != prev) & 0xffu;
+            if (jj % kBatch == 0) {
+                const int last = __shfl_sync(kFull, slots, 31);
+                slots = slots_next;
+                slots_next = load_slots(jj + kBatch);
+                int prev = __shfl_up_sync(kFull, slots, 1);
+                if (lane == 0) prev = last;
+                changes = __ballot_sync(kFull, slots != prev);
+            }
+            const uint32_t chg_mask = (changes >> (jj % kBatch * kStepPages)) & ((1u << kStepPages) - 1u);
 
-            ok = mbar_wait(bar_s_full(i), static_cast<uint32_t>(jj & 1), abort_flag, p.status);
+            const uint32_t t_sb = t_s + static_cast<uint32_t>((jj & 1) * kStepKeys);
+            ok = mbar_wait(bar_s_full(i, jj & 1), static_cast<uint32_t>((jj >> 1) & 1), abort_flag, p.status);
             if (!ok) break;
             tc_fence_after();
 
-            // the row's 128 scores
-            uint32_t su[kTileKeys];
+            // the row's 64 scores
+            uint32_t su[kStepKeys];
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-                tmem_ld32_issue(t_s + static_cast<uint32_t>(k * 32), reinterpret_cast<uint32_t(&)[32]>(su[k * 32]));
+            for (int k = 0; k < kStepKeys / 32; ++k)
+                tmem_ld32_issue(t_sb + static_cast<uint32_t>(k * 32), reinterpret_cast<uint32_t(&)[32]>(su[k * 32]));
             tmem_ld_wait();
 #pragma unroll
-            for (int k = 0; k < 4; ++k) tmem_ld32_arrived(reinterpret_cast<uint32_t(&)[32]>(su[k * 32]));
-            float s[kTileKeys];
+            for (int k = 0; k < kStepKeys / 32; ++k) tmem_ld32_arrived(reinterpret_cast<uint32_t(&)[32]>(su[k * 32]));
+            float s[kStepKeys];
 #pragma unroll
-            for (int x = 0; x < kTileKeys; ++x) s[x] = __uint_as_float(su[x]);
+            for (int x = 0; x < kStepKeys; ++x) s[x] = __uint_as_float(su[x]);
 
             // hide keys after the causal limit (page padding is hidden in S already)
-            if (!cached) {
-                const int kbase = (j - ep.n_ctiles) * kTileKeys;
+            if (j >= n_csteps) {
+                const int kbase = (j - n_csteps) * kStepKeys;
                 const int vis = c - kbase + 1;                      // visible keys of this row
                 const int vis_lo = c_lo - kbase + 1;                // <= vis of every row of the tile
-                if (vis_lo < kTileKeys) {
+                if (vis_lo < kStepKeys) {
 #pragma unroll
-                    for (int x = 0; x < kTileKeys; ++x)
+                    for (int x = 0; x < kStepKeys; ++x)
                         if (x >= vis) s[x] = kNegInf;
                 }
             }
 
-            // row maximum: eight independent chains
-            float mx8[kPagesPerTile];
+            // row maximum: four independent chains
+            float mx4[kStepPages];
 #pragma unroll
-            for (int k = 0; k < kPagesPerTile; ++k) {
+            for (int k = 0; k < kStepPages; ++k) {
                 float a = fmax3(s[k * 16], s[k * 16 + 1], s[k * 16 + 2]);
 #pragma unroll
                 for (int x = 3; x < 15; x += 2) a = fmax3(a, s[k * 16 + x], s[k * 16 + x + 1]);
-                mx8[k] = fmaxf(a, s[k * 16 + 15]);
+                mx4[k] = fmaxf(a, s[k * 16 + 15]);
             }
-            const float m_cand = fmax3(fmax3(mx8[0], mx8[1], mx8[2]), fmax3(mx8[3], mx8[4], mx8[5]), fmaxf(mx8[6], mx8[7])) * scale;
+            const float m_cand = fmaxf(fmax3(mx4[0], mx4[1], mx4[2]), mx4[3]) * scale;
 
             // The reference moves only when the row maximum has grown by more than the threshold (probabilities
             // stay below 2^threshold meanwhile); then the sums and the accumulator O_i are rescaled.  O_i holds
@@ -477,6 +479,9 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                 acc *= alpha;
                 m = m_new;
                 if (jj > 0) {
+                    ok = mbar_wait(bar_pv_done(i), static_cast<uint32_t>((jj - 1) & 1), abort_flag, p.status);
+                    if (!ok) break;
+                    tc_fence_after();
 #pragma unroll 1
                     for (int k = 0; k < D / 32; ++k) {
                         uint32_t o[32];
@@ -492,10 +497,11 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
             // p = exp2(s * scale - m) in fp32; bf16 pairs (even key in the low half) into P_i, 32 keys per store, handed
             // to the MMA warp in two halves.  The page sums (of the fp32 values) are taken along the way: their adds
             // fill issue slots that the exponentials leave free.
+            await_turn(jj);
             const uint64_t sc2 = pack2(scale, scale), nm2 = pack2(-m_use, -m_use);
-            uint64_t ps2[kPagesPerTile];
+            uint64_t ps2[kStepPages];
 #pragma unroll
-            for (int ch = 0; ch < 4; ++ch) {
+            for (int ch = 0; ch < kStepKeys / 32; ++ch) {
                 uint32_t pk[16];
 #pragma unroll
                 for (int x = 0; x < 16; ++x) {
@@ -508,39 +514,40 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                     pk[x] = pack_bf16(a0, a1);
                     ps2[e] = (x & 7) ? add2(ps2[e], p2) : p2;
                 }
-                tmem_st16(t_s + static_cast<uint32_t>(ch * 16), pk);
-                if (ch & 1) {
-                    tmem_st_wait();
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(bar_p_half(i, ch >> 1));
-                }
+                tmem_st16(t_sb + static_cast<uint32_t>(ch * 16), pk);
             }
+            pass_turn(jj);
+            tmem_st_wait();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_p_full(i, jj & 1));
 
             // under the MMAs: row sum, slots
-            float ps[kPagesPerTile];
+            float ps[kStepPages];
 #pragma unroll
-            for (int e = 0; e < kPagesPerTile; ++e) {
+            for (int e = 0; e < kStepPages; ++e) {
                 float lo, hi;
                 unpack2(ps2[e], lo, hi);
                 ps[e] = lo + hi;
             }
-            const float tot = ((ps[0] + ps[1]) + (ps[2] + ps[3])) + ((ps[4] + ps[5]) + (ps[6] + ps[7]));
+            const float tot = (ps[0] + ps[1]) + (ps[2] + ps[3]);
             l += tot;
             if (chg_mask == 0u) {
                 acc += tot;
             } else {
 #pragma unroll
-                for (int e = 0; e < kPagesPerTile; ++e) {
+                for (int e = 0; e < kStepPages; ++e) {
                     if ((chg_mask >> e) & 1u) {
                         park(m_use);
                         acc = 0.f;
-                        cur_slot = __shfl_sync(kFull, meta >> 8, e);
+                        cur_slot = __shfl_sync(kFull, slots, jj % kBatch * kStepPages + e);
                     }
                     acc += ps[e];
                 }
             }
         }
+
+        for (; jj < n_steps; ++jj) { await_turn(jj); pass_turn(jj); }      // error path only: the other tile's warp may be waiting
 
         // ---- per-row results ----
         const float m_use = (m == kNegInf) ? 0.f : m;
@@ -596,9 +603,9 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
         if (p.n_splits > 1) {
             first_slot = G + 1;
             last_slot = -1;
-            if (n_tiles > 0) {
-                first_slot = (j_beg < ep.n_ctiles) ? (__ldg(p.stream_meta + ep.stream_off + j_beg * kPagesPerTile) >> 8) : G;
-                last_slot = (j_end > ep.n_ctiles) ? G : (__ldg(p.stream_meta + ep.stream_off + j_end * kPagesPerTile - 1) >> 8);
+            if (n_steps > 0) {
+                first_slot = (j_beg < n_csteps) ? (__ldg(p.stream_meta + ep.stream_off + j_beg * kStepPages) >> 8) : G;
+                last_slot = (j_end > n_csteps) ? G : (__ldg(p.stream_meta + ep.stream_off + j_end * kStepPages - 1) >> 8);
             }
         }
 
@@ -611,7 +618,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                     if (park_smem) finish_masses(lse, kNegInf, 0, G);
                     else if (row_valid) p.lse_out[rh] = lse;
                 }
-                if (n_tiles > 0) {
+                if (n_steps > 0) {
                     const float inv = (l > 0.f) ? 1.f / l : 0.f;
                     ok = mbar_wait(bar_o_done(i), 0, abort_flag, p.status);
                     if (ok) {
@@ -648,7 +655,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                             if (sl < first_slot || sl > last_slot) slots[sl] = kNegInf;
                     }
                 }
-                if (n_tiles > 0) {
+                if (n_steps > 0) {
                     const float inv = (l > 0.f) ? 1.f / l : 0.f;
                     ok = mbar_wait(bar_o_done(i), 0, abort_flag, p.status);
                     if (ok) {
@@ -672,10 +679,10 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                     const uint32_t mine = sbase + static_cast<uint32_t>(C::kXpeerOff + (i * 128 + r) * 16);
                     peer_push4(peer_addr(mine, peer), m_use, l, bnd, 0.f, peer_addr(bar_peer_ml, peer));
                 }
-                constexpr uint32_t kRingOff = kQTiles * C::kTileBytes;
+                constexpr uint32_t kRingOff = C::kRingOff;
                 constexpr uint32_t kExportStageOff = 65536;         // upper half of the ring (4 stages x 32 KB)
                 const uint32_t warp_off = kRingOff + static_cast<uint32_t>(q4 * 16384);
-                if (i != it.split && n_tiles > 0) {
+                if (i != it.split && n_steps > 0) {
                     // This CTA finishes Q tile `it.split`; the accumulator of the other tile goes to the peer, which
                     // finishes that one.  It goes as it is (relative to this CTA's own reference; the peer learns the
                     // weight from the row sums above), so that nothing but the last MMA stands before it: staged
@@ -734,7 +741,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                         }
                     }
                 }
-                if (ok && i == it.split && n_tiles > 0) {
+                if (ok && i == it.split && n_steps > 0) {
                     // this CTA finishes the tile: its own accumulator and what the peer sent, each with its weight;
                     // thread (warp, lane) reads what thread (warp, lane) of the peer wrote
                     ok = mbar_wait(bar_o_done(i), 0, abort_flag, p.status);

@@ -90,8 +90,8 @@ struct MapCache {
     CUtensorMap map[kSlots];
     bool used[kSlots] = {};
     uint32_t turn = 0;
-    // 3-D bf16 map [d2][d1][d0] with box {b0, b1, b2}
-    bool get(CUtensorMap *out, const void *base, const cuuint64_t *dims, const cuuint64_t *strides, const cuuint32_t *box)
+    // bf16 map [..][d2][d1][d0] of rank 3 or 4 with box {b0, b1, b2, ..}; the boxes in use tell the ranks apart
+    bool get(CUtensorMap *out, const void *base, const cuuint64_t *dims, const cuuint64_t *strides, const cuuint32_t *box, int rank = 3)
     {
         const MapKey k{base, dims[0], dims[1], dims[2], box[0], box[1], box[2]};
         const size_t h = (reinterpret_cast<uintptr_t>(base) >> 8) * 0x9E3779B97F4A7C15ull >> 56;
@@ -101,7 +101,7 @@ struct MapCache {
             if (used[i] && key[i] == k) { *out = map[i]; return true; }
             if (victim < 0 && (!used[i] || key[i].base == base)) victim = i;
         }
-        if (!encode_map(out, base, 3, dims, strides, box)) return false;
+        if (!encode_map(out, base, rank, dims, strides, box)) return false;
         const int i = victim >= 0 ? victim : static_cast<int>((h + (turn++ & 3u)) % kSlots);
         key[i] = k;
         map[i] = *out;
@@ -131,7 +131,8 @@ struct enl_cache {
     uint8_t *kpool = nullptr, *vpool = nullptr;
     std::vector<int32_t> free_pages;        // stack of free page ids (page 0 is never in it)
     std::vector<Group> groups;
-    std::vector<CUtensorMap> tm_k, tm_v;    // per layer
+    std::vector<CUtensorMap> tm_k, tm_v;    // per layer, boxes of 64 channels of a page of a head
+    std::vector<CUtensorMap> tm_k4, tm_v4;  // and of a page of a head, for attn_kernel
     uint64_t epoch = 0;                     // bumped by every store
 
     // gather plan: host image (pinned when there is a GPU), device copy, capacities
@@ -336,13 +337,21 @@ extern "C" int enl_cache_create(const enl_cache_desc_t *desc, enl_cache_t **out)
 
     c->tm_k.resize(d.n_layers);
     c->tm_v.resize(d.n_layers);
+    c->tm_k4.resize(d.n_layers);
+    c->tm_v4.resize(d.n_layers);
     const cuuint64_t dims[2] = {static_cast<cuuint64_t>(d.head_dim),
                                 static_cast<cuuint64_t>(c->n_pages) * d.n_kv_heads * kPageTokens};
     const cuuint64_t strides[1] = {static_cast<cuuint64_t>(d.head_dim) * 2};
     const cuuint32_t box[2] = {64, kPageTokens};
+    const cuuint64_t row = strides[0];
+    const cuuint64_t dims4[4] = {64, 8, static_cast<cuuint64_t>(d.head_dim / 64), dims[1] / 8};
+    const cuuint64_t strides4[3] = {row, 128, row * 8};
+    const cuuint32_t box4[4] = {64, 8, static_cast<cuuint32_t>(d.head_dim / 64), 2};
     for (int l = 0; l < d.n_layers; ++l) {
         if (!encode_map(&c->tm_k[l], c->kpool + c->layer_bytes * l, 2, dims, strides, box) ||
-            !encode_map(&c->tm_v[l], c->vpool + c->layer_bytes * l, 2, dims, strides, box)) {
+            !encode_map(&c->tm_v[l], c->vpool + c->layer_bytes * l, 2, dims, strides, box) ||
+            !encode_map(&c->tm_k4[l], c->kpool + c->layer_bytes * l, 4, dims4, strides4, box4) ||
+            !encode_map(&c->tm_v4[l], c->vpool + c->layer_bytes * l, 4, dims4, strides4, box4)) {
             destroy(c);
             return ENL_E_CUDA;
         }
@@ -1069,17 +1078,22 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         const cuuint64_t qs[2] = {static_cast<cuuint64_t>(d.head_dim) * 2,
                                   static_cast<cuuint64_t>(d.head_dim) * 2 * d.n_q_heads};
         const cuuint32_t qb[3] = {64, static_cast<cuuint32_t>(c->rep), static_cast<cuuint32_t>(kTileRows / c->rep)};
-        const cuuint64_t nd[3] = {static_cast<cuuint64_t>(d.head_dim), static_cast<cuuint64_t>(d.n_kv_heads),
-                                  static_cast<cuuint64_t>(a->n_new)};
-        const cuuint64_t ns[2] = {static_cast<cuuint64_t>(d.head_dim) * 2,
-                                  static_cast<cuuint64_t>(d.head_dim) * 2 * d.n_kv_heads};
-        const cuuint32_t nb[3] = {64, 1, kTileKeys};
-        if (!c->maps.get(&p.tm_q, a->q, qd, qs, qb) || !c->maps.get(&p.tm_knew, a->k_new, nd, ns, nb) ||
-            !c->maps.get(&p.tm_vnew, a->v_new, nd, ns, nb))
-            return ENL_E_CUDA;
+        const cuuint64_t n_new = static_cast<cuuint64_t>(a->n_new), head = static_cast<cuuint64_t>(d.head_dim) * 2, token = head * d.n_kv_heads;
+        const cuuint64_t n_heads = static_cast<cuuint64_t>(d.n_kv_heads), n_halves = static_cast<cuuint64_t>(d.head_dim / 64);
+        bool okm = c->maps.get(&p.tm_q, a->q, qd, qs, qb);
+        if (mass_only) {
+            const cuuint64_t nd[3] = {static_cast<cuuint64_t>(d.head_dim), n_heads, n_new}, ns[2] = {head, token};
+            const cuuint32_t nb[3] = {64, 1, kTileKeys};
+            okm = okm && c->maps.get(&p.tm_knew, a->k_new, nd, ns, nb);
+        } else {
+            const cuuint64_t nd[4] = {64, n_new, n_halves, n_heads}, ns[3] = {token, 128, head};
+            const cuuint32_t nb[4] = {64, 8, static_cast<cuuint32_t>(n_halves), 1};
+            okm = okm && c->maps.get(&p.tm_knew, a->k_new, nd, ns, nb, 4) && c->maps.get(&p.tm_vnew, a->v_new, nd, ns, nb, 4);
+        }
+        if (!okm) return ENL_E_CUDA;
     }
-    p.tm_kpool = c->tm_k[a->layer];
-    p.tm_vpool = c->tm_v[a->layer];
+    p.tm_kpool = mass_only ? c->tm_k[a->layer] : c->tm_k4[a->layer];
+    p.tm_vpool = c->tm_v4[a->layer];
     p.items = reinterpret_cast<const Item *>(c->plan_dev + c->off_items);
     p.eps = reinterpret_cast<const EpInfo *>(c->plan_dev + c->off_eps);
     p.stream_page = reinterpret_cast<const int32_t *>(c->plan_dev + c->off_stream);

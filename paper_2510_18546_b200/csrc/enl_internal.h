@@ -10,6 +10,7 @@ namespace enl {
 constexpr int kPageTokens = 16;     // tokens per page: one TMA box of 16 rows x 128 B per 64 channels
 constexpr int kTileKeys   = 128;    // keys per KV tile (8 pages)
 constexpr int kPagesPerTile = kTileKeys / kPageTokens;
+constexpr int kStepKeys   = 64;     // keys that attn_kernel takes at once
 constexpr int kTileRows   = 128;    // query rows per Q tile = (128 / rep) tokens x rep q heads of one kv head
 constexpr int kQTiles     = 2;      // Q tiles per CTA (they share every K/V tile the CTA loads)
 constexpr int kZeroPage   = 0;      // page 0 is never handed out: all zeros, target of null stream entries
@@ -35,9 +36,11 @@ struct Item {
 // Kernel parameters (passed by value as a __grid_constant__).
 struct AttnParams {
     CUtensorMap tm_q;       // [n_q][Hq][D]      box {64, rep, 128/rep}
-    CUtensorMap tm_knew;    // [n_new][Hkv][D]   box {64, 1, 128}
+    // Boxes that leave a block of 8 rows x 128 bytes per 64 channels and then the next 8 rows: eight rows of a head of new tokens
+    // (channel, token, 64-channel block, head), both groups of a page of a head (channel, row of 8, 64-channel block, group of 8 rows)
+    CUtensorMap tm_knew;    // [n_new][Hkv][D]   box {64, 8, D/64, 1}
     CUtensorMap tm_vnew;
-    CUtensorMap tm_kpool;   // [pages*Hkv*16][D] box {64, 16}   (one layer)
+    CUtensorMap tm_kpool;   // [pages*Hkv*2][8][D] box {64, 8, D/64, 2}   (one layer)
     CUtensorMap tm_vpool;
     const Item   *items;
     const EpInfo *eps;
