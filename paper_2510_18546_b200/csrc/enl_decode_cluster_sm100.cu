@@ -7,14 +7,15 @@
 // streaming kernel spends 6 of its 8.6 us on merging -- partial results to memory, a fence, a counter, and the last CTA
 // reading them back (0.9 + 1.9 us), while the next launch cannot even start.  Here the splits of one (episode, kv head) are
 // the CTAs of one thread-block cluster: each merges its warps in its own shared memory and pushes what the others need of
-// the result into theirs; behind the cluster barrier every CTA adds up its share of the output out of its own shared memory
-// and writes it out.  And two CTAs fit an SM (12 warps of 80 registers, ~110 KB), so the next launch is resident while this
+// the result into theirs, with st.async, whose bytes the receiver's barrier counts: the receiver adds up its share of the output as soon
+// as it is there, nobody fences and nobody waits for a second cluster barrier (its release waits for every earlier store, ~0.5 us).
+// And two CTAs fit an SM (12 warps of 80 registers, ~110 KB), so the next launch is resident while this
 // one runs: its set-up and its first pages (from the pool, which only this library writes) are done before its wait for the
-// previous kernel ends.
-// Measured per launch in a chain of 20 layers (32 q / 8 kv heads, 24 groups, masses wanted, streaming kernel -> this one): D 128,
-// 640 keys 9.2 -> 6.0 us, 2200 keys 10.2 -> 8.1, 4900 keys 11.9 -> 10.1, 16 episodes of 3160 keys 38.1 -> 37.8, 8 of 3200
-// 24.5 -> 22.3; D 64, the same, 8.6 -> 5.5, 9.1 -> 6.9, 10.3 -> 8.5, 28.7 -> 22.8, 20.2 -> 14.7; contiguous keys (the entry point
-// that allocates nothing), D 128, 2500 keys 91 -> 9.3 (10.2 where every layer's keys come from memory).
+// previous kernel ends.  Where its last clusters have to wait for an SM (sixteens of eight kv heads), the set-up itself counts: each warp
+// asks for its first page before anything else, and prefetches are dealt to the warps (start to wait 2.7 -> 1.8 us).
+// Measured per launch in a chain of 20 layers (32 q / 8 kv heads, 24 groups; streaming kernel, this one with cluster barriers, now):
+// D 128 with masses, 640 keys 9.2, 6.0, 5.4 us, 2560 keys 10.2, 8.3, 6.9; without, 640 keys 5.0, 4.6, 2560 keys 6.7, 5.9; D 64 with
+// masses, 640 keys 8.6, 5.6, 4.7, 2560 keys 9.1, 7.3, 5.7; contiguous keys (the entry point that allocates nothing), 2500 keys 91, 10.2, 9.0.
 //
 // Per page, all in registers of one warp:
 //   S^T = K Q^T        mma.sync m16n8k16, A = the 16 keys (ldmatrix), B = the rep query rows padded to 8
@@ -43,21 +44,39 @@ constexpr int kMaxRep  = 8;                               // q heads per kv head
 constexpr int kPrefetchPages = 24;                        // pages per CTA asked into the L2 before the previous kernel has ended
 constexpr float kRescaleThreshold = 8.0f;                 // log2 units
 
-__device__ __forceinline__ float peer_f32(uint32_t addr)
+// Stores into a peer's shared memory whose completion is counted (in bytes) on a barrier of the peer: neither side needs a
+// fence or a round trip.  Not for a cluster of one: that is launched without clusters, where these instructions are illegal.
+__device__ __forceinline__ void peer_push(uint32_t addr, float v, uint32_t bar)
 {
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
-    return v;
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(addr), "f"(v), "r"(bar) : "memory");
 }
-__device__ __forceinline__ void peer_push(uint32_t addr, float v)
+__device__ __forceinline__ void peer_push4(uint32_t addr, float4 v, uint32_t bar)
 {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
+                 ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(bar) : "memory");
 }
-__device__ __forceinline__ void peer_push4(uint32_t addr, float4 v)
+// Waits for what the peers push.  No CTA may leave before it has arrived, so a wait of its own that ran out does not cut this one short:
+// its limit covers that of the peers' waits, after which they push whatever they have.
+__device__ __forceinline__ void wait_for_peers(uint32_t bar, int32_t *status)
 {
-    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+    unsigned long long t0 = 0;
+    for (uint32_t spins = 1;; ++spins) {
+        uint32_t done;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(done) : "r"(bar) : "memory");
+        if (__all_sync(0xffffffffu, done != 0u)) return;
+        if ((spins & 15u) == 0u) {
+            const unsigned long long now = global_ns();
+            if (t0 == 0) t0 = now;
+            if (__any_sync(0xffffffffu, now - t0 > 4 * kWaitLimitNs)) { atomicExch(status, 2); return; }
+        }
+    }
 }
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+// (nothing to publish but barriers, which fence.mbarrier_init has: no wait for earlier stores)
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 // the 8 x 8 matrix of 16-bit values that the warp holds, transposed
 __device__ __forceinline__ uint32_t transpose8x8(uint32_t x)
@@ -76,13 +95,15 @@ struct Cfg {
     static constexpr int kORow       = D + 4;                          // row of a warp's output: no two rows of a store share banks
     static_assert(kWarps * kMaxRep * kORow * 4 <= kRingBytes, "the warps' outputs fit the idle ring");
     static constexpr int kBarOff     = kRingBytes;                     // [warp][stage]
-    static constexpr int kRngOff     = kBarOff + kWarps * kStages * 8; // [kMaxCluster] (first slot, slots)
+    static constexpr int kInBarOff   = kBarOff + kWarps * kStages * 8; // what the cluster sends has arrived: outputs, shares of a slot
+    static constexpr int kRngOff     = kInBarOff + 16;                 // [kMaxCluster] (first slot, slots)
     static constexpr int kMiscOff    = kRngOff + kMaxCluster * 8;
     // wm[warp][rep], wl[warp][rep], cm[rep], cl[rep], warp weights[rep][kMaxCluster], log2-sum-exps (then weights) of the
     // cluster's CTAs[rep][kMaxCluster], ctrs[2], flags[2]
     static constexpr int kMiscBytes  = (2 * kWarps * kMaxRep + 2 * kMaxRep + 2 * kMaxRep * kMaxCluster + 4) * 4;
     static constexpr int kQOff       = kMiscOff + kMiscBytes;          // [D / 16][32 lanes] B fragments of the query rows
-    static constexpr int kInOff      = kQOff + D / 16 * 32 * 8;        // [CTA][float4]: what the cluster's CTAs send for this CTA's share of the output
+    static constexpr int kShareOff   = kQOff + D / 16 * 32 * 8;        // [kMaxCluster][kMaxRep]: the cluster's shares of this CTA's last slot
+    static constexpr int kInOff      = kShareOff + kMaxCluster * kMaxRep * 4;        // [CTA][float4]: what the cluster's CTAs send for this CTA's share of the output
     static_assert(kInOff % 16 == 0, "alignment");
     // parked slot sums: a warp's pages come in stream order, so it parks each slot it meets once
     static __host__ __device__ constexpr int ent_cap(int pages, int slots)
@@ -121,7 +142,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     float *cl = cm + kMaxRep;
     float *ww = cl + kMaxRep;                                                 // [kMaxRep][kMaxCluster]: weights of the warps
     float *cw = ww + kMaxRep * kMaxCluster;                                   // [kMaxRep][kMaxCluster]: log2-sum-exps of the cluster's CTAs
-    int *ctrs = reinterpret_cast<int *>(cw + kMaxRep * kMaxCluster);          // [0] next page to hand out, [1] parked entries
+    int *ctrs = reinterpret_cast<int *>(cw + kMaxRep * kMaxCluster);          // [0] next page to hand out, [1] parked entries, [3] see `owner`
     volatile int *abort_flag = ctrs + 2;
     const int rep = p.rep, rep2 = (rep + 1) & ~1;
     const int n_ent_cap = C::ent_cap(p.list_pages, p.list_slots);
@@ -130,6 +151,8 @@ __global__ void __launch_bounds__(kThreads, 2)
     int2 *pg_list = reinterpret_cast<int2 *>(ent_slot + ((n_ent_cap + 1) & ~1));   // the CTA's pages in stream order
     float *cslot = reinterpret_cast<float *>(pg_list + p.list_pages);         // [slot][kMaxRep]: shares of the range's sum
     const uint32_t bar0 = sbase + C::kBarOff;
+    const uint32_t bar_in = sbase + C::kInBarOff, bar_share = bar_in + 8;
+    const float *share_in = reinterpret_cast<const float *>(smem + C::kShareOff);
     auto bar_full = [&](int s) { return bar0 + 8u * (warp * kStages + s); };
     auto stage_addr = [&](int s) { return sbase + static_cast<uint32_t>((warp * kStages + s) * C::kStageBytes); };
 
@@ -157,8 +180,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     int total;
     if constexpr (kStatic) total = prm.page_off[G + 1];
     else total = n_cached + (ep.n_new + kPageTokens - 1) / kPageTokens;
-    const int pg_beg = static_cast<int>(static_cast<long long>(total) * split / n_splits);
-    const int pg_end = static_cast<int>(static_cast<long long>(total) * (split + 1) / n_splits);
+    const int pg_beg = total * split >> ls, pg_end = total * (split + 1) >> ls;   // (at most kMaxCluster * kClusterMaxPages pages)
     const int n_cta = pg_end - pg_beg;                                        // <= p.list_pages (host guarantees)
 
     // page e of the stream: (page id, or -1 - first row of the caller's keys; slot << 8 | valid keys)
@@ -177,29 +199,6 @@ __global__ void __launch_bounds__(kThreads, 2)
             return make_int2(-1 - r, (G << 8) | min(kPageTokens, ep.n_new - r));
         }
     };
-
-    if (threadIdx.x == 0) { *abort_flag = 0; ctrs[0] = kWarps; ctrs[1] = 0; }
-    // The slot range of every CTA of the cluster (the same arithmetic as that CTA uses): the merge looks up whose table holds a slot.
-    if (static_cast<int>(threadIdx.x) < n_splits) {
-        const int k = threadIdx.x;
-        const int b0 = static_cast<int>(static_cast<long long>(total) * k / n_splits);
-        const int b1 = static_cast<int>(static_cast<long long>(total) * (k + 1) / n_splits);
-        int2 r = make_int2(0, 0);
-        if (b1 > b0) {
-            const int s0 = entry(b0).y >> 8;
-            r = make_int2(s0, (entry(b1 - 1).y >> 8) - s0 + 1);
-        }
-        rng_tab[k] = r;
-    }
-    for (int i = threadIdx.x; i < n_cta; i += kThreads) pg_list[i] = entry(pg_beg + i);
-    if (lane == 0) {
-        for (int s = 0; s < kStages; ++s) mbar_init(bar_full(s), 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    }
-    __syncthreads();
-    cluster_arrive();                                                        // every CTA of the cluster has started (waited for before the first store to a peer)
-    pdl_trigger();
 
     const uint64_t pol = policy_evict_first();
     // K or V of one page into this warp's ring
@@ -224,12 +223,60 @@ __global__ void __launch_bounds__(kThreads, 2)
     // come in between, so the first cached page of every warp is fetched for good; what else comes first is asked into the L2
     // (which observes nothing: the L2 is the point of coherence).  The first round is handed out statically.
     int cur = warp;
-    const int pg0 = cur < n_cta ? pg_list[cur].x : -1;
-    if (lane == 0 && pg0 >= 0) { issue(false, pg0); issue(true, pg0); }
-    for (int i = threadIdx.x; i < min(n_cta, kPrefetchPages) * 2 * kHalves; i += kThreads) {
-        const int pg = pg_list[i / (2 * kHalves)].x, r = i % (2 * kHalves), x = (r % kHalves) * 64;
-        if (pg < 0) tma_prefetch_3d(r >= kHalves ? &p.tm_vnew : &p.tm_knew, x, kvh, ep.new_off + (-1 - pg));
-        else if (i >= kWarps * 2 * kHalves) tma_prefetch_2d(r >= kHalves ? &p.tm_vpool : &p.tm_kpool, x, (pg * p.Hkv + kvh) * kPageTokens);
+    const int2 first = cur < n_cta ? entry(pg_beg + cur) : make_int2(-1, 0);
+    const int pg0 = first.x;
+    if (lane == 0) {
+        for (int s = 0; s < kStages; ++s) mbar_init(bar_full(s), 1);
+        if (warp == 0) {
+            mbar_init(bar_in, 1);
+            mbar_init(bar_share, 1);
+            mbar_expect_tx(bar_in, static_cast<uint32_t>(rep * (D + n_splits) * 4));
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        if (pg0 >= 0) { issue(false, pg0); issue(true, pg0); }
+    }
+    if (threadIdx.x == 0) { *abort_flag = 0; ctrs[0] = kWarps; ctrs[1] = 0; }
+    // The slot range of every CTA of the cluster (the same arithmetic as that CTA uses): the merge looks up whose table holds a slot.
+    if (static_cast<int>(threadIdx.x) < n_splits) {
+        const int k = threadIdx.x;
+        const int b0 = total * k >> ls, b1 = total * (k + 1) >> ls;
+        int2 r = make_int2(0, 0);
+        if (b1 > b0) {
+            const int s0 = entry(b0).y >> 8;
+            r = make_int2(s0, (entry(b1 - 1).y >> 8) - s0 + 1);
+        }
+        rng_tab[k] = r;
+    }
+    for (int i = threadIdx.x; i < n_cta; i += kThreads) pg_list[i] = entry(pg_beg + i);
+    __syncthreads();
+    cluster_arrive_relaxed();                                                // every CTA of the cluster has started (waited for before the first store to a peer)
+    pdl_trigger();
+    int slot_first = 0, n_local = 0;                                         // slots the CTA's range touches
+    if (n_cta > 0) {
+        slot_first = pg_list[0].y >> 8;
+        n_local = (pg_list[n_cta - 1].y >> 8) - slot_first + 1;
+    }
+    // The CTA in whose range a slot begins writes its mass; the CTAs behind whose ranges the slot reaches into send their shares.  Which
+    // CTA wants this one's share of its first slot (-1: this one does), and how many send theirs of its last?
+    if (p.mass && warp == kWarps - 1) {
+        const int2 r = lane < n_splits ? rng_tab[lane] : make_int2(0, 0);
+        const int last = r.x + r.y - 1;
+        const uint32_t into = __ballot_sync(0xffffffffu, lane < split && r.y > 0 && last == slot_first);
+        const uint32_t after = __ballot_sync(0xffffffffu, lane > split && r.y > 0 && r.x == slot_first + n_local - 1);
+        if (lane == 0) {
+            ctrs[3] = n_cta > 0 ? __ffs(into) - 1 : -1;
+            const bool wanted = n_local > 1 || (n_local == 1 && into == 0u);
+            mbar_expect_tx(bar_share, wanted ? static_cast<uint32_t>(__popc(after) * rep * 4) : 0u);
+        }
+    }
+    // (a warp takes a page: a box costs the warp that asks for it some 50 cycles)
+    for (int i = warp; i < min(n_cta, kPrefetchPages); i += kWarps) {
+        const int pg = pg_list[i].x, x = (lane % kHalves) * 64;
+        if (lane < 2 * kHalves) {
+            if (pg < 0) tma_prefetch_3d(lane >= kHalves ? &p.tm_vnew : &p.tm_knew, x, kvh, ep.new_off + (-1 - pg));
+            else if (i >= kWarps) tma_prefetch_2d(lane >= kHalves ? &p.tm_vpool : &p.tm_kpool, x, (pg * p.Hkv + kvh) * kPageTokens);
+        }
     }
     const uint8_t *q_rows = static_cast<const uint8_t *>(p.q) + (static_cast<long long>(ep.q_off) * p.Hq + kvh * rep) * D * 2;
     if (static_cast<int>(threadIdx.x) * 128 < rep * D * 2)
@@ -391,12 +438,7 @@ __global__ void __launch_bounds__(kThreads, 2)
         *reinterpret_cast<float2 *>(wm + warp * kMaxRep + 2 * tq) = make_float2(m[0], m[1]);
         *reinterpret_cast<float2 *>(wl + warp * kMaxRep + 2 * tq) = make_float2(lsum[0], lsum[1]);
     }
-    // slots the CTA's range touched, and their table cleared for the merge of the parked sums
-    int slot_first = 0, n_local = 0;
-    if (n_cta > 0) {
-        slot_first = pg_list[0].y >> 8;
-        n_local = (pg_list[n_cta - 1].y >> 8) - slot_first + 1;
-    }
+    // the table of the CTA's slots cleared for the merge of the parked sums
     for (int idx = threadIdx.x; idx < n_local * kMaxRep; idx += kThreads) cslot[idx] = 0.f;
     __syncthreads();                                                         // every stage consumed: the ring is free
     // (after an expired wait the CTA goes on with whatever it has: its peers wait for it at the cluster's barriers)
@@ -436,7 +478,8 @@ __global__ void __launch_bounds__(kThreads, 2)
     cluster_wait();                                                          // they have all started
     if (static_cast<int>(threadIdx.x) < (rep << ls)) {
         const int h = threadIdx.x >> ls, k = threadIdx.x & (n_splits - 1);
-        peer_push(peer_addr(smem_u32(cw + h * kMaxCluster + split), k), cm[h]);
+        if (n_splits == 1) cw[h * kMaxCluster] = cm[h];
+        else peer_push(peer_addr(smem_u32(cw + h * kMaxCluster + split), k), cm[h], peer_addr(bar_in, k));
     }
     const int n_f4 = rep * (D / 4);                                          // the rep output rows as float4 (16 .. 256)
     const int lf = 31 - __clz(n_f4) - ls;                                    // log2 of a CTA's share of them
@@ -452,7 +495,8 @@ __global__ void __launch_bounds__(kThreads, 2)
         const float inv = cl[h];
         a.x *= inv; a.y *= inv; a.z *= inv; a.w *= inv;
         const int owner = ff >> lf, at = (split << lf) + (ff & ((1 << lf) - 1));
-        peer_push4(peer_addr(sbase + C::kInOff + at * 16, owner), a);
+        if (n_splits == 1) *reinterpret_cast<float4 *>(smem + C::kInOff + at * 16) = a;
+        else peer_push4(peer_addr(sbase + C::kInOff + at * 16, owner), a, peer_addr(bar_in, owner));
     }
     // parked sums -> shares of the range's sum.  No slot's sum exceeds it, so the shares are at most 1 and add up without a
     // maximum pass (a share below 2^-126 counts as nothing).
@@ -464,8 +508,14 @@ __global__ void __launch_bounds__(kThreads, 2)
             if (v != kNegInf) atomicAdd(&cslot[(ent_slot[e] - slot_first) * kMaxRep + h], ex2(v - cm[h]));
         }
     }
-    cluster_arrive();
-    cluster_wait();
+    if (p.mass) {
+        __syncthreads();                                                     // the shares are complete
+        const int owner = ctrs[3];
+        if (owner >= 0 && static_cast<int>(threadIdx.x) < rep)
+            peer_push(peer_addr(sbase + C::kShareOff + (split * kMaxRep + threadIdx.x) * 4, owner), cslot[threadIdx.x], peer_addr(bar_share, owner));
+    }
+    if (n_splits == 1) __syncthreads();
+    else wait_for_peers(bar_in, p.status);
 
     // ---- merge the CTAs of the cluster: every CTA takes its share of the rows, thread (float4, CTA) ----
     const long long row_h0 = static_cast<long long>(ep.q_off) * p.Hq + kvh * rep;             // + h: (row, head) index
@@ -499,9 +549,8 @@ __global__ void __launch_bounds__(kThreads, 2)
         }
     }
     if (!p.mass) return;
-    // Masses: every CTA writes the slots whose pages begin in its range (and the empty ones behind them).  Only a slot that
-    // reaches into the ranges behind needs anything of the peers: their shares of their first slot, read where they are, so
-    // that nobody may leave before the others have.
+    // Masses: every CTA writes the slots whose pages begin in its range (and the empty ones behind them), its last slot with
+    // what the CTAs behind have sent.
     float *wt = wm;                                                          // [kMaxRep][kMaxCluster] (the warps' words are spent)
     static_assert(kMaxRep * kMaxCluster <= 2 * kWarps * kMaxRep && kMaxRep * kMaxCluster <= 128 && kThreads >= 256 + 128, "weights");
     if (threadIdx.x >= 256) {                                                // the warps that have no output to write
@@ -510,6 +559,7 @@ __global__ void __launch_bounds__(kThreads, 2)
         if (h < rep) wt[h * kMaxCluster + k] = w;
     }
     __syncthreads();
+    if (n_splits > 1) wait_for_peers(bar_share, p.status);
     if (n_cta > 0) {
         int s0 = slot_first, s1 = G + 1;                                     // this CTA's slots
         if (split == 0) s0 = 0;
@@ -531,13 +581,11 @@ __global__ void __launch_bounds__(kThreads, 2)
                 sum = w[split] * cslot[(s - slot_first) * kMaxRep + h];
                 if (s == slot_first + n_local - 1)
                     for (int k = split + 1; k < n_splits && rng_tab[k].x <= s; ++k)
-                        if (rng_tab[k].y > 0 && rng_tab[k].x == s) sum += w[k] * peer_f32(peer_addr(smem_u32(cslot + h), k));
+                        if (rng_tab[k].y > 0 && rng_tab[k].x == s) sum += w[k] * share_in[k * kMaxRep + h];
             }
             p.mass[(row_h0 + h) * p.mass_stride + s] = sum;
         }
     }
-    cluster_arrive();
-    cluster_wait();
 }
 
 template <int D, bool kStatic, typename P>

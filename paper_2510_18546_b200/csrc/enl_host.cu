@@ -749,7 +749,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
             // 9.9 / 11.8, 11.3 / 12.4, 15.0 / 15.6, 20.0 / 19.3; 18.2 / 23.1, so there the line could lie at some 100 pages.  With few
             // kv heads, too: D 128, 10k keys, 2 kv heads 10.5 / 15.7, 4 kv heads 12.3 / 14.9.
             const int n = B * d.n_kv_heads;
-            for (int i = widest_cluster_log(n, most, has_mass); i >= 0 && !cluster; --i) {
+            for (int i = widest_cluster_log(n, most, false); i >= 0 && !cluster; --i) {
                 if ((1 << i) > fewest) continue;
                 list_pages = (ceil_div(most, 1 << i) + 1) & ~1;
                 if (list_pages > kClusterMaxPages) break;

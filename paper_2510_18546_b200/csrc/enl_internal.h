@@ -251,15 +251,16 @@ struct ClusterCaps {
     int get(int i, int smem) const { return smem <= kClusterPairSmem ? two[i] : one[i]; }
 };
 // log2 of the widest cluster worth having for `heads` (kv heads x episodes) streams of up to `pages` pages.  Sixteen CTAs read a
-// stream fastest, but clusters of eight start and merge faster.  Measured (one token, 24 groups, sixteens against eights, us):
-//   8 kv heads, D 128, 640 keys (a page a warp) 5.87 against 4.97, with masses 7.17 against 5.97; 1280 keys (two pages) 6.20
-//     against 6.31, with masses 7.46 against 7.39; 2560 keys 6.66 against 7.10, with masses 8.09 against 8.33
-//   8 kv heads, D 64, the same sizes: 5.16 / 4.44, 6.42 / 5.62; 5.32 / 5.34, 6.57 / 6.42; 5.76 / 5.99, 7.03 / 7.27
-//   6 kv heads, D 128, with masses: 640 keys 6.44 / 6.20, 1280 keys 6.67 / 7.40, 2560 keys 7.12 / 8.87
-//   2 kv heads, D 128: 640 keys 4.62 / 4.52, 960 keys 4.70 / 4.65
-// So a page a warp is where eights are the better ones, most of all at eight streams, whose sixteens leave an SM no room; the two pages
-// that the rule grants calls with masses are about even at eight streams and lose at five and six.
-inline int widest_cluster_log(int heads, int pages, bool masses) { return heads > 4 && pages <= 8 * 12 * (masses ? 2 : 1) ? 3 : 4; }
+// stream fastest, but from eight streams on they leave the next launch room for six of its eight clusters only, and clusters of eight
+// merge faster.  Measured (one token, 24 groups, sixteens against eights, us; without masses, with masses):
+//   8 kv heads, D 128, 640 keys (a page a warp) 5.05 / 4.59, 5.81 / 5.43; 1280 keys (two pages) 5.33 / 6.14, 6.19 / 6.81; 2560 keys
+//     5.88 / 6.92, 6.85 / 7.83;  D 64, the same sizes: 4.37 / 3.93, 5.06 / 4.69; 4.51 / 4.95, 5.30 / 5.66; 4.81 / 5.60, 5.73 / 6.53
+//   6 kv heads, D 128, 640 keys 4.70 / 5.01, 5.51 / 5.51; 2560 keys 5.77 / 7.27, 6.75 / 8.10;  5 kv heads 4.61 / 4.78, 5.39 / 5.53;
+//     5.51 / 7.19, 6.48 / 8.02
+// two_pages: up to two pages a warp are eights', too.  For contiguous keys with masses (none of whose pages is fetched before the kernel
+// before has ended), where the two are about even: 8 kv heads, D 128, 640 keys 6.43 / 5.92, 1280 keys 6.98 / 7.67, 2560 keys 8.86 / 8.34
+// (20 layers of 2500 keys in segments of 40..120: 10.2 / 9.0); D 64 5.79 / 5.27, 6.16 / 6.36, 6.73 / 7.21.
+inline int widest_cluster_log(int heads, int pages, bool two_pages) { return heads >= 8 && pages <= 8 * 12 * (two_pages ? 2 : 1) ? 3 : 4; }
 // Opt the kernel for pool pages, and the one for contiguous keys, in on the current device and ask for its capacities there.
 cudaError_t prepare_decode_cluster(int head_dim, ClusterCaps *caps);
 cudaError_t prepare_decode_static(int head_dim, ClusterCaps *caps);
