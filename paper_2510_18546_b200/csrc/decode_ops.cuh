@@ -38,6 +38,13 @@ __device__ __forceinline__ uint64_t policy_evict_first()
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
     return pol;
 }
+// Where the 16-byte chunk ch of row `row` of a page lies: two groups of 8 rows, a group being one swizzled 8 x 128-byte block per
+// 64 channels (the layout of the boxes that fetch a page).
+template <int D>
+__device__ __forceinline__ uint32_t page_chunk(uint32_t base, int row, int ch)
+{
+    return base + static_cast<uint32_t>((row >> 3) * (D * 16) + (ch >> 3) * 1024 + (row & 7) * 128 + (((ch & 7) ^ (row & 7)) << 4));
+}
 __device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t (&r)[4])
 {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"

@@ -43,6 +43,7 @@ struct Cfg {
     static constexpr int kHalves    = D / 64;             // 64-channel (128-byte) column blocks
     static constexpr int kHalfBytes = 128 * 128;          // 128 rows x 128 B
     static constexpr int kTileBytes = kHalves * kHalfBytes;
+    static constexpr int kGroupBytes = kHalves * 1024;     // K: eight rows, one 8 x 128-byte block per 64 channels
     static constexpr int kStages    = 4;
     static constexpr int kBarOff    = (kQTiles + kStages) * kTileBytes;
     // operands of the MMA that hides page padding, 16 bytes per row: 1 for 8 queries, 0 or -inf for every key of a stage
@@ -137,17 +138,30 @@ __global__ void __launch_bounds__(kThreads, 1) mass_kernel(const __grid_constant
                     tma_load_3d(q_addr(i) + hf * C::kHalfBytes, &p.tm_q, hf * 64, it.kvh * rep,
                                 ep.q_off + it.t0 + i * tile_tokens, bar_q_full);
         }
+        // page words (id; slot << 8 | valid keys) of 32 pages at a time, one per lane, fetched four tiles ahead
+        constexpr int kBatch = 32 / kPagesPerTile;
+        auto words = [&](int t, int &id, int &meta) {
+            const int e = (j_beg + t) * kPagesPerTile + lane;
+            id = kZeroPage;
+            meta = kPageTokens;
+            if (e < ep.n_ctiles * kPagesPerTile) {
+                id = __ldg(p.stream_page + ep.stream_off + e);
+                meta = __ldg(p.stream_meta + ep.stream_off + e);
+            }
+        };
+        int id_cur = 0, meta_cur = 0, id_next, meta_next;
+        words(0, id_next, meta_next);
         int jj = 0;
         for (; jj < n_tiles && ok; ++jj) {
             const int j = j_beg + jj, st = jj % C::kStages;
             const bool cached = j < ep.n_ctiles;
-            // lane = (64-channel half, page): every box of a tile leaves in one instruction
-            const int hf = lane / kPagesPerTile;
-            int row = 0, valid = 0;
-            if (cached && hf < C::kHalves) {
-                row = (p.stream_page[ep.stream_off + j * kPagesPerTile + lane % kPagesPerTile] * p.Hkv + it.kvh) * kPageTokens;
-                valid = __ldg(p.stream_meta + ep.stream_off + j * kPagesPerTile + lane % kPagesPerTile) & 0xff;
+            if (jj % kBatch == 0) {
+                id_cur = id_next;
+                meta_cur = meta_next;
+                words(jj + kBatch, id_next, meta_next);
             }
+            const int at = jj % kBatch * kPagesPerTile + lane % kPagesPerTile;
+            const int row8 = (__shfl_sync(kFull, id_cur, at) * p.Hkv + it.kvh) * 2, valid = __shfl_sync(kFull, meta_cur, at) & 0xff;
             if (jj >= C::kStages) {
                 ok = mbar_wait(bar_k_empty(st), static_cast<uint32_t>((jj / C::kStages - 1) & 1), abort_flag, p.status);
                 if (!ok) break;
@@ -165,12 +179,11 @@ __global__ void __launch_bounds__(kThreads, 1) mass_kernel(const __grid_constant
             if (lane == 0) mbar_expect_tx(bar_k_full(st), static_cast<uint32_t>(C::kTileBytes));
             __syncwarp();
             if (cached) {
-                if (hf < C::kHalves)
-                    tma_load_2d(stage_addr(st) + hf * C::kHalfBytes + (lane % kPagesPerTile) * (kPageTokens * 128), &p.tm_kpool,
-                                hf * 64, row, bar_k_full(st));
-            } else if (lane < C::kHalves) {
-                tma_load_3d(stage_addr(st) + lane * C::kHalfBytes, &p.tm_knew, lane * 64, it.kvh,
-                            ep.new_off + (j - ep.n_ctiles) * kTileKeys, bar_k_full(st));
+                if (lane < kPagesPerTile)
+                    tma_load_4d(stage_addr(st) + static_cast<uint32_t>(lane * 2 * C::kGroupBytes), &p.tm_kpool, 0, 0, 0, row8, bar_k_full(st));
+            } else if (lane < kTileKeys / 8) {
+                tma_load_4d(stage_addr(st) + static_cast<uint32_t>(lane * C::kGroupBytes), &p.tm_knew, 0,
+                            ep.new_off + (j - ep.n_ctiles) * kTileKeys + lane * 8, 0, it.kvh, bar_k_full(st));
             }
         }
         // error path only: let the copies already in flight land before the CTA retires
@@ -183,7 +196,7 @@ __global__ void __launch_bounds__(kThreads, 1) mass_kernel(const __grid_constant
         // ================= MMA issuer =================
         constexpr uint32_t idesc_qk = make_idesc(kTileKeys, false);
         constexpr uint32_t kTileUnits = C::kTileBytes >> 4;
-        const uint64_t dq0 = smem_desc(q_addr(0), 16), dk0 = smem_desc(stage_addr(0), 16);
+        const uint64_t dq0 = smem_desc(q_addr(0), 16), dk0 = smem_desc(stage_addr(0), 16, C::kGroupBytes);
         const uint32_t dq_lo = static_cast<uint32_t>(dq0), dq_hi = static_cast<uint32_t>(dq0 >> 32);
         const uint32_t dk_lo = static_cast<uint32_t>(dk0), dk_hi = static_cast<uint32_t>(dk0 >> 32);
         const uint64_t d_ones = smem_desc_plain(sbase + C::kOnesOff, 0u), d_hide = smem_desc_plain(sbase + C::kHideOff, 128u);
@@ -202,9 +215,11 @@ __global__ void __launch_bounds__(kThreads, 1) mass_kernel(const __grid_constant
                             static_cast<uint32_t>(d_hide >> 32), idesc_qk, 0u);
 #pragma unroll
                 for (int kk = 0; kk < D / 16; ++kk) {
-                    const uint32_t off = static_cast<uint32_t>((kk >> 2) * (C::kHalfBytes >> 4) + (kk & 3) * 2);   // 32 bytes per 16 channels
-                    mma_ss2(tmem_base + static_cast<uint32_t>((2 * buf + i) * 128), dq_lo + static_cast<uint32_t>(i) * kTileUnits + off, dq_hi,
-                            dk_lo + static_cast<uint32_t>(st) * kTileUnits + off, dk_hi, idesc_qk, kk > 0 || hide ? 1u : 0u);
+                    const uint32_t in_row = static_cast<uint32_t>((kk & 3) * 2);                       // 32 bytes per 16 channels
+                    mma_ss2(tmem_base + static_cast<uint32_t>((2 * buf + i) * 128),
+                            dq_lo + static_cast<uint32_t>(i) * kTileUnits + static_cast<uint32_t>((kk >> 2) * (C::kHalfBytes >> 4)) + in_row, dq_hi,
+                            dk_lo + static_cast<uint32_t>(st) * kTileUnits + static_cast<uint32_t>((kk >> 2) * (1024 >> 4)) + in_row, dk_hi,
+                            idesc_qk, kk > 0 || hide ? 1u : 0u);
                 }
                 tc_commit(bar_s_full(i, buf));
             }

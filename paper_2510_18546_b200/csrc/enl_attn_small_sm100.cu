@@ -58,7 +58,6 @@ __global__ void __launch_bounds__(kThreads, 1) small_kernel(const __grid_constan
 {
     using C = Cfg<D, kRowGroups>;
     constexpr int kKeyRanges = C::kKeyRanges, kRows = C::kRows;
-    constexpr int kHalves = D / 64;                       // TMA boxes (64 channels) per page
     constexpr int kSteps  = D / 16;                       // k16 steps of Q K^T
     constexpr int kNB     = D / 8;                        // 8-channel blocks of O
     extern __shared__ uint8_t smem_raw[];
@@ -125,14 +124,15 @@ __global__ void __launch_bounds__(kThreads, 1) small_kernel(const __grid_constan
     auto issue = [&](int i, int pg) {
         const uint32_t full = bar0 + 8u * i, dst = sbase + static_cast<uint32_t>(i * 2 * C::kStageBytes);
         mbar_expect_tx(full, 2u * C::kStageBytes);
+        // (no evict-first hint: the row blocks of a kv head share its pages)
+        if (pg >= 0) {
+            tma_load_4d(dst, &p.tm_kpool, 0, 0, 0, (pg * p.Hkv + kvh) * 2, full);
+            tma_load_4d(dst + C::kStageBytes, &p.tm_vpool, 0, 0, 0, (pg * p.Hkv + kvh) * 2, full);
+        } else {
 #pragma unroll
-        for (int x = 0; x < 2 * kHalves; ++x) {
-            const bool v = x >= kHalves;
-            const int ch = (x % kHalves) * 64;
-            const uint32_t at = dst + static_cast<uint32_t>(x * kPageTokens * 128);
-            // (no evict-first hint: the row blocks of a kv head share its pages)
-            if (pg >= 0) tma_load_2d(at, v ? &p.tm_vpool : &p.tm_kpool, ch, (pg * p.Hkv + kvh) * kPageTokens, full);
-            else tma_load_3d(at, v ? &p.tm_vnew : &p.tm_knew, ch, kvh, ep.new_off + (-1 - pg), full);
+            for (int x = 0; x < 4; ++x)                                       // eight rows of K or V
+                tma_load_4d(dst + static_cast<uint32_t>(x * (C::kStageBytes / 2)), x < 2 ? &p.tm_knew : &p.tm_vnew, 0,
+                            ep.new_off + (-1 - pg) + (x & 1) * 8, 0, kvh, full);
         }
     };
     // page i is fetched by lane 0 of warp i % kWarps: the cached ones while the previous kernel still runs
@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(kThreads, 1) small_kernel(const __grid_constan
             for (int nb = 0; nb < 2; ++nb) {
                 const int row = nb * 8 + (lane & 7), ch = kq * 4 + (lane >> 3);
                 uint32_t b[4];
-                ldsm_x4(base + (ch >> 3) * (kPageTokens * 128) + row * 128 + (((ch & 7) ^ (row & 7)) << 4), b);
+                ldsm_x4(page_chunk<D>(base, row, ch), b);
                 mma_bf16(c[nb], qa[2 * kq], b[0], b[1]);
                 mma_bf16(c2[nb], qa[2 * kq + 1], b[2], b[3]);
             }
@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(kThreads, 1) small_kernel(const __grid_constan
         for (int nq = 0; nq < kNB / 2; ++nq) {                                // two 8-channel blocks per ldmatrix
             const int ch = nq * 2 + (lane >> 4);
             uint32_t b[4];
-            ldsm_x4_trans(vbase + (ch >> 3) * (kPageTokens * 128) + row * 128 + (((ch & 7) ^ (row & 7)) << 4), b);
+            ldsm_x4_trans(page_chunk<D>(vbase, row, ch), b);
             mma_bf16(o[2 * nq], pa, b[0], b[1]);
             mma_bf16(o[2 * nq + 1], pa, b[2], b[3]);
         }

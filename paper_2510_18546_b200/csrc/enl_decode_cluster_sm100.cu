@@ -125,7 +125,6 @@ __global__ void __launch_bounds__(kThreads, 2)
     decode_cluster_kernel(const __grid_constant__ std::conditional_t<kStatic, StaticDecodeParams, ClusterDecodeParams> prm)
 {
     using C = Cfg<D>;
-    constexpr int kHalves = D / 64;                       // TMA boxes (64 channels) per page
     constexpr int kMB     = D / 16;                       // 16-channel blocks of O^T
     const ClusterDecodeParams &p = common(prm);
     extern __shared__ uint8_t smem_raw[];
@@ -208,15 +207,12 @@ __global__ void __launch_bounds__(kThreads, 2)
         mbar_expect_tx(full, static_cast<uint32_t>(C::kStageBytes));
         if (!kStatic && page >= 0) {
             const CUtensorMap *tm = is_v ? &p.tm_vpool : &p.tm_kpool;
-            const int row = (page * p.Hkv + kvh) * kPageTokens;
-#pragma unroll
-            for (int hf = 0; hf < kHalves; ++hf) tma_load_2d(dst + hf * (kPageTokens * 128), tm, hf * 64, row, full, pol);
+            tma_load_4d(dst, tm, 0, 0, 0, (page * p.Hkv + kvh) * 2, full, pol);
         } else {
             const CUtensorMap *tm = is_v ? &p.tm_vnew : &p.tm_knew;
             const int krow = ep.new_off + (-1 - page);                       // rows past the tensor's end read as zero
-#pragma unroll
-            for (int hf = 0; hf < kHalves; ++hf)
-                tma_load_3d(dst + hf * (kPageTokens * 128), tm, hf * 64, kvh, krow, full, pol);
+            tma_load_4d(dst, tm, 0, krow, 0, kvh, full, pol);
+            tma_load_4d(dst + C::kStageBytes / 2, tm, 0, krow + 8, 0, kvh, full, pol);
         }
     };
     // While the previous kernel of the stream still runs: the pool is written by launches of this library only, and none has
@@ -272,10 +268,11 @@ __global__ void __launch_bounds__(kThreads, 2)
     }
     // (a warp takes a page: a box costs the warp that asks for it some 50 cycles)
     for (int i = warp; i < min(n_cta, kPrefetchPages); i += kWarps) {
-        const int pg = pg_list[i].x, x = (lane % kHalves) * 64;
-        if (lane < 2 * kHalves) {
-            if (pg < 0) tma_prefetch_3d(lane >= kHalves ? &p.tm_vnew : &p.tm_knew, x, kvh, ep.new_off + (-1 - pg));
-            else if (i >= kWarps) tma_prefetch_2d(lane >= kHalves ? &p.tm_vpool : &p.tm_kpool, x, (pg * p.Hkv + kvh) * kPageTokens);
+        const int pg = pg_list[i].x;
+        if (pg < 0) {
+            if (lane < 4) tma_prefetch_4d((lane & 1) ? &p.tm_vnew : &p.tm_knew, 0, ep.new_off + (-1 - pg) + (lane >> 1) * 8, 0, kvh);
+        } else if (i >= kWarps && lane < 2) {
+            tma_prefetch_4d((lane & 1) ? &p.tm_vpool : &p.tm_kpool, 0, 0, 0, (pg * p.Hkv + kvh) * 2);
         }
     }
     const uint8_t *q_rows = static_cast<const uint8_t *>(p.q) + (static_cast<long long>(ep.q_off) * p.Hq + kvh * rep) * D * 2;
@@ -348,7 +345,7 @@ __global__ void __launch_bounds__(kThreads, 2)
             for (int ks = 0; ks < D / 16; ++ks) {
                 const int ch = 2 * ks + (lane >> 4);
                 uint32_t a[4];
-                ldsm_x4(base + (ch >> 3) * (kPageTokens * 128) + row * 128 + (((ch & 7) ^ (row & 7)) << 4), a);
+                ldsm_x4(page_chunk<D>(base, row, ch), a);
                 const uint2 qv = qfrag[ks * 32 + lane];
                 mma_bf16((ks & 1) ? c2 : c, a, qv.x, qv.y);
             }
@@ -418,7 +415,7 @@ __global__ void __launch_bounds__(kThreads, 2)
         for (int mb = 0; mb < kMB; ++mb) {
             const int ch = 2 * mb + ((lane >> 3) & 1);
             uint32_t a[4];
-            ldsm_x4_trans(base + (ch >> 3) * (kPageTokens * 128) + row * 128 + (((ch & 7) ^ (row & 7)) << 4), a);
+            ldsm_x4_trans(page_chunk<D>(base, row, ch), a);
 #pragma unroll
             for (int t = 0; t < kTerms; ++t) mma_bf16(o[mb], a, b0[t], b1[t]);
         }

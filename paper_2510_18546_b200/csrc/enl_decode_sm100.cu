@@ -74,7 +74,6 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(const __grid_consta
 {
     using C = DecCfg<D>;
     constexpr int kChunks = D / 8;                        // 16-byte chunks per row
-    constexpr int kHalves = D / 64;                       // TMA boxes (64 channels) per page
     constexpr int kNB     = D / 8;                        // n-blocks of the PV product
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
@@ -172,11 +171,9 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(const __grid_consta
     // the stream below then starts on hits.
     {
         const int n_pf = min(n_cta, kPrefetchPages);
-        for (int i = threadIdx.x; i < n_pf * 2 * kHalves; i += kThreads) {
-            const int pg = pg_list[i / (2 * kHalves)].x;
-            const int r = i % (2 * kHalves);
-            if (pg >= 0)
-                tma_prefetch_2d(r >= kHalves ? &p.tm_vpool : &p.tm_kpool, (r % kHalves) * 64, (pg * p.Hkv + it.kvh) * kPageTokens);
+        for (int i = threadIdx.x; i < n_pf * 2; i += kThreads) {
+            const int pg = pg_list[i / 2].x;
+            if (pg >= 0) tma_prefetch_4d((i & 1) ? &p.tm_vpool : &p.tm_kpool, 0, 0, 0, (pg * p.Hkv + it.kvh) * 2);
         }
     }
 
@@ -200,15 +197,12 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(const __grid_consta
         mbar_expect_tx(full, static_cast<uint32_t>(C::kStageBytes));
         if (page >= 0) {
             const CUtensorMap *tm = is_v ? &p.tm_vpool : &p.tm_kpool;
-            const int row = (page * p.Hkv + it.kvh) * kPageTokens;
-#pragma unroll
-            for (int hf = 0; hf < kHalves; ++hf) tma_load_2d(dst + hf * (kPageTokens * 128), tm, hf * 64, row, full, pol);
+            tma_load_4d(dst, tm, 0, 0, 0, (page * p.Hkv + it.kvh) * 2, full, pol);
         } else {
             const CUtensorMap *tm = is_v ? &p.tm_vnew : &p.tm_knew;
             const int krow = ep.new_off + (-1 - page) * kPageTokens;         // rows past the tensor's end read as zero
-#pragma unroll
-            for (int hf = 0; hf < kHalves; ++hf)
-                tma_load_3d(dst + hf * (kPageTokens * 128), tm, hf * 64, it.kvh, krow, full, pol);
+            tma_load_4d(dst, tm, 0, krow, 0, it.kvh, full, pol);
+            tma_load_4d(dst + C::kStageBytes / 2, tm, 0, krow + 8, 0, it.kvh, full, pol);
         }
     };
     // the next page of the CTA that nobody has taken yet (CTA-relative index; >= n_cta: none left)
@@ -285,9 +279,8 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(const __grid_consta
 #pragma unroll
             for (int kq = 0; kq < kChunks / 4; ++kq) {                       // four 8-channel chunks = two k16 steps
                 const int ch = kq * 4 + (lane >> 3);
-                const uint32_t addr = base + (ch >> 3) * (kPageTokens * 128) + row * 128 + (((ch & 7) ^ (row & 7)) << 4);
                 uint32_t b[4];
-                ldsm_x4(addr, b);
+                ldsm_x4(page_chunk<D>(base, row, ch), b);
                 mma_bf16(c[nb][0], c[nb][1], z0, z1, qa[2 * kq][0], qa[2 * kq][1], b[0], b[1]);
                 mma_bf16(c[nb][0], c[nb][1], z0, z1, qa[2 * kq + 1][0], qa[2 * kq + 1][1], b[2], b[3]);
             }
@@ -333,9 +326,8 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(const __grid_consta
 #pragma unroll
         for (int nq = 0; nq < kNB / 2; ++nq) {                               // two 8-channel n-blocks per ldmatrix
             const int ch = nq * 2 + (lane >> 4);
-            const uint32_t addr = base + (ch >> 3) * (kPageTokens * 128) + row * 128 + (((ch & 7) ^ (row & 7)) << 4);
             uint32_t b[4];
-            ldsm_x4_trans(addr, b);
+            ldsm_x4_trans(page_chunk<D>(base, row, ch), b);
             mma_bf16(o[2 * nq][0], o[2 * nq][1], z0, z1, a0, a2, b[0], b[1]);
             mma_bf16(o[2 * nq + 1][0], o[2 * nq + 1][1], z0, z1, a0, a2, b[2], b[3]);
         }

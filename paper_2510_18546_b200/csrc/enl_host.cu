@@ -110,14 +110,22 @@ struct MapCache {
     }
 };
 
+// a caller's [n][Hkv][D] keys or values, fetched by eight rows of a head
+struct KeyMapShape {
+    cuuint64_t dims[4], strides[3];
+    cuuint32_t box[4];
+    KeyMapShape(int D, int Hkv, int n)
+        : dims{64, static_cast<cuuint64_t>(n), static_cast<cuuint64_t>(D / 64), static_cast<cuuint64_t>(Hkv)},
+          strides{static_cast<cuuint64_t>(D) * 2 * Hkv, 128, static_cast<cuuint64_t>(D) * 2},
+          box{64, 8, static_cast<cuuint32_t>(D / 64), 1} {}
+};
+
 }  // namespace
 
 bool enl::encode_key_map(CUtensorMap *tm, const void *base, int D, int Hkv, int n)
 {
-    const cuuint64_t dims[3] = {static_cast<cuuint64_t>(D), static_cast<cuuint64_t>(Hkv), static_cast<cuuint64_t>(n)};
-    const cuuint64_t strides[2] = {static_cast<cuuint64_t>(D) * 2, static_cast<cuuint64_t>(D) * 2 * Hkv};
-    const cuuint32_t box[3] = {64, 1, kPageTokens};
-    return encode_map(tm, base, 3, dims, strides, box);
+    const KeyMapShape k(D, Hkv, n);
+    return encode_map(tm, base, 4, k.dims, k.strides, k.box);
 }
 
 struct enl_cache {
@@ -131,8 +139,7 @@ struct enl_cache {
     uint8_t *kpool = nullptr, *vpool = nullptr;
     std::vector<int32_t> free_pages;        // stack of free page ids (page 0 is never in it)
     std::vector<Group> groups;
-    std::vector<CUtensorMap> tm_k, tm_v;    // per layer, boxes of 64 channels of a page of a head
-    std::vector<CUtensorMap> tm_k4, tm_v4;  // and of a page of a head, for attn_kernel
+    std::vector<CUtensorMap> tm_k, tm_v;    // per layer
     uint64_t epoch = 0;                     // bumped by every store
 
     // gather plan: host image (pinned when there is a GPU), device copy, capacities
@@ -337,21 +344,13 @@ extern "C" int enl_cache_create(const enl_cache_desc_t *desc, enl_cache_t **out)
 
     c->tm_k.resize(d.n_layers);
     c->tm_v.resize(d.n_layers);
-    c->tm_k4.resize(d.n_layers);
-    c->tm_v4.resize(d.n_layers);
-    const cuuint64_t dims[2] = {static_cast<cuuint64_t>(d.head_dim),
-                                static_cast<cuuint64_t>(c->n_pages) * d.n_kv_heads * kPageTokens};
-    const cuuint64_t strides[1] = {static_cast<cuuint64_t>(d.head_dim) * 2};
-    const cuuint32_t box[2] = {64, kPageTokens};
-    const cuuint64_t row = strides[0];
-    const cuuint64_t dims4[4] = {64, 8, static_cast<cuuint64_t>(d.head_dim / 64), dims[1] / 8};
-    const cuuint64_t strides4[3] = {row, 128, row * 8};
-    const cuuint32_t box4[4] = {64, 8, static_cast<cuuint32_t>(d.head_dim / 64), 2};
+    const cuuint64_t row = static_cast<cuuint64_t>(d.head_dim) * 2;
+    const cuuint64_t dims[4] = {64, 8, static_cast<cuuint64_t>(d.head_dim / 64), static_cast<cuuint64_t>(c->n_pages) * d.n_kv_heads * (kPageTokens / 8)};
+    const cuuint64_t strides[3] = {row, 128, row * 8};
+    const cuuint32_t box[4] = {64, 8, static_cast<cuuint32_t>(d.head_dim / 64), kPageTokens / 8};
     for (int l = 0; l < d.n_layers; ++l) {
-        if (!encode_map(&c->tm_k[l], c->kpool + c->layer_bytes * l, 2, dims, strides, box) ||
-            !encode_map(&c->tm_v[l], c->vpool + c->layer_bytes * l, 2, dims, strides, box) ||
-            !encode_map(&c->tm_k4[l], c->kpool + c->layer_bytes * l, 4, dims4, strides4, box4) ||
-            !encode_map(&c->tm_v4[l], c->vpool + c->layer_bytes * l, 4, dims4, strides4, box4)) {
+        if (!encode_map(&c->tm_k[l], c->kpool + c->layer_bytes * l, 4, dims, strides, box) ||
+            !encode_map(&c->tm_v[l], c->vpool + c->layer_bytes * l, 4, dims, strides, box)) {
             destroy(c);
             return ENL_E_CUDA;
         }
@@ -993,12 +992,8 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
     if (c->plan_small_blocks || (c->plan_decode && c->plan_cluster)) {
         SmallParams dp;
         std::memset(&dp, 0, sizeof dp);
-        const cuuint64_t nd[3] = {static_cast<cuuint64_t>(d.head_dim), static_cast<cuuint64_t>(d.n_kv_heads),
-                                  static_cast<cuuint64_t>(a->n_new)};
-        const cuuint64_t ns[2] = {static_cast<cuuint64_t>(d.head_dim) * 2,
-                                  static_cast<cuuint64_t>(d.head_dim) * 2 * d.n_kv_heads};
-        const cuuint32_t nb[3] = {64, 1, kPageTokens};
-        if (!c->maps.get(&dp.tm_knew, a->k_new, nd, ns, nb) || !c->maps.get(&dp.tm_vnew, a->v_new, nd, ns, nb))
+        const KeyMapShape km(d.head_dim, d.n_kv_heads, a->n_new);
+        if (!c->maps.get(&dp.tm_knew, a->k_new, km.dims, km.strides, km.box, 4) || !c->maps.get(&dp.tm_vnew, a->v_new, km.dims, km.strides, km.box, 4))
             return ENL_E_CUDA;
         dp.tm_kpool = c->tm_k[a->layer];
         dp.tm_vpool = c->tm_v[a->layer];
@@ -1030,12 +1025,8 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
     if (c->plan_decode) {
         DecodeParams dp;
         std::memset(&dp, 0, sizeof dp);
-        const cuuint64_t nd[3] = {static_cast<cuuint64_t>(d.head_dim), static_cast<cuuint64_t>(d.n_kv_heads),
-                                  static_cast<cuuint64_t>(a->n_new)};
-        const cuuint64_t ns[2] = {static_cast<cuuint64_t>(d.head_dim) * 2,
-                                  static_cast<cuuint64_t>(d.head_dim) * 2 * d.n_kv_heads};
-        const cuuint32_t nb[3] = {64, 1, kPageTokens};
-        if (!c->maps.get(&dp.tm_knew, a->k_new, nd, ns, nb) || !c->maps.get(&dp.tm_vnew, a->v_new, nd, ns, nb))
+        const KeyMapShape km(d.head_dim, d.n_kv_heads, a->n_new);
+        if (!c->maps.get(&dp.tm_knew, a->k_new, km.dims, km.strides, km.box, 4) || !c->maps.get(&dp.tm_vnew, a->v_new, km.dims, km.strides, km.box, 4))
             return ENL_E_CUDA;
         dp.tm_kpool = c->tm_k[a->layer];
         dp.tm_vpool = c->tm_v[a->layer];
@@ -1078,22 +1069,13 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         const cuuint64_t qs[2] = {static_cast<cuuint64_t>(d.head_dim) * 2,
                                   static_cast<cuuint64_t>(d.head_dim) * 2 * d.n_q_heads};
         const cuuint32_t qb[3] = {64, static_cast<cuuint32_t>(c->rep), static_cast<cuuint32_t>(kTileRows / c->rep)};
-        const cuuint64_t n_new = static_cast<cuuint64_t>(a->n_new), head = static_cast<cuuint64_t>(d.head_dim) * 2, token = head * d.n_kv_heads;
-        const cuuint64_t n_heads = static_cast<cuuint64_t>(d.n_kv_heads), n_halves = static_cast<cuuint64_t>(d.head_dim / 64);
-        bool okm = c->maps.get(&p.tm_q, a->q, qd, qs, qb);
-        if (mass_only) {
-            const cuuint64_t nd[3] = {static_cast<cuuint64_t>(d.head_dim), n_heads, n_new}, ns[2] = {head, token};
-            const cuuint32_t nb[3] = {64, 1, kTileKeys};
-            okm = okm && c->maps.get(&p.tm_knew, a->k_new, nd, ns, nb);
-        } else {
-            const cuuint64_t nd[4] = {64, n_new, n_halves, n_heads}, ns[3] = {token, 128, head};
-            const cuuint32_t nb[4] = {64, 8, static_cast<cuuint32_t>(n_halves), 1};
-            okm = okm && c->maps.get(&p.tm_knew, a->k_new, nd, ns, nb, 4) && c->maps.get(&p.tm_vnew, a->v_new, nd, ns, nb, 4);
-        }
-        if (!okm) return ENL_E_CUDA;
+        const KeyMapShape km(d.head_dim, d.n_kv_heads, a->n_new);
+        if (!c->maps.get(&p.tm_q, a->q, qd, qs, qb) || !c->maps.get(&p.tm_knew, a->k_new, km.dims, km.strides, km.box, 4) ||
+            !c->maps.get(&p.tm_vnew, a->v_new, km.dims, km.strides, km.box, 4))
+            return ENL_E_CUDA;
     }
-    p.tm_kpool = mass_only ? c->tm_k[a->layer] : c->tm_k4[a->layer];
-    p.tm_vpool = c->tm_v4[a->layer];
+    p.tm_kpool = c->tm_k[a->layer];
+    p.tm_vpool = c->tm_v[a->layer];
     p.items = reinterpret_cast<const Item *>(c->plan_dev + c->off_items);
     p.eps = reinterpret_cast<const EpInfo *>(c->plan_dev + c->off_eps);
     p.stream_page = reinterpret_cast<const int32_t *>(c->plan_dev + c->off_stream);

@@ -33,14 +33,19 @@ struct Item {
     int32_t split;          // KV split index in [0, n_splits)
 };
 
+// How keys and values are fetched: by boxes that leave one swizzled block of 8 rows x 128 bytes per 64 channels, and then the next 8 rows.
+//   pool (a layer), dims {64 channels, 8 rows, D/64 blocks, groups of 8 rows}, box {64, 8, D/64, 2}: a page of a kv head, 16 D contiguous
+//     values, in one box
+//   a caller's [n][Hkv][D], dims {64 channels, n rows, D/64 blocks, Hkv heads}, box {64, 8, D/64, 1}: eight rows of a head
+// A box costs the warp that asks for it some 50 cycles, so a box of half as much (64 channels of a page, as a two-dimensional map gives
+// them) had every producer take twice as long.
+
 // Kernel parameters (passed by value as a __grid_constant__).
 struct AttnParams {
     CUtensorMap tm_q;       // [n_q][Hq][D]      box {64, rep, 128/rep}
-    // Boxes that leave a block of 8 rows x 128 bytes per 64 channels and then the next 8 rows: eight rows of a head of new tokens
-    // (channel, token, 64-channel block, head), both groups of a page of a head (channel, row of 8, 64-channel block, group of 8 rows)
-    CUtensorMap tm_knew;    // [n_new][Hkv][D]   box {64, 8, D/64, 1}
+    CUtensorMap tm_knew;    // [n_new][Hkv][D]: eight rows of a head (see above)
     CUtensorMap tm_vnew;
-    CUtensorMap tm_kpool;   // [pages*Hkv*2][8][D] box {64, 8, D/64, 2}   (one layer)
+    CUtensorMap tm_kpool;   // one layer: a page of a head
     CUtensorMap tm_vpool;
     const Item   *items;
     const EpInfo *eps;
@@ -69,8 +74,8 @@ struct AttnParams {
 // Masses without outputs (see enl_attn_mass_sm100.cu)
 struct MassParams {
     CUtensorMap tm_q;       // [n_q][Hq][D]      box {64, rep, 128/rep}
-    CUtensorMap tm_knew;    // [n_new][Hkv][D]   box {64, 1, 128}
-    CUtensorMap tm_kpool;   // [pages*Hkv*16][D] box {64, 16}   (one layer)
+    CUtensorMap tm_knew;    // as in AttnParams
+    CUtensorMap tm_kpool;
     const Item   *items;
     const EpInfo *eps;
     const int32_t *stream_page;
@@ -95,9 +100,9 @@ constexpr int kDecodeMaxPages = 256;
 constexpr int kMaxSplits      = 64;
 
 struct DecodeParams {
-    CUtensorMap tm_knew;    // [n_new][Hkv][D]   box {64, 1, 16}
+    CUtensorMap tm_knew;    // as in AttnParams
     CUtensorMap tm_vnew;
-    CUtensorMap tm_kpool;   // [pages*Hkv*16][D] box {64, 16}   (one layer)
+    CUtensorMap tm_kpool;
     CUtensorMap tm_vpool;
     EpInfo ep0;             // episode 0 (used when the call has one episode; grid = splits x kv heads x episodes)
     const EpInfo *eps;
@@ -121,9 +126,9 @@ struct DecodeParams {
 
 // The same for calls whose splits fit a thread-block cluster (see enl_decode_cluster_sm100.cu): no partial results in memory.
 struct ClusterDecodeParams {
-    CUtensorMap tm_knew;    // [n_new][Hkv][D]   box {64, 1, 16}
+    CUtensorMap tm_knew;    // as in AttnParams
     CUtensorMap tm_vnew;
-    CUtensorMap tm_kpool;   // [pages*Hkv*16][D] box {64, 16}   (one layer)
+    CUtensorMap tm_kpool;
     CUtensorMap tm_vpool;
     EpInfo ep0;             // episode 0 (used when the call has one episode; grid = cluster x kv heads x episodes)
     const EpInfo *eps;
@@ -227,7 +232,7 @@ struct FinishParams {
 constexpr int kFinishSplits = 8;
 cudaError_t launch_mass_finish(const FinishParams &p, cudaStream_t st);
 
-// Tensor map of a caller's [n][Hkv][D] bf16 keys or values with boxes of one head's 16 rows x 64 channels (in enl_host.cu)
+// Tensor map of a caller's [n][Hkv][D] bf16 keys or values with boxes of eight rows of a head (in enl_host.cu)
 bool encode_key_map(CUtensorMap *tm, const void *base, int D, int Hkv, int n);
 
 // launchers (defined in the .cu files of the kernels)
