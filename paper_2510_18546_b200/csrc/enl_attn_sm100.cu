@@ -18,7 +18,7 @@
 // Roles (12 warps): warps 0-3 are the softmax warpgroup of Q tile 0, warps 4-7 that of Q tile 1: one
 // thread per query row holds the row's 64 scores of a step in registers, so the row maximum, the
 // exponentials and the four page sums need no exchange between threads.  Warps 8 and 10 fetch K and V, warps 9 and 11 issue the
-// MMAs of tile 0 and tile 1 (9 owns the TMEM).
+// MMAs of tile 0 and tile 1 (9 owns the TMEM).  A softmax warpgroup and its issuer are a walker.
 //
 // What bounds it, and why it is split like this (all cycles per 128 keys and pair of Q tiles, 64 groups, 1024 rows; the tensor pipe
 // needs 2176, the special-function unit 2048):
@@ -35,6 +35,11 @@
 // Not kept: exponentials on the FMA pipe, a quarter of them 270 thousand cycles (the warps have issue slots, but a step is one chain);
 // the maximum beside the exponentials, with the reference a step behind: 6700 against 5860 us a pass; tiles of 128 keys with all of the
 // above: the same on long calls, 8 % slower on the planner's, whose ends waste half a tile.
+//
+// Calls with few CTAs run the second form (kHalves): a CTA has one Q tile, its two walkers take the first and the second half of its steps
+// and put outputs and slots together at the end, in TMEM lanes that both read: twice as many CTAs, or half as many splits to merge through
+// memory, and no walker idle where a call has fewer rows than two tiles.  With masses, 2560 keys: 41 rows 16.6 -> 15.4 us, 128 rows
+// 22.6 -> 19.1, 256 rows 28.3 -> 26.2; 512 rows at head_dim 64, which has no pairs of CTAs, 39.0 -> 34.1.
 //
 // TMEM columns: S0 [0,128) S1 [128,256), two buffers of 64 columns each, O0 [256,384) O1 [384,512); P_i (bf16 pairs) overwrites the
 // first 32 columns of the buffer that held its scores once these are in registers.
@@ -85,7 +90,7 @@ struct Cfg {
 };
 
 // ---- the kernel ----------------------------------------------------------------------------
-template <int D>
+template <int D, bool kHalves>
 __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant__ AttnParams p)
 {
     using C = Cfg<D>;
@@ -126,7 +131,9 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
     const EpInfo ep = p.eps[it.ep];
     const int rep = p.rep;
     const int tile_tokens = kTileRows / rep;
-    const int t_hi = min(it.t0 + kQTiles * tile_tokens, ep.n_q);        // exclusive
+    // Calls with few CTAs (kHalves): one Q tile per CTA, and the two walkers (softmax warpgroup + issuer) take half of its steps each
+    // and put their results together at the end.  Else a walker has a Q tile of its own and walks all the steps.
+    const int t_hi = min(it.t0 + (kHalves ? 1 : kQTiles) * tile_tokens, ep.n_q);    // exclusive
     const int n_qt = (t_hi - it.t0 > tile_tokens) ? 2 : 1;
     const int c_max = ep.n_new - ep.n_q + t_hi - 1;                      // last new key any row sees
     const int n_csteps = (ep.n_entries + kStepPages - 1) / kStepPages;  // steps over cached pages
@@ -134,14 +141,21 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
     const int j_beg = static_cast<int>(static_cast<long long>(total_steps) * it.split / p.n_splits);
     const int j_end = static_cast<int>(static_cast<long long>(total_steps) * (it.split + 1) / p.n_splits);
     const int n_steps = j_end - j_beg;
+    const int n_walk = kHalves ? min(2, n_steps) : n_qt;                  // walkers with work
+    // walker i: its steps and the first of them; in the order in which K and V are fetched, its step jj is number place_of(i, jj), and
+    // number v is step step_of(v) of the stream
+    auto count_of = [&](int i) { return kHalves ? (n_steps + 1 - i) >> 1 : n_steps; };
+    auto first_of = [&](int i) { return kHalves && i ? j_beg + ((n_steps + 1) >> 1) : j_beg; };
+    auto place_of = [&](int i, int jj) { return kHalves ? 2 * jj + i : jj; };
+    auto step_of = [&](int v) { return kHalves ? first_of(v & 1) + (v >> 1) : j_beg + v; };
 
     // ---- set-up ----
     if (threadIdx.x == 0) {
         *abort_flag = 0;
         mbar_init(bar_q_full, 1);
         for (int x = 0; x < C::kRing; ++x) {
-            mbar_init(bar_k_full(x), 1); mbar_init(bar_k_empty(x), n_qt);
-            mbar_init(bar_v_full(x), 1); mbar_init(bar_v_empty(x), n_qt);
+            mbar_init(bar_k_full(x), 1); mbar_init(bar_k_empty(x), kHalves ? 1 : n_qt);
+            mbar_init(bar_v_full(x), 1); mbar_init(bar_v_empty(x), kHalves ? 1 : n_qt);
         }
         for (int i = 0; i < kQTiles; ++i) {
             for (int b = 0; b < 2; ++b) {
@@ -174,7 +188,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    const bool pair = p.pair_merge != 0;
+    const bool pair = !kHalves && p.pair_merge != 0;
     if (pair) cluster_sync_all();                // the peer's barriers exist before anything is sent to them
     // everything above touched only shared memory, TMEM and the gather plan; from here on the caller's tensors,
     // the pool and the scratch are read and written, so the previous kernel of the stream must have finished
@@ -185,13 +199,13 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
     if ((warp == kKWarp || warp == kVWarp) && n_steps > 0 && static_cast<int>(blockIdx.x) < p.first_wave) {
         if (warp == kKWarp && lane < n_qt * C::kHalves)
             tma_prefetch_3d(&p.tm_q, (lane % C::kHalves) * 64, it.kvh * rep, ep.q_off + it.t0 + (lane / C::kHalves) * tile_tokens);
-        const int j = j_beg + lane / kStepPages;
-        if (lane < C::kRing * kStepPages && j < min(j_end, n_csteps))
+        const int v = lane / kStepPages, j = step_of(v);
+        if (v < min(C::kRing, n_steps) && j < n_csteps)
             tma_prefetch_4d(warp == kKWarp ? &p.tm_kpool : &p.tm_vpool, 0, 0, 0,
                             (p.stream_page[ep.stream_off + j * kStepPages + lane % kStepPages] * p.Hkv + it.kvh) * 2);
-        const int jn = max(j_beg, n_csteps) + lane / 8;              // new tokens: eight rows a box
-        if (jn < min(j_beg + C::kRing, j_end))
-            tma_prefetch_4d(warp == kKWarp ? &p.tm_knew : &p.tm_vnew, 0, ep.new_off + (jn - n_csteps) * kStepKeys + lane % 8 * 8, 0, it.kvh);
+        const int vn = lane / (kStepKeys / 8), jn = step_of(vn);     // new tokens: eight rows a box
+        if (vn < min(C::kRing, n_steps) && jn >= n_csteps)
+            tma_prefetch_4d(warp == kKWarp ? &p.tm_knew : &p.tm_vnew, 0, ep.new_off + (jn - n_csteps) * kStepKeys + lane % (kStepKeys / 8) * 8, 0, it.kvh);
     }
     pdl_wait();
 
@@ -215,31 +229,31 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                         tma_load_3d(q_addr(i) + hf * C::kHalfBytes, &p.tm_q, hf * 64, it.kvh * rep,
                                     ep.q_off + it.t0 + i * tile_tokens, bar_q_full);
             }
-            // Page words (id; slot << 8 | valid keys) of 32 pages at a time, one per lane, fetched eight steps ahead: a load in
-            // every step kept the ring waiting for the L2.
+            // Page words (id; slot << 8 | valid keys) of 32 pages at a time, one per lane, fetched eight steps ahead (of either walker): a
+            // load in every step kept the ring waiting for the L2.
             constexpr int kBatch = 32 / kStepPages;
-            auto words = [&](int jj, int &id, int &meta) {
-                const int e = (j_beg + jj) * kStepPages + lane;
-                id = kZeroPage;
-                meta = kPageTokens;
+            struct Words { int id, meta; };
+            auto words = [&](int j) {
+                const int e = j * kStepPages + lane;
+                Words w = {kZeroPage, kPageTokens};
                 if (e < n_csteps * kStepPages) {
-                    id = __ldg(p.stream_page + ep.stream_off + e);
-                    meta = __ldg(p.stream_meta + ep.stream_off + e);
+                    w.id = __ldg(p.stream_page + ep.stream_off + e);
+                    w.meta = __ldg(p.stream_meta + ep.stream_off + e);
                 }
+                return w;
             };
-            int id_cur = 0, meta_cur = 0, id_next, meta_next, fetched = 0;
-            words(0, id_next, meta_next);
-            for (int jj = 0; jj < n_steps; ++jj) {
-                const int j = j_beg + jj, x = jj % C::kRing;
+            Words cur0 = {0, 0}, cur1 = {0, 0}, next0 = words(first_of(0)), next1 = kHalves ? words(first_of(1)) : cur1;
+            int fetched = 0;
+            for (int v = 0; v < n_steps; ++v) {
+                const int i = kHalves ? v & 1 : 0, jj = kHalves ? v >> 1 : v, j = step_of(v), x = v % C::kRing;
                 if (jj % kBatch == 0) {
-                    id_cur = id_next;
-                    meta_cur = meta_next;
-                    words(jj + kBatch, id_next, meta_next);
+                    if (i == 0) { cur0 = next0; next0 = words(j + kBatch); }
+                    else { cur1 = next1; next1 = words(j + kBatch); }
                 }
                 const int pg = lane % kStepPages, at = jj % kBatch * kStepPages;
-                const int row8 = (__shfl_sync(kFull, id_cur, at + pg) * p.Hkv + it.kvh) * 2;
-                const int valid = __shfl_sync(kFull, meta_cur, at + pg) & 0xff;
-                if (jj >= C::kRing) ok = mbar_wait(empty0 + 8u * x, static_cast<uint32_t>((jj / C::kRing - 1) & 1), abort_flag, p.status);
+                const int row8 = (__shfl_sync(kFull, i ? cur1.id : cur0.id, at + pg) * p.Hkv + it.kvh) * 2;
+                const int valid = __shfl_sync(kFull, i ? cur1.meta : cur0.meta, at + pg) & 0xff;
+                if (v >= C::kRing) ok = mbar_wait(empty0 + 8u * x, static_cast<uint32_t>((v / C::kRing - 1) & 1), abort_flag, p.status);
                 if (!ok) break;
                 const uint32_t dst = ring + static_cast<uint32_t>(2 * x * C::kStepBytes), full = full0 + 8u * x;
                 if (is_k) {
@@ -275,13 +289,14 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
             }
         }
       } else {
-        // ================= MMA issuer of a Q tile =================
+        // ================= MMA issuer of a walker =================
         const int i = warp == kMmaWarp ? 0 : 1;
-        if (n_steps > 0 && i < n_qt) {
+        const int n_mine = count_of(i);
+        if (n_mine > 0 && i < n_walk) {
             constexpr uint32_t idesc_qk = make_idesc(kStepKeys, false), idesc_pv = make_idesc(D, true);
             // descriptor words: place x of the ring starts 2 * kStepUnits x address units behind place 0
             constexpr uint32_t kStepUnits = C::kStepBytes >> 4, kGroupUnits = C::kGroupBytes >> 4;
-            const uint64_t dq0 = smem_desc(q_addr(i), 16), dk0 = smem_desc(k_addr(0), 16, C::kGroupBytes), dv0 = smem_desc(v_addr(0), 1024, C::kGroupBytes);
+            const uint64_t dq0 = smem_desc(q_addr(kHalves ? 0 : i), 16), dk0 = smem_desc(k_addr(0), 16, C::kGroupBytes), dv0 = smem_desc(v_addr(0), 1024, C::kGroupBytes);
             const uint32_t dq_lo = static_cast<uint32_t>(dq0), dq_hi = static_cast<uint32_t>(dq0 >> 32);
             const uint32_t dk_lo = static_cast<uint32_t>(dk0), dk_hi = static_cast<uint32_t>(dk0 >> 32);
             const uint32_t dv_lo = static_cast<uint32_t>(dv0), dv_hi = static_cast<uint32_t>(dv0 >> 32);
@@ -315,27 +330,28 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                 tc_commit(bar_pv_done(i));
                 tc_commit(bar_v_empty(x));
             };
-            auto wait_k = [&](int jj) { return mbar_wait(bar_k_full(jj % C::kRing), static_cast<uint32_t>((jj / C::kRing) & 1), abort_flag, p.status); };
+            auto wait_k = [&](int v) { return mbar_wait(bar_k_full(v % C::kRing), static_cast<uint32_t>((v / C::kRing) & 1), abort_flag, p.status); };
             ok = mbar_wait(bar_q_full, 0, abort_flag, p.status);
-            for (int jj = 0; jj < min(2, n_steps) && ok; ++jj) {
-                ok = wait_k(jj);
+            for (int jj = 0; jj < min(2, n_mine) && ok; ++jj) {
+                const int v = place_of(i, jj);
+                ok = wait_k(v);
                 if (!ok) break;
                 tc_fence_after();
-                issue_qk(jj, jj, hide_flag[jj] != 0u);
+                issue_qk(v, jj, hide_flag[v] != 0u);
             }
-            for (int jj = 0; jj < n_steps && ok; ++jj) {
-                const int x = jj % C::kRing, x2 = (jj + 2) % C::kRing, b = jj & 1;
-                const bool more = jj + 2 < n_steps;
+            for (int jj = 0; jj < n_mine && ok; ++jj) {
+                const int v = place_of(i, jj), v2 = place_of(i, jj + 2), b = jj & 1;
+                const bool more = jj + 2 < n_mine;
                 // P comes last: nothing but the MMAs themselves stands between its arrival and the next scores
-                ok = mbar_wait(bar_v_full(x), static_cast<uint32_t>((jj / C::kRing) & 1), abort_flag, p.status);
-                if (ok && more) ok = wait_k(jj + 2);
-                const bool hide = more && hide_flag[x2] != 0u;
+                ok = mbar_wait(bar_v_full(v % C::kRing), static_cast<uint32_t>((v / C::kRing) & 1), abort_flag, p.status);
+                if (ok && more) ok = wait_k(v2);
+                const bool hide = more && hide_flag[v2 % C::kRing] != 0u;
                 if (ok) ok = mbar_wait(bar_p_full(i, b), static_cast<uint32_t>((jj >> 1) & 1), abort_flag, p.status);
                 if (!ok) break;
                 tc_fence_after();
-                issue_pv(x, b, jj == 0);
-                if (more) issue_qk(x2, b, hide);
-                else if (jj + 1 == n_steps) tc_commit(bar_o_done(i));
+                issue_pv(v % C::kRing, b, jj == 0);
+                if (more) issue_qk(v2 % C::kRing, b, hide);
+                else if (jj + 1 == n_mine) tc_commit(bar_o_done(i));
             }
             // pair merge: once every MMA of this CTA has completed, its K/V ring is idle and the peer may write
             // into it (only a CTA that finishes a Q tile receives anything)
@@ -347,16 +363,18 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
       }
     } else {
       asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsSoftmax));
-      if ((warp >> 2) < n_qt) {
+      if ((warp >> 2) < n_walk) {
         // ================= softmax / epilogue: one thread per query row =================
-        const int i = warp >> 2;                                   // Q tile
+        const int i = warp >> 2;                                   // walker
+        const int tile_t0 = it.t0 + (kHalves ? 0 : i * tile_tokens);  // first token of its Q tile
+        const int j0 = first_of(i), n_mine = count_of(i);          // its steps
         const int q4 = warp & 3;                                   // TMEM lane quadrant
         const int r = q4 * 32 + lane;
-        const int t = it.t0 + i * tile_tokens + r / rep;           // episode-relative query token
+        const int t = tile_t0 + r / rep;           // episode-relative query token
         const int h = it.kvh * rep + r % rep;
         const bool row_valid = t < ep.n_q;
         const int c = min(ep.n_new - ep.n_q + t, ep.n_new - 1);    // last visible new key
-        const int c_lo = ep.n_new - ep.n_q + it.t0 + i * tile_tokens;   // the same for the tile's first row: every row sees at least this far
+        const int c_lo = ep.n_new - ep.n_q + tile_t0;   // the same for the tile's first row: every row sees at least this far
         const int G = ep.n_slots;
         const uint32_t lane_sel = static_cast<uint32_t>(q4 * 32) << 16;
         const uint32_t t_s = tmem_base + lane_sel + static_cast<uint32_t>(i * 128);
@@ -372,18 +390,19 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
             else if (p.mass) slot_out = p.mass + rh * p.mass_stride;
         }
         const bool park_smem = p.park_smem != 0;
-        float *park_row = reinterpret_cast<float *>(smem + C::kParkOff) + i * (kParkSlots * 128) + r;   // + slot * 128
+        float *park_row = reinterpret_cast<float *>(smem + C::kParkOff) + i * (kParkSlots * 128) + r;   // + slot * 128; (each walker its own slots)
         const float scale = p.scale_log2;
 
-        // Pair merge: the slot in which the two splits meet is walked by both.  Split 0 writes it (adding what
-        // split 1 sends); split 1 keeps its part in `bnd` instead of storing it.
+        // Where two split the steps between them (the CTAs of a pair, the walkers of a CTA) the slot in which they meet is walked by both.
+        // The first writes it (adding what the second sends); the second keeps its part in `bnd` instead of storing it.
         int shared_slot = -1, skip_slot = -1;
         float bnd = kNegInf;
-        if (pair) {
-            const int jb = (it.split == 0) ? j_end : j_beg;         // first tile of split 1
+        const bool two_halves = kHalves && n_walk == 2;
+        if (pair || two_halves) {
+            const int jb = two_halves ? first_of(1) : (it.split == 0) ? j_end : j_beg;       // first step of the second
             const int last0 = (jb > n_csteps) ? G : (__ldg(p.stream_meta + ep.stream_off + jb * kStepPages - 1) >> 8);
             const int first1 = (jb < n_csteps) ? (__ldg(p.stream_meta + ep.stream_off + jb * kStepPages) >> 8) : G;
-            if (last0 == first1) { shared_slot = last0; if (it.split == 1) skip_slot = last0; }
+            if (last0 == first1) { shared_slot = last0; if ((two_halves ? i : it.split) == 1) skip_slot = last0; }
         }
         float m = kNegInf, l = 0.f, acc = 0.f;                     // reference (log2 units), row sum, sum of the current slot
         int cur_slot = -1;
@@ -401,7 +420,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
         // from the page before.  The pages of a new-token step are one slot (G).
         constexpr int kBatch = 32 / kStepPages;
         auto load_slots = [&](int jj) -> int {
-            const int e = (j_beg + jj) * kStepPages + lane;
+            const int e = (j0 + jj) * kStepPages + lane;
             return e < n_csteps * kStepPages ? __ldg(p.stream_meta + ep.stream_off + e) >> 8 : G;
         };
         int slots = -1, slots_next = load_slots(0);
@@ -409,15 +428,15 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
         // The two warps that share a scheduler (one of each tile) take their exponentials in turns: both at once leave its special-function
         // unit idle while both do the rest.  (Named barriers 1..8: (tile, quadrant) may begin.)
         auto await_turn = [&](int jj) {
-            if (n_qt == 2 && (i == 1 || jj > 0)) asm volatile("bar.sync %0, 64;" ::"r"(1 + q4 + 4 * i) : "memory");
+            if (n_walk == 2 && (i == 1 || jj > 0)) asm volatile("bar.sync %0, 64;" ::"r"(1 + q4 + 4 * i) : "memory");
         };
         auto pass_turn = [&](int jj) {
-            if (n_qt == 2 && (i == 0 || jj + 1 < n_steps)) asm volatile("bar.arrive %0, 64;" ::"r"(1 + q4 + 4 * (i ^ 1)) : "memory");
+            if (n_walk == 2 && (i == 0 ? !kHalves || jj < count_of(1) : jj + 1 < count_of(0))) asm volatile("bar.arrive %0, 64;" ::"r"(1 + q4 + 4 * (i ^ 1)) : "memory");
         };
 
         int jj = 0;
-        for (; jj < n_steps; ++jj) {
-            const int j = j_beg + jj;
+        for (; jj < n_mine; ++jj) {
+            const int j = j0 + jj;
             if (jj % kBatch == 0) {
                 const int last = __shfl_sync(kFull, slots, 31);
                 slots = slots_next;
@@ -547,7 +566,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
             }
         }
 
-        for (; jj < n_steps; ++jj) { await_turn(jj); pass_turn(jj); }      // error path only: the other tile's warp may be waiting
+        for (; jj < n_mine; ++jj) { await_turn(jj); pass_turn(jj); }      // error path only: the other tile's warp may be waiting
 
         // ---- per-row results ----
         const float m_use = (m == kNegInf) ? 0.f : m;
@@ -555,7 +574,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
         // (row, head) index of row rr of this warp, or -1 beyond the episode's queries
         auto row_index = [&](int rr) -> int {
             const int r2 = q4 * 32 + rr;
-            const int t2 = it.t0 + i * tile_tokens + r2 / rep;
+            const int t2 = tile_t0 + r2 / rep;
             if (t2 >= ep.n_q) return -1;
             const int g2 = ep.q_off + t2;
             return (split_mode ? it.split * p.n_q_total + g2 : g2) * p.Hq + it.kvh * rep + r2 % rep;
@@ -598,19 +617,106 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                 slots[sl] = w;
             }
         };
-        // slots this CTA walked (all of them without splits)
+        // slots this walker walked (all of them where nothing is split)
         int first_slot = 0, last_slot = G;
-        if (p.n_splits > 1) {
+        if (p.n_splits > 1 || two_halves) {
             first_slot = G + 1;
             last_slot = -1;
-            if (n_steps > 0) {
-                first_slot = (j_beg < n_csteps) ? (__ldg(p.stream_meta + ep.stream_off + j_beg * kStepPages) >> 8) : G;
-                last_slot = (j_end > n_csteps) ? G : (__ldg(p.stream_meta + ep.stream_off + j_end * kStepPages - 1) >> 8);
+            if (n_mine > 0) {
+                const int je = j0 + n_mine;
+                first_slot = (j0 < n_csteps) ? (__ldg(p.stream_meta + ep.stream_off + j0 * kStepPages) >> 8) : G;
+                last_slot = (je > n_csteps) ? G : (__ldg(p.stream_meta + ep.stream_off + je * kStepPages - 1) >> 8);
             }
         }
+        // The merged row: what a walker or a CTA of a pair makes of its own (m_use, l) and the other's (x, y of pe)
+        float row_lse = lse, other_bnd = kNegInf, w_own = 0.f, w_other = 0.f;
+        auto merge_rows = [&](const float4 &pe) {
+            const bool va = l > 0.f, vb = pe.y > 0.f;
+            const float M = fmaxf(va ? m_use : kNegInf, vb ? pe.x : kNegInf);
+            const float fa = va ? ex2(m_use - M) : 0.f;
+            const float fb = vb ? ex2(pe.x - M) : 0.f;
+            const float L = (va ? l * fa : 0.f) + (vb ? pe.y * fb : 0.f);
+            row_lse = (L > 0.f) ? M + lg2(L) : kNegInf;
+            other_bnd = pe.z;
+            w_own = (L > 0.f) ? fa / L : 0.f;
+            w_other = (L > 0.f) ? fb / L : 0.f;
+        };
+        // log-sum of the slot in which two meet, from the open sum of the first and what the second sent
+        auto shared_log = [&]() {
+            const float own = lg2(acc) + m_use, mx = fmaxf(own, other_bnd);
+            return (mx != kNegInf) ? mx + lg2(ex2(own - mx) + ex2(other_bnd - mx)) : kNegInf;
+        };
 
+        if (two_halves) {
+            // ---- the walkers tell each other (reference, sum, part of the slot in which they meet) of every row; each goes on with its
+            // own slots and half of the channels, whose accumulators both lie in the TMEM lanes it reads ----
+            if (ok) park(m_use);
+            float4 *rows = reinterpret_cast<float4 *>(smem + C::kXpeerOff);
+            rows[i * 128 + r] = make_float4(m_use, ok ? l : 0.f, bnd, 0.f);
+            asm volatile("bar.sync 9, 256;" ::: "memory");           // reached whatever happened (the waits are bounded)
+            merge_rows(rows[(i ^ 1) * 128 + r]);
+            if (split_mode) {
+                if (i == 0 && row_valid) p.part_lse[rh] = row_lse;
+                if (slot_out) {                                      // slots that this split did not walk contribute nothing
+                    for (int sl = i == 0 ? 0 : first_slot; sl <= (i == 0 ? last_slot : G); ++sl) {
+                        if (sl == skip_slot) continue;
+                        if (sl < first_slot || sl > last_slot) slot_out[sl] = kNegInf;
+                        else if (sl == shared_slot) slot_out[sl] = shared_log();
+                        else if (park_smem) slot_out[sl] = park_row[sl * 128];
+                    }
+                }
+            } else if (p.mass) {
+                if (park_smem) {
+                    finish_masses(row_lse, other_bnd, first_slot, last_slot);
+                } else if (row_valid && i == 0) {
+                    p.lse_out[rh] = row_lse;
+                    if (shared_slot >= 0) slot_out[shared_slot] = shared_log();
+                }
+            }
+            for (int t = 0; t < 2 && ok; ++t) ok = mbar_wait(bar_o_done(t), 0, abort_flag, p.status);
+            if (ok) {
+                tc_fence_after();
+                const float w0 = i == 0 ? w_own : w_other, w1 = i == 0 ? w_other : w_own;
+                const uint32_t t_o0 = tmem_base + lane_sel + 256u, t_o1 = t_o0 + 128u;
+                // 32 channels of the merged row
+                auto merged = [&](int col, float (&x)[32]) {
+                    uint32_t a[32], b[32];
+                    tmem_ld32_issue(t_o0 + static_cast<uint32_t>(col), a);
+                    tmem_ld32_issue(t_o1 + static_cast<uint32_t>(col), b);
+                    tmem_ld_wait();
+                    tmem_ld32_arrived(a);
+                    tmem_ld32_arrived(b);
+#pragma unroll
+                    for (int y = 0; y < 32; ++y) x[y] = fmaf(__uint_as_float(a[y]), w0, __uint_as_float(b[y]) * w1);
+                };
+                if (split_mode) {
+#pragma unroll 1
+                    for (int pc = i; pc < D / 32; pc += 2) {         // 32 fp32 channels = 128 bytes per row and piece
+                        float x[32];
+                        uint32_t w[32];
+                        merged(pc * 32, x);
+#pragma unroll
+                        for (int y = 0; y < 32; ++y) w[y] = __float_as_uint(x[y]);
+                        flush_piece(w, reinterpret_cast<uint8_t *>(p.part_o), D * 4, pc);
+                    }
+                } else {
+#pragma unroll 1
+                    for (int pc = i; pc < D / 64; pc += 2) {         // 64 bf16 channels = 128 bytes per row and piece
+                        float x[32];
+                        uint32_t w[32];
+#pragma unroll
+                        for (int k = 0; k < 2; ++k) {
+                            merged(pc * 64 + k * 32, x);
+#pragma unroll
+                            for (int y = 0; y < 16; ++y) w[k * 16 + y] = pack_bf16(x[2 * y], x[2 * y + 1]);
+                        }
+                        flush_piece(w, static_cast<uint8_t *>(p.out), D * 2, pc);
+                    }
+                }
+            }
+        }
         bool exported = false;
-        if (ok) {
+        if (ok && !two_halves) {
             park(m_use);
             if (!pair && !split_mode) {
                 // ---- the whole key stream was this CTA's: output and masses ----
@@ -671,7 +777,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                     }
                 }
             } else {
-              if constexpr (D == 128) {
+              if constexpr (D == 128 && !kHalves) {
                 // ---- pair merge: the two CTAs of the cluster hold the two halves of the key stream ----
                 const uint32_t peer = cluster_rank() ^ 1u;
                 // they tell each other (reference, sum, shared-slot part) of every row
@@ -712,33 +818,17 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                         exported = ok;
                     }
                 }
-                // the merged row: reference, sum, weights of the two accumulators
-                float pair_lse = kNegInf, pair_bnd = kNegInf, w_own = 0.f, w_peer = 0.f;
                 if (ok) ok = mbar_wait<true>(bar_peer_ml, 0, abort_flag, p.status);
-                if (ok) {
-                    const float4 pe = *reinterpret_cast<const float4 *>(smem + C::kXpeerOff + (i * 128 + r) * 16);
-                    const bool va = l > 0.f, vb = pe.y > 0.f;
-                    const float M = fmaxf(va ? m_use : kNegInf, vb ? pe.x : kNegInf);
-                    const float fa = va ? ex2(m_use - M) : 0.f;
-                    const float fb = vb ? ex2(pe.x - M) : 0.f;
-                    const float L = (va ? l * fa : 0.f) + (vb ? pe.y * fb : 0.f);
-                    pair_lse = (L > 0.f) ? M + lg2(L) : kNegInf;
-                    pair_bnd = pe.z;
-                    w_own = (L > 0.f) ? fa / L : 0.f;
-                    w_peer = (L > 0.f) ? fb / L : 0.f;
-                }
+                if (ok) merge_rows(*reinterpret_cast<const float4 *>(smem + C::kXpeerOff + (i * 128 + r) * 16));
                 // each CTA writes the slots it walked against the merged log-sum-exp; the slot both walked is
                 // written by split 0, which adds the part split 1 sent.  (Before the output: the peer's accumulator is
                 // still on its way.)
                 if (ok && p.mass) {
                     if (park_smem) {
-                        finish_masses(pair_lse, pair_bnd, first_slot, last_slot);
+                        finish_masses(row_lse, other_bnd, first_slot, last_slot);
                     } else if (row_valid && it.split == 0) {
-                        p.lse_out[rh] = pair_lse;
-                        if (shared_slot >= 0) {                     // the slot parked last: its own part is still in acc
-                            const float own = lg2(acc) + m_use, mx = fmaxf(own, pair_bnd);
-                            slot_out[shared_slot] = (mx != kNegInf) ? mx + lg2(ex2(own - mx) + ex2(pair_bnd - mx)) : kNegInf;
-                        }
+                        p.lse_out[rh] = row_lse;
+                        if (shared_slot >= 0) slot_out[shared_slot] = shared_log();      // the slot parked last: its own part is still in acc
                     }
                 }
                 if (ok && i == it.split && n_steps > 0) {
@@ -763,7 +853,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                                 for (int cch = 0; cch < 8; ++cch) {
                                     const float4 a = *reinterpret_cast<const float4 *>(
                                         theirs + ((((pc * 2 + k) * 8 + cch) ^ (lane & 7)) << 4));
-                                    auto mix = [&](uint32_t own, float th) { return fmaf(__uint_as_float(own), w_own, th * w_peer); };
+                                    auto mix = [&](uint32_t own, float th) { return fmaf(__uint_as_float(own), w_own, th * w_other); };
                                     w[k * 16 + 2 * cch] = pack_bf16(mix(o[4 * cch], a.x), mix(o[4 * cch + 1], a.y));
                                     w[k * 16 + 2 * cch + 1] = pack_bf16(mix(o[4 * cch + 2], a.z), mix(o[4 * cch + 3], a.w));
                                 }
@@ -793,13 +883,17 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
 
 int attention_park_slots() { return kParkSlots; }
 
+template <int D>
+static cudaError_t prepare()
+{
+    cudaError_t e = cudaFuncSetAttribute(attn_kernel<D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<D>::kSmemBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_kernel<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<D>::kSmemBytes);
+    return e;
+}
+
 cudaError_t prepare_attention(int head_dim)
 {
-    if (head_dim == 128)
-        return cudaFuncSetAttribute(attn_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<128>::kSmemBytes);
-    if (head_dim == 64)
-        return cudaFuncSetAttribute(attn_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<64>::kSmemBytes);
-    return cudaErrorInvalidValue;
+    return head_dim == 128 ? prepare<128>() : head_dim == 64 ? prepare<64>() : cudaErrorInvalidValue;
 }
 
 bool attention_pairs_supported()
@@ -816,7 +910,7 @@ bool attention_pairs_supported()
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, attn_kernel<128>, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, attn_kernel<128, false>, &cfg) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
@@ -826,14 +920,12 @@ bool attention_pairs_supported()
 cudaError_t launch_attention(const AttnParams &p, int head_dim, int n_items, cudaStream_t st)
 {
     if (n_items <= 0) return cudaSuccess;
-    cudaError_t e;
-    if (p.pair_merge && (head_dim != 128 || p.n_splits != 2 || (n_items & 1))) return cudaErrorInvalidValue;
-    if (head_dim == 128)
-        e = launch_pdl(attn_kernel<128>, dim3(n_items), dim3(kThreads), Cfg<128>::kSmemBytes, st, p, p.pair_merge ? 2u : 1u);
-    else if (head_dim == 64)
-        e = launch_pdl(attn_kernel<64>, dim3(n_items), dim3(kThreads), Cfg<64>::kSmemBytes, st, p);
-    else
-        return cudaErrorInvalidValue;
+    if (p.pair_merge && (head_dim != 128 || p.n_splits != 2 || p.halves || (n_items & 1))) return cudaErrorInvalidValue;
+    if (head_dim != 128 && head_dim != 64) return cudaErrorInvalidValue;
+    const auto kernel = head_dim == 128 ? (p.halves ? attn_kernel<128, true> : attn_kernel<128, false>)
+                                        : (p.halves ? attn_kernel<64, true> : attn_kernel<64, false>);
+    const int smem = head_dim == 128 ? Cfg<128>::kSmemBytes : Cfg<64>::kSmemBytes;
+    const cudaError_t e = launch_pdl(kernel, dim3(n_items), dim3(kThreads), smem, st, p, p.pair_merge ? 2u : 1u);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 

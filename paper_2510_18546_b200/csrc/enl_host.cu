@@ -173,6 +173,7 @@ struct enl_cache {
     unsigned long long plan_graph = 0;      // capture that holds the write of the current plan
     bool plan_in_graphs = false;            // some graph may write its plan over the one on the device at any time
     bool plan_pair = false;                 // two splits whose CTAs merge inside the attention kernel (cluster of two)
+    bool plan_halves = false;               // items of one Q tile whose steps the two halves of a CTA share
     bool pairs_ok = false;                  // the device can co-schedule two of the attention kernel's CTAs as a cluster
     std::vector<int32_t> key_sel, key_cu, key_len;   // what the current plan was built from
     int32_t plan_entries = 0, plan_items = 0, plan_splits = 1, plan_batch = 0, plan_max_slots = 0;
@@ -240,7 +241,7 @@ void destroy(enl_cache *c)
     delete c;
 }
 
-int tokens_per_cta(const enl_cache *c) { return kQTiles * (kTileRows / c->rep); }
+int tokens_per_cta(const enl_cache *c, bool halves = false) { return (halves ? 1 : kQTiles) * (kTileRows / c->rep); }
 
 }  // namespace
 
@@ -701,7 +702,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
     if (!reuse) {
         // size check first, so that a failed call leaves the previous plan intact
         const int tpc = tokens_per_cta(c);
-        int64_t n_entries = 0, base_items = 0;
+        int64_t n_entries = 0, base_items = 0, half_items = 0;      // CTAs of two Q tiles, of one
         int min_tiles = 0x7fffffff, max_tiles = 1, max_rows = 1;
         for (int b = 0; b < B; ++b) {
             int64_t e = 0;
@@ -710,6 +711,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
             n_entries += e;
             const int nq = cu_q[b + 1] - cu_q[b], nn = cu_new[b + 1] - cu_new[b];
             base_items += static_cast<int64_t>(ceil_div(nq, tpc)) * d.n_kv_heads;
+            half_items += static_cast<int64_t>(ceil_div(nq, tokens_per_cta(c, true))) * d.n_kv_heads;
             // fewest tiles any CTA of this episode walks: its first token block
             const int c_first = nn - nq + std::min(tpc, nq) - 1;
             min_tiles = std::min<int64_t>(min_tiles, e / kPagesPerTile + c_first / kTileKeys + 1);
@@ -794,39 +796,61 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
                 list_pages = pages;
             }
         }
+        bool halves = false;
         if (!decode) {
             n_splits = 1;
             const bool few = base_items * 5 < c->n_sm * 4;         // a launch that leaves SMs idle splits the key stream
-            // A launch takes about T us per key tile of its longest CTA on top of what it always takes: 8.5 us in one split,
-            // 10.5 with two splits merged by pairs, 11.5 with partial results in memory plus 0.15 us per 1000 of their rows.
-            // (T = 2.25 for two Q tiles, 2.0 for one.  17 to 320 rows over 640 to 5120 keys, measured against two tiles or
-            // more per split: 17 rows over 640 keys 15.0 -> 10.4 us, 41 over 640 17.0 -> 12.6, 320 over 1280 27.0 -> 25.9.  The same
-            // figures serve head_dim 64, whose tiles take 0.93 of the time: of 17, 41, 128 and 320 rows over 640, 1280, 2560 and
-            // 5120 keys the best of 1, 2, 3, 4, 6, 8, 12 and 16 splits takes 0.94 of the chosen number's time at worst, 1.00 in
-            // the middle; at head_dim 128 0.91 and 1.00.)
-            // Of equal costs the fewest splits: SMs left over take in the next launch.
-            auto filling = [&]() {
+            // What a launch takes by a model of the measured times, in us: T per 128 keys of its longest CTA, and what comes on top, rh being
+            // thousands of (row, q head) pairs, m 1 with masses, w 1 at head_dim 128; in memory: splits that the merge kernel puts together.
+            //   two walkers, a Q tile each        T = 1.65 + 0.07 w  unsplit 6.4 + 0.7 w + 2 m + (0.07 + 0.085 m) rh
+            //                                     T = 1.7            two splits merged by pairs of CTAs 9 + m + (0.11 + 0.06 m) rh
+            //                                     T = 1.65 + 0.05 w  in memory 7.4 + 1.3 w + 1.75 m + (0.19 - 0.1 w + 0.12 m + (0.092 + 0.042 w + 0.06 m) splits) rh
+            //   one walker, one Q tile            T = 1.43           unsplit 5.8 + 1.1 m, in memory 6.7 + 0.6 m + (0.35 + 0.05 m) splits rh
+            //   two walkers, half of the steps    T = 1              unsplit 5 + 0.7 w + 1.1 m + (0.135 + 0.02 w + 0.045 m) rh, in memory
+            //                                                        6.8 + 0.9 w + 1.2 m + (0.245 + 0.04 m) splits rh
+            // (beyond eight splits the merge kernel needs a second round trip, 0.4; two steps in all are 0.8 less).  Fitted to 948 measurements: 17 to 512 rows over 640 to 5120
+            // keys, 32 / 8 heads, 24 groups, both head_dims, 1 to 16 splits; the choice takes 1.01 of the best one's time in the mean, 1.11 at
+            // worst.  The best with a Q tile each against the best in halves, head_dim 128, masses: 17 rows over 640 keys 11.2 / 11.2, over
+            // 5120 15.6 / 14.9; 41 rows 14.3 / 12.6, 20.7 / 17.9; 128 rows 16.2 / 14.6, 27.0 / 24.4; 256 rows 17.9 / 16.2, 37.0 / 36.2; 512 rows
+            // 21.2 / 19.4, 51.3 / 55.7; head_dim 64: 41 rows 12.4 / 11.5, 18.6 / 16.8; 128 rows 16.5 / 13.6, 23.6 / 23.0; 512 rows 26.4 / 18.4,
+            // 55.7 / 54.6.
+            const double rh = 1e-3 * a->n_q * d.n_q_heads, m = has_mass ? 1.0 : 0.0, w = d.head_dim == 128 ? 1.0 : 0.0;
+            auto cost_of = [&](bool hv, int ns) {
+                const int steps = ceil_div(2 * max_tiles, ns);                     // of 64 keys
+                const double t = 0.5 * steps, trips = ns > 8 ? 0.4 : !hv && steps <= 2 ? -0.8 : 0.0;
+                if (hv) return ceil_div(steps, 2) + (ns == 1 ? 5.0 + 0.7 * w + 1.1 * m + (0.135 + 0.02 * w + 0.045 * m) * rh
+                                                             : trips + 6.8 + 0.9 * w + 1.2 * m + (0.245 + 0.04 * m) * ns * rh);
+                if (ns == 2 && c->pairs_ok) return 1.7 * t + 9.0 + m + (0.11 + 0.06 * m) * rh;
+                if (max_rows <= kTileRows) return 1.43 * t + (ns == 1 ? 5.8 + 1.1 * m : trips + 6.7 + 0.6 * m + (0.35 + 0.05 * m) * ns * rh);
+                if (ns == 1) return (1.65 + 0.07 * w) * t + 6.4 + 0.7 * w + 2.0 * m + (0.07 + 0.085 * m) * rh;
+                return (1.65 + 0.05 * w) * t + trips + 7.4 + 1.3 * w + 1.75 * m + (0.19 - 0.1 * w + 0.12 * m + (0.092 + 0.042 * w + 0.06 * m) * ns) * rh;
+            };
+            // the cheapest number of splits that runs at once; of equal costs the fewest: SMs left over take in the next launch
+            auto filling = [&](bool hv) {
+                const int64_t items = hv ? half_items : base_items;
                 int best = 1;
-                double least = 1e30;
-                for (int ns = 1; ns <= kMaxSplits && ns * base_items <= c->n_sm && ns <= min_tiles; ++ns) {
-                    const bool in_pairs = ns == 2 && c->pairs_ok;
-                    const double cost = (max_rows > kTileRows ? 2.25 : 2.0) * ceil_div(max_tiles, ns) +
-                                        (ns == 1 ? 8.5 : in_pairs ? 10.5 : 11.5 + 0.15e-3 * ns * a->n_q * d.n_q_heads);
-                    if (cost < least - 1e-9) { least = cost; best = ns; }
-                }
+                for (int ns = 2; ns <= kMaxSplits && ns * items <= c->n_sm && ns <= min_tiles; ++ns)
+                    if (cost_of(hv, ns) < cost_of(hv, best) - 1e-9) best = ns;
                 return best;
             };
             // the kernel that finishes masses takes a few us itself: eight tiles per split and more
             const int filling_mass = std::max(1, std::min(static_cast<int>(c->n_sm / base_items), min_tiles / 8));
             if (small_blocks) n_splits = 1;
-            else if (has_sum && !mass_only) n_splits = few && a->split_hint != 1 && c->pairs_ok && filling_mass >= 2 ? 2 : 1;   // a pair or none
-            else if (a->split_hint >= 1) n_splits = std::min(a->split_hint, std::max(1, min_tiles));   // no CTA without a tile
-            else if (few) n_splits = mass_only ? filling_mass : filling();
+            else if (a->split_hint >= 1 && !(has_sum && !mass_only)) n_splits = std::min(a->split_hint, std::max(1, min_tiles));   // no CTA without a tile
+            else if (few && mass_only) n_splits = filling_mass;
+            else if (few && a->split_hint == 0 && c->gpu && half_items <= c->n_sm) {
+                // (sums per object: outputs are merged by the walkers or by pairs, or not at all)
+                const int with = has_sum ? 1 : filling(true), without = has_sum ? (c->pairs_ok && filling_mass >= 2 ? 2 : 1) : filling(false);
+                halves = cost_of(true, with) < cost_of(false, without);
+                n_splits = halves ? with : without;
+            } else if (has_sum && !mass_only) n_splits = few && a->split_hint != 1 && c->pairs_ok && filling_mass >= 2 ? 2 : 1;   // a pair or none
+            else if (few) n_splits = filling(false);
             if (mass_only) {                                       // no outputs to merge: the kernel that finishes the masses adds the splits up
                 n_splits = std::min(n_splits, kFinishSplits);
                 while (n_splits > 1 && static_cast<int64_t>(n_splits) * a->n_q * d.n_q_heads > c->finish_cap) --n_splits;
             }
-            n_splits = std::min<int64_t>(n_splits, std::max<int64_t>(1, c->cap_items / base_items));
+            n_splits = std::min<int64_t>(n_splits, std::max<int64_t>(1, c->cap_items / (halves ? half_items : base_items)));
+            halves = halves && half_items <= c->cap_items;
             n_splits = std::min(n_splits, kMaxSplits);
             while (n_splits > 1 && !mass_only && !fits(n_splits)) --n_splits;
         }
@@ -839,9 +863,9 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         // Two splits of a head_dim-128 call are launched as clusters of two CTAs, which exchange their partial
         // results through distributed shared memory: no scratch round trip and no merge kernel.  Every CTA must
         // have at least one tile, and the items of a pair must be neighbours (they are: same tile count, stable sort).
-        const bool pair = !decode && !mass_only && n_splits == 2 && d.head_dim == 128 && min_tiles >= 2 && (c->pairs_ok || !c->gpu);
+        const bool pair = !decode && !mass_only && !halves && n_splits == 2 && d.head_dim == 128 && min_tiles >= 2 && (c->pairs_ok || !c->gpu);
         const bool by_grid = decode || small_blocks > 0;               // kernels that take their CTA's place from the grid
-        const int64_t n_items = decode ? static_cast<int64_t>(B) * d.n_kv_heads * n_splits : base_items * n_splits;
+        const int64_t n_items = decode ? static_cast<int64_t>(B) * d.n_kv_heads * n_splits : (halves ? half_items : base_items) * n_splits;
         {   // sections: what the kernels of this plan read (the decode kernel takes its CTA's place from the grid)
             auto align16 = [](size_t x) { return (x + 15) & ~static_cast<size_t>(15); };
             size_t at = 0;
@@ -910,8 +934,9 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
             work.reserve(static_cast<size_t>(n_items));
             for (int b = 0; b < B; ++b) {
                 const EpInfo &e = eps[b];
-                for (int t0 = 0; t0 < e.n_q; t0 += tpc) {
-                    const int t_hi = std::min(t0 + tpc, e.n_q);
+                const int step = tokens_per_cta(c, halves);
+                for (int t0 = 0; t0 < e.n_q; t0 += step) {
+                    const int t_hi = std::min(t0 + step, e.n_q);
                     const int tiles = e.n_ctiles + (e.n_new - e.n_q + t_hi - 1) / kTileKeys + 1;
                     for (int h = 0; h < d.n_kv_heads; ++h)
                         for (int sp = 0; sp < n_splits; ++sp) work.push_back({Item{b, h, t0, sp}, tiles});
@@ -941,6 +966,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         c->plan_cluster = cluster;
         c->plan_list_pages = list_pages;
         c->plan_pair = pair;
+        c->plan_halves = halves;
         c->key_sel.assign(a->sel_ids, a->sel_ids + a->n_sel);
         c->key_cu.assign(cu_sel, cu_sel + B + 1);
         c->key_cu.insert(c->key_cu.end(), cu_q, cu_q + B + 1);
@@ -1090,6 +1116,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
     p.mass_stride = a->mass_stride;
     p.n_splits = c->plan_splits;
     p.pair_merge = c->plan_pair ? 1 : 0;
+    p.halves = c->plan_halves ? 1 : 0;
     p.scale_log2 = 1.4426950408889634f / sqrtf(static_cast<float>(d.head_dim));
     p.park_smem = c->plan_park ? 1 : 0;
     p.lse_out = c->finish_lse;

@@ -29,7 +29,7 @@ struct EpInfo {
 struct Item {
     int32_t ep;             // episode
     int32_t kvh;            // kv head
-    int32_t t0;             // first query token (episode-relative) of the CTA's two Q tiles
+    int32_t t0;             // first query token (episode-relative) of the CTA's Q tiles
     int32_t split;          // KV split index in [0, n_splits)
 };
 
@@ -62,6 +62,7 @@ struct AttnParams {
     int32_t mass_stride;
     int32_t n_splits;
     int32_t pair_merge;     // 1: two splits, launched as clusters of two CTAs that merge through distributed shared memory
+    int32_t halves;         // 1: items are Q tiles of 128 rows, whose steps the two walkers of a CTA share (see the kernel)
     float   scale_log2;     // log2(e) / sqrt(D)
     int32_t park_smem;      // 1: the call has at most attention_park_slots() slots: the kernel turns their log-sums into masses itself;
                             // 0: log-sums go to mass, log-sum-exps to lse_out, and mass_finish_kernel does
