@@ -744,11 +744,12 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         if (decode && a->split_hint == 0) {
             // Splits merged by a thread-block cluster: the widest one worth having of which all (episode, kv head) pairs' run at
             // once.  When they do not fill one and a half CTAs per SM the streaming kernel, whose CTAs keep more in flight, is faster
-            // from some 40 pages per CTA on; below, and wherever they do, its merge through memory costs more.  Measured with masses
-            // (clusters against streaming, us), one episode, 8 kv heads, D 128: 2200 keys 8.1 / 10.2, 7000 keys 12.3 / 13.3, 10k keys
-            // (40 pages) 14.6 / 14.4, 20k keys 21.1 / 19.4, 33k keys 30.0 / 26.3; four episodes of 9900 keys 29.3 / 30.3.  D 64: 6.9 / 9.1,
-            // 9.9 / 11.8, 11.3 / 12.4, 15.0 / 15.6, 20.0 / 19.3; 18.2 / 23.1, so there the line could lie at some 100 pages.  With few
-            // kv heads, too: D 128, 10k keys, 2 kv heads 10.5 / 15.7, 4 kv heads 12.3 / 14.9.
+            // from some number of pages per CTA on; below, and wherever they do, its merge through memory costs more.  Measured (clusters
+            // against streaming, us, without masses, with masses), D 128: 8 kv heads, 12k keys (47 pages) 13.1 / 14.5, 14.2 / 15.1, 16k (62)
+            // 15.8 / 16.3, 17.0 / 17.0, 27k (105) 23.2 / 22.4, 24.6 / 23.4; 6 kv heads, 16k 14.0 / 14.6, 15.3 / 15.2, 20k 16.2 / 16.2,
+            // 17.5 / 16.9; 4 kv heads, 20k (78) 14.9 / 15.5, 16.0 / 17.7, 27k 18.3 / 17.6, 19.3 / 19.5; two episodes of 12k keys (clusters of
+            // eight, 94) 19.4 / 21.1, 20.5 / 21.6.  D 64: 4 kv heads, 20k 11.3 / 11.6, 11.3 / 14.0, 33k (129) 16.2 / 13.5, 15.0 / 15.5; 8 kv heads,
+            // 33k 17.4 / 18.3, 18.7 / 19.2.
             const int n = B * d.n_kv_heads;
             for (int i = widest_cluster_log(n, most, false); i >= 0 && !cluster; --i) {
                 if ((1 << i) > fewest) continue;
@@ -758,7 +759,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
                 // (where the streaming kernel would need a second wave too, one here is the better one: 8 episodes of 9900 keys
                 // 56 against 82 us)
                 if (cap < n && !(cap > 0 && n * need > c->n_sm && (n << i) <= 2 * c->n_sm)) continue;
-                if (2 * (n << i) < 3 * c->n_sm && list_pages > 40) break;
+                if (2 * (n << i) < 3 * c->n_sm && list_pages > (d.head_dim == 64 ? 112 : i < 4 || n <= 4 ? 88 : 64)) break;
                 cluster = 1 << i;
             }
         }
