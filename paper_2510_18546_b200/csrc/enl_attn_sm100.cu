@@ -130,7 +130,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
     const Item it = p.items[blockIdx.x];
     const EpInfo ep = p.eps[it.ep];
     const int rep = p.rep;
-    const int tile_tokens = kTileRows / rep;
+    const int lr = 31 - __clz(rep);                                      // a power of two
+    const int tile_tokens = kTileRows >> lr;
     // Calls with few CTAs (kHalves): one Q tile per CTA, and the two walkers (softmax warpgroup + issuer) take half of its steps each
     // and put their results together at the end.  Else a walker has a Q tile of its own and walks all the steps.
     const int t_hi = min(it.t0 + (kHalves ? 1 : kQTiles) * tile_tokens, ep.n_q);    // exclusive
@@ -193,21 +194,21 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
     // everything above touched only shared memory, TMEM and the gather plan; from here on the caller's tensors,
     // the pool and the scratch are read and written, so the previous kernel of the stream must have finished
     pdl_trigger();
-    // While the previous kernel drains, ask what the first steps need into the L2: the Q tiles and a ring full of
-    // K and V (new tokens only when the stream starts with them).
-    // (Only CTAs of the first wave wait for the previous kernel; for the others this would be loads issued twice.)
-    if ((warp == kKWarp || warp == kVWarp) && n_steps > 0 && static_cast<int>(blockIdx.x) < p.first_wave) {
+    // While the previous kernel drains, the producers (which wait for it later) fetch the cached pages of the first steps: the pool is
+    // written by launches of this library only, and none has come in between.  What else comes first is asked into the L2: the Q tiles and
+    // new tokens.  (Only CTAs of the first wave wait for the previous kernel; for the others this would be loads issued twice.)
+    // How many steps: with none a launch took 2.4 us from the wait to its first scores (the page words' round trip and then the pages').
+    // Two steps leave the planner's layer at 29.3 us (none 30.5, four 29.7); where the kernel before is the one that merges the splits,
+    // whose reads more loads hold up, one: 128 rows over 2560 keys 19.0 -> 18.35 us, with two steps 18.6, with four 19.3.
+    const bool producer = warp == kKWarp || warp == kVWarp;
+    if (producer && n_steps > 0 && static_cast<int>(blockIdx.x) < p.first_wave) {
         if (warp == kKWarp && lane < n_qt * C::kHalves)
             tma_prefetch_3d(&p.tm_q, (lane % C::kHalves) * 64, it.kvh * rep, ep.q_off + it.t0 + (lane / C::kHalves) * tile_tokens);
-        const int v = lane / kStepPages, j = step_of(v);
-        if (v < min(C::kRing, n_steps) && j < n_csteps)
-            tma_prefetch_4d(warp == kKWarp ? &p.tm_kpool : &p.tm_vpool, 0, 0, 0,
-                            (p.stream_page[ep.stream_off + j * kStepPages + lane % kStepPages] * p.Hkv + it.kvh) * 2);
-        const int vn = lane / (kStepKeys / 8), jn = step_of(vn);     // new tokens: eight rows a box
+        const int vn = lane / (kStepKeys / 8), jn = step_of(vn);     // eight rows a box
         if (vn < min(C::kRing, n_steps) && jn >= n_csteps)
             tma_prefetch_4d(warp == kKWarp ? &p.tm_knew : &p.tm_vnew, 0, ep.new_off + (jn - n_csteps) * kStepKeys + lane % (kStepKeys / 8) * 8, 0, it.kvh);
     }
-    pdl_wait();
+    if (!producer) pdl_wait();
 
     bool ok = true;
 
@@ -222,13 +223,21 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
         const uint32_t ring = is_k ? k_addr(0) : v_addr(0), full0 = is_k ? bar_k_full(0) : bar_v_full(0),
                        empty0 = is_k ? bar_k_empty(0) : bar_v_empty(0);
         if (n_steps > 0) {
-            if (is_k && lane == 0) {
-                mbar_expect_tx(bar_q_full, static_cast<uint32_t>(n_qt * C::kTileBytes));
-                for (int i = 0; i < n_qt; ++i)
-                    for (int hf = 0; hf < C::kHalves; ++hf)
-                        tma_load_3d(q_addr(i) + hf * C::kHalfBytes, &p.tm_q, hf * 64, it.kvh * rep,
-                                    ep.q_off + it.t0 + i * tile_tokens, bar_q_full);
-            }
+            // before anything of the caller's: the wait for the previous kernel, and then the Q tiles first
+            const int early = p.wait_first || static_cast<int>(blockIdx.x) >= p.first_wave ? 0 : p.n_splits > 1 && !pair ? 1 : 2;   // nothing to wait for: Q first
+            bool waited = false;
+            auto wait_previous = [&]() {
+                pdl_wait();
+                waited = true;
+                if (is_k && lane == 0) {
+                    mbar_expect_tx(bar_q_full, static_cast<uint32_t>(n_qt * C::kTileBytes));
+                    for (int i = 0; i < n_qt; ++i)
+                        for (int hf = 0; hf < C::kHalves; ++hf)
+                            tma_load_3d(q_addr(i) + hf * C::kHalfBytes, &p.tm_q, hf * 64, it.kvh * rep,
+                                        ep.q_off + it.t0 + i * tile_tokens, bar_q_full);
+                }
+                __syncwarp();
+            };
             // Page words (id; slot << 8 | valid keys) of 32 pages at a time, one per lane, fetched eight steps ahead (of either walker): a
             // load in every step kept the ring waiting for the L2.
             constexpr int kBatch = 32 / kStepPages;
@@ -250,6 +259,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                     if (i == 0) { cur0 = next0; next0 = words(j + kBatch); }
                     else { cur1 = next1; next1 = words(j + kBatch); }
                 }
+                if (!waited && (v >= early || j >= n_csteps)) wait_previous();
                 const int pg = lane % kStepPages, at = jj % kBatch * kStepPages;
                 const int row8 = (__shfl_sync(kFull, i ? cur1.id : cur0.id, at + pg) * p.Hkv + it.kvh) * 2;
                 const int valid = __shfl_sync(kFull, i ? cur1.meta : cur0.meta, at + pg) & 0xff;
@@ -279,6 +289,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                 }
                 ++fetched;
             }
+            if (!waited) wait_previous();
             // error path only: let the copies already in flight land before the CTA retires
             if (!ok) {
                 for (int f = max(0, fetched - C::kRing); f < fetched; ++f) {
@@ -370,8 +381,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
         const int j0 = first_of(i), n_mine = count_of(i);          // its steps
         const int q4 = warp & 3;                                   // TMEM lane quadrant
         const int r = q4 * 32 + lane;
-        const int t = tile_t0 + r / rep;           // episode-relative query token
-        const int h = it.kvh * rep + r % rep;
+        const int t = tile_t0 + (r >> lr);           // episode-relative query token
+        const int h = it.kvh * rep + (r & (rep - 1));
         const bool row_valid = t < ep.n_q;
         const int c = min(ep.n_new - ep.n_q + t, ep.n_new - 1);    // last visible new key
         const int c_lo = ep.n_new - ep.n_q + tile_t0;   // the same for the tile's first row: every row sees at least this far
@@ -574,10 +585,10 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
         // (row, head) index of row rr of this warp, or -1 beyond the episode's queries
         auto row_index = [&](int rr) -> int {
             const int r2 = q4 * 32 + rr;
-            const int t2 = tile_t0 + r2 / rep;
+            const int t2 = tile_t0 + (r2 >> lr);
             if (t2 >= ep.n_q) return -1;
             const int g2 = ep.q_off + t2;
-            return (split_mode ? it.split * p.n_q_total + g2 : g2) * p.Hq + it.kvh * rep + r2 % rep;
+            return (split_mode ? it.split * p.n_q_total + g2 : g2) * p.Hq + it.kvh * rep + (r2 & (rep - 1));
         };
         // The warp's 32 rows x 128 bytes leave through the (idle) shared memory of the Q tile: row-per-thread
         // stores would touch 32 different rows per instruction.  Each thread stages its own 128 bytes, 16-byte
