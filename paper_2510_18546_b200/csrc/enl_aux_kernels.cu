@@ -154,12 +154,12 @@ __global__ void __launch_bounds__(256) combine_kernel(const CombineParams p)
 
 // Masses of the attention kernel's calls with many slots, of scoring passes and of per-object sums: the attention kernel has
 // left every slot's log2-sum in the mass buffer and every row's log2-sum-exp beside it.  One warp per 32 (row, head) pairs and
-// 32 slots, lanes over the slots: every access is a coalesced line, eight pairs' lines in flight.  Bandwidth-bound: reads and
+// 32 slots, lanes over the slots: every access is a coalesced line, kLoads pairs' lines in flight.  Bandwidth-bound: reads and
 // writes every mass once.  Four layers of 1024 rows x 32 heads over 1000 groups (131 MB of masses each): 9.4 -> 8.5 ms against
 // finishing them inside the attention kernel.
 // With mass_sum the masses of one object's rows are added up on the way and leave as one atomic add per warp, object and slot
 // (Sec. 3.3 consumes only averages over an object's tokens and the q heads).
-template <bool kSplits, bool kSums>
+template <bool kSplits, bool kSums, int kLoads>
 __global__ void __launch_bounds__(256) mass_finish_kernel(const FinishParams p)
 {
     const int lane = threadIdx.x & 31;
@@ -215,15 +215,15 @@ __global__ void __launch_bounds__(256) mass_finish_kernel(const FinishParams p)
     auto turn = [&](auto one_row) {
         constexpr bool kOneRow = decltype(one_row)::value;  // the pairs have one slot count and one object
         if (kOneRow) run_obj = obj;
-        for (int x0 = 0; x0 < n_here; x0 += 16) {                   // (loads in flight: with 8 four layers of 512 rows over 200 groups take 475 us, 16 and 32: 471)
-            float v[16];
+        for (int x0 = 0; x0 < n_here; x0 += kLoads) {
+            float v[kLoads];
 #pragma unroll
-            for (int u = 0; u < 16; ++u) {
+            for (int u = 0; u < kLoads; ++u) {
                 const int g = kOneRow ? G : __shfl_sync(0xffffffffu, G, x0 + u);
                 v[u] = s <= g ? __ldcg(col + static_cast<long long>(x0 + u) * p.mass_stride) : ninf;
             }
 #pragma unroll
-            for (int u = 0; u < 16; ++u) {
+            for (int u = 0; u < kLoads; ++u) {
                 const int x = x0 + u, g = kOneRow ? G : __shfl_sync(0xffffffffu, G, x);
                 const float ref = __shfl_sync(0xffffffffu, lse, x);
                 float w = (ref != ninf) ? ex2f(v[u] - ref) : 0.f;
@@ -402,13 +402,20 @@ cudaError_t launch_mass_finish(const FinishParams &p, cudaStream_t st)
     if (pairs <= 0) return cudaSuccess;
     if (p.n_splits > kFinishSplits) return cudaErrorInvalidValue;
     const dim3 grid(static_cast<unsigned>((pairs + 255) / 256), static_cast<unsigned>(p.max_slots / 32 + 1));
-    cudaError_t e;
-    if (p.n_splits > 1)
-        e = p.mass_sum ? launch_pdl(mass_finish_kernel<true, true>, grid, dim3(256), 0, st, p)
-                       : launch_pdl(mass_finish_kernel<true, false>, grid, dim3(256), 0, st, p);
-    else
-        e = p.mass_sum ? launch_pdl(mass_finish_kernel<false, true>, grid, dim3(256), 0, st, p)
-                       : launch_pdl(mass_finish_kernel<false, false>, grid, dim3(256), 0, st, p);
+    // Loads in flight per warp: sixteen where a multiprocessor has few warps to hide a round trip with, eight where the grid fills it.
+    // Four layers with outputs, 8 -> 16 loads: 448 CTAs (512 rows over 200 groups) 467 -> 440 us, 896 CTAs (1024 rows) 799 -> 805,
+    // 1280 CTAs 1132 -> 1177, 4096 CTAs (1000 groups) 3735 -> 3817; averages only, 896 CTAs 597 -> 602.
+    constexpr unsigned kFewCtas = 4 * 148;
+    const bool few = static_cast<unsigned long long>(grid.x) * grid.y <= kFewCtas;
+    auto launch = [&](auto loads) {
+        constexpr int kLoads = decltype(loads)::value;
+        if (p.n_splits > 1)
+            return p.mass_sum ? launch_pdl(mass_finish_kernel<true, true, kLoads>, grid, dim3(256), 0, st, p)
+                              : launch_pdl(mass_finish_kernel<true, false, kLoads>, grid, dim3(256), 0, st, p);
+        return p.mass_sum ? launch_pdl(mass_finish_kernel<false, true, kLoads>, grid, dim3(256), 0, st, p)
+                          : launch_pdl(mass_finish_kernel<false, false, kLoads>, grid, dim3(256), 0, st, p);
+    };
+    const cudaError_t e = few ? launch(std::integral_constant<int, 16>{}) : launch(std::integral_constant<int, 8>{});
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
