@@ -191,8 +191,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
     const uint32_t tmem_base = *tmem_slot;
     const bool pair = !kHalves && p.pair_merge != 0;
     if (pair) cluster_sync_all();                // the peer's barriers exist before anything is sent to them
-    // everything above touched only shared memory, TMEM and the gather plan; from here on the caller's tensors,
-    // the pool and the scratch are read and written, so the previous kernel of the stream must have finished
+    // Everything above touched only shared memory, TMEM and the gather plan.  From here on the pool is read, which the previous kernel of
+    // the stream leaves alone (wait_first), and the caller's tensors and the scratch are, for which it must have finished.
     pdl_trigger();
     // While the previous kernel drains, the producers (which wait for it later) fetch the cached pages of the first steps: the pool is
     // written by launches of this library only, and none has come in between.  What else comes first is asked into the L2: the Q tiles and
@@ -499,8 +499,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
             const float m_cand = fmaxf(fmax3(mx4[0], mx4[1], mx4[2]), mx4[3]) * scale;
 
             // The reference moves only when the row maximum has grown by more than the threshold (probabilities
-            // stay below 2^threshold meanwhile); then the sums and the accumulator O_i are rescaled.  O_i holds
-            // the tiles so far and no MMA touches it now: S_i of this tile completed after P_i V of the previous.
+            // stay below 2^threshold meanwhile); then the sums and the accumulator O_i are rescaled.  S_i of this
+            // step may have been made before P_i V of the previous one, so that one is waited for first: seldom.
             const bool need = m_cand > m + kRescaleThreshold;       // also true when m == -inf < m_cand
             if (__any_sync(kFull, need)) {
                 const float m_new = fmaxf(m, m_cand);
@@ -525,7 +525,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
             const float m_use = (m == kNegInf) ? 0.f : m;
 
             // p = exp2(s * scale - m) in fp32; bf16 pairs (even key in the low half) into P_i, 32 keys per store, handed
-            // to the MMA warp in two halves.  The page sums (of the fp32 values) are taken along the way: their adds
+            // to the issuer once a step.  The page sums (of the fp32 values) are taken along the way: their adds
             // fill issue slots that the exponentials leave free.
             await_turn(jj);
             const uint64_t sc2 = pack2(scale, scale), nm2 = pack2(-m_use, -m_use);
