@@ -172,6 +172,7 @@ struct enl_cache {
     unsigned long long settled_graph = 0;   // capture that holds an attention launch behind everything written so far
     unsigned long long plan_graph = 0;      // capture that holds the write of the current plan
     bool plan_in_graphs = false;            // some graph may write its plan over the one on the device at any time
+    bool pool_in_graphs = false;            // some graph holds launches that write the pool: it may run before any call outside it
     bool plan_pair = false;                 // two splits whose CTAs merge inside the attention kernel (cluster of two)
     bool plan_halves = false;               // items of one Q tile whose steps the two halves of a CTA share
     bool pairs_ok = false;                  // the device can co-schedule two of the attention kernel's CTAs as a cluster
@@ -209,7 +210,13 @@ struct enl_cache {
     int32_t *h_meta() { return reinterpret_cast<int32_t *>(plan_host + off_meta); }
     int32_t *h_rowslots() { return reinterpret_cast<int32_t *>(plan_host + off_rowslots); }
     uint8_t *h_chg() { return plan_host + off_chg; }
-    void pool_written() { written = true; settled_graph = 0; }
+    // A launch that writes the pool is about to be enqueued (captured: a graph that does so is being made).
+    void pool_written(bool captured)
+    {
+        written = true;
+        settled_graph = 0;
+        pool_in_graphs = pool_in_graphs || captured;
+    }
     int32_t *h_rowobj() { return reinterpret_cast<int32_t *>(plan_host + off_rowobj); }
 };
 
@@ -505,9 +512,9 @@ extern "C" int enl_group_store(enl_cache_t *c, int32_t group_id, int32_t layer, 
     ++c->epoch;
 
     if (!c->gpu || n_tokens == 0) return ENL_OK;
-    c->pool_written();
     DeviceGuard dg(c->d.device);
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    c->pool_written(capture_of(st) != 0);
     if (join_loads(c, st, -1) != ENL_OK) return ENL_E_CUDA;
     const size_t row_bytes = static_cast<size_t>(c->d.n_kv_heads) * c->d.head_dim * 2;
     int pos = first_pos;
@@ -573,9 +580,9 @@ extern "C" int enl_group_store_all_layers(enl_cache_t *c, int32_t group_id, int3
     ++c->epoch;
 
     if (!c->gpu || n_tokens == 0) return ENL_OK;
-    c->pool_written();
     DeviceGuard dg(c->d.device);
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    c->pool_written(capture_of(st) != 0);
     if (join_loads(c, st, -1) != ENL_OK) return ENL_E_CUDA;
     const size_t row_bytes = static_cast<size_t>(c->d.n_kv_heads) * c->d.head_dim * 2;
     for (int layer0 = 0; layer0 < L; layer0 += kScatterLayers) {
@@ -1011,8 +1018,9 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
     }
     // Launches that find plan and pool as the attention launch before left them may read both before the kernel before them
     // has ended.  Ones that do not wait for it first and hold their own successor back until then, so that this carries over:
-    // from an attention launch that was made, not from one that was refused.
-    const bool wait_first = graph ? c->settled_graph != graph : c->written;
+    // from an attention launch that was made, not from one that was refused.  A graph that stores may have run right before any call
+    // outside it, so once there is one those calls always wait.
+    const bool wait_first = graph ? c->settled_graph != graph : c->written || c->pool_in_graphs;
     auto settled = [&]() { if (graph) c->settled_graph = graph; else c->written = false; };
 
     const int slot_stride = c->plan_max_slots + 1;
@@ -1457,7 +1465,7 @@ extern "C" int enl_step_prepare(enl_cache_t *c, const int32_t *sel_ids, int32_t 
             g.resident = true;                                         // host copy stays current until the next store
             stt.bytes_h2d += static_cast<int64_t>(np) * page_bytes_of(c) * 2 * c->d.n_layers;
         }
-        c->pool_written();
+        c->pool_written(c->gpu && capture_of(st) != 0);
         const int rc = enqueue_loads(c, n, st);
         if (rc != ENL_OK) return rc;
     }

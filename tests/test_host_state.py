@@ -158,3 +158,28 @@ def test_captured_plan_of_any_size_is_part_of_the_graph(host):
     host.fake_capture(0)
     c.store(2, 89000)
     assert c.waits("prefill") == (1, True)
+
+
+@pytest.mark.parametrize("all_layers", [False, True])
+@pytest.mark.parametrize("route", sorted(Cache.ROUTES))
+def test_captured_store_is_waited_for_whenever_its_graph_may_have_run(host, route, all_layers):
+    """A captured store writes the pool when its graph runs, however often that is: calls outside the graph and in other graphs cannot
+    know, so their launches read nothing of the pool before what the stream holds has ended."""
+    c = Cache(host)
+    assert c.waits(route)[0] == 1 and c.waits(route, layer=1) == (0, False)
+    host.fake_capture(7)
+    if all_layers:
+        rows = (ctypes.c_void_p * 2)(1 << 20, 1 << 20)
+        assert host.enl_group_store_all_layers(c.h, 1, 64, rows, rows, 0, None) == enl.ENL_OK
+    else:
+        c.store(1, 64)
+    host.fake_capture(0)
+    for layer in (0, 1, 0, 1):                                  # the graph may have run before each of these
+        assert c.waits(route, layer)[0] == 1
+    c.store(1, 60)
+    for layer in (0, 1):
+        assert c.waits(route, layer)[0] == 1
+    host.fake_capture(8)                                        # a graph's first launch waits for all that ran before the graph
+    assert c.waits(route)[0] == 1 and c.waits(route, layer=1) == (0, False)
+    host.fake_capture(0)
+    assert c.waits(route)[0] == 1
