@@ -72,28 +72,39 @@ bool encode_map(CUtensorMap *tm, const void *base, int rank, const cuuint64_t *d
 
 inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 
-// Tensor maps of the caller's tensors, kept by (pointer, shape): a planning step calls enl_attend once per layer with
+// Tensor maps of the caller's tensors, kept by what they are made from: a planning step calls enl_attend once per layer with
 // tensors that come back step after step, and encoding three maps per call is most of the host time of a call whose
 // gather plan is reused.
+// The key is all that a map is made from.
 struct MapKey {
     const void *base;
-    uint64_t d0, d1, d2;
-    uint32_t b0, b1, b2;
+    cuuint64_t dims[4], strides[3];
+    cuuint32_t box[4];
+    int rank;
+    MapKey() : base(nullptr), dims{}, strides{}, box{}, rank(0) {}
+    MapKey(const void *b, int r, const cuuint64_t *d, const cuuint64_t *s, const cuuint32_t *x) : MapKey()
+    {
+        base = b;
+        rank = r;
+        for (int i = 0; i < r; ++i) { dims[i] = d[i]; box[i] = x[i]; }
+        for (int i = 0; i + 1 < r; ++i) strides[i] = s[i];
+    }
     bool operator==(const MapKey &o) const
     {
-        return base == o.base && d0 == o.d0 && d1 == o.d1 && d2 == o.d2 && b0 == o.b0 && b1 == o.b1 && b2 == o.b2;
+        return base == o.base && rank == o.rank && std::equal(dims, dims + 4, o.dims) && std::equal(strides, strides + 3, o.strides) &&
+               std::equal(box, box + 4, o.box);
     }
 };
 struct MapCache {
     static constexpr int kSlots = 256;
-    MapKey key[kSlots] = {};
+    MapKey key[kSlots];
     CUtensorMap map[kSlots];
     bool used[kSlots] = {};
     uint32_t turn = 0;
-    // bf16 map [..][d2][d1][d0] of rank 3 or 4 with box {b0, b1, b2, ..}; the boxes in use tell the ranks apart
+    // bf16 map [..][d2][d1][d0] of rank 3 or 4 with box {b0, b1, b2, ..}
     bool get(CUtensorMap *out, const void *base, const cuuint64_t *dims, const cuuint64_t *strides, const cuuint32_t *box, int rank = 3)
     {
-        const MapKey k{base, dims[0], dims[1], dims[2], box[0], box[1], box[2]};
+        const MapKey k(base, rank, dims, strides, box);
         const size_t h = (reinterpret_cast<uintptr_t>(base) >> 8) * 0x9E3779B97F4A7C15ull >> 56;
         int victim = -1;                                    // the same tensor with another length (decoding), else a free slot
         for (int probe = 0; probe < 4; ++probe) {
