@@ -396,17 +396,17 @@ cudaError_t launch_page_scatter_layers(void *kpool, void *vpool, size_t layer_by
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-cudaError_t launch_mass_finish(const FinishParams &p, cudaStream_t st)
+cudaError_t launch_mass_finish(const FinishParams &p, int n_sm, cudaStream_t st)
 {
     const long long pairs = static_cast<long long>(p.n_q_total) * p.Hq;
     if (pairs <= 0) return cudaSuccess;
     if (p.n_splits > kFinishSplits) return cudaErrorInvalidValue;
     const dim3 grid(static_cast<unsigned>((pairs + 255) / 256), static_cast<unsigned>(p.max_slots / 32 + 1));
-    // Loads in flight per warp: sixteen where a multiprocessor has few warps to hide a round trip with, eight where the grid fills it.
+    // Loads in flight per warp: sixteen where a multiprocessor has few warps to hide a round trip with (up to four CTAs each), eight where
+    // the grid fills it.  148 multiprocessors:
     // Four layers with outputs, 8 -> 16 loads: 448 CTAs (512 rows over 200 groups) 467 -> 440 us, 896 CTAs (1024 rows) 799 -> 805,
     // 1280 CTAs 1132 -> 1177, 4096 CTAs (1000 groups) 3735 -> 3817; averages only, 896 CTAs 597 -> 602.
-    constexpr unsigned kFewCtas = 4 * 148;
-    const bool few = static_cast<unsigned long long>(grid.x) * grid.y <= kFewCtas;
+    const bool few = static_cast<long long>(grid.x) * grid.y <= 4ll * n_sm;
     auto launch = [&](auto loads) {
         constexpr int kLoads = decltype(loads)::value;
         if (p.n_splits > 1)

@@ -1190,7 +1190,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         fp.sum_stride = a->sum_stride;
         fp.n_splits = mass_only ? p.n_splits : 1;
         fp.max_slots = c->plan_max_slots;
-        if (launch_mass_finish(fp, st) != cudaSuccess) { cudaGetLastError(); return ENL_E_CUDA; }
+        if (launch_mass_finish(fp, c->n_sm, st) != cudaSuccess) { cudaGetLastError(); return ENL_E_CUDA; }
     }
     if (scratch_merge) {
         CombineParams cp;

@@ -231,7 +231,8 @@ struct FinishParams {
     int32_t n_q_total, Hq, mass_stride, sum_stride, n_splits, max_slots;
 };
 constexpr int kFinishSplits = 8;
-cudaError_t launch_mass_finish(const FinishParams &p, cudaStream_t st);
+// n_sm: multiprocessors of the device
+cudaError_t launch_mass_finish(const FinishParams &p, int n_sm, cudaStream_t st);
 
 // Tensor map of a caller's [n][Hkv][D] bf16 keys or values with boxes of eight rows of a head (in enl_host.cu)
 bool encode_key_map(CUtensorMap *tm, const void *base, int D, int Hkv, int n);

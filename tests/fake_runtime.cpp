@@ -130,7 +130,7 @@ cudaError_t launch_mass(const MassParams &p, int, int, cudaStream_t) { return no
 cudaError_t launch_small(const SmallParams &p, int, int, int, int, cudaStream_t) { return note('a', p.wait_first); }
 cudaError_t launch_decode(const DecodeParams &p, int, int, cudaStream_t) { return note('d', p.wait_first); }
 cudaError_t launch_combine(const CombineParams &, cudaStream_t) { return note('b', 0); }
-cudaError_t launch_mass_finish(const FinishParams &, cudaStream_t) { return note('f', 0); }
+cudaError_t launch_mass_finish(const FinishParams &, int, cudaStream_t) { return note('f', 0); }
 cudaError_t launch_plan_write(void *, const void *, size_t bytes, cudaStream_t) { return note('w', 0, bytes); }
 cudaError_t launch_page_scatter(void *, void *, const void *, const void *, const PageRun &, int, int, int, int, int, int, cudaStream_t) { return note('s', 0); }
 cudaError_t launch_page_scatter_layers(void *, void *, size_t, int, int, const LayerSrc &, size_t, const PageRun &, int, int, int, int, int, int,

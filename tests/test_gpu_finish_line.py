@@ -1,4 +1,4 @@
-"""Masses finished by a launch of their own, just below and above the grid size (592 CTAs) where it keeps sixteen or eight loads in flight:
+"""Masses finished by a launch of their own, just below and above the grid size (four CTAs per multiprocessor) where it keeps sixteen or eight loads in flight:
 with outputs (no splits), without (key ranges split), with the objects' sums."""
 import pytest
 import torch
@@ -10,8 +10,10 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("mass_only", [False, True])
-@pytest.mark.parametrize("n_q", [941, 944, 945])            # 590 CTAs (a ragged and a full last one) and 595
-def test_masses_around_the_line(n_q, mass_only):
+@pytest.mark.parametrize("over", [-3, 0, 1])                # the last row block below the line ragged or full; a row beyond it
+def test_masses_around_the_line(over, mass_only):
+    # a CTA finishes 8 rows x 32 heads and 32 slots, so five CTAs are one row block over the 131 slots
+    n_q = 4 * torch.cuda.get_device_properties(0).multi_processor_count // 5 * 8 + over
     sizes = [1 + (i * 5) % 3 for i in range(130)]           # five slot blocks
     wl = synth.make_small(73, 1, 32, 8, 64, [sizes], [list(range(130))], [n_q], [n_q], name="finish")
     cuts = [0, 1, n_q // 3, n_q - 40]                       # the last rows belong to no object
