@@ -722,9 +722,11 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         const int tpc = tokens_per_cta(c);
         int64_t n_entries = 0, base_items = 0, half_items = 0;      // CTAs of two Q tiles, of one
         int min_tiles = 0x7fffffff, max_tiles = 1, max_rows = 1;
+        int64_t min_steps = 0x7fffffff, min_half_steps = 0x7fffffff;       // fewest steps of 64 keys that a CTA of either form walks
         for (int b = 0; b < B; ++b) {
             int64_t e = 0;
             for (int s = cu_sel[b]; s < cu_sel[b + 1]; ++s) e += std::max(1, ceil_div(sel_len[s], kPageTokens));
+            const int64_t cached_steps = (e + kStepKeys / kPageTokens - 1) / (kStepKeys / kPageTokens);
             e = (e + kPagesPerTile - 1) / kPagesPerTile * kPagesPerTile;
             n_entries += e;
             const int nq = cu_q[b + 1] - cu_q[b], nn = cu_new[b + 1] - cu_new[b];
@@ -732,6 +734,9 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
             half_items += static_cast<int64_t>(ceil_div(nq, tokens_per_cta(c, true))) * d.n_kv_heads;
             // fewest tiles any CTA of this episode walks: its first token block
             const int c_first = nn - nq + std::min(tpc, nq) - 1;
+            const int c_half = nn - nq + std::min(tokens_per_cta(c, true), nq) - 1;
+            min_steps = std::min<int64_t>(min_steps, cached_steps + c_first / kStepKeys + 1);
+            min_half_steps = std::min<int64_t>(min_half_steps, cached_steps + c_half / kStepKeys + 1);
             min_tiles = std::min<int64_t>(min_tiles, e / kPagesPerTile + c_first / kTileKeys + 1);
             max_tiles = std::max<int64_t>(max_tiles, e / kPagesPerTile + (nn - 1) / kTileKeys + 1);
             max_rows = std::max(max_rows, std::min(nq, tpc) * c->rep);
@@ -871,6 +876,10 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
             n_splits = std::min<int64_t>(n_splits, std::max<int64_t>(1, c->cap_items / (halves ? half_items : base_items)));
             halves = halves && half_items <= c->cap_items;
             n_splits = std::min(n_splits, kMaxSplits);
+            // Every CTA walks a step at least: attn_kernel writes nothing for a range without keys.  (The bounds above see to it already: a
+            // first block of one Q tile sees at most 128 new keys less than one of two, and what is left has at least as many steps of 64
+            // keys as the longer one has tiles of 128.)
+            if (!mass_only) n_splits = static_cast<int>(std::min<int64_t>(n_splits, halves ? min_half_steps : min_steps));
             while (n_splits > 1 && !mass_only && !fits(n_splits)) --n_splits;
         }
 

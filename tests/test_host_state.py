@@ -183,3 +183,40 @@ def test_captured_store_is_waited_for_whenever_its_graph_may_have_run(host, rout
     assert c.waits(route)[0] == 1 and c.waits(route, layer=1) == (0, False)
     host.fake_capture(0)
     assert c.waits(route)[0] == 1
+
+
+@pytest.mark.parametrize("heads", [(1, 1), (2, 1), (4, 1), (8, 1), (16, 1), (8, 2), (32, 8)])
+@pytest.mark.parametrize("D", [64, 128])
+def test_no_cta_without_keys(host, heads, D):
+    """The attention kernel writes nothing for a range of keys without a step of 64: no plan has one, in whichever form."""
+    hq, hkv = heads
+    h = ctypes.c_void_p()
+    d = enl.CacheDesc(1, hq, hkv, D, 0, 4, 8192, enl.ENL_BF16, 0, 4, 2048, 0)
+    assert host.enl_cache_create(ctypes.byref(d), ctypes.byref(h)) == enl.ENL_OK
+    halves = 0
+    for n in (1, 16, 60, 70, 130, 1000):
+        assert host.enl_group_store(h, 0, 0, n, ctypes.c_void_p(1 << 20), ctypes.c_void_p(1 << 21), 0, None) == enl.ENL_OK
+        for n_q in (2, 17, 63, 64, 65, 127, 128, 129, 255, 256, 257, 500):
+            for prior in (0, 1, 63, 64, 65, 127, 128, 129):
+                for hint in (0, 64):
+                    for n_sel in (0, 1):
+                        ids = np.zeros(1, np.int32)
+                        a = enl.AttendArgs()
+                        a.batch, a.n_sel, a.n_q, a.n_new, a.split_hint, a.sel_ids = 1, n_sel, n_q, n_q + prior, hint, ids.ctypes.data
+                        a.q, a.k_new, a.v_new, a.out, a.group_mass = ((1 << 20) * i for i in range(1, 6))
+                        a.mass_stride, a.flags = 2, enl.ENL_PLAN_ONLY
+                        assert host.enl_attend(h, ctypes.byref(a), None) == enl.ENL_OK
+                        out = [ctypes.c_int32() for _ in range(4)]
+                        assert host.enl_plan_inspect(h, 0, None, None, ctypes.byref(out[0]), 0, None, None, *(ctypes.byref(x) for x in out[1:])) == enl.ENL_OK
+                        _, n_splits, n_items, kind = (x.value for x in out)
+                        tile = 128 // (hq // hkv)
+                        if n_items != -(-n_q // (2 * tile)) * hkv * n_splits or kind == 3:
+                            if kind == 3 or n_items == 0:
+                                continue
+                            assert n_items == -(-n_q // tile) * hkv * n_splits
+                            halves += 1
+                        first = min(tile, n_q)                  # the fewest rows a first block may have
+                        pages = -(-n // 16) if n_sel else 0
+                        assert n_splits <= -(-pages // 4) + (prior + first - 1) // 64 + 1, (n, n_q, prior, hint, n_sel)
+    assert halves > 0
+    host.enl_cache_free(h)
