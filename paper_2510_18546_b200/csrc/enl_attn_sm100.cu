@@ -628,6 +628,18 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                 slots[sl] = w;
             }
         };
+        // Slots [from, to) of the warp's rows in the partial results: a row at a time, lanes over the slots.  (A thread per row, whose
+        // stores of a warp lie in 32 rows, took the masses of 128 rows over 400 groups in 17 splits, 8 heads, from 56 to 81 us.)
+        auto clear_slots = [&](int from, int to) {
+            __syncwarp();
+#pragma unroll 1
+            for (int rr = 0; rr < 32; ++rr) {
+                const int ri = __shfl_sync(kFull, my_ridx, rr);
+                if (ri < 0) continue;
+                float *slots = p.part_slot + static_cast<long long>(ri) * p.mass_stride;
+                for (int sl = from + lane; sl < to; sl += 32) slots[sl] = kNegInf;
+            }
+        };
         // slots this walker walked (all of them where nothing is split)
         int first_slot = 0, last_slot = G;
         if (p.n_splits > 1 || two_halves) {
@@ -668,13 +680,14 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
             merge_rows(rows[(i ^ 1) * 128 + r]);
             if (split_mode) {
                 if (i == 0 && row_valid) p.part_lse[rh] = row_lse;
-                if (slot_out) {                                      // slots that this split did not walk contribute nothing
-                    for (int sl = i == 0 ? 0 : first_slot; sl <= (i == 0 ? last_slot : G); ++sl) {
-                        if (sl == skip_slot) continue;
-                        if (sl < first_slot || sl > last_slot) slot_out[sl] = kNegInf;
-                        else if (sl == shared_slot) slot_out[sl] = shared_log();
-                        else if (park_smem) slot_out[sl] = park_row[sl * 128];
-                    }
+                if (park_smem) {                                     // slots that this split did not walk contribute nothing
+                    if (slot_out)
+                        for (int sl = i == 0 ? 0 : first_slot; sl <= (i == 0 ? last_slot : G); ++sl)
+                            if (sl != skip_slot)
+                                slot_out[sl] = (sl < first_slot || sl > last_slot) ? kNegInf : sl == shared_slot ? shared_log() : park_row[sl * 128];
+                } else if (p.part_slot) {
+                    if (slot_out && i == 0 && shared_slot >= 0) slot_out[shared_slot] = shared_log();
+                    clear_slots(i == 0 ? 0 : last_slot + 1, i == 0 ? first_slot : G + 1);
                 }
             } else if (p.mass) {
                 if (park_smem) {
@@ -761,16 +774,9 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                     if (slot_out)
                         for (int sl = 0; sl <= G; ++sl)
                             slot_out[sl] = (sl < first_slot || sl > last_slot) ? kNegInf : park_row[sl * 128];
-                } else if (p.part_slot) {
-                    __syncwarp();
-#pragma unroll 1
-                    for (int rr = 0; rr < 32; ++rr) {               // slots this split did not walk contribute nothing
-                        const int ri = __shfl_sync(kFull, my_ridx, rr);
-                        if (ri < 0) continue;
-                        float *slots = p.part_slot + static_cast<long long>(ri) * p.mass_stride;
-                        for (int sl = lane; sl <= G; sl += 32)
-                            if (sl < first_slot || sl > last_slot) slots[sl] = kNegInf;
-                    }
+                } else if (p.part_slot) {                           // slots this split did not walk contribute nothing
+                    clear_slots(0, first_slot);
+                    clear_slots(last_slot + 1, G + 1);
                 }
                 if (n_steps > 0) {
                     const float inv = (l > 0.f) ? 1.f / l : 0.f;
