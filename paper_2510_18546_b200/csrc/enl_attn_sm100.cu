@@ -401,6 +401,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
             else if (p.mass) slot_out = p.mass + rh * p.mass_stride;
         }
         const bool park_smem = p.park_smem != 0;
+        const bool want_slots = (split_mode ? p.part_slot : p.mass) != nullptr;
+        float *slot_global = park_smem ? nullptr : slot_out;
         float *park_row = reinterpret_cast<float *>(smem + C::kParkOff) + i * (kParkSlots * 128) + r;   // + slot * 128; (each walker its own slots)
         const float scale = p.scale_log2;
 
@@ -416,15 +418,18 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
             if (last0 == first1) { shared_slot = last0; if ((two_halves ? i : it.split) == 1) skip_slot = last0; }
         }
         float m = kNegInf, l = 0.f, acc = 0.f;                     // reference (log2 units), row sum, sum of the current slot
-        int cur_slot = -1;
-        // the slot that ends parks its log2-sum-exp
-        auto park = [&](float m_ref) {
-            if (cur_slot >= 0) {
-                const float v = lg2(acc) + m_ref;
-                if (cur_slot == skip_slot) bnd = v;
-                else if (park_smem) park_row[cur_slot * 128] = v;
-                else if (slot_out) slot_out[cur_slot] = v;
-            }
+        int cur_slot = 0;
+        // The slot that ends (if `ends`, the same for the whole warp) parks its log2-sum-exp; the one behind it is the next in the list, since
+        // every slot has a page.  Predicated stores and no shuffle: what comes back through the queue of the special-function unit, which the
+        // other tile's warp keeps full, costs a hundred cycles and more.  (Branches with a shuffle and a logarithm per slot: 310 cycles of a
+        // step of 1950, groups of two pages; 600 rows over 400 such groups 282 -> 256 us.  Slots staged in shared memory and written out a row
+        // at a time: 330.  Without masses nothing is parked: 266 -> 237.)
+        auto park = [&](bool ends, float v) {
+            const bool mine = ends && cur_slot != skip_slot;
+            if (mine && park_smem) park_row[cur_slot * 128] = v;
+            if (mine && slot_global) slot_global[cur_slot] = v;
+            bnd = ends && !mine ? v : bnd;
+            cur_slot += ends ? 1 : 0;
         };
 
         // Slots of 32 pages at a time, one per lane, fetched eight steps ahead, and a warp-uniform mask of those pages whose slot differs
@@ -434,7 +439,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
             const int e = (j0 + jj) * kStepPages + lane;
             return e < n_csteps * kStepPages ? __ldg(p.stream_meta + ep.stream_off + e) >> 8 : G;
         };
-        int slots = -1, slots_next = load_slots(0);
+        int slots_next = load_slots(0), slots = __shfl_sync(kFull, slots_next, 0);
+        cur_slot = slots;
         uint32_t changes = 0;
         // The two warps that share a scheduler (one of each tile) take their exponentials in turns: both at once leave its special-function
         // unit idle while both do the rest.  (Named barriers 1..8: (tile, quadrant) may begin.)
@@ -454,7 +460,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                 slots_next = load_slots(jj + kBatch);
                 int prev = __shfl_up_sync(kFull, slots, 1);
                 if (lane == 0) prev = last;
-                changes = __ballot_sync(kFull, slots != prev);
+                changes = want_slots ? __ballot_sync(kFull, slots != prev) : 0u;
             }
             const uint32_t chg_mask = (changes >> (jj % kBatch * kStepPages)) & ((1u << kStepPages) - 1u);
 
@@ -567,12 +573,9 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
             } else {
 #pragma unroll
                 for (int e = 0; e < kStepPages; ++e) {
-                    if ((chg_mask >> e) & 1u) {
-                        park(m_use);
-                        acc = 0.f;
-                        cur_slot = __shfl_sync(kFull, slots, jj % kBatch * kStepPages + e);
-                    }
-                    acc += ps[e];
+                    const bool ends = (chg_mask >> e) & 1u;
+                    park(ends, lg2(acc) + m_use);
+                    acc = (ends ? 0.f : acc) + ps[e];
                 }
             }
         }
@@ -628,18 +631,6 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                 slots[sl] = w;
             }
         };
-        // Slots [from, to) of the warp's rows in the partial results: a row at a time, lanes over the slots.  (A thread per row, whose
-        // stores of a warp lie in 32 rows, took the masses of 128 rows over 400 groups in 17 splits, 8 heads, from 56 to 81 us.)
-        auto clear_slots = [&](int from, int to) {
-            __syncwarp();
-#pragma unroll 1
-            for (int rr = 0; rr < 32; ++rr) {
-                const int ri = __shfl_sync(kFull, my_ridx, rr);
-                if (ri < 0) continue;
-                float *slots = p.part_slot + static_cast<long long>(ri) * p.mass_stride;
-                for (int sl = from + lane; sl < to; sl += 32) slots[sl] = kNegInf;
-            }
-        };
         // slots this walker walked (all of them where nothing is split)
         int first_slot = 0, last_slot = G;
         if (p.n_splits > 1 || two_halves) {
@@ -651,6 +642,20 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                 last_slot = (je > n_csteps) ? G : (__ldg(p.stream_meta + ep.stream_off + je * kStepPages - 1) >> 8);
             }
         }
+        // Slots of the warp's rows in the partial results, those in [from, to) that were not walked: a row at a time, lanes over the slots.
+        // (A thread per row, whose stores of a warp lie in 32 rows, took the masses of 128 rows over 400 groups in 17 splits, 8 heads,
+        // from 56 to 81 us.)
+        auto clear_slots = [&](int from, int to) {
+            __syncwarp();
+#pragma unroll 1
+            for (int rr = 0; rr < 32; ++rr) {
+                const int ri = __shfl_sync(kFull, my_ridx, rr);
+                if (ri < 0) continue;
+                float *slots = p.part_slot + static_cast<long long>(ri) * p.mass_stride;
+                for (int sl = from + lane; sl < to; sl += 32)
+                    if (sl < first_slot || sl > last_slot) slots[sl] = kNegInf;
+            }
+        };
         // The merged row: what a walker or a CTA of a pair makes of its own (m_use, l) and the other's (x, y of pe)
         float row_lse = lse, other_bnd = kNegInf, w_own = 0.f, w_other = 0.f;
         auto merge_rows = [&](const float4 &pe) {
@@ -673,7 +678,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
         if (two_halves) {
             // ---- the walkers tell each other (reference, sum, part of the slot in which they meet) of every row; each goes on with its
             // own slots and half of the channels, whose accumulators both lie in the TMEM lanes it reads ----
-            if (ok) park(m_use);
+            if (ok) park(true, lg2(acc) + m_use);
             float4 *rows = reinterpret_cast<float4 *>(smem + C::kXpeerOff);
             rows[i * 128 + r] = make_float4(m_use, ok ? l : 0.f, bnd, 0.f);
             asm volatile("bar.sync 9, 256;" ::: "memory");           // reached whatever happened (the waits are bounded)
@@ -741,7 +746,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
         }
         bool exported = false;
         if (ok && !two_halves) {
-            park(m_use);
+            park(n_mine > 0, lg2(acc) + m_use);
             if (!pair && !split_mode) {
                 // ---- the whole key stream was this CTA's: output and masses ----
                 if (p.mass) {
@@ -775,8 +780,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                         for (int sl = 0; sl <= G; ++sl)
                             slot_out[sl] = (sl < first_slot || sl > last_slot) ? kNegInf : park_row[sl * 128];
                 } else if (p.part_slot) {                           // slots this split did not walk contribute nothing
-                    clear_slots(0, first_slot);
-                    clear_slots(last_slot + 1, G + 1);
+                    clear_slots(0, G + 1);
                 }
                 if (n_steps > 0) {
                     const float inv = (l > 0.f) ? 1.f / l : 0.f;
