@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(kThreads, 1) mass_kernel(const __grid_constant
                 words(jj + kBatch, id_next, meta_next);
             }
             const int at = jj % kBatch * kPagesPerTile + lane % kPagesPerTile;
-            const int row8 = (__shfl_sync(kFull, id_cur, at) * p.Hkv + it.kvh) * 2, valid = __shfl_sync(kFull, meta_cur, at) & 0xff;
+            const int group = (__shfl_sync(kFull, id_cur, at) * p.Hkv + it.kvh) * kPageGroups<D>, valid = __shfl_sync(kFull, meta_cur, at) & 0xff;
             if (jj >= C::kStages) {
                 ok = mbar_wait(bar_k_empty(st), static_cast<uint32_t>((jj / C::kStages - 1) & 1), abort_flag, p.status);
                 if (!ok) break;
@@ -180,10 +180,10 @@ __global__ void __launch_bounds__(kThreads, 1) mass_kernel(const __grid_constant
             __syncwarp();
             if (cached) {
                 if (lane < kPagesPerTile)
-                    tma_load_4d(stage_addr(st) + static_cast<uint32_t>(lane * 2 * C::kGroupBytes), &p.tm_kpool, 0, 0, 0, row8, bar_k_full(st));
-            } else if (lane < kTileKeys / 8) {
-                tma_load_4d(stage_addr(st) + static_cast<uint32_t>(lane * C::kGroupBytes), &p.tm_knew, 0,
-                            ep.new_off + (j - ep.n_ctiles) * kTileKeys + lane * 8, 0, it.kvh, bar_k_full(st));
+                    tma_load_4d(stage_addr(st) + static_cast<uint32_t>(lane * 2 * C::kGroupBytes), &p.tm_kpool, 0, 0, 0, group, bar_k_full(st));
+            } else if (lane < kTileKeys / kBoxRows<D>) {
+                tma_load_4d(stage_addr(st) + static_cast<uint32_t>(lane * (kBoxRows<D> * D * 2)), &p.tm_knew, 0,
+                            ep.new_off + (j - ep.n_ctiles) * kTileKeys + lane * kBoxRows<D>, 0, it.kvh, bar_k_full(st));
             }
         }
         // error path only: let the copies already in flight land before the CTA retires

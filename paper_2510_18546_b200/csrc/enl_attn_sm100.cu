@@ -204,9 +204,10 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
     if (producer && n_steps > 0 && static_cast<int>(blockIdx.x) < p.first_wave) {
         if (warp == kKWarp && lane < n_qt * C::kHalves)
             tma_prefetch_3d(&p.tm_q, (lane % C::kHalves) * 64, it.kvh * rep, ep.q_off + it.t0 + (lane / C::kHalves) * tile_tokens);
-        const int vn = lane / (kStepKeys / 8), jn = step_of(vn);     // eight rows a box
+        constexpr int kBoxes = kStepKeys / kBoxRows<D>;              // of a step
+        const int vn = lane / kBoxes, jn = step_of(vn);
         if (vn < min(C::kRing, n_steps) && jn >= n_csteps)
-            tma_prefetch_4d(warp == kKWarp ? &p.tm_knew : &p.tm_vnew, 0, ep.new_off + (jn - n_csteps) * kStepKeys + lane % (kStepKeys / 8) * 8, 0, it.kvh);
+            tma_prefetch_4d(warp == kKWarp ? &p.tm_knew : &p.tm_vnew, 0, ep.new_off + (jn - n_csteps) * kStepKeys + lane % kBoxes * kBoxRows<D>, 0, it.kvh);
     }
     if (!producer) pdl_wait();
 
@@ -261,7 +262,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                 }
                 if (!waited && (v >= early || j >= n_csteps)) wait_previous();
                 const int pg = lane % kStepPages, at = jj % kBatch * kStepPages;
-                const int row8 = (__shfl_sync(kFull, i ? cur1.id : cur0.id, at + pg) * p.Hkv + it.kvh) * 2;
+                const int group = (__shfl_sync(kFull, i ? cur1.id : cur0.id, at + pg) * p.Hkv + it.kvh) * kPageGroups<D>;
                 const int valid = __shfl_sync(kFull, i ? cur1.meta : cur0.meta, at + pg) & 0xff;
                 if (v >= C::kRing) ok = mbar_wait(empty0 + 8u * x, static_cast<uint32_t>((v / C::kRing - 1) & 1), abort_flag, p.status);
                 if (!ok) break;
@@ -282,10 +283,10 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                 }
                 if (lane == 0) mbar_expect_tx(full, static_cast<uint32_t>(C::kStepBytes));
                 if (j < n_csteps) {
-                    if (lane < kStepPages) tma_load_4d(dst + static_cast<uint32_t>(lane * 2 * C::kGroupBytes), tm_pool, 0, 0, 0, row8, full);
-                } else if (lane < 8) {
-                    tma_load_4d(dst + static_cast<uint32_t>(lane * C::kGroupBytes), tm_new, 0,
-                                ep.new_off + (j - n_csteps) * kStepKeys + lane * 8, 0, it.kvh, full);
+                    if (lane < kStepPages) tma_load_4d(dst + static_cast<uint32_t>(lane * 2 * C::kGroupBytes), tm_pool, 0, 0, 0, group, full);
+                } else if (lane < kStepKeys / kBoxRows<D>) {
+                    tma_load_4d(dst + static_cast<uint32_t>(lane * (kBoxRows<D> * D * 2)), tm_new, 0,
+                                ep.new_off + (j - n_csteps) * kStepKeys + lane * kBoxRows<D>, 0, it.kvh, full);
                 }
                 ++fetched;
             }

@@ -126,13 +126,13 @@ __global__ void __launch_bounds__(kThreads, 1) small_kernel(const __grid_constan
         mbar_expect_tx(full, 2u * C::kStageBytes);
         // (no evict-first hint: the row blocks of a kv head share its pages)
         if (pg >= 0) {
-            tma_load_4d(dst, &p.tm_kpool, 0, 0, 0, (pg * p.Hkv + kvh) * 2, full);
-            tma_load_4d(dst + C::kStageBytes, &p.tm_vpool, 0, 0, 0, (pg * p.Hkv + kvh) * 2, full);
+            tma_load_4d(dst, &p.tm_kpool, 0, 0, 0, (pg * p.Hkv + kvh) * kPageGroups<D>, full);
+            tma_load_4d(dst + C::kStageBytes, &p.tm_vpool, 0, 0, 0, (pg * p.Hkv + kvh) * kPageGroups<D>, full);
         } else {
 #pragma unroll
-            for (int x = 0; x < 4; ++x)                                       // eight rows of K or V
-                tma_load_4d(dst + static_cast<uint32_t>(x * (C::kStageBytes / 2)), x < 2 ? &p.tm_knew : &p.tm_vnew, 0,
-                            ep.new_off + (-1 - pg) + (x & 1) * 8, 0, kvh, full);
+            for (int x = 0; x < 2 * kPageGroups<D>; ++x)                      // a group of rows of K or V
+                tma_load_4d(dst + static_cast<uint32_t>(x * (C::kStageBytes / kPageGroups<D>)), x < kPageGroups<D> ? &p.tm_knew : &p.tm_vnew, 0,
+                            ep.new_off + (-1 - pg) + x % kPageGroups<D> * kBoxRows<D>, 0, kvh, full);
         }
     };
     // page i is fetched by lane 0 of warp i % kWarps: the cached ones while the previous kernel still runs

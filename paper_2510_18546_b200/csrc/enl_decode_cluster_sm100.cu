@@ -207,12 +207,12 @@ __global__ void __launch_bounds__(kThreads, 2)
         mbar_expect_tx(full, static_cast<uint32_t>(C::kStageBytes));
         if (!kStatic && page >= 0) {
             const CUtensorMap *tm = is_v ? &p.tm_vpool : &p.tm_kpool;
-            tma_load_4d(dst, tm, 0, 0, 0, (page * p.Hkv + kvh) * 2, full, pol);
+            tma_load_4d(dst, tm, 0, 0, 0, (page * p.Hkv + kvh) * kPageGroups<D>, full, pol);
         } else {
             const CUtensorMap *tm = is_v ? &p.tm_vnew : &p.tm_knew;
             const int krow = ep.new_off + (-1 - page);                       // rows past the tensor's end read as zero
             tma_load_4d(dst, tm, 0, krow, 0, kvh, full, pol);
-            tma_load_4d(dst + C::kStageBytes / 2, tm, 0, krow + 8, 0, kvh, full, pol);
+            if constexpr (kPageGroups<D> == 2) tma_load_4d(dst + C::kStageBytes / 2, tm, 0, krow + kBoxRows<D>, 0, kvh, full, pol);
         }
     };
     // While the previous kernel of the stream still runs: the pool is written by launches of this library only, and none has
@@ -270,9 +270,10 @@ __global__ void __launch_bounds__(kThreads, 2)
     for (int i = warp; i < min(n_cta, kPrefetchPages); i += kWarps) {
         const int pg = pg_list[i].x;
         if (pg < 0) {
-            if (lane < 4) tma_prefetch_4d((lane & 1) ? &p.tm_vnew : &p.tm_knew, 0, ep.new_off + (-1 - pg) + (lane >> 1) * 8, 0, kvh);
+            if (lane < 2 * kPageGroups<D>)
+                tma_prefetch_4d((lane & 1) ? &p.tm_vnew : &p.tm_knew, 0, ep.new_off + (-1 - pg) + (lane >> 1) * kBoxRows<D>, 0, kvh);
         } else if (i >= kWarps && lane < 2) {
-            tma_prefetch_4d((lane & 1) ? &p.tm_vpool : &p.tm_kpool, 0, 0, 0, (pg * p.Hkv + kvh) * 2);
+            tma_prefetch_4d((lane & 1) ? &p.tm_vpool : &p.tm_kpool, 0, 0, 0, (pg * p.Hkv + kvh) * kPageGroups<D>);
         }
     }
     const uint8_t *q_rows = static_cast<const uint8_t *>(p.q) + (static_cast<long long>(ep.q_off) * p.Hq + kvh * rep) * D * 2;

@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(const __grid_consta
         const int n_pf = min(n_cta, kPrefetchPages);
         for (int i = threadIdx.x; i < n_pf * 2; i += kThreads) {
             const int pg = pg_list[i / 2].x;
-            if (pg >= 0) tma_prefetch_4d((i & 1) ? &p.tm_vpool : &p.tm_kpool, 0, 0, 0, (pg * p.Hkv + it.kvh) * 2);
+            if (pg >= 0) tma_prefetch_4d((i & 1) ? &p.tm_vpool : &p.tm_kpool, 0, 0, 0, (pg * p.Hkv + it.kvh) * kPageGroups<D>);
         }
     }
 
@@ -197,12 +197,12 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(const __grid_consta
         mbar_expect_tx(full, static_cast<uint32_t>(C::kStageBytes));
         if (page >= 0) {
             const CUtensorMap *tm = is_v ? &p.tm_vpool : &p.tm_kpool;
-            tma_load_4d(dst, tm, 0, 0, 0, (page * p.Hkv + it.kvh) * 2, full, pol);
+            tma_load_4d(dst, tm, 0, 0, 0, (page * p.Hkv + it.kvh) * kPageGroups<D>, full, pol);
         } else {
             const CUtensorMap *tm = is_v ? &p.tm_vnew : &p.tm_knew;
             const int krow = ep.new_off + (-1 - page) * kPageTokens;         // rows past the tensor's end read as zero
             tma_load_4d(dst, tm, 0, krow, 0, it.kvh, full, pol);
-            tma_load_4d(dst + C::kStageBytes / 2, tm, 0, krow + 8, 0, it.kvh, full, pol);
+            if constexpr (kPageGroups<D> == 2) tma_load_4d(dst + C::kStageBytes / 2, tm, 0, krow + kBoxRows<D>, 0, it.kvh, full, pol);
         }
     };
     // the next page of the CTA that nobody has taken yet (CTA-relative index; >= n_cta: none left)

@@ -121,14 +121,14 @@ struct MapCache {
     }
 };
 
-// a caller's [n][Hkv][D] keys or values, fetched by eight rows of a head
+// a caller's [n][Hkv][D] keys or values, fetched by a few rows of a head
 struct KeyMapShape {
     cuuint64_t dims[4], strides[3];
     cuuint32_t box[4];
     KeyMapShape(int D, int Hkv, int n)
         : dims{64, static_cast<cuuint64_t>(n), static_cast<cuuint64_t>(D / 64), static_cast<cuuint64_t>(Hkv)},
           strides{static_cast<cuuint64_t>(D) * 2 * Hkv, 128, static_cast<cuuint64_t>(D) * 2},
-          box{64, 8, static_cast<cuuint32_t>(D / 64), 1} {}
+          box{64, static_cast<cuuint32_t>(box_rows(D)), static_cast<cuuint32_t>(D / 64), 1} {}
 };
 
 }  // namespace
@@ -364,9 +364,10 @@ extern "C" int enl_cache_create(const enl_cache_desc_t *desc, enl_cache_t **out)
     c->tm_k.resize(d.n_layers);
     c->tm_v.resize(d.n_layers);
     const cuuint64_t row = static_cast<cuuint64_t>(d.head_dim) * 2;
-    const cuuint64_t dims[4] = {64, 8, static_cast<cuuint64_t>(d.head_dim / 64), static_cast<cuuint64_t>(c->n_pages) * d.n_kv_heads * (kPageTokens / 8)};
-    const cuuint64_t strides[3] = {row, 128, row * 8};
-    const cuuint32_t box[4] = {64, 8, static_cast<cuuint32_t>(d.head_dim / 64), kPageTokens / 8};
+    const cuuint32_t group = box_rows(d.head_dim), page_groups = kPageTokens / group;
+    const cuuint64_t dims[4] = {64, group, static_cast<cuuint64_t>(d.head_dim / 64), static_cast<cuuint64_t>(c->n_pages) * d.n_kv_heads * page_groups};
+    const cuuint64_t strides[3] = {row, 128, row * group};
+    const cuuint32_t box[4] = {64, group, static_cast<cuuint32_t>(d.head_dim / 64), page_groups};
     for (int l = 0; l < d.n_layers; ++l) {
         if (!encode_map(&c->tm_k[l], c->kpool + c->layer_bytes * l, 4, dims, strides, box) ||
             !encode_map(&c->tm_v[l], c->vpool + c->layer_bytes * l, 4, dims, strides, box)) {

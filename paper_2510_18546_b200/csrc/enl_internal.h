@@ -7,7 +7,7 @@
 
 namespace enl {
 
-constexpr int kPageTokens = 16;     // tokens per page: one TMA box of 16 rows x 128 B per 64 channels
+constexpr int kPageTokens = 16;     // tokens per page: one TMA box per kv head (see below)
 constexpr int kTileKeys   = 128;    // keys per KV tile (8 pages)
 constexpr int kPagesPerTile = kTileKeys / kPageTokens;
 constexpr int kStepKeys   = 64;     // keys that attn_kernel takes at once
@@ -34,16 +34,21 @@ struct Item {
 };
 
 // How keys and values are fetched: by boxes that leave one swizzled block of 8 rows x 128 bytes per 64 channels, and then the next 8 rows.
-//   pool (a layer), dims {64 channels, 8 rows, D/64 blocks, groups of 8 rows}, box {64, 8, D/64, 2}: a page of a kv head, 16 D contiguous
-//     values, in one box
-//   a caller's [n][Hkv][D], dims {64 channels, n rows, D/64 blocks, Hkv heads}, box {64, 8, D/64, 1}: eight rows of a head
+// With R = kBoxRows, the rows of 64 channels that lie behind one another in such a box (8, at head_dim 64 all 16 of a page):
+//   pool (a layer), dims {64 channels, R rows, D/64 blocks, groups of R rows}, box {64, R, D/64, 16/R}: a page of a kv head, 16 D contiguous
+//     values, in one box; its last coordinate is (page * Hkv + head) * kPageGroups
+//   a caller's [n][Hkv][D], dims {64 channels, n rows, D/64 blocks, Hkv heads}, box {64, R, D/64, 1}: R rows of a head
 // A box costs the warp that asks for it some 50 cycles, so a box of half as much (64 channels of a page, as a two-dimensional map gives
-// them) had every producer take twice as long.
+// them) had every producer take twice as long.  (Groups of eight at head_dim 64, too, are up to 4 % slower: one token over two streams of
+// 16000 keys, 8 kv heads, 19.0 against 19.7 us.)
+constexpr int box_rows(int D) { return 1024 / D; }
+template <int D> constexpr int kBoxRows = box_rows(D);
+template <int D> constexpr int kPageGroups = kPageTokens / kBoxRows<D>;
 
 // Kernel parameters (passed by value as a __grid_constant__).
 struct AttnParams {
     CUtensorMap tm_q;       // [n_q][Hq][D]      box {64, rep, 128/rep}
-    CUtensorMap tm_knew;    // [n_new][Hkv][D]: eight rows of a head (see above)
+    CUtensorMap tm_knew;    // [n_new][Hkv][D]: rows of a head (see above)
     CUtensorMap tm_vnew;
     CUtensorMap tm_kpool;   // one layer: a page of a head
     CUtensorMap tm_vpool;
@@ -234,7 +239,7 @@ constexpr int kFinishSplits = 8;
 // n_sm: multiprocessors of the device
 cudaError_t launch_mass_finish(const FinishParams &p, int n_sm, cudaStream_t st);
 
-// Tensor map of a caller's [n][Hkv][D] bf16 keys or values with boxes of eight rows of a head (in enl_host.cu)
+// Tensor map of a caller's [n][Hkv][D] bf16 keys or values with boxes of box_rows(D) rows of a head (in enl_host.cu)
 bool encode_key_map(CUtensorMap *tm, const void *base, int D, int Hkv, int n);
 
 // launchers (defined in the .cu files of the kernels)
