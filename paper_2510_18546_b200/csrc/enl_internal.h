@@ -256,7 +256,7 @@ cudaError_t prepare_small(int head_dim);
 // row_groups: 1, 2 or 4 groups of 16 query rows (tokens x q heads of a kv head) per CTA
 cudaError_t launch_small(const SmallParams &p, int head_dim, int row_groups, int row_blocks, int batch, cudaStream_t st);
 int decode_cluster_smem(int head_dim, int list_pages, int list_slots, int rep);
-constexpr int kClusterPairSmem = 113800;      // two CTAs of up to this much fit an SM
+constexpr int kClusterPairSmem = 115712;      // two CTAs of up to this much fit an SM (228 KB, of which a CTA takes 1 KB for itself)
 // How many clusters of 2^i CTAs the current device runs at once: with two CTAs per SM, and with one (larger lists).
 struct ClusterCaps {
     int two[5], one[5];
