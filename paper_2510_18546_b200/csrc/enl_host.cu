@@ -775,7 +775,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
             // eight, 94) 19.4 / 21.1, 20.5 / 21.6.  D 64: 4 kv heads, 20k 11.3 / 11.6, 11.3 / 14.0, 33k (129) 16.2 / 13.5, 15.0 / 15.5; 8 kv heads,
             // 33k 17.4 / 18.3, 18.7 / 19.2.
             const int n = B * d.n_kv_heads;
-            for (int i = widest_cluster_log(n, most, false); i >= 0 && !cluster; --i) {
+            for (int i = widest_cluster_log(n, most); i >= 0 && !cluster; --i) {
                 if ((1 << i) > fewest) continue;
                 list_pages = (ceil_div(most, 1 << i) + 1) & ~1;
                 if (list_pages > kClusterMaxPages) break;

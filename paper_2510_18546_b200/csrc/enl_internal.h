@@ -269,10 +269,10 @@ struct ClusterCaps {
 //     5.88 / 6.92, 6.85 / 7.83;  D 64, the same sizes: 4.37 / 3.93, 5.06 / 4.69; 4.51 / 4.95, 5.30 / 5.66; 4.81 / 5.60, 5.73 / 6.53
 //   6 kv heads, D 128, 640 keys 4.70 / 5.01, 5.51 / 5.51; 2560 keys 5.77 / 7.27, 6.75 / 8.10;  5 kv heads 4.61 / 4.78, 5.39 / 5.53;
 //     5.51 / 7.19, 6.48 / 8.02
-// two_pages: up to two pages a warp are eights', too.  For contiguous keys with masses (none of whose pages is fetched before the kernel
-// before has ended), where the two are about even: 8 kv heads, D 128, 640 keys 6.43 / 5.92, 1280 keys 6.98 / 7.67, 2560 keys 8.86 / 8.34
-// (20 layers of 2500 keys in segments of 40..120: 10.2 / 9.0); D 64 5.79 / 5.27, 6.16 / 6.36, 6.73 / 7.21.
-inline int widest_cluster_log(int heads, int pages, bool two_pages) { return heads >= 8 && pages <= 8 * 12 * (two_pages ? 2 : 1) ? 3 : 4; }
+// Contiguous keys (24 segments and new keys), with masses: 8 kv heads, D 128, 75 pages 7.07 / 6.66, 92 pages 7.22 /
+//     6.84, 108 pages 7.45 / 8.36, 176 pages 9.27 / 9.75, 261 pages 11.28 / 11.85; D 64, 86 pages 6.31 / 5.86, 106 pages 6.44 / 6.69, 188 pages
+//     7.02 / 7.53; one q head per kv head, D 128, 73 pages 6.68 / 6.52, 108 pages 7.05 / 8.10; eight, 79 pages 7.55 / 7.16, 106 pages 7.93 / 8.66
+inline int widest_cluster_log(int heads, int pages) { return heads >= 8 && pages <= 8 * 12 ? 3 : 4; }
 // Opt the kernel for pool pages, and the one for contiguous keys, in on the current device and ask for its capacities there.
 cudaError_t prepare_decode_cluster(int head_dim, ClusterCaps *caps);
 cudaError_t prepare_decode_static(int head_dim, ClusterCaps *caps);

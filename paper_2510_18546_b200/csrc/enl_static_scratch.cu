@@ -249,7 +249,7 @@ extern "C" int enl_attend_static(const enl_static_args_t *a, void *cuda_stream)
         sp.page_off[a->n_seg + 1] = pages;
         // the widest cluster of which all kv heads' run at once, else (many kv heads) the narrowest that holds the lists
         int cluster = 0, list_pages = 0;
-        for (int i = 0; i <= enl::widest_cluster_log(a->n_kv_heads, pages, a->group_mass != nullptr) && info; ++i) {
+        for (int i = 0; i <= enl::widest_cluster_log(a->n_kv_heads, pages) && info; ++i) {
             const int lp = ((pages + (1 << i) - 1) / (1 << i) + 1) & ~1;
             if ((1 << i) > pages || lp > enl::kClusterMaxPages) continue;
             const int cap = info->caps.get(i, enl::decode_cluster_smem(a->head_dim, lp, a->n_seg + 1, rep));
