@@ -58,8 +58,8 @@ STEP = {
     "slots_of_one_key": dict(Hq=16, Hkv=8, D=64, pool=[[1] * 200], n_new=[17]),
     "empty_groups": dict(Hq=4, Hkv=4, D=128, pool=[[0, 0, 300, 0, 17, 0, 0]], n_new=[40]),
     "long_new": dict(Hq=32, Hkv=8, D=128, pool=[[90, 33]], n_new=[700]),
-    "below_the_line": dict(Hq=32, Hkv=8, D=128, pool=[[639 * 16 // 4] * 4], n_new=[16]),
-    "above_the_line": dict(Hq=32, Hkv=8, D=128, pool=[[656 * 16 // 4] * 4], n_new=[16]),
+    "below_the_line": dict(Hq=32, Hkv=8, D=128, pool=[[1008 * 16 // 4] * 4], n_new=[16]),
+    "above_the_line": dict(Hq=32, Hkv=8, D=128, pool=[[1032 * 16 // 4] * 4], n_new=[16]),
     "batch": dict(Hq=8, Hkv=2, D=128, pool=[[30, 60, 90], [5, 5, 5, 5], [200], [], [700, 1]], n_new=[1, 10, 129, 16, 33]),
     "eights_at_most": dict(Hq=32, Hkv=8, D=128, pool=[[90 * 16 // 4] * 4], n_new=[96]),
     "eights_with_masses": dict(Hq=32, Hkv=8, D=128, pool=[[47 * 16] * 4], n_new=[64]),
