@@ -9,7 +9,7 @@
 
 namespace {
 
-struct Record { char kind; int wait_first; size_t bytes; };      // launch ('w' plan write, 's' store, 'a' attention ...)
+struct Record { char kind; int wait_first; size_t bytes; int halves; };   // launch ('w' plan write, 's' store, 'a' attention ...)
 Record g_log[4096];
 int g_n_log;
 int g_heap;                      // allocations of the library's code since the last look
@@ -18,10 +18,10 @@ int g_wait_expires;              // the next one-token kernel gives up on a wait
 unsigned long long g_capture;    // the stream is being captured (as this graph)
 bool g_captured_event;           // the last record of any event was captured
 
-cudaError_t note(char kind, int wait_first, size_t bytes = 0)
+cudaError_t note(char kind, int wait_first, size_t bytes = 0, int halves = 0)
 {
     if (g_fail_kind == kind) return cudaErrorInvalidValue;
-    if (g_n_log < 4096) g_log[g_n_log++] = Record{kind, wait_first, bytes};
+    if (g_n_log < 4096) g_log[g_n_log++] = Record{kind, wait_first, bytes, halves};
     return cudaSuccess;
 }
 CUresult encode(CUtensorMap *tm, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
@@ -49,6 +49,7 @@ void fake_clear() { g_n_log = 0; }
 int fake_launches() { return g_n_log; }
 int fake_kind(int i) { return g_log[i].kind; }
 int fake_wait_first(int i) { return g_log[i].wait_first; }
+int fake_halves(int i) { return g_log[i].halves; }
 long long fake_bytes(int i) { return static_cast<long long>(g_log[i].bytes); }
 
 // ---- CUDA runtime ---------------------------------------------------------------------------------------------------------
@@ -125,7 +126,7 @@ cudaError_t cudaGetDriverEntryPoint(const char *, void **fn, unsigned long long,
 
 // ---- launchers of the kernels that are not linked ---------------------------------------------------------------------------
 namespace enl {
-cudaError_t launch_attention(const AttnParams &p, int, int, cudaStream_t) { return note('a', p.wait_first); }
+cudaError_t launch_attention(const AttnParams &p, int, int, cudaStream_t) { return note('a', p.wait_first, 0, p.halves); }
 cudaError_t launch_mass(const MassParams &p, int, int, cudaStream_t) { return note('m', p.wait_first); }
 cudaError_t launch_small(const SmallParams &p, int, int, int, int, cudaStream_t) { return note('a', p.wait_first); }
 cudaError_t launch_decode(const DecodeParams &p, int, int, cudaStream_t) { return note('d', p.wait_first); }

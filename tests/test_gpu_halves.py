@@ -1,5 +1,6 @@
 """Prefill calls with few CTAs: a Q tile per CTA whose key steps its two walkers share.  Where the halves meet (inside a group, between two,
-at an empty one, in the new tokens), odd numbers of steps, one row to several tiles, with and without splits on top."""
+at an empty one, in the new tokens), odd numbers of steps, one row to several tiles, with and without splits on top (`splits`), slots that
+fit shared memory and more.  (That these calls are planned as such is checked without a GPU, in test_host_state.py.)"""
 import numpy as np
 import pytest
 import torch
@@ -10,17 +11,21 @@ from tests.helpers import Session, check_close
 pytestmark = pytest.mark.gpu
 
 CASES = {
-    "meet_inside_a_group": dict(Hq=8, Hkv=2, D=128, pool=[[30, 500, 20]], n_q=[70], n_new=[70]),
-    "meet_between_groups": dict(Hq=8, Hkv=2, D=128, pool=[[256, 256]], n_q=[40], n_new=[40]),
-    "meet_at_an_empty_group": dict(Hq=8, Hkv=2, D=128, pool=[[240, 0, 0, 224]], n_q=[40], n_new=[40]),
-    "meet_in_the_new_tokens": dict(Hq=8, Hkv=2, D=128, pool=[[100]], n_q=[400], n_new=[400]),
-    "slots_in_the_mass_buffer": dict(Hq=8, Hkv=2, D=128, pool=[[5 + (i * 7) % 23 for i in range(40)]], n_q=[100], n_new=[100]),
-    "rows_of_one_tile": dict(Hq=32, Hkv=8, D=128, pool=[[400, 33]], n_q=[17], n_new=[17]),
-    "one_row_beyond_a_tile": dict(Hq=32, Hkv=8, D=128, pool=[[400, 33, 7]], n_q=[33], n_new=[95]),
-    "odd_steps_d64": dict(Hq=8, Hkv=2, D=64, pool=[[64 * 7]], n_q=[65], n_new=[65]),
-    "rep1": dict(Hq=2, Hkv=2, D=64, pool=[[300, 200]], n_q=[140], n_new=[140]),
-    "rep8_long": dict(Hq=8, Hkv=1, D=128, pool=[[2000, 45, 1100]], n_q=[40], n_new=[40]),
-    "batch": dict(Hq=8, Hkv=2, D=128, pool=[[300, 60, 90], [5, 5, 450], [400]], n_q=[70, 3, 129], n_new=[70, 10, 129]),
+    "meet_inside_a_group": dict(Hq=8, Hkv=2, D=128, pool=[[30, 500, 20]], n_q=[70], n_new=[70], splits=True),
+    "meet_between_groups": dict(Hq=8, Hkv=2, D=128, pool=[[256, 256]], n_q=[40], n_new=[40], splits=True),
+    "meet_at_an_empty_group": dict(Hq=8, Hkv=2, D=128, pool=[[240, 0, 0, 224]], n_q=[40], n_new=[40], splits=True),
+    "meet_in_the_new_tokens": dict(Hq=8, Hkv=2, D=128, pool=[[100]], n_q=[400], n_new=[400], splits=False),
+    "slots_in_the_mass_buffer": dict(Hq=8, Hkv=2, D=128, pool=[[5 + (i * 7) % 23 for i in range(40)]], n_q=[100], n_new=[100], splits=True),
+    "rows_of_one_tile": dict(Hq=32, Hkv=8, D=128, pool=[[3000, 33]], n_q=[17], n_new=[17], splits=True),
+    "one_row_beyond_a_tile": dict(Hq=32, Hkv=8, D=128, pool=[[400, 33, 7]], n_q=[33], n_new=[95], splits=True),
+    "odd_steps_d64": dict(Hq=8, Hkv=2, D=64, pool=[[64 * 7]], n_q=[65], n_new=[65], splits=True),
+    "rep1": dict(Hq=2, Hkv=2, D=64, pool=[[300, 200]], n_q=[140], n_new=[140], splits=True),
+    "rep8_long": dict(Hq=8, Hkv=1, D=128, pool=[[2000, 45, 1100]], n_q=[40], n_new=[40], splits=True),
+    "unsplit_inside_a_group": dict(Hq=32, Hkv=8, D=128, pool=[[30, 500, 20]], n_q=[310], n_new=[310], splits=False),
+    "unsplit_d64": dict(Hq=16, Hkv=16, D=64, pool=[[100, 77, 200]], n_q=[600], n_new=[650], splits=False),
+    "unsplit_slots_in_the_mass_buffer": dict(Hq=32, Hkv=8, D=128, pool=[[5 + (i * 7) % 23 for i in range(40)]], n_q=[310], n_new=[310], splits=False),
+    "unsplit_ends_in_the_mass_buffer": dict(Hq=32, Hkv=8, D=128, pool=[[16] * 60], n_q=[297], n_new=[300], splits=False),
+    "batch": dict(Hq=8, Hkv=2, D=128, pool=[[300, 60, 90], [5, 5, 450], [400]], n_q=[70, 3, 129], n_new=[70, 10, 129], splits=True),
 }
 
 
@@ -39,7 +44,8 @@ def test_halves(name, want_mass):
         assert enl.enl_cache_status(s.cache) == enl.ENL_OK
         p = enl.enl_plan_inspect(s.cache)
         tokens = 128 // (c["Hq"] // c["Hkv"])
-        assert p["n_items"] == sum(-(-x // tokens) for x in c["n_q"]) * c["Hkv"] * p["n_splits"] and p["merge_kind"] in (0, 1)
+        assert p["n_items"] == sum(-(-x // tokens) for x in c["n_q"]) * c["Hkv"] * p["n_splits"]
+        assert p["merge_kind"] == (1 if c["splits"] else 0)
         for b in range(n):
             ro, rm, _ = s.oracle(0, b, q[cq[b]:cq[b + 1]], kn[cn[b]:cn[b + 1]], vn[cn[b]:cn[b + 1]])
             G = len(wl.sel_local[b])

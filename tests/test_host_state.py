@@ -9,6 +9,7 @@ import pytest
 
 from paper_2510_18546_b200 import build as enl_build
 from paper_2510_18546_b200 import enl
+from tests.test_gpu_halves import CASES as HALVES
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 SOURCES = ["enl_host.cu", "enl_static_scratch.cu", "enl_decode_cluster_sm100.cu"]
@@ -219,4 +220,35 @@ def test_no_cta_without_keys(host, heads, D):
                         pages = -(-n // 16) if n_sel else 0
                         assert n_splits <= -(-pages // 4) + (prior + first - 1) // 64 + 1, (n, n_q, prior, hint, n_sel)
     assert halves > 0
+    host.enl_cache_free(h)
+
+
+@pytest.mark.parametrize("want_mass", [True, False])
+@pytest.mark.parametrize("name", sorted(HALVES))
+def test_form_of_the_calls_that_test_halves(host, name, want_mass):
+    """The calls whose results are checked on the GPU as calls with few CTAs are planned as such: the walkers share the steps, with the
+    splits on top that the case says."""
+    c = HALVES[name]
+    n = len(c["pool"])
+    lens = [x for pool in c["pool"] for x in pool]
+    h = ctypes.c_void_p()
+    d = enl.CacheDesc(1, c["Hq"], c["Hkv"], c["D"], 0, len(lens), sum(lens), enl.ENL_BF16, 0, n, sum(c["n_q"]), 0)
+    assert host.enl_cache_create(ctypes.byref(d), ctypes.byref(h)) == enl.ENL_OK
+    for g, x in enumerate(lens):
+        assert host.enl_group_store(h, g, 0, x, ctypes.c_void_p(1 << 20), ctypes.c_void_p(1 << 21), 0, None) == enl.ENL_OK
+    ids = np.arange(len(lens), dtype=np.int32)
+    cu = [np.concatenate([[0], np.cumsum(x)]).astype(np.int32) for x in ([len(x) for x in c["pool"]], c["n_q"], c["n_new"])]
+    a = enl.AttendArgs()
+    a.batch, a.n_sel, a.n_q, a.n_new = n, len(ids), sum(c["n_q"]), sum(c["n_new"])
+    a.sel_ids, a.mass_stride = ids.ctypes.data, max(len(x) for x in c["pool"]) + 1
+    a.cu_sel, a.cu_q, a.cu_new = (x.ctypes.data for x in cu)
+    a.q, a.k_new, a.v_new, a.out = ((1 << 20) * i for i in range(1, 5))
+    a.group_mass = (1 << 20) * 5 if want_mass else None
+    host.fake_clear()
+    assert host.enl_attend(h, ctypes.byref(a), None) == enl.ENL_OK
+    (i,) = [i for i in range(host.fake_launches()) if chr(host.fake_kind(i)) == "a"]
+    assert host.fake_halves(i) == 1
+    out = [ctypes.c_int32() for _ in range(4)]
+    assert host.enl_plan_inspect(h, 0, None, None, ctypes.byref(out[0]), 0, None, None, *(ctypes.byref(x) for x in out[1:])) == enl.ENL_OK
+    assert (out[1].value > 1) == c["splits"]
     host.enl_cache_free(h)

@@ -235,6 +235,36 @@ def test_mass_sums_from_the_attention_kernel_match_the_oracle(shape):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("lens", [[1500, 700, 300, 900, 17, 0, 40], [3600], [100] * 36])
+def test_object_sums_with_outputs_in_pairs(lens):
+    """Outputs, masses and the objects' sums of a call whose two splits are merged by pairs of CTAs: the log-sums go to the mass buffer, the
+    slot in which the splits meet (within a group here) from one of them, and the kernel behind finishes and sums."""
+    from tests.helpers import MASS_MAX_ABS, Session, check_close
+    from paper_2510_18546_b200 import synth
+    n_q, G = 70, len(lens)
+    wl = synth.make_small(55, 1, 32, 8, 128, [lens], [list(range(G))], [n_q], [n_q + 9], name="sums in pairs")
+    cuts = [0, 1, 40, 66]                               # the last rows belong to no object
+    with Session(wl, [0]) as s:
+        q, kn, vn = wl.new_qkv(0, s.device)
+        out = torch.full_like(q, float("nan"))
+        mass = torch.full((n_q, 32, G + 1), float("nan"), device=s.device)
+        sums = torch.zeros(len(cuts) - 1, G + 1, device=s.device)
+        enl.enl_attend(s.cache, 0, wl.sel_ids(), q, kn, vn, out, mass, group_mass_sum=sums, obj_off=cuts)
+        torch.cuda.synchronize()
+        assert enl.enl_cache_status(s.cache) == enl.ENL_OK
+        p = enl.enl_plan_inspect(s.cache)
+        assert p["n_splits"] == 2 and p["merge_kind"] == 2
+        ro, rm, _ = s.oracle(0, 0, q, kn, vn)
+        check_close(out, ro, mass, rm, what="sums in pairs")
+        for o in range(len(cuts) - 1):
+            n = (cuts[o + 1] - cuts[o]) * 32
+            want = mass[cuts[o]:cuts[o + 1]].double().sum((0, 1))
+            # fp32 sums of n addends that are not negative: relative error below n * 2^-24
+            assert ((sums[o].double() - want).abs() <= want * n * 2.0 ** -24 + 1e-30).all()
+            assert (np.abs(sums[o].cpu().numpy() / n - rm[cuts[o]:cuts[o + 1]].mean((0, 1))) <= MASS_MAX_ABS).all()
+
+
+@pytest.mark.gpu
 def test_mass_only_and_sum_argument_errors():
     from tests.helpers import Session
     from paper_2510_18546_b200 import synth
