@@ -356,3 +356,42 @@ def test_graphs_and_calls_beside_them(n_q, pages):
             ks, vs = ([x[g] for g in lists[i]] for x in s.host_kv[(0, 0)])
             ro, _ = orc.attend_slots(4, 1, 64, ks, vs, q.cpu(), kn.cpu(), vn.cpu(), rows=rows)
             check_close(out[rows], ro, None, None, what=f"{wl.name}, list {i}")
+
+
+@pytest.mark.parametrize("n_q", [1, 20, 300])
+def test_captured_stores_are_seen_by_calls_outside_the_graph(n_q):
+    """A graph that stores runs before, between and directly in front of calls outside it, with other rows every time: each call sees what
+    the graph has written last."""
+    lens = [64, 200, 48]
+    wl = synth.make_small(66, 1, 8, 2, 128, [lens], [[0, 1, 2]], [n_q], [n_q], name=f"captured store, {n_q} rows")
+    with Session(wl, [0]) as s:
+        q, kn, vn = wl.new_qkv(0, s.device)
+        k, v = (x.clone() for x in wl.pool_kv(0, 0, s.device))
+        rows_k, rows_v = k[64:264].clone(), v[64:264].clone()
+
+        def attend():
+            out = torch.empty_like(q)
+            enl.enl_attend(s.cache, 0, [0, 1, 2], q, kn, vn, out, stream=torch.cuda.current_stream().cuda_stream)
+            return out
+
+        attend()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            enl.enl_group_store(s.cache, 1, 0, rows_k, rows_v, stream=torch.cuda.current_stream().cuda_stream)
+        gen = torch.Generator(device=s.device).manual_seed(7)
+        got = []
+        for _ in range(4):
+            for _ in range(2):                          # launches that nothing has been written between
+                attend()
+            rows_k.copy_(torch.randn(200, 2, 128, generator=gen, device=s.device))
+            graph.replay()
+            got.append((rows_k.cpu(), attend(), attend()))
+        torch.cuda.synchronize()
+        assert enl.enl_cache_status(s.cache) == enl.ENL_OK
+        rows = sorted({0, n_q // 2, n_q - 1})
+        for now, *outs in got:
+            ks = [k[:64].cpu(), now, k[264:].cpu()]
+            vs = [v[:64].cpu(), v[64:264].cpu(), v[264:].cpu()]
+            ro, _ = orc.attend_slots(8, 2, 128, ks, vs, q.cpu(), kn.cpu(), vn.cpu(), rows=rows)
+            for out in outs:
+                check_close(out[rows], ro, None, None, what=wl.name)
