@@ -66,11 +66,11 @@ constexpr float kRescaleThreshold = 8.0f;     // log2 units: p stays below 2^8 b
 
 template <int D>
 struct Cfg {
-    static constexpr int kHalves    = D / 64;             // 64-channel (128-byte) column blocks
-    static constexpr int kHalfBytes = 128 * 128;          // Q tile: 128 rows x 128 B
-    static constexpr int kTileBytes = kHalves * kHalfBytes;
+    static constexpr int kBlocks    = D / 64;             // 64-channel (128-byte) column blocks
+    static constexpr int kBlockBytes = 128 * 128;          // Q tile: 128 rows x 128 B
+    static constexpr int kTileBytes = kBlocks * kBlockBytes;
     // K or V of a step: eight groups of 8 rows, a group being one 8 x 128-byte block per 64 channels
-    static constexpr int kGroupBytes = kHalves * 1024;
+    static constexpr int kGroupBytes = kBlocks * 1024;
     static constexpr int kStepBytes = kStepKeys / 8 * kGroupBytes;
     static constexpr int kRing      = 4;                  // steps whose K (and whose V) are in shared memory at once
     static constexpr int kRingOff   = kQTiles * kTileBytes;
@@ -202,8 +202,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
     // whose reads more loads hold up, one: 128 rows over 2560 keys 19.0 -> 18.35 us, with two steps 18.6, with four 19.3.
     const bool producer = warp == kKWarp || warp == kVWarp;
     if (producer && n_steps > 0 && static_cast<int>(blockIdx.x) < p.first_wave) {
-        if (warp == kKWarp && lane < n_qt * C::kHalves)
-            tma_prefetch_3d(&p.tm_q, (lane % C::kHalves) * 64, it.kvh * rep, ep.q_off + it.t0 + (lane / C::kHalves) * tile_tokens);
+        if (warp == kKWarp && lane < n_qt * C::kBlocks)
+            tma_prefetch_3d(&p.tm_q, (lane % C::kBlocks) * 64, it.kvh * rep, ep.q_off + it.t0 + (lane / C::kBlocks) * tile_tokens);
         constexpr int kBoxes = kStepKeys / kBoxRows<D>;              // of a step
         const int vn = lane / kBoxes, jn = step_of(vn);
         if (vn < min(C::kRing, n_steps) && jn >= n_csteps)
@@ -233,8 +233,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                 if (is_k && lane == 0) {
                     mbar_expect_tx(bar_q_full, static_cast<uint32_t>(n_qt * C::kTileBytes));
                     for (int i = 0; i < n_qt; ++i)
-                        for (int hf = 0; hf < C::kHalves; ++hf)
-                            tma_load_3d(q_addr(i) + hf * C::kHalfBytes, &p.tm_q, hf * 64, it.kvh * rep,
+                        for (int b = 0; b < C::kBlocks; ++b)
+                            tma_load_3d(q_addr(i) + b * C::kBlockBytes, &p.tm_q, b * 64, it.kvh * rep,
                                         ep.q_off + it.t0 + i * tile_tokens, bar_q_full);
                 }
                 __syncwarp();
@@ -326,7 +326,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
 #pragma unroll
                 for (int kk = 0; kk < D / 16; ++kk) {
                     const uint32_t in_row = static_cast<uint32_t>((kk & 3) * 2);                       // 32 bytes per 16 channels
-                    mma_ss2(d, dq_lo + static_cast<uint32_t>((kk >> 2) * (C::kHalfBytes >> 4)) + in_row, dq_hi,
+                    mma_ss2(d, dq_lo + static_cast<uint32_t>((kk >> 2) * (C::kBlockBytes >> 4)) + in_row, dq_hi,
                             ka + static_cast<uint32_t>((kk >> 2) * (1024 >> 4)) + in_row, dk_hi, idesc_qk, kk > 0 || hide ? 1u : 0u);
                 }
                 tc_commit(bar_s_full(i, b));
