@@ -632,7 +632,10 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                 slots[sl] = w;
             }
         };
-        // slots this walker walked (all of them where nothing is split)
+        // Slots this walker walked (all of them where nothing is split).  Beyond kParkSlots the kernel that merges splits is told which slots a
+        // split has written of a row, and the others are left as they were: clearing them took the masses of 128 rows over 400 groups in 17
+        // splits (8 heads) 30 us of 81 a thread per row, and reading them as long again.
+        int2 *range_out = slot_out && p.part_rng && h == 0 ? p.part_rng + static_cast<long long>(it.split) * p.n_q_total + grow : nullptr;
         int first_slot = 0, last_slot = G;
         if (p.n_splits > 1 || two_halves) {
             first_slot = G + 1;
@@ -643,20 +646,6 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                 last_slot = (je > n_csteps) ? G : (__ldg(p.stream_meta + ep.stream_off + je * kStepPages - 1) >> 8);
             }
         }
-        // Slots of the warp's rows in the partial results, those in [from, to) that were not walked: a row at a time, lanes over the slots.
-        // (A thread per row, whose stores of a warp lie in 32 rows, took the masses of 128 rows over 400 groups in 17 splits, 8 heads,
-        // from 56 to 81 us.)
-        auto clear_slots = [&](int from, int to) {
-            __syncwarp();
-#pragma unroll 1
-            for (int rr = 0; rr < 32; ++rr) {
-                const int ri = __shfl_sync(kFull, my_ridx, rr);
-                if (ri < 0) continue;
-                float *slots = p.part_slot + static_cast<long long>(ri) * p.mass_stride;
-                for (int sl = from + lane; sl < to; sl += 32)
-                    if (sl < first_slot || sl > last_slot) slots[sl] = kNegInf;
-            }
-        };
         // The merged row: what a walker or a CTA of a pair makes of its own (m_use, l) and the other's (x, y of pe)
         float row_lse = lse, other_bnd = kNegInf, w_own = 0.f, w_other = 0.f;
         auto merge_rows = [&](const float4 &pe) {
@@ -686,14 +675,15 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
             merge_rows(rows[(i ^ 1) * 128 + r]);
             if (split_mode) {
                 if (i == 0 && row_valid) p.part_lse[rh] = row_lse;
-                if (park_smem) {                                     // slots that this split did not walk contribute nothing
-                    if (slot_out)
+                if (slot_out) {
+                    if (park_smem) {                                 // slots that this split did not walk contribute nothing
                         for (int sl = i == 0 ? 0 : first_slot; sl <= (i == 0 ? last_slot : G); ++sl)
                             if (sl != skip_slot)
                                 slot_out[sl] = (sl < first_slot || sl > last_slot) ? kNegInf : sl == shared_slot ? shared_log() : park_row[sl * 128];
-                } else if (p.part_slot) {
-                    if (slot_out && i == 0 && shared_slot >= 0) slot_out[shared_slot] = shared_log();
-                    clear_slots(i == 0 ? 0 : last_slot + 1, i == 0 ? first_slot : G + 1);
+                    } else {
+                        if (i == 0 && shared_slot >= 0) slot_out[shared_slot] = shared_log();
+                        if (range_out) *(i == 0 ? &range_out->x : &range_out->y) = i == 0 ? first_slot : last_slot;
+                    }
                 }
             } else if (p.mass) {
                 if (park_smem) {
@@ -776,12 +766,12 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
             } else if (split_mode) {
                 // ---- partial results for the merge kernel: O / l in fp32, the row's log-sum-exp, raw slot log-sums ----
                 if (row_valid) p.part_lse[rh] = lse;
-                if (p.part_slot && park_smem) {
-                    if (slot_out)
+                if (slot_out) {
+                    if (park_smem)                                   // slots that this split did not walk contribute nothing
                         for (int sl = 0; sl <= G; ++sl)
                             slot_out[sl] = (sl < first_slot || sl > last_slot) ? kNegInf : park_row[sl * 128];
-                } else if (p.part_slot) {                           // slots this split did not walk contribute nothing
-                    clear_slots(0, G + 1);
+                    else if (range_out)
+                        *range_out = make_int2(first_slot, last_slot);
                 }
                 if (n_steps > 0) {
                     const float inv = (l > 0.f) ? 1.f / l : 0.f;

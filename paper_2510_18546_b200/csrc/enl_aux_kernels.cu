@@ -82,7 +82,9 @@ __global__ void __launch_bounds__(256) combine_kernel(const CombineParams p)
     pdl_wait();                                             // the partial results come from the previous kernel
     if (rh >= split_stride) return;
     const float ninf = -__builtin_huge_valf();
-    const int G = p.mass ? p.row_slots[static_cast<int>(rh / p.Hq)] : -1;
+    const int row = static_cast<int>(rh / p.Hq);
+    const int G = p.mass ? p.row_slots[row] : -1;
+    const int G0 = p.part_rng ? -1 : G;                     // slots whose log-sums come along with the outputs
     const float *o0 = p.part_o + rh * D + lane * V;
     const float *s0 = p.part_slot ? p.part_slot + rh * p.slot_stride + lane : nullptr;
     float ov[kBatch][V], sv[kBatch];
@@ -97,13 +99,18 @@ __global__ void __launch_bounds__(256) combine_kernel(const CombineParams p)
                 const float2 t = __ldcg(reinterpret_cast<const float2 *>(o0 + k * split_stride * D));
                 ov[j][0] = t.x; ov[j][1] = t.y;
             }
-            sv[j] = (lane <= G && k0 + j < p.n_splits) ? __ldcg(s0 + k * split_stride * p.slot_stride) : ninf;
+            sv[j] = (lane <= G0 && k0 + j < p.n_splits) ? __ldcg(s0 + k * split_stride * p.slot_stride) : ninf;
         }
     };
     fetch(0);
     // every lane needs every split's log-sum-exp: lane k loads split k (and k + 32), then shuffles
     const float my0 = lane < p.n_splits ? __ldcg(p.part_lse + lane * split_stride + rh) : ninf;
     const float my1 = lane + 32 < p.n_splits ? __ldcg(p.part_lse + (lane + 32) * split_stride + rh) : ninf;
+    int2 r0 = make_int2(0, -1), r1 = r0;                    // slots that the splits have written of this row
+    if (p.part_rng) {
+        if (lane < p.n_splits) r0 = __ldcg(p.part_rng + static_cast<long long>(lane) * p.n_q_total + row);
+        if (lane + 32 < p.n_splits) r1 = __ldcg(p.part_rng + static_cast<long long>(lane + 32) * p.n_q_total + row);
+    }
     float mx = fmaxf(my0, my1);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -138,6 +145,36 @@ __global__ void __launch_bounds__(256) combine_kernel(const CombineParams p)
         *reinterpret_cast<__nv_bfloat162 *>(dst + x) = __floats2bfloat162_rn(acc[x], acc[x + 1]);
     if (!p.mass) return;
     float *masses = p.mass + rh * p.mass_stride;
+    if (p.part_rng) {
+        // Many slots, most of them in one split only: of every 64 slots (two a lane), the splits whose ranges reach into them, four at a time.
+        // (All splits of every slot, which the attention kernel then has to clear: 17 rows over 400 groups in 60 splits, 4 heads, 66 us and not 28.)
+        for (int s = 0; s <= G; s += 64) {                  // warp-uniform
+            uint32_t m0 = __ballot_sync(0xffffffffu, r0.x <= s + 63 && r0.y >= s), m1 = __ballot_sync(0xffffffffu, r1.x <= s + 63 && r1.y >= s);
+            const int s_lo = s + lane, s_hi = s_lo + 32;
+            float mass_lo = 0.f, mass_hi = 0.f;
+            while ((m0 | m1) != 0u) {
+                float lo[4], hi[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int k = m0 ? __ffs(m0) - 1 : m1 ? __ffs(m1) + 31 : -1;
+                    const int first = __shfl_sync(0xffffffffu, k < 32 ? r0.x : r1.x, k & 31), last = __shfl_sync(0xffffffffu, k < 32 ? r0.y : r1.y, k & 31);
+                    const float *sk = s0 + s + k * split_stride * p.slot_stride;
+                    lo[u] = (k >= 0 && s_lo >= first && s_lo <= last) ? __ldcg(sk) : ninf;
+                    hi[u] = (k >= 0 && s_hi >= first && s_hi <= last) ? __ldcg(sk + 32) : ninf;
+                    if (m0) m0 &= m0 - 1u;
+                    else m1 &= m1 - 1u;
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    mass_lo += ex2f(lo[u] - lse_s);
+                    mass_hi += ex2f(hi[u] - lse_s);
+                }
+            }
+            if (s_lo <= G) masses[s_lo] = mass_lo;
+            if (s_hi <= G) masses[s_hi] = mass_hi;
+        }
+        return;
+    }
     if (lane <= G) masses[lane] = mass;
     for (int s = 32; s <= G; s += 32) {                     // warp-uniform
         mass = 0.f;

@@ -746,9 +746,9 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
 
         const int slot_stride = max_slots + 1;
         const int64_t per_rh = d.head_dim + 1 + (has_mass ? slot_stride : 0);      // scratch floats per (split, row, head)
-        auto fits = [&](int ns) {      // partial O, log-sum-exp and slot log-sums, plus the decode kernel's slot ranges
+        auto fits = [&](int ns) {      // partial O, log-sum-exp and slot log-sums, plus the ranges of slots
             return static_cast<int64_t>(ns) * a->n_q * d.n_q_heads * per_rh * 4 +
-                   static_cast<int64_t>(ns) * B * d.n_kv_heads * 8 + 16 <= d.scratch_bytes;
+                   static_cast<int64_t>(ns) * std::max(B * d.n_kv_heads, a->n_q) * 8 + 16 <= d.scratch_bytes;
         };
         // One query token per episode: the streaming decode kernel, whose CTAs cover at most kDecodeMaxPages pages each (the
         // last one of a kv head to finish merges their partial results), or the one merged by clusters.
@@ -1158,6 +1158,10 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         p.part_o = c->scratch;
         p.part_lse = c->scratch + rows * d.head_dim;
         p.part_slot = has_mass ? c->scratch + rows * (d.head_dim + 1) : nullptr;
+        if (has_mass && !c->plan_park) {
+            const size_t used = rows * (d.head_dim + 1 + slot_stride);                       // floats
+            p.part_rng = reinterpret_cast<int2 *>(c->scratch + ((used + 1) & ~static_cast<size_t>(1)));
+        }
         p.mass_stride = slot_stride;                 // the partial slot buffer is packed
     }
     if (mass_only) {
@@ -1207,6 +1211,7 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
         cp.part_o = p.part_o;
         cp.part_lse = p.part_lse;
         cp.part_slot = p.part_slot;
+        cp.part_rng = p.part_rng;
         cp.out = a->out;
         cp.mass = a->group_mass;
         cp.row_slots = reinterpret_cast<const int32_t *>(c->plan_dev + c->off_rowslots);

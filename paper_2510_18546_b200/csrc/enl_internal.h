@@ -60,7 +60,8 @@ struct AttnParams {
     float  *mass;           // fp32 or null
     float  *part_o;         // split mode: [split][row][Hq][D] fp32 (normalised by the split's own sum)
     float  *part_lse;       // split mode: [split][row][Hq] log2-sum-exp of the split
-    float  *part_slot;      // split mode: [split][row][Hq][mass_stride] per-slot log2-sum-exp
+    float  *part_slot;      // split mode: [split][row][Hq][mass_stride] per-slot log2-sum-exp (with part_rng only of the slots that the split has walked)
+    int2   *part_rng;       // split mode, log-sums not parked in shared memory: [split][row] first and last of them (the same for all heads)
     int32_t *status;        // device word: nonzero = a bounded wait expired
     int32_t n_q_total;      // rows over the batch
     int32_t Hq, Hkv, rep;   // rep = Hq / Hkv
@@ -169,6 +170,7 @@ struct StaticDecodeParams {
 
 struct CombineParams {
     const float *part_o, *part_lse, *part_slot;
+    const int2 *part_rng;       // [split][row]: first and last slot that the split has written, or null: all are
     void  *out;
     float *mass;
     const int32_t *row_slots;   // [n_q_total]: G_b of the row's episode

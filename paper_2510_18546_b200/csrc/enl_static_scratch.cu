@@ -309,6 +309,7 @@ extern "C" int enl_attend_static(const enl_static_args_t *a, void *cuda_stream)
     cp.part_o = p.part_o;
     cp.part_lse = p.part_lse;
     cp.part_slot = p.part_slot;
+    cp.part_rng = nullptr;
     cp.out = a->out;
     cp.mass = a->group_mass;
     cp.row_slots = p.row_slots;

@@ -395,3 +395,23 @@ def test_captured_stores_are_seen_by_calls_outside_the_graph(n_q):
             ro, _ = orc.attend_slots(8, 2, 128, ks, vs, q.cpu(), kn.cpu(), vn.cpu(), rows=rows)
             for out in outs:
                 check_close(out[rows], ro, None, None, what=wl.name)
+
+
+@pytest.mark.parametrize("splits", [3, 5, 33, 40])
+@pytest.mark.parametrize("groups", [25, 31, 32, 63, 64, 65, 130])
+def test_masses_of_splits_merged_in_memory(groups, splits):
+    """More slots than fit shared memory, each in one or two of the splits: the merge takes them from where the splits have walked them, 64 at a
+    time.  The scratch buffer holds another call's partial results, so slots that a split has not written are anything."""
+    lens = [max(1, 2 * 5400 // groups * (1 + i % 3) // 4) for i in range(groups)]
+    lens[groups // 2] = 0
+    wl = synth.make_small(67, 1, 4, 1, 64, [lens], [list(range(groups))], [40], [50], name=f"{groups} groups in {splits} splits")
+    with Session(wl, [0]) as s:
+        q, kn, vn = wl.new_qkv(0, s.device)
+        s.attend(0, q * 3, kn, vn, split_hint=splits, sel_override=list(range(groups))[::-1])
+        out, mass, _ = s.attend(0, q, kn, vn, split_hint=splits)
+        torch.cuda.synchronize()
+        assert enl.enl_cache_status(s.cache) == enl.ENL_OK
+        p = enl.enl_plan_inspect(s.cache)
+        assert p["n_splits"] == splits and p["merge_kind"] == 1
+        ro, rm, _ = s.oracle(0, 0, q, kn, vn)
+        check_close(out, ro, mass, rm, what=wl.name)
