@@ -31,7 +31,8 @@
 //    per page needed 3800.
 //  * Turns: the warps of the two tiles that share a scheduler take their exponentials one after the other (a named barrier).  Left alone
 //    the tiles fall into step, both wanting the special-function unit and then both not: 4150 against 3500.
-// Long calls 251 -> 238 thousand cycles a launch (then at the power cap), the planner's 512 rows over 24 groups 33.5 -> 31.0 us.
+// Together: long calls 251 -> 238 thousand cycles a launch (then at the power cap), the planner's 512 rows over 24 groups 33.5 -> 31.0 us
+// (29.9 to 30.3 with the early pages and a start that takes no division).
 // Not kept: exponentials on the FMA pipe, a quarter of them 270 thousand cycles (the warps have issue slots, but a step is one chain);
 // the maximum beside the exponentials, with the reference a step behind: 6700 against 5860 us a pass; tiles of 128 keys with all of the
 // above: the same on long calls, 8 % slower on the planner's, whose ends waste half a tile.
@@ -198,7 +199,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
     // written by launches of this library only, and none has come in between.  What else comes first is asked into the L2: the Q tiles and
     // new tokens.  (Only CTAs of the first wave wait for the previous kernel; for the others this would be loads issued twice.)
     // How many steps: with none a launch took 2.4 us from the wait to its first scores (the page words' round trip and then the pages').
-    // Two steps leave the planner's layer at 29.3 us (none 30.5, four 29.7); where the kernel before is the one that merges the splits,
+    // With two steps the planner's layer took 29.3 us where none took 30.5 and four 29.7; where the kernel before is the one that merges the splits,
     // whose reads more loads hold up, one: 128 rows over 2560 keys 19.0 -> 18.35 us, with two steps 18.6, with four 19.3.
     const bool producer = warp == kKWarp || warp == kVWarp;
     if (producer && n_steps > 0 && static_cast<int>(blockIdx.x) < p.first_wave) {
@@ -210,6 +211,16 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
             tma_prefetch_4d(warp == kKWarp ? &p.tm_knew : &p.tm_vnew, 0, ep.new_off + (jn - n_csteps) * kStepKeys + lane % kBoxes * kBoxRows<D>, 0, it.kvh);
     }
     if (!producer) pdl_wait();
+    // Beyond kParkSlots the kernel that merges splits is told which slots a split writes of a row, and the others are left as they were:
+    // clearing them took 30 us of the 81 that the masses of 128 rows over 400 groups in 17 splits (8 heads) did a thread per row, and
+    // reading them as long again.  (Here, by a warp that would only wait now: the softmax warps have no registers to spare; from their
+    // epilogue a layer of the planner's took 0.8 % longer, from the producers' end the loop 3 to 8 %.)
+    if (warp == kMmaWarp + 2 && it.kvh == 0 && p.part_rng && n_steps > 0) {
+        const int first = j_beg < n_csteps ? __ldg(p.stream_meta + ep.stream_off + j_beg * kStepPages) >> 8 : ep.n_slots;
+        const int last = j_end > n_csteps ? ep.n_slots : __ldg(p.stream_meta + ep.stream_off + j_end * kStepPages - 1) >> 8;
+        for (int t = it.t0 + lane; t < t_hi; t += 32)
+            p.part_rng[static_cast<long long>(it.split) * p.n_q_total + ep.q_off + t] = make_int2(first, last);
+    }
 
     bool ok = true;
 
@@ -392,18 +403,13 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
         const uint32_t t_s = tmem_base + lane_sel + static_cast<uint32_t>(i * 128);
         const uint32_t t_o = tmem_base + lane_sel + static_cast<uint32_t>(256 + i * 128);
         const bool split_mode = p.n_splits > 1 && !pair;
-        const long long grow = static_cast<long long>(ep.q_off) + t;   // global query row
-        const long long rh = (split_mode ? (static_cast<long long>(it.split) * p.n_q_total + grow) : grow) * p.Hq + h;
         // Where this row's slot log-sums are parked until the row's total is known: shared memory when the call has few
         // slots (one store per slot end, no round trip to the L2 at the end), else the buffer that takes the result.
-        float *slot_out = nullptr;
-        if (row_valid) {
-            if (split_mode) { if (p.part_slot) slot_out = p.part_slot + rh * p.mass_stride; }
-            else if (p.mass) slot_out = p.mass + rh * p.mass_stride;
-        }
-        const bool park_smem = p.park_smem != 0;
-        const bool want_slots = (split_mode ? p.part_slot : p.mass) != nullptr;
-        float *slot_global = park_smem ? nullptr : slot_out;
+        float *const slot_rows = split_mode ? p.part_slot : p.mass;
+        const bool park_smem = p.park_smem != 0, want_slots = slot_rows != nullptr;
+        float *slot_global = nullptr;
+        if (row_valid && want_slots && !park_smem)
+            slot_global = slot_rows + (static_cast<long long>((split_mode ? it.split * p.n_q_total : 0) + ep.q_off + t) * p.Hq + h) * p.mass_stride;
         float *park_row = reinterpret_cast<float *>(smem + C::kParkOff) + i * (kParkSlots * 128) + r;   // + slot * 128; (each walker its own slots)
         const float scale = p.scale_log2;
 
@@ -621,6 +627,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
         // mass_finish_kernel: it reads and writes them at memory speed, while here every 32 slots of a warp cost a memory round trip with
         // the tensor pipe idle: 245 of 2300 us of a scoring pass over 1000 groups.)
         const int my_ridx = row_index(lane);
+        const long long rh = my_ridx;
+        float *const slot_out = my_ridx >= 0 && slot_rows ? slot_rows + rh * p.mass_stride : nullptr;
         auto finish_masses = [&](float ref, float extra, int first, int last) {
             if (my_ridx < 0) return;
             float *slots = p.mass + static_cast<long long>(my_ridx) * p.mass_stride;
@@ -632,10 +640,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                 slots[sl] = w;
             }
         };
-        // Slots this walker walked (all of them where nothing is split).  Beyond kParkSlots the kernel that merges splits is told which slots a
-        // split has written of a row, and the others are left as they were: clearing them took the masses of 128 rows over 400 groups in 17
-        // splits (8 heads) 30 us of 81 a thread per row, and reading them as long again.
-        int2 *range_out = slot_out && p.part_rng && h == 0 ? p.part_rng + static_cast<long long>(it.split) * p.n_q_total + grow : nullptr;
+        // slots this walker walked (all of them where nothing is split)
         int first_slot = 0, last_slot = G;
         if (p.n_splits > 1 || two_halves) {
             first_slot = G + 1;
@@ -674,21 +679,20 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
             asm volatile("bar.sync 9, 256;" ::: "memory");           // reached whatever happened (the waits are bounded)
             merge_rows(rows[(i ^ 1) * 128 + r]);
             if (split_mode) {
-                if (i == 0 && row_valid) p.part_lse[rh] = row_lse;
+                if (i == 0 && my_ridx >= 0) p.part_lse[rh] = row_lse;
                 if (slot_out) {
                     if (park_smem) {                                 // slots that this split did not walk contribute nothing
                         for (int sl = i == 0 ? 0 : first_slot; sl <= (i == 0 ? last_slot : G); ++sl)
                             if (sl != skip_slot)
                                 slot_out[sl] = (sl < first_slot || sl > last_slot) ? kNegInf : sl == shared_slot ? shared_log() : park_row[sl * 128];
-                    } else {
-                        if (i == 0 && shared_slot >= 0) slot_out[shared_slot] = shared_log();
-                        if (range_out) *(i == 0 ? &range_out->x : &range_out->y) = i == 0 ? first_slot : last_slot;
+                    } else if (i == 0 && shared_slot >= 0) {
+                        slot_out[shared_slot] = shared_log();
                     }
                 }
             } else if (p.mass) {
                 if (park_smem) {
                     finish_masses(row_lse, other_bnd, first_slot, last_slot);
-                } else if (row_valid && i == 0) {
+                } else if (my_ridx >= 0 && i == 0) {
                     p.lse_out[rh] = row_lse;
                     if (shared_slot >= 0) slot_out[shared_slot] = shared_log();
                 }
@@ -742,7 +746,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                 // ---- the whole key stream was this CTA's: output and masses ----
                 if (p.mass) {
                     if (park_smem) finish_masses(lse, kNegInf, 0, G);
-                    else if (row_valid) p.lse_out[rh] = lse;
+                    else if (my_ridx >= 0) p.lse_out[rh] = lse;
                 }
                 if (n_steps > 0) {
                     const float inv = (l > 0.f) ? 1.f / l : 0.f;
@@ -765,13 +769,11 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                 }
             } else if (split_mode) {
                 // ---- partial results for the merge kernel: O / l in fp32, the row's log-sum-exp, raw slot log-sums ----
-                if (row_valid) p.part_lse[rh] = lse;
+                if (my_ridx >= 0) p.part_lse[rh] = lse;
                 if (slot_out) {
                     if (park_smem)                                   // slots that this split did not walk contribute nothing
                         for (int sl = 0; sl <= G; ++sl)
                             slot_out[sl] = (sl < first_slot || sl > last_slot) ? kNegInf : park_row[sl * 128];
-                    else if (range_out)
-                        *range_out = make_int2(first_slot, last_slot);
                 }
                 if (n_steps > 0) {
                     const float inv = (l > 0.f) ? 1.f / l : 0.f;
@@ -838,7 +840,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
                 if (ok && p.mass) {
                     if (park_smem) {
                         finish_masses(row_lse, other_bnd, first_slot, last_slot);
-                    } else if (row_valid && it.split == 0) {
+                    } else if (my_ridx >= 0 && it.split == 0) {
                         p.lse_out[rh] = row_lse;
                         if (shared_slot >= 0) slot_out[shared_slot] = shared_log();      // the slot parked last: its own part is still in acc
                     }
