@@ -33,12 +33,12 @@ import torch
 
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 
-# dram__bytes_read.sum + dram__bytes_write.sum per attention launch from the ncu capture summarised in
-# profiles/ (same kernel, same workload shape); None until a capture exists for the workload.
+# dram__bytes_read.sum + dram__bytes_write.sum per attention launch from an ncu capture of the same kernel and workload shape;
+# None until a capture exists for the workload.
 NCU_TRAFFIC_BYTES = {
-    "planner": 15.42e6 + 0.0,         # attn_kernel<128> incl. the in-kernel split merge, profiles/attn_kernel_planner.md
-    "long": 44.84e6 + 1.59e6,         # attn_kernel<128>, one launch, profiles/attn_kernel_planner.md
-    "decode": 140.64e6 + 3.75e6,      # decode_kernel<128>, profiles/decode_kernel_decode.md
+    "planner": 15.41e6 + 0.0,         # attn_kernel<128> incl. the in-kernel split merge
+    "long": 45.14e6 + 2.06e6,         # attn_kernel<128>, one launch
+    "decode": 140.64e6 + 3.75e6,      # decode_kernel<128>
 }
 
 

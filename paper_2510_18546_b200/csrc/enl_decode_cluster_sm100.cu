@@ -15,7 +15,7 @@
 // asks for its first page before anything else, and prefetches are dealt to the warps (start to wait 2.7 -> 1.8 us).
 // Measured per launch in a chain of 20 layers (32 q / 8 kv heads, 24 groups; streaming kernel, this one with cluster barriers, now):
 // D 128 with masses, 640 keys 9.2, 6.0, 5.4 us, 2560 keys 10.2, 8.3, 6.9; without, 640 keys 5.0, 4.6, 2560 keys 6.7, 5.9; D 64 with
-// masses, 640 keys 8.6, 5.6, 4.7, 2560 keys 9.1, 7.3, 5.7; contiguous keys (the entry point that allocates nothing), 2500 keys 91, 10.2, 9.0.
+// masses, 640 keys 8.6, 5.6, 4.7, 2560 keys 9.1, 7.3, 5.7; contiguous keys (the entry point that allocates nothing), 2500 keys 91, 10.2, 8.9.
 //
 // Per page, all in registers of one warp:
 //   S^T = K Q^T        mma.sync m16n8k16, A = the 16 keys (ldmatrix), B = the rep query rows padded to 8

@@ -835,7 +835,8 @@ extern "C" int enl_attend(enl_cache_t *c, const enl_attend_args_t *a, void *cuda
             //                                                        6.8 + 0.9 w + 1.2 m + (0.245 + 0.04 m) splits rh
             // (beyond eight splits the merge kernel needs a second round trip, 0.4; two steps in all are 0.8 less).  Fitted to 948 measurements: 17 to 512 rows over 640 to 5120
             // keys, 32 / 8 heads, 24 groups, both head_dims, 1 to 16 splits; the choice takes 1.01 of the best one's time in the mean, 1.11 at
-            // worst.  The best with a Q tile each against the best in halves, head_dim 128, masses: 17 rows over 640 keys 11.2 / 11.2, over
+            // worst.  (Elsewhere only its outcome has been compared: 708 calls of 4 / 1 to 64 / 8 heads, up to 16 episodes, 400 groups and 60 splits against
+            // the code before the form in halves existed: 0.81 of the time in the geometric mean, 1.04 at worst.)  The best with a Q tile each against the best in halves, head_dim 128, masses: 17 rows over 640 keys 11.2 / 11.2, over
             // 5120 15.6 / 14.9; 41 rows 14.3 / 12.6, 20.7 / 17.9; 128 rows 16.2 / 14.6, 27.0 / 24.4; 256 rows 17.9 / 16.2, 37.0 / 36.2; 512 rows
             // 21.2 / 19.4, 51.3 / 55.7; head_dim 64: 41 rows 12.4 / 11.5, 18.6 / 16.8; 128 rows 16.5 / 13.6, 23.6 / 23.0; 512 rows 26.4 / 18.4,
             // 55.7 / 54.6.
